@@ -8,6 +8,7 @@
 #include <mutex>
 
 #include "sd_kernels.cuh"
+#include "sd_sweep.cuh"
 #include "sd_greedy.cuh"
 #include "sd_errpos.cuh"
 #include "sd_lmhead.cuh"
@@ -75,8 +76,10 @@ int elem_bytes(int dtype) { return dtype == SD_DTYPE_F32 ? 4 : 2; }
 int vec_elems(int dtype) { return 16 / elem_bytes(dtype); }
 
 struct WorkspaceLayout {
-    size_t ticket, wstatus, sticky, accept, rowc, region_sums, hint_part, total;
+    size_t ticket, wstatus, sticky, arrived, accept, rowc, region_sums, part, hint_part, total;
     int NRmax;   // room for region sums per row: enough for either path at any cluster size
+    int slices;  // items per row of the two sweeps (0: the layout has no room for them)
+    int hint_stride;
 };
 
 bool shape_ok(int B, int k, int V) {
@@ -85,22 +88,45 @@ bool shape_ok(int B, int k, int V) {
     return n < 4.0e18L && (long double)B * (k + 1) < 2.0e9L;
 }
 
-WorkspaceLayout workspace_layout(int B, int k, int V, int dtype, bool with_hint = false) {
+// Sampling regions per item of the two sweeps: four per warp where that leaves enough items for every SM
+// (nominally 888 blocks at a time), down to one per warp for the smallest calls, and so many that a row
+// never falls into more than kMaxSlices items.  Measured on 288 rows of 128 256 bf16 entries: three per
+// warp 63.4 us, four 61.6 us, five 63.7 us (more items cost more prologues and merges, fewer leave the last
+// wave of blocks emptier).
+int sweep_regions(long long units, int V, int dtype) {
+    const int fast_elems = kRegionVecs * vec_elems(dtype);
+    const long long R = ((long long)V + fast_elems - 1) / fast_elems;
+    long long ri = (units * R / 888 + kSweepWarps - 1) / kSweepWarps * kSweepWarps;
+    if (ri < kSweepWarps) ri = kSweepWarps;
+    if (ri > 4 * kSweepWarps) ri = 4 * kSweepWarps;
+    long long s = (R + ri - 1) / ri;
+    if (s > kMaxSlices) s = kMaxSlices;
+    return (int)((R + s - 1) / s);
+}
+
+// sweeps = false: the layout without room for the two sweeps (what a buffer of that size is still good for).
+WorkspaceLayout workspace_layout(int B, int k, int V, int dtype, bool with_hint = false, bool sweeps = true) {
     WorkspaceLayout L;
     // room for region sums per row: enough for either path (the fast path's regions are 64 vectors,
     // 256 fp32 or 512 bf16 entries; the generic path's 512 entries)
     const int fast_elems = kRegionVecs * vec_elems(dtype);
     const int per = fast_elems < kGenericRegionElems ? fast_elems : kGenericRegionElems;
+    const size_t units = (size_t)B * (k + 1);
     L.NRmax = (V + per - 1) / per;
+    const int ri = sweep_regions((long long)units, V, dtype), R = (V + fast_elems - 1) / fast_elems;
+    L.slices = sweeps ? (R + ri - 1) / ri : 0;
+    L.hint_stride = L.slices > kMaxCluster ? L.slices : kMaxCluster;
     size_t off = 0;
     L.ticket = off;      off = align_up(off + (size_t)B * 4, kAlign);
     L.wstatus = off;     off = align_up(off + (size_t)B * 4, kAlign);
     L.sticky = off;      off = align_up(off + 4, kAlign);
+    L.arrived = off;     off = align_up(off + (sweeps ? units * 4 : 0), kAlign);
     L.accept = off;      off = align_up(off + (size_t)B * k, kAlign);
-    L.rowc = off;        off = align_up(off + (size_t)B * (k + 1) * sizeof(RowConst), kAlign);
-    L.region_sums = off; off = align_up(off + (size_t)B * (k + 1) * L.NRmax * 4, kAlign);
+    L.rowc = off;        off = align_up(off + units * sizeof(RowConst), kAlign);
+    L.region_sums = off; off = align_up(off + units * L.NRmax * 4, kAlign);
+    L.part = off;        off = align_up(off + units * L.slices * sizeof(PartialStats), kAlign);
     L.hint_part = off;
-    if (with_hint) off = align_up(off + (size_t)B * (k + 1) * kMaxCluster * 8, kAlign);
+    if (with_hint) off = align_up(off + units * L.hint_stride * 8, kAlign);
     L.total = off;
     return L;
 }
@@ -219,6 +245,68 @@ int launch_stream(DeviceState& d, const Params& P, int C, int G, int lag, cudaSt
     SD_CUDA(cudaLaunchKernelEx(&cfg, kern, P, lag, prefetch));
     tl_info[0] = 1; tl_info[1] = C; tl_info[2] = kStreamThreads; tl_info[3] = stream_smem<DT>();
     tl_info[4] = G * C; tl_info[5] = 1;
+    return SD_OK;
+}
+
+// Does a call that reads `bytes` of logits take the two sweeps (else the cluster kernel)?  The sweeps read
+// them twice, and what is beyond L2 from HBM both times.  For bf16 that is the better bargain at every size
+// measured, because the cluster kernel is held up by its exponentials; for fp32, half as many to the byte,
+// up to about 450 MB.  Cluster kernel / sweeps in us (step, 128 256 entries):
+//     bf16  16x5 rows (37 MB) 43.0 / 28.1,  64x9 124 / 117,  128x7 191 / 172,  256x7 340 / 333
+//     fp32  8x5 (37 MB) 32.7 / 24.5,  32x7 (214 MB) 96.4 / 80.1,  64x7 (427 MB) 165 / 158,  96x7 (640 MB) 206 / 234
+// At the small end the two launches more cost the calling thread 5 us, which a caller that issues rounds
+// back to back pays instead of the GPU (one sequence: 24 us a call with one launch, 29 us with three).
+// The ensemble stays with the cluster kernel, whose units share a target row: 3 learners on 32 sequences,
+// 8 tokens, bf16 151 / 151; on 16 sequences, 4 tokens, fp32 67.7 / 72.3.
+// Options that only the cluster kernel has, off their defaults, choose the cluster kernel.
+bool use_sweeps(int dtype, double bytes) {
+    if (option(SD_OPT_CLUSTER) != 0 || option(SD_OPT_LAG) != -1 || option(SD_OPT_PREFETCH) != 0 ||
+        option(SD_OPT_L2_BUDGET_MIB) != kL2BudgetMiB || option(SD_OPT_WAIT_POLLS) != (long long)kWaitLimit)
+        return false;
+    return dtype == SD_DTYPE_BF16 ? bytes >= 32e6 : bytes >= 48e6 && bytes <= 450e6;
+}
+
+// Launch of a kernel whose blocks come as those of the kernel before it on the stream go.
+template <class K, class... A>
+cudaError_t launch_following(K kern, dim3 grid, int threads, cudaStream_t stream, const A&... args) {
+    cudaLaunchConfig_t cfg;
+    memset(&cfg, 0, sizeof cfg);
+    cfg.gridDim = grid;
+    cfg.blockDim = dim3((unsigned)threads, 1, 1);
+    cfg.stream = stream;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, kern, args...);
+}
+
+template <int DT, int MODE>
+int launch_sweeps_of(const Params& P, const Sweep& S, long long units, cudaStream_t stream) {
+    sd_sweep_stats_kernel<DT><<<dim3((unsigned)units, (unsigned)S.slices), kSweepThreads, 0, stream>>>(P, S);
+    SD_CUDA(cudaGetLastError());
+    SD_CUDA(launch_following(sd_sweep_rows_kernel<DT>, dim3((unsigned)P.B), kSweepThreads, stream, P, S));
+    // the rows that are drawn from, then (if anything of them is wanted) all rows
+    const bool all = MODE != kSweepErrors && (P.grad || MODE == kSweepHint || S.all_rows);
+    const unsigned second = (unsigned)S.draw_blocks + (all ? (unsigned)(units * S.slices) : 0u);
+    SD_CUDA(launch_following(sd_sweep_grad_kernel<DT, MODE>, dim3(second), kSweepThreads, stream, P, S));
+    return SD_OK;
+}
+
+template <int MODE>
+int launch_sweeps(const Params& P, Sweep& S, long long units, int dtype, cudaStream_t stream) {
+    S.regions = (P.NR + S.slices - 1) / S.slices;
+    // What the first sweep reads last stays in L2 for the second, which starts there: 80 MiB of 126 (measured
+    // on 288 rows of 128 256 bf16 entries: 0 MiB 70.5 us, 48 69.7, 64 69.1, 80 68.4, 96 68.8, before the draws
+    // went first).
+    S.kept = (80u << 20) / (unsigned)(S.regions * kRegionVecs * 32);
+    S.draw_blocks = P.B * S.slices;
+    const int rc = dtype == SD_DTYPE_F32 ? launch_sweeps_of<SD_DTYPE_F32, MODE>(P, S, units, stream)
+                                         : launch_sweeps_of<SD_DTYPE_BF16, MODE>(P, S, units, stream);
+    if (rc != SD_OK) return rc;
+    tl_info[0] = 1; tl_info[1] = 1; tl_info[2] = kSweepThreads; tl_info[3] = 0;
+    tl_info[4] = (int)(units * S.slices); tl_info[5] = 3;
     return SD_OK;
 }
 
@@ -346,18 +434,34 @@ int run_device(DeviceState& d, const void* T, const void* D, const int32_t* x, c
     P.hint = hint;
     P.hint_err = hint_err;
     P.hint_part = hint ? reinterpret_cast<double*>(ws + L.hint_part) : nullptr;
+    P.hint_stride = L.hint_stride;
 
-    if (!clean) SD_CUDA(cudaMemsetAsync(ws, 0, L.accept, stream));   // tickets, status words, sticky flag
-    if (status) SD_CUDA(cudaMemsetAsync(status, 0, (size_t)B * 4, stream));   // bits are ORed in on the device
+    if (!clean) SD_CUDA(cudaMemsetAsync(ws, 0, L.accept, stream));   // tickets, status words, sticky flag, counters
 
     const size_t row_bytes = (size_t)V * elem_bytes(dtype);
     const bool fast = (row_bytes % 16 == 0) && aligned(T, 16) && aligned(D, 16) && (!grad || aligned(grad, 16)) &&
                       (!hint || aligned(hint, 16)) && option(SD_OPT_FORCE_GENERIC) == 0;
+    const long long units = (long long)B * (k + 1);
+    if (fast && L.slices > 0 && use_sweeps(dtype, (double)B * (2 * k + 1) * (double)row_bytes)) {
+        // (the status words are cleared by the first sweep)
+        Sweep S;
+        S.slices = L.slices;
+        S.part = reinterpret_cast<PartialStats*>(ws + L.part);
+        S.arrived = reinterpret_cast<uint32_t*>(ws + L.arrived);
+        S.all_rows = acc_prob != nullptr;
+        P.blocks_per_unit = L.slices;
+        P.RE = kRegionVecs * vec_elems(dtype);
+        P.NR = (V + P.RE - 1) / P.RE;
+        return hint ? launch_sweeps<kSweepHint>(P, S, units, dtype, stream)
+                    : launch_sweeps<kSweepStepMode>(P, S, units, dtype, stream);
+    }
+    if (status) SD_CUDA(cudaMemsetAsync(status, 0, (size_t)B * 4, stream));   // bits are ORed in on the device
     int C = 0, G = 0, lag = 0, per = 0;
-    if (fast) C = choose_stream(d, V, (long long)B * (k + 1), dtype, &G, &per, &lag);
+    if (fast) C = choose_stream(d, V, units, dtype, &G, &per, &lag);
     int rc;
     if (C > 0) {
         P.blocks_per_unit = C;
+        P.tickets = (uint32_t)C * (uint32_t)(k + 1);
         P.RE = per * vec_elems(dtype);
         P.NR = (V + P.RE - 1) / P.RE;
         if (hint)
@@ -368,12 +472,39 @@ int run_device(DeviceState& d, const void* T, const void* D, const int32_t* x, c
                                        : launch_stream<SD_DTYPE_BF16>(d, P, C, G, lag, stream, false, nullptr);
     } else {
         P.blocks_per_unit = 1;
+        P.tickets = (uint32_t)(k + 1);
         P.RE = kGenericRegionElems;
         P.NR = (V + P.RE - 1) / P.RE;
         rc = dtype == SD_DTYPE_F32 ? launch_generic<SD_DTYPE_F32>(P, stream)
                                    : launch_generic<SD_DTYPE_BF16>(P, stream);
     }
     return rc;
+}
+
+// Is work on `stream` being captured?  (Nothing may be allocated then.)
+bool capturing(cudaStream_t stream) {
+    cudaStreamCaptureStatus st = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(stream, &st) != cudaSuccess) {
+        (void)cudaGetLastError();
+        return false;
+    }
+    return st != cudaStreamCaptureStatusNone;
+}
+
+// The library's own scratch, at least `need` bytes of it (grown on demand).
+int own_scratch(DeviceState* d, size_t need) {
+    if (d->ws_bytes >= need) return SD_OK;
+    if (d->ws) {
+        SD_CUDA(cudaDeviceSynchronize());
+        SD_CUDA(cudaFree(d->ws));
+        d->ws = nullptr;
+        d->ws_bytes = 0;
+    }
+    const size_t want = align_up(need + need / 4, 1 << 20);
+    SD_CUDA(cudaMalloc(&d->ws, want));
+    d->ws_bytes = want;
+    d->ws_zero_bytes = 0;
+    return SD_OK;
 }
 
 int run_cached(const void* T, const void* D, const int32_t* x, const float* u, float tau, int B, int k, int V,
@@ -384,20 +515,12 @@ int run_cached(const void* T, const void* D, const int32_t* x, const float* u, f
     DeviceState* d = nullptr;
     rc = current_device(&dev, &d);
     if (rc != SD_OK) return rc;
-    const WorkspaceLayout L = workspace_layout(B, k, V, dtype);
+    WorkspaceLayout L = workspace_layout(B, k, V, dtype);
     std::lock_guard<std::mutex> lock(d->mu);
-    if (d->ws_bytes < L.total) {
-        if (d->ws) {
-            SD_CUDA(cudaDeviceSynchronize());
-            SD_CUDA(cudaFree(d->ws));
-            d->ws = nullptr;
-            d->ws_bytes = 0;
-        }
-        const size_t want = align_up(L.total + L.total / 4, 1 << 20);
-        SD_CUDA(cudaMalloc(&d->ws, want));
-        d->ws_bytes = want;
-        d->ws_zero_bytes = 0;
-    }
+    if (d->ws_bytes < L.total && capturing(static_cast<cudaStream_t>(stream)))
+        L = workspace_layout(B, k, V, dtype, false, false);   // what there is may do for the cluster kernel
+    rc = own_scratch(d, L.total);
+    if (rc != SD_OK) return rc;
     // the head of this layout (tickets, status words, error flag) must be zero on entry; the kernel
     // leaves it zero again and dirties everything behind it
     const bool clean = d->ws_zero_bytes >= L.accept;
@@ -510,7 +633,8 @@ int sd_verify_feedback_ex(const void* target_logits, const void* draft_logits, c
     int rc = check_args(target_logits, draft_logits, draft_tokens, uniforms, temperature, B, k, V, dtype,
                         out_accept_len, out_tokens, out_loss, out_grad_draft, out_acc_prob, out_status);
     if (rc != SD_OK) return rc;
-    const WorkspaceLayout L = workspace_layout(B, k, V, dtype);
+    WorkspaceLayout L = workspace_layout(B, k, V, dtype);
+    if (workspace_bytes < L.total) L = workspace_layout(B, k, V, dtype, false, false);
     if (!workspace || !aligned(workspace, kAlign) || workspace_bytes < L.total) return SD_ERR_WORKSPACE;
     int dev;
     DeviceState* d = nullptr;
@@ -537,7 +661,8 @@ int sd_verify_feedback_hint(const void* target_logits, const void* draft_logits,
     if (rc != SD_OK) return rc;
     if (!hint || !out_hint_err) return SD_ERR_NULL;
     if (!aligned(hint, (size_t)elem_bytes(dtype)) || !aligned(out_hint_err, 4)) return SD_ERR_ALIGN;
-    const WorkspaceLayout L = workspace_layout(B, k, V, dtype, true);
+    WorkspaceLayout L = workspace_layout(B, k, V, dtype, true);
+    if (workspace_bytes < L.total) L = workspace_layout(B, k, V, dtype, true, false);
     if (!workspace || !aligned(workspace, kAlign) || workspace_bytes < L.total) return SD_ERR_WORKSPACE;
     int dev;
     DeviceState* d = nullptr;
@@ -557,7 +682,8 @@ int sd_verify_feedback_static(const void* target_logits, const void* draft_logit
     int rc = check_args(target_logits, draft_logits, draft_tokens, uniforms, temperature, B, k, V, dtype,
                         out_accept_len, out_tokens, out_loss, out_grad_draft, out_acc_prob, out_status);
     if (rc != SD_OK) return rc;
-    const WorkspaceLayout L = workspace_layout(B, k, V, dtype);
+    WorkspaceLayout L = workspace_layout(B, k, V, dtype);
+    if (L.total > (size_t)SD_STATIC_SCRATCH_BYTES) L = workspace_layout(B, k, V, dtype, false, false);
     if (L.total > (size_t)SD_STATIC_SCRATCH_BYTES) {
         snprintf(tl_cuda_error, sizeof tl_cuda_error,
                  "this shape needs %zu bytes of scratch, the built-in scratch has %d: use sd_verify_feedback_ex",
@@ -610,12 +736,8 @@ int sd_ensemble_feedback(const void* target_logits, const void* const* draft_log
     cudaStream_t st = static_cast<cudaStream_t>(stream);
     unsigned char* ws = static_cast<unsigned char*>(workspace);
     if (!ws) {
-        if (!d->ws) {
-            const size_t want = 1 << 20;
-            SD_CUDA(cudaMalloc(&d->ws, want));
-            d->ws_bytes = want;
-            d->ws_zero_bytes = 0;
-        }
+        rc = own_scratch(d, SD_ENSEMBLE_SCRATCH_BYTES);
+        if (rc != SD_OK) return rc;
         ws = static_cast<unsigned char*>(d->ws);
         d->ws_zero_bytes = 0;      // the flag word of this call sits where other entry points expect zeros
     }
@@ -666,7 +788,8 @@ int sd_verify_error_feedback(const void* target_logits, const void* draft_logits
     if (row_bytes % 16 != 0 || !aligned(target_logits, 16) || !aligned(draft_logits, 16) ||
         (out_error_grad && !aligned(out_error_grad, 16)))
         return SD_ERR_ALIGN;
-    const WorkspaceLayout L = workspace_layout(B, k, V, dtype);
+    WorkspaceLayout L = workspace_layout(B, k, V, dtype);
+    if (workspace && workspace_bytes < L.total) L = workspace_layout(B, k, V, dtype, false, false);
     if (workspace && (!aligned(workspace, kAlign) || workspace_bytes < L.total)) return SD_ERR_WORKSPACE;
     int dev;
     DeviceState* d = nullptr;
@@ -675,21 +798,15 @@ int sd_verify_error_feedback(const void* target_logits, const void* draft_logits
     std::lock_guard<std::mutex> lock(d->mu);
     cudaStream_t st = static_cast<cudaStream_t>(stream);
     unsigned char* ws = static_cast<unsigned char*>(workspace);
+    bool clean = false;
     if (!ws) {
         // the library's own scratch, shared with the other entry points and grown on demand
-        if (d->ws_bytes < L.total) {
-            if (d->ws) {
-                SD_CUDA(cudaDeviceSynchronize());
-                SD_CUDA(cudaFree(d->ws));
-                d->ws = nullptr;
-                d->ws_bytes = 0;
-            }
-            const size_t want = align_up(L.total + L.total / 4, 1 << 20);
-            SD_CUDA(cudaMalloc(&d->ws, want));
-            d->ws_bytes = want;
-        }
+        if (d->ws_bytes < L.total && capturing(st)) L = workspace_layout(B, k, V, dtype, false, false);
+        rc = own_scratch(d, L.total);
+        if (rc != SD_OK) return rc;
         ws = static_cast<unsigned char*>(d->ws);
-        d->ws_zero_bytes = 0;     // cleared below for this call; what it leaves behind is not tracked
+        clean = d->ws_zero_bytes >= L.accept;
+        d->ws_zero_bytes = 0;
     }
     Params P;
     memset(&P, 0, sizeof P);
@@ -707,14 +824,29 @@ int sd_verify_error_feedback(const void* target_logits, const void* draft_logits
     P.rowc = reinterpret_cast<RowConst*>(ws + L.rowc);
     P.region_sums = reinterpret_cast<float*>(ws + L.region_sums);
     P.wait_polls = wait_polls();
-    SD_CUDA(cudaMemsetAsync(ws, 0, L.accept, st));   // tickets, status words, sticky flag
+    if (!clean) SD_CUDA(cudaMemsetAsync(ws, 0, L.accept, st));   // tickets, status words, sticky flag, counters
+    const long long units = (long long)B * (k + 1);
+    P.RE = kRegionVecs * vec_elems(dtype);
+    P.NR = (V + P.RE - 1) / P.RE;
+    // (the rule of the full step, so that both give the same bits)
+    if (L.slices > 0 && use_sweeps(dtype, (double)B * (2 * k + 1) * (double)row_bytes)) {
+        Sweep S;
+        S.slices = L.slices;
+        S.part = reinterpret_cast<PartialStats*>(ws + L.part);
+        S.arrived = reinterpret_cast<uint32_t*>(ws + L.arrived);
+        S.all_rows = 0;
+        P.blocks_per_unit = L.slices;
+        rc = launch_sweeps<kSweepErrors>(P, S, units, dtype, st);
+        if (rc != SD_OK) return rc;
+        if (!workspace) d->ws_zero_bytes = L.accept;
+        tl_info[0] = 4;
+        return SD_OK;
+    }
     if (out_status) SD_CUDA(cudaMemsetAsync(out_status, 0, (size_t)B * 4, st));   // bits are ORed in on the device
     int G = 0, lag = 0, per = 0;
-    const int C = choose_stream(*d, V, (long long)B * (k + 1), dtype, &G, &per, &lag);
+    const int C = choose_stream(*d, V, units, dtype, &G, &per, &lag);
     if (C <= 0) return SD_ERR_CUDA;
     P.blocks_per_unit = C;
-    P.RE = per * vec_elems(dtype);
-    P.NR = (V + P.RE - 1) / P.RE;
     rc = dtype == SD_DTYPE_F32 ? launch_stream<SD_DTYPE_F32, false, true>(*d, P, C, G, lag, st, false, nullptr)
                                : launch_stream<SD_DTYPE_BF16, false, true>(*d, P, C, G, lag, st, false, nullptr);
     if (rc != SD_OK) return rc;

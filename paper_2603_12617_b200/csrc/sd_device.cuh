@@ -103,12 +103,14 @@ struct Params {
     uint8_t* accept;         // [B*k]
     RowConst* rowc;          // [B*(k+1)]
     float* region_sums;      // [B*(k+1)*NR] mass of each sampling region of each row
-    int blocks_per_unit;     // blocks that take a ticket per (sequence, row)
+    int blocks_per_unit;     // blocks that work on a (sequence, row)
+    uint32_t tickets;        // tickets of a sequence: whoever takes the last one draws its token
     uint32_t wait_polls;     // polls after which a bounded wait gives up (kWaitLimit unless a caller asks otherwise)
     // hint error of the optimistic update (null: not asked for)
     const void* hint;        // [B,k,V] the last round's gradient, in the dtype of the logits
     float* hint_err;         // [B,k] sum_v (hint - this round's gradient)^2
-    double* hint_part;       // workspace [B*(k+1)][kMaxCluster]: each block's share of a row's sum
+    double* hint_part;       // workspace [B*(k+1)][hint_stride]: each block's share of a row's sum
+    int hint_stride;
     // online ensemble: feedback of `learners` draft models against one target (0: the plain step).
     // Then loss is [learners,B,k], D and grad above are unused, and nothing is verified or drawn.
     int learners;
@@ -652,8 +654,10 @@ __device__ int draw_row_slow(const Params& P, const RowConst& rc, int mode, size
 
 // FAST: the regions are those of the fast path (kRegionVecs vectors, rows of whole vectors);
 // otherwise those of the generic path (kGenericRegionElems entries, any alignment).
-template <int DT, bool FAST>
-__device__ __noinline__ void resolve_sequence(const Params& P, int b) {
+// KNOWN: the accept length and the constants of its row are the caller's (and the sums over whole rows for
+// hint error and acceptance probability somebody else's business).
+template <int DT, bool FAST, bool KNOWN = false>
+__device__ __noinline__ void resolve_sequence(const Params& P, int b, int known_n = 0, RowConst known_rc = RowConst{}) {
     constexpr int PER = FAST ? kRegionVecs * Elem<DT>::VEC / 32 : kGenericRegionElems / 32;
     const int lane = threadIdx.x & 31;
     const int k = P.k, NR = P.NR;
@@ -670,8 +674,8 @@ __device__ __noinline__ void resolve_sequence(const Params& P, int b) {
     }
 
     // accept length: first rejected position
-    int n = k;
-    for (int i0 = 0; i0 < k; i0 += 32) {
+    int n = KNOWN ? known_n : k;
+    for (int i0 = 0; !KNOWN && i0 < k; i0 += 32) {
         const int i = i0 + lane;
         const bool rej = (i < k) && (__ldcg(P.accept + b * k + i) == 0);
         const unsigned m = __ballot_sync(0xffffffffu, rej);
@@ -680,9 +684,9 @@ __device__ __noinline__ void resolve_sequence(const Params& P, int b) {
     uint32_t flags = 0;
 
     // hint error per position: the shares of the blocks that worked on the row, in their order
-    if (P.hint_err) {
+    if (!KNOWN && P.hint_err) {
         for (int i = lane; i < k; i += 32) {
-            const double* hp = P.hint_part + (size_t)(b * (k + 1) + i) * kMaxCluster;
+            const double* hp = P.hint_part + (size_t)(b * (k + 1) + i) * P.hint_stride;
             double e = 0.0;
             for (int r = 0; r < P.blocks_per_unit; ++r) e += __ldcg(hp + r);
             P.hint_err[b * k + i] = (float)e;
@@ -690,7 +694,7 @@ __device__ __noinline__ void resolve_sequence(const Params& P, int b) {
     }
 
     // diagnostic: acceptance probability 1 - sum max(0,p-q) per position (Eq. 1)
-    if (P.acc_prob) {
+    if (!KNOWN && P.acc_prob) {
         for (int i = 0; i < k; ++i) {
             const float* rsi = P.region_sums + (size_t)(b * (k + 1) + i) * NR;
             double part = 0.0;
@@ -710,8 +714,11 @@ __device__ __noinline__ void resolve_sequence(const Params& P, int b) {
     const int unit = b * (k + 1) + n;
     if (!SD_IN(unit, P.B * (k + 1), 23) || !SD_IN(n, k + 1, 23)) return;
     const float* rs = P.region_sums + (size_t)unit * NR;
-    const float4 rcv = __ldcg(reinterpret_cast<const float4*>(P.rowc + unit));
-    const RowConst rc{rcv.x, rcv.y, rcv.z, rcv.w};
+    RowConst rc = known_rc;
+    if constexpr (!KNOWN) {
+        const float4 rcv = __ldcg(reinterpret_cast<const float4*>(P.rowc + unit));
+        rc = RowConst{rcv.x, rcv.y, rcv.z, rcv.w};
+    }
     const size_t offT = (size_t)unit * P.V;
     const size_t offD = (size_t)(b * k + (bonus ? 0 : n)) * P.V;
     const double uk = (double)uk_f;
@@ -818,14 +825,12 @@ __device__ __noinline__ void resolve_sequence(const Params& P, int b) {
     }
 }
 
-// Tickets of one block for sequence b: `n` of the (k+1) * blocks_per_unit tickets of the
-// sequence at once, by one thread, after everything the tickets stand for has been ordered before
+// Tickets of one block for sequence b: `n` of the sequence's tickets at once, by one thread, after everything the tickets stand for has been ordered before
 // this thread.  True if these were the last tickets of the sequence.
 __device__ __forceinline__ bool take_tickets(const Params& P, int b, uint32_t n) {
     __threadfence();
-    const uint32_t total = (uint32_t)(P.k + 1) * (uint32_t)P.blocks_per_unit;
     const uint32_t old = atomicAdd(P.ticket + b, n);
-    const bool last = (old + n == total);
+    const bool last = (old + n == P.tickets);
     if (last) __threadfence();
     return last;
 }

@@ -388,8 +388,9 @@ __device__ __forceinline__ void pass1_region(const uint4* st, int nv, int lane, 
 // Pass 2 of a region held in registers: gradient out (gdst = where the region's part of the
 // gradient row starts, or null) and the region's mass (sum of max(0,p-q)/tau, or of p on the
 // bonus row), in every lane.  HINT: hq holds the region of the hint (the last round's gradient), and
-// this lane's sum of squared differences between hint and gradient is added to herr.
-template <int DT, bool BONUS, bool HINT>
+// this lane's sum of squared differences between hint and gradient is added to herr.  MASS = false: the
+// region's mass is not wanted.
+template <int DT, bool BONUS, bool HINT, bool MASS = true>
 __device__ __forceinline__ float pass2_region_impl(const uint4 (&rt)[kRegionRows], const uint4 (&rd)[kRegionRows], int nv,
                                                    int lane, float c, const RowConst& rc, typename Elem<DT>::type* gdst,
                                                    const uint4 (&hq)[kRegionRows], float& herr) {
@@ -410,7 +411,7 @@ __device__ __forceinline__ float pass2_region_impl(const uint4 (&rt)[kRegionRows
                 const float2 g2 = grad_elem2(make_float2(tv[z], tv[z + 1]), make_float2(dv[z], dv[z + 1]), c, rc);
                 gv[z] = g2.x;
                 gv[z + 1] = g2.y;
-                acc = __fadd2_rn(acc, make_float2(fmaxf(-g2.x, 0.f), fmaxf(-g2.y, 0.f)));
+                if constexpr (MASS) acc = __fadd2_rn(acc, make_float2(fmaxf(-g2.x, 0.f), fmaxf(-g2.y, 0.f)));
             }
             if (gdst && vi < nv) store_streaming(gdst + (size_t)vi * VEC, E::pack(gv));
             if constexpr (HINT) {
@@ -432,6 +433,7 @@ __device__ __forceinline__ float pass2_region_impl(const uint4 (&rt)[kRegionRows
             ms[g] = tree_sum<VEC>(r);
         }
     }
+    if constexpr (!MASS) return 0.f;
     float mass = tree_sum<kRegionRows>(ms);
 #pragma unroll
     for (int off = 16; off > 0; off >>= 1) mass += __shfl_xor_sync(0xffffffffu, mass, off);
@@ -641,7 +643,7 @@ sd_stream_kernel(const __grid_constant__ Params P, const int lag_stages, const i
                 // this block's share of the row's hint error: the warps' shares in their order, in fp64
                 double hp = (lane < kConsumerWarps) ? (double)sh.hpart[dslot][lane] : 0.0;
                 hp = warp_sum(hp);
-                if (lane == 0 && !bonus) P.hint_part[(size_t)unit * kMaxCluster + rank] = hp;
+                if (lane == 0 && !bonus) P.hint_part[(size_t)unit * P.hint_stride + rank] = hp;
             }
             ++seg;
             const bool leaves = (i == P.k) || (j == nu - 1);   // last unit of the sequence in this cluster
@@ -1002,7 +1004,7 @@ __global__ void __launch_bounds__(kGenericThreads) sd_generic_kernel(const __gri
     if (tid == 0 && P.hint && !bonus) {
         double e = 0.0;
         for (int w = 0; w < kGenericWarps; ++w) e += (double)sh.hpart[w];
-        P.hint_part[(size_t)unit * kMaxCluster] = e;
+        P.hint_part[(size_t)unit * P.hint_stride] = e;
     }
     if (tid == 0) sh.last = take_tickets(P, b, 1u) ? 1 : 0;
     __syncthreads();

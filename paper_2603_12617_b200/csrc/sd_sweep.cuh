@@ -1,0 +1,333 @@
+// The step as two sweeps over the logits, grids of small independent blocks: no cluster, no ring, nobody
+// waits for anybody.  A unit (sequence, row) is cut into `slices` items of the same number of sampling
+// regions, a block takes one item, a warp every eighth region of it, straight from global memory into
+// registers.  Three kernels, each of which comes in as the one before goes out:
+//
+//   sd_sweep_stats_kernel  softmax sums of every item to the workspace.
+//   sd_sweep_rows_kernel   merges the items of every row in slice order and reports the rows: constants,
+//                          losses, rejection tests.
+//   sd_sweep_grad_kernel   gradient of every pair row; masses of the sampling regions only for the one row
+//                          per sequence that the extra token is drawn from (bonus rows that are not drawn
+//                          from cost nothing).  The block that brings that row's last item draws.
+//
+// The second sweep runs through the items backwards: what the first one read last, and asked L2 to keep,
+// is still there.
+//
+// What bounds it: HBM, the exponentials close behind.  Measured alone, the first sweep's loop reads 5.6 TB/s
+// and the second's reads and writes 6.1 TB/s; their arithmetic (144 and 141 instructions per region and
+// warp, 64 cycles of exponentials per region and SM) hides behind the copies with 48 warps an SM.
+// sd_stream_kernel reads every logit from HBM once, but its 28 consumer warps share one ring and all blocks
+// read at the same time and compute at the same time, so at bf16, where the exponentials take as long as
+// the reads, it moves 2.9 TB/s.  Step on 32 sequences, 8 draft tokens, 128 256 bf16 entries: 71.1 us there,
+// 61.6 us here (first sweep 31, rows 3, second 28); 64 sequences, 4 tokens, 151 936: 93.4 and 74.7 us; one
+// sequence, 4 tokens, 32 000 fp32: 16.5 and 14.5 us.  The rule which of the two a call takes is use_sweeps
+// (host).
+//
+// Tried and dropped, on the first of these: one persistent kernel whose warps take both passes of an item
+// from per-warp rings of bulk copies (82 us: many 1 KiB copies in flight slow each other down) or of
+// cp.async (99: their instructions), from registers in teams of blocks that wait for their row (71), and
+// from a queue that mixes first and second passes so that the second hits L2 (70: an SM has no more
+// instruction slots for both than for one).
+#pragma once
+
+#include "sd_kernels.cuh"
+
+namespace sdv {
+
+constexpr int kSweepWarps = 8;
+constexpr int kSweepThreads = kSweepWarps * 32;
+constexpr int kMaxSlices = 32;                  // items of a row: one warp merges them, one per lane
+constexpr int kSweepStep = kSweepWarps * kRegionVecs;   // vectors from a warp's region to its next
+
+struct Sweep {
+    int slices;              // items per unit (1..kMaxSlices)
+    int regions;             // sampling regions per item (the last item of a unit may have fewer)
+    PartialStats* part;      // workspace [units][slices]
+    uint32_t* arrived;       // workspace [units], zero on entry and zero again on exit
+    unsigned kept;           // items, from the last one backwards, that L2 is asked to keep between the sweeps
+    int all_rows;            // second sweep: masses of every row wanted (acceptance probabilities)
+    int draw_blocks;         // second sweep: its first blocks, those of the rows that are drawn from
+};
+
+// What the second sweep is for.
+enum SweepMode { kSweepStepMode = 0, kSweepErrors = 1, kSweepHint = 2 };
+
+__device__ __forceinline__ uint4 load_l2(const uint4* p, uint64_t policy) {
+    uint4 v;
+    asm volatile("ld.global.L1::no_allocate.L2::cache_hint.v4.u32 {%0,%1,%2,%3}, [%4], %5;"
+                 : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "l"(p), "l"(policy));
+    return v;
+}
+// Programmatic dependent launch: let the next kernel's blocks come as soon as there is room / wait until
+// the kernel before has finished and its writes are visible.
+__device__ __forceinline__ void launch_dependents() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+__device__ __forceinline__ void await_previous_kernel() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+
+// Sums of the lanes of a warp that share the references (RT, RD) into *out, in fp64 and a fixed order.
+// The three sums are folded into one register pair on the way (a lane keeps what its half of the warp is
+// responsible for): 6 exchanges of a double instead of the 15 of warp_sum_lanes.
+__device__ __forceinline__ void warp_post_lanes(const LaneSums& ls, float RT, float RD, int lane, PartialStats* out) {
+    const double T = (double)ls.sT, W = (double)ls.w;
+    double D = (double)ls.sD;
+    const bool hi = (lane & 16) != 0, odd = (lane & 8) != 0;
+    double a = hi ? W : T;
+    a += shfl_xor_f64(hi ? T : W, 16);       // lanes 0-15: T, lanes 16-31: W
+    D += shfl_xor_f64(D, 16);                // both halves: D
+    double v = odd ? D : a;
+    v += shfl_xor_f64(odd ? a : D, 8);       // lanes 0-7: T, 16-23: W, 8-15 and 24-31: D
+#pragma unroll
+    for (int off = 4; off > 0; off >>= 1) v += shfl_xor_f64(v, off);
+    if (lane == 0) { out->RT = RT; out->RD = RD; out->sT = v; }
+    if (lane == 8) out->sD = v;
+    if (lane == 16) out->w = v;
+}
+
+__device__ __forceinline__ PartialStats load_partial_cg(const PartialStats* p) {
+    PartialStats r;
+    const float4 a = __ldcg(reinterpret_cast<const float4*>(p)), b = __ldcg(reinterpret_cast<const float4*>(p) + 1);
+    memcpy(&r, &a, 16);
+    memcpy(reinterpret_cast<char*>(&r) + 16, &b, 16);
+    return r;
+}
+
+// Pass 1 of a warp's regions of an item: gT and gD lead to the first of them, `nvec` vectors of the item lie
+// from there on.  (Fetching the next region while this one is worked on was measured as well: no faster,
+// the other warps of the SM hide the loads.)
+template <int DT, bool BONUS>
+__device__ __forceinline__ void sweep_pass1(const uint4* gT, const uint4* gD, int nvec, int lane, float c, uint64_t policy,
+                                            Pass1State& s) {
+    constexpr float kTooLarge = 1.152921504606846976e18f;   // 2^60
+    bool first = true;
+    for (; nvec >= kRegionVecs; gT += kSweepStep, gD += kSweepStep, nvec -= kSweepStep, first = false) {
+        uint4 rt[kRegionRows], rd[kRegionRows];
+#pragma unroll
+        for (int g = 0; g < kRegionRows; ++g) {
+            rt[g] = load_l2(gT + g * 32 + lane, policy);
+            if (!BONUS) rd[g] = load_l2(gD + g * 32 + lane, policy);
+        }
+        if (first) raise_references<DT, BONUS>(rt, rd, c, s);
+        float sT, sD, sW;
+        region_sums_of<DT, BONUS, false>(rt, rd, c, s.RT, s.RD, sT, sD, sW);
+        // masked target entries (NaN) or entries far above the references: maxima first, then the sums
+        if (__any_sync(0xffffffffu, !(sT < kTooLarge) || !(sD < kTooLarge) || sW != sW)) {
+            s = pass1_region_again<DT, BONUS>(gT, gD, kRegionVecs, lane, c, s);
+            continue;
+        }
+        s.ls.sT += sT;
+        s.ls.sD += sD;
+        s.ls.w += sW;
+    }
+    if (nvec > 0) s = pass1_region_again<DT, BONUS>(gT, gD, nvec, lane, c, s);   // cut short by the end of the row
+}
+
+// One block per item: blockIdx.x = unit, blockIdx.y = slice.
+template <int DT>
+__global__ void __launch_bounds__(kSweepThreads, 6)
+sd_sweep_stats_kernel(const __grid_constant__ Params P, const __grid_constant__ Sweep S) {
+    using E = Elem<DT>;
+    using ET = typename E::type;
+    __shared__ PartialStats wpart[kSweepWarps];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    launch_dependents();
+    const int unit = blockIdx.x, slice = blockIdx.y;
+    const UnitRef ur = unit_ref<false>(P, unit);
+    const int v0 = slice * S.regions * kRegionVecs + warp * kRegionVecs;
+    int nvec = min((slice + 1) * S.regions * kRegionVecs, P.V / E::VEC) - v0;
+    if (nvec > 0 && !SD_IN((long long)(v0 + nvec) * E::VEC - 1, P.V, 10)) nvec = 0;
+    if (!SD_IN(ur.t_row, (long long)P.B * (P.k + 1), 10) ||
+        !SD_IN(ur.d_row, (long long)P.B * P.k, 11)) nvec = 0;
+    const uint4* const gT = reinterpret_cast<const uint4*>(reinterpret_cast<const ET*>(P.T) + ur.t_row * P.V) + v0;
+    const uint4* const gD = reinterpret_cast<const uint4*>(reinterpret_cast<const ET*>(P.D) + ur.d_row * P.V) + v0;
+    Pass1State ps;
+    ps.RT = ps.RD = kEmptyRef;
+    ps.ls.init();
+    const unsigned from_end = (gridDim.y - 1u - blockIdx.y) * gridDim.x + (gridDim.x - 1u - blockIdx.x);
+    const uint64_t policy = from_end < S.kept ? policy_keep() : policy_discard();
+    if (ur.bonus) sweep_pass1<DT, true>(gT, gD, nvec, lane, P.c, policy, ps);
+    else          sweep_pass1<DT, false>(gT, gD, nvec, lane, P.c, policy, ps);
+    warp_post_lanes(ps.ls, ps.RT, ps.RD, lane, &wpart[warp]);
+    __syncthreads();
+    if (warp == 0) {
+        const PartialStats item = warp_merge_lanes(lane < kSweepWarps ? wpart[lane] : empty_partial());
+        if (lane == 0 && SD_IN((long long)unit * S.slices + slice, (long long)total_units<false>(P) * S.slices, 26))
+            S.part[(size_t)unit * S.slices + slice] = item;
+    }
+}
+
+// A block per sequence, a warp per row.
+template <int DT>
+__global__ void __launch_bounds__(kSweepThreads)
+sd_sweep_rows_kernel(const __grid_constant__ Params P, const __grid_constant__ Sweep S) {
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int b = blockIdx.x;
+    launch_dependents();
+    for (int i = warp; i <= P.k; i += kSweepWarps) {
+        const int unit = b * (P.k + 1) + i;
+        AcceptOperands aop;
+        aop.valid = false;
+        if (lane == 0 && i < P.k) aop = load_accept_operands<DT>(P, b, i);   // (inputs of the call)
+        await_previous_kernel();
+        const PartialStats row = warp_merge_lanes(lane < S.slices ? load_partial_cg(S.part + (size_t)unit * S.slices + lane)
+                                                                  : empty_partial());
+        if (lane == 0) {
+            if (P.status && i == 0) P.status[b] = 0;      // the words are ORed in by the second sweep
+            finish_row(P, b, i, row, row_constants(P, i == P.k, row), aop);
+        }
+    }
+}
+
+// Pass 2 of a warp's regions of an item.
+template <int DT, bool BONUS, bool HINT, bool MASS>
+__device__ __forceinline__ void sweep_pass2(const uint4* gT, const uint4* gD, const uint4* gH, typename Elem<DT>::type* gdst,
+                                            float* rsum, int nvec, int lane, float c, uint64_t policy, const RowConst& rc,
+                                            float& herr) {
+    using E = Elem<DT>;
+    for (; nvec > 0; gT += kSweepStep, gD += kSweepStep, nvec -= kSweepStep) {
+        uint4 rt[kRegionRows], rd[kRegionRows], hq[kRegionRows];
+        float mass;
+        if (nvec >= kRegionVecs) {
+#pragma unroll
+            for (int g = 0; g < kRegionRows; ++g) {
+                rt[g] = load_l2(gT + g * 32 + lane, policy);
+                if (!BONUS) rd[g] = load_l2(gD + g * 32 + lane, policy);
+                if (HINT) hq[g] = __ldcs(gH + g * 32 + lane);
+            }
+            mass = pass2_region_impl<DT, BONUS, HINT, MASS>(rt, rd, kRegionVecs, lane, c, rc, gdst, hq, herr);
+        } else {
+#pragma unroll
+            for (int g = 0; g < kRegionRows; ++g) {
+                const int vi = g * 32 + lane;
+                rt[g] = vi < nvec ? load_l2(gT + vi, policy) : E::masked();
+                rd[g] = (!BONUS && vi < nvec) ? load_l2(gD + vi, policy) : E::masked();
+                if (HINT) hq[g] = vi < nvec ? __ldcs(gH + vi) : make_uint4(0u, 0u, 0u, 0u);
+            }
+            mass = pass2_region_impl<DT, BONUS, HINT, MASS>(rt, rd, nvec, lane, c, rc, gdst, hq, herr);
+        }
+        if constexpr (MASS) {
+            if (lane == 0) *rsum = mass;
+            rsum += kSweepWarps;
+        }
+        if (gdst) gdst += (size_t)kSweepStep * E::VEC;
+        if (HINT) gH += kSweepStep;
+    }
+}
+
+// A row of the second sweep whose sums over the whole row are wanted, by the warp of the block that brought
+// its last item: hint error, acceptance probability, the draw.
+template <int DT, bool HINT>
+__device__ __noinline__ void sweep_row_done(const Params& P, const Sweep& S, int unit, int n, const RowConst rc) {
+    const int lane = threadIdx.x & 31;
+    const UnitRef ur = unit_ref<false>(P, unit);
+    if (HINT && !ur.bonus) {
+        // the items' shares in their order
+        double e = 0.0;
+        const double* hp = P.hint_part + (size_t)unit * P.hint_stride;
+        for (int i = 0; i < S.slices; ++i) e += __ldcg(hp + i);
+        if (lane == 0) P.hint_err[ur.d_row] = (float)e;
+    }
+    if (S.all_rows && !ur.bonus) {
+        // diagnostic: acceptance probability 1 - sum max(0,p-q) of the position
+        const float* rs = P.region_sums + (size_t)unit * P.NR;
+        double part = 0.0;
+        for (int j = lane; j < P.NR; j += 32) part += (double)__ldcg(rs + j);
+        const double R = warp_sum(part) * (double)P.tau;
+        if (lane == 0) P.acc_prob[ur.d_row] = (float)(1.0 - R);
+    }
+    if (ur.i == n) resolve_sequence<DT, true, true>(P, ur.b, n, rc);
+}
+
+// One block per item.  The first S.draw_blocks blocks take the rows that are drawn from (so that the draws,
+// chains of dependent reads, are over long before the sweep is); the rest all other pair rows, from the
+// last item of the first sweep backwards.
+template <int DT, int MODE>
+__global__ void __launch_bounds__(kSweepThreads, MODE == kSweepHint ? 4 : 6)
+sd_sweep_grad_kernel(const __grid_constant__ Params P, const __grid_constant__ Sweep S) {
+    using E = Elem<DT>;
+    using ET = typename E::type;
+    constexpr bool ERR = MODE == kSweepErrors, HINT = MODE == kSweepHint;
+    __shared__ float hpart[kSweepWarps];
+    __shared__ int is_last;
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const bool draws = (int)blockIdx.x < S.draw_blocks;
+    int unit, slice, b, n = P.k;
+    if (draws) {
+        b = (int)blockIdx.x / S.slices;
+        slice = (int)blockIdx.x - b * S.slices;
+        unit = 0;
+    } else {
+        const int units = total_units<false>(P), id = (int)(gridDim.x - 1u - blockIdx.x);
+        slice = id / units;
+        unit = id - slice * units;
+        b = unit / (P.k + 1);
+    }
+    await_previous_kernel();
+
+    // the first rejected position of the sequence
+    for (int i0 = 0; i0 < P.k; i0 += 32) {
+        const unsigned m = __ballot_sync(0xffffffffu, i0 + lane < P.k && P.accept[b * P.k + i0 + lane] == 0);
+        if (m) { n = i0 + __ffs(m) - 1; break; }
+    }
+    if (draws) unit = b * (P.k + 1) + n;
+    else if (unit - b * (P.k + 1) == n) return;      // the first blocks have it
+    const UnitRef ur = unit_ref<false>(P, unit);
+    if (!draws && ur.bonus) return;
+    const RowConst rc = P.rowc[unit];
+    const int v0 = (slice * S.regions + warp) * kRegionVecs;
+    int nvec = min((slice + 1) * S.regions * kRegionVecs, P.V / E::VEC) - v0;
+    if (nvec > 0 && !SD_IN((long long)(v0 + nvec) * E::VEC - 1, P.V, 12)) nvec = 0;
+    if (!SD_IN(ur.t_row, (long long)P.B * (P.k + 1), 12) ||
+        !SD_IN(ur.d_row, (long long)P.B * P.k, 12)) nvec = 0;
+    const size_t offD = ur.d_row * P.V + (size_t)v0 * E::VEC;
+    const size_t offG = ERR ? (size_t)b * P.V + (size_t)v0 * E::VEC : offD;
+    const uint4* const gT = reinterpret_cast<const uint4*>(reinterpret_cast<const ET*>(P.T) + ur.t_row * P.V) + v0;
+    const uint4* const gD = reinterpret_cast<const uint4*>(reinterpret_cast<const ET*>(P.D) + offD);
+    ET* const gdst = (P.grad && !ur.bonus) ? reinterpret_cast<ET*>(P.grad) + offG : nullptr;
+    const uint64_t policy = policy_discard();
+    if (!draws && !HINT && !S.all_rows) {
+        float unused = 0.f;
+        sweep_pass2<DT, false, false, false>(gT, gD, nullptr, gdst, nullptr, nvec, lane, P.c, policy, rc, unused);
+        return;
+    }
+    float herr = 0.f;
+    float* const rsum = P.region_sums + (size_t)unit * P.NR + slice * S.regions + warp;
+    if (ur.bonus) {
+        sweep_pass2<DT, true, false, true>(gT, gD, nullptr, nullptr, rsum, nvec, lane, P.c, policy, rc, herr);
+        if (ERR && P.grad) {
+            // no error position: a zero row
+            uint4* z = reinterpret_cast<uint4*>(reinterpret_cast<ET*>(P.grad) + offG);
+            for (; nvec > 0; nvec -= kSweepStep, z += kSweepStep) {
+#pragma unroll
+                for (int g = 0; g < kRegionRows; ++g)
+                    if (g * 32 + lane < nvec) __stcs(z + g * 32 + lane, make_uint4(0u, 0u, 0u, 0u));
+            }
+        }
+    } else {
+        const uint4* const gH = HINT ? reinterpret_cast<const uint4*>(reinterpret_cast<const ET*>(P.hint) + offD) : nullptr;
+        sweep_pass2<DT, false, HINT, true>(gT, gD, gH, gdst, rsum, nvec, lane, P.c, policy, rc, herr);
+    }
+    if constexpr (HINT) {
+#pragma unroll
+        for (int off = 16; off > 0; off >>= 1) herr += __shfl_xor_sync(0xffffffffu, herr, off);
+        if (lane == 0) hpart[warp] = herr;
+    }
+    __syncthreads();
+    if (warp != 0) return;
+    if (lane == 0) {
+        if (HINT && !ur.bonus) {
+            // this item's share of the row's hint error: the warps' shares in their order, in fp64
+            double e = 0.0;
+            for (int w = 0; w < kSweepWarps; ++w) e += (double)hpart[w];
+            P.hint_part[(size_t)unit * P.hint_stride + slice] = e;
+        }
+        __threadfence();
+        is_last = atomicAdd(S.arrived + unit, 1u) == (uint32_t)S.slices - 1u;
+        if (is_last) {
+            __threadfence();
+            S.arrived[unit] = 0;
+        }
+    }
+    __syncwarp();
+    if (is_last) sweep_row_done<DT, HINT>(P, S, unit, n, rc);
+}
+
+}  // namespace sdv

@@ -1,0 +1,64 @@
+"""The two sweeps (csrc/sd_sweep.cuh) at the sizes where their cuts can go wrong -- rows of one vector, of
+one region more or less than an item or a warp's step, of the most items a row may have -- against the
+oracle, and against the cluster kernel that a workspace without room for them selects."""
+import numpy as np
+import pytest
+import torch
+
+from paper_2603_12617_b200 import synth
+from test_parity_gpu import check, oracle_of, to_device
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def binding():
+    import __graft_entry__ as entry
+    entry.build()
+    from paper_2603_12617_b200 import binding as b
+    return b
+
+
+# A region is 64 vectors: 256 fp32 or 512 bf16 entries; an item is 8 to 32 regions, a row at most 32 items.
+# (Small batches take the cluster kernel, so these are just large enough: about 32 MB of bf16, 48 MB of fp32.)
+SHAPES = [(6400, 2, 504, "bf16"),                  # less than a region
+          (1300, 2, 512 * 8 - 8, "bf16"), (1300, 2, 512 * 8 + 8, "bf16"), (4100, 1, 1024 - 4, "f32"),
+          (64, 1, 256 * 257, "f32"), (2, 64, 65536 + 8, "bf16"), (150, 1, 256 * 129 + 4, "f32"),
+          (1, 1, 5500008, "bf16")]                 # the most items a row may have
+
+
+@pytest.mark.parametrize("B,k,V,dtype", SHAPES)
+def test_sweeps_match_the_oracle(binding, B, k, V, dtype):
+    cfg = synth.custom_config(B=B, k=k, V=V, dtype=dtype, tau=0.9, index=97)
+    inp = synth.make_inputs(cfg)
+    T, D, x, u = to_device(inp)
+    ref = oracle_of(inp)
+    ex = binding.sd_verify_feedback_ex(T, D, x, u, inp.tau)            # masses of every row (acceptance probabilities)
+    info = binding.sd_launch_info()
+    assert info["path"] == 1 and info["kernels"] == 3
+    check(inp, ex, ref, max_band_frac=1.0)
+    out = binding.sd_verify_feedback(T, D, x, u, inp.tau)              # masses of the drawn rows only
+    only = binding.sd_verify_feedback(T, D, x, u, inp.tau, want_loss=False, want_grad=False)
+    err = binding.sd_verify_error_feedback(T, D, x, u, inp.tau)
+    torch.cuda.synchronize()
+    for o in (out, only, err):
+        assert torch.equal(o.accept_len, ex.accept_len) and torch.equal(o.tokens, ex.tokens)
+    assert torch.equal(out.grad_draft, ex.grad_draft) and torch.equal(out.loss, ex.loss) and torch.equal(err.loss, ex.loss)
+    n = ex.accept_len.long()
+    rows = torch.where((n < k)[:, None], ex.grad_draft[torch.arange(B, device="cuda"), n.clamp(max=k - 1)], 0)
+    assert torch.equal(err.error_grad, rows)
+
+
+@pytest.mark.parametrize("dtype", ["f32", "bf16"])
+def test_a_workspace_without_room_for_the_sweeps_takes_the_cluster_kernel(binding, dtype):
+    """Callers that sized their workspace before there were sweeps are served as before."""
+    B, k, V = 40, 3, 512 * 128 if dtype == "bf16" else 256 * 192
+    cfg = synth.custom_config(B=B, k=k, V=V, dtype=dtype, index=98)
+    inp = synth.make_inputs(cfg)
+    T, D, x, u = to_device(inp)
+    code = binding.SD_DTYPE_F32 if dtype == "f32" else binding.SD_DTYPE_BF16
+    small = torch.empty(binding.sd_workspace_bytes(B, k, V, code) - 256, dtype=torch.uint8, device="cuda")
+    out = binding.sd_verify_feedback_ex(T, D, x, u, inp.tau, workspace=small)
+    assert binding.sd_launch_info()["kernels"] == 1
+    torch.cuda.synchronize()
+    check(inp, out, oracle_of(inp), max_band_frac=1.0)
