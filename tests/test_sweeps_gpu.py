@@ -62,3 +62,45 @@ def test_a_workspace_without_room_for_the_sweeps_takes_the_cluster_kernel(bindin
     assert binding.sd_launch_info()["kernels"] == 1
     torch.cuda.synchronize()
     check(inp, out, oracle_of(inp), max_band_frac=1.0)
+
+
+def _at(t, lead):
+    """The tensor's values `lead` elements past a 16-byte boundary."""
+    buf = torch.empty(t.numel() + lead, dtype=t.dtype, device=t.device)
+    v = buf[lead:].view(t.shape)
+    v.copy_(t)
+    return v
+
+
+@pytest.mark.parametrize("B,k,V,dtype,leadT,leadD", [
+    (3, 2, 50257, "bf16", 0, 0), (2, 3, 30001, "f32", 0, 0), (5, 2, 4097, "bf16", 1, 6), (4, 3, 2051, "f32", 2, 1),
+    (2, 2, 512 * 65 + 1, "bf16", 7, 7), (2, 2, 512 * 65 - 1, "bf16", 3, 0), (3, 1, 256 * 33 + 2, "f32", 0, 3), (1, 1, 4095 + 8, "bf16", 5, 2)])
+def test_rows_that_are_not_whole_vectors(binding, B, k, V, dtype, leadT, leadD):
+    """Every row starts elsewhere within a vector, target and draft differently."""
+    cfg = synth.custom_config(B=B, k=k, V=V, dtype=dtype, tau=0.8, index=99)
+    inp = synth.make_inputs(cfg)
+    T, D, x, u = to_device(inp)
+    T, D = _at(T, leadT), _at(D, leadD)
+    ref = oracle_of(inp)
+
+    def outputs(lead):
+        guard = torch.full((B * k * V + lead + 8,), -7.0, dtype=D.dtype, device="cuda")
+        grad = guard[lead:lead + B * k * V].view(B, k, V)
+        return guard, binding.StepOutputs(
+            accept_len=torch.empty(B, dtype=torch.int32, device="cuda"), tokens=torch.empty((B, k + 1), dtype=torch.int32, device="cuda"),
+            loss=torch.empty((B, k), device="cuda"), grad_draft=grad, acc_prob=torch.empty((B, k), device="cuda"),
+            status=torch.empty(B, dtype=torch.int32, device="cuda"))
+    guard, out = outputs(leadD)
+    binding.sd_verify_feedback_ex(T, D, x, u, inp.tau, out=out)
+    info = binding.sd_launch_info()
+    assert info["path"] == 1 and info["kernels"] == 3
+    check(inp, out, ref, max_band_frac=1.0)
+    assert (guard[:leadD] == -7).all() and (guard[leadD + B * k * V:] == -7).all()
+    only = binding.sd_verify_feedback(T, D, x, u, inp.tau, want_loss=False, want_grad=False)
+    torch.cuda.synchronize()
+    assert torch.equal(only.accept_len, out.accept_len) and torch.equal(only.tokens, out.tokens)
+    # a gradient that starts elsewhere than the draft: element-wise kernel
+    _, out2 = outputs(leadD + 1)
+    binding.sd_verify_feedback_ex(T, D, x, u, inp.tau, out=out2)
+    assert binding.sd_launch_info()["path"] == 0
+    check(inp, out2, ref, max_band_frac=1.0)
