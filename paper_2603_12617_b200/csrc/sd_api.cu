@@ -932,9 +932,10 @@ int sd_verify_greedy(const void* target_logits, const int32_t* draft_tokens, int
     P.accept_len = out_accept_len; P.tokens = out_tokens; P.argmax = out_argmax;
     P.ticket = reinterpret_cast<uint32_t*>(ws);
     P.keys = reinterpret_cast<unsigned long long*>(ws + kAlign);
-    const int item_elems = kGreedyItemVecs * vec_elems(dtype);
-    P.items_per_row = (V + item_elems - 1) / item_elems;
-    P.vectorised = (((size_t)V * es) % 16 == 0 && aligned(target_logits, 16)) ? 1 : 0;
+    // (a row that does not start on a 16-byte boundary is read from the one before it)
+    const int vec = vec_elems(dtype), item_elems = kGreedyItemVecs * vec;
+    const bool whole = V % vec == 0 && aligned(target_logits, 16);
+    P.items_per_row = (int)(((long long)V + (whole ? 0 : vec - 1) + item_elems - 1) / item_elems);
     const long long items = (long long)B * (k + 1) * P.items_per_row;
     // blocks per SM: 4 of 256 threads, 8 loads of 16 bytes in flight per thread, measured best among 2..8
     // on the largest workload (more blocks disturb the DRAM page locality of the streams);
