@@ -1168,10 +1168,10 @@ int sd_vp_finish(const void* target_shard, const void* draft_shard, const int32_
     sd_vp_rows_kernel<<<(unsigned)B, 96, 0, st>>>(P);
     const int slices = (P.NR + kVpSliceRegions - 1) / kVpSliceRegions;
     const unsigned grid = (unsigned)B * (unsigned)(k + 1) * (unsigned)slices;
-    if (dtype == SD_DTYPE_F32) sd_vp_grad_kernel<SD_DTYPE_F32><<<grid, kVpThreads, 0, st>>>(P, slices);
-    else                       sd_vp_grad_kernel<SD_DTYPE_BF16><<<grid, kVpThreads, 0, st>>>(P, slices);
-    sd_vp_mass_kernel<<<(unsigned)B, 32, 0, st>>>(P);
     SD_CUDA(cudaGetLastError());
+    SD_CUDA(dtype == SD_DTYPE_F32 ? launch_following(sd_vp_grad_kernel<SD_DTYPE_F32>, dim3(grid), kVpThreads, st, P, slices)
+                                  : launch_following(sd_vp_grad_kernel<SD_DTYPE_BF16>, dim3(grid), kVpThreads, st, P, slices));
+    SD_CUDA(launch_following(sd_vp_mass_kernel, dim3((unsigned)B), 32, st, P));
     tl_info[0] = 6; tl_info[1] = 1; tl_info[2] = kVpThreads; tl_info[3] = 0; tl_info[4] = (int)grid; tl_info[5] = 3;
     return SD_OK;
 }
