@@ -128,31 +128,50 @@ def _dtype_code(t: torch.Tensor) -> int:
 
 
 def _ptr(t: Optional[torch.Tensor]):
-    return None if t is None else ctypes.c_void_p(t.data_ptr())
+    return None if t is None else t.data_ptr()      # (the argument types make a void* of it)
+
+
+class _OnDevice:
+    """``torch.cuda.device(dev)``, but free of charge when ``dev`` is the current device already."""
+    __slots__ = ("guard",)
+
+    def __init__(self, dev: torch.device):
+        index = dev.index
+        self.guard = None if index is None or index == torch.cuda.current_device() else torch.cuda.device(dev)
+
+    def __enter__(self):
+        if self.guard is not None:
+            self.guard.__enter__()
+
+    def __exit__(self, *exc):
+        if self.guard is not None:
+            return self.guard.__exit__(*exc)
+        return False
 
 
 def _shapes(target_logits, draft_logits, draft_tokens, uniforms):
-    if target_logits.dim() != 3 or draft_logits.dim() != 3:
+    t_shape, d_shape = target_logits.shape, draft_logits.shape
+    if len(t_shape) != 3 or len(d_shape) != 3:
         raise ValueError("logits must be [B,k+1,V] and [B,k,V]")
-    B, k1, V = target_logits.shape
+    B, k1, V = t_shape
     k = k1 - 1
-    if tuple(draft_logits.shape) != (B, k, V):
-        raise ValueError(f"draft logits {tuple(draft_logits.shape)} do not match target {tuple(target_logits.shape)}")
-    if tuple(draft_tokens.shape) != (B, k) or draft_tokens.dtype != torch.int32:
+    if d_shape != (B, k, V):
+        raise ValueError(f"draft logits {tuple(d_shape)} do not match target {tuple(t_shape)}")
+    if draft_tokens.shape != (B, k) or draft_tokens.dtype != torch.int32:
         raise ValueError("draft_tokens must be int32 [B,k]")
-    if tuple(uniforms.shape) != (B, k + 1) or uniforms.dtype != torch.float32:
+    if uniforms.shape != (B, k1) or uniforms.dtype != torch.float32:
         raise ValueError("uniforms must be float32 [B,k+1]")
     if draft_logits.dtype != target_logits.dtype:
         raise TypeError("target and draft logits must have the same dtype")
-    for t in (target_logits, draft_logits, draft_tokens, uniforms):
-        if not t.is_contiguous():
-            raise ValueError("inputs must be contiguous")
+    if not (target_logits.is_contiguous() and draft_logits.is_contiguous() and draft_tokens.is_contiguous()
+            and uniforms.is_contiguous()):
+        raise ValueError("inputs must be contiguous")
     return B, k, V
 
 
 def _stream_ptr(stream: Optional[torch.cuda.Stream]):
-    s = torch.cuda.current_stream() if stream is None else stream
-    return ctypes.c_void_p(s.cuda_stream)
+    # the raw handle of the current stream: a Stream object would be made only to be asked for it
+    return torch._C._cuda_getCurrentRawStream(torch.cuda.current_device()) if stream is None else stream.cuda_stream
 
 
 def sd_version() -> int:
@@ -213,7 +232,7 @@ def sd_verify_feedback(target_logits: torch.Tensor, draft_logits: torch.Tensor,
             grad_draft=torch.empty_like(draft_logits) if want_grad else None)
     fn = _lib.sd_verify_feedback if target_logits.dtype == torch.float32 else _lib.sd_verify_feedback_bf16
     _dtype_code(target_logits)
-    with torch.cuda.device(dev):
+    with _OnDevice(dev):
         rc = fn(_ptr(target_logits), _ptr(draft_logits), _ptr(draft_tokens), _ptr(uniforms),
                 float(temperature), B, k, V, _ptr(out.accept_len), _ptr(out.tokens), _ptr(out.loss),
                 _ptr(out.grad_draft), _stream_ptr(stream))
@@ -242,7 +261,7 @@ def sd_verify_feedback_ex(target_logits: torch.Tensor, draft_logits: torch.Tenso
             grad_draft=torch.empty_like(draft_logits) if want_grad else None,
             acc_prob=torch.empty((B, k), dtype=torch.float32, device=dev) if want_acc_prob else None,
             status=torch.empty(B, dtype=torch.int32, device=dev) if want_status else None)
-    with torch.cuda.device(dev):
+    with _OnDevice(dev):
         rc = _lib.sd_verify_feedback_ex(
             _ptr(target_logits), _ptr(draft_logits), _ptr(draft_tokens), _ptr(uniforms), float(temperature),
             B, k, V, code, _ptr(out.accept_len), _ptr(out.tokens), _ptr(out.loss), _ptr(out.grad_draft),
@@ -277,7 +296,7 @@ def sd_verify_feedback_hint(target_logits: torch.Tensor, draft_logits: torch.Ten
         grad_draft=grad_out if grad_out is not None else torch.empty_like(draft_logits),
         status=torch.empty(B, dtype=torch.int32, device=dev),
         hint_err=torch.empty((B, k), dtype=torch.float32, device=dev))
-    with torch.cuda.device(dev):
+    with _OnDevice(dev):
         rc = _lib.sd_verify_feedback_hint(
             _ptr(target_logits), _ptr(draft_logits), _ptr(draft_tokens), _ptr(uniforms), float(temperature),
             B, k, V, code, _ptr(hint), _ptr(out.accept_len), _ptr(out.tokens), _ptr(out.loss), _ptr(out.grad_draft),
@@ -317,7 +336,7 @@ def sd_verify_greedy(target_logits: torch.Tensor, draft_tokens: torch.Tensor, *,
         out = GreedyOutputs(accept_len=torch.empty(B, dtype=torch.int32, device=dev),
                             tokens=torch.empty((B, k + 1), dtype=torch.int32, device=dev),
                             argmax=torch.empty((B, k + 1), dtype=torch.int32, device=dev) if want_argmax else None)
-    with torch.cuda.device(dev):
+    with _OnDevice(dev):
         rc = _lib.sd_verify_greedy(_ptr(target_logits), _ptr(draft_tokens), B, k, V, code, _ptr(out.accept_len),
                                    _ptr(out.tokens), _ptr(out.argmax), _ptr(workspace),
                                    0 if workspace is None else workspace.numel() * workspace.element_size(),
@@ -354,7 +373,7 @@ def sd_verify_error_feedback(target_logits: torch.Tensor, draft_logits: torch.Te
             loss=torch.empty((B, k), dtype=torch.float32, device=dev) if want_loss else None,
             error_grad=torch.empty((B, V), dtype=target_logits.dtype, device=dev) if want_grad else None,
             status=torch.empty(B, dtype=torch.int32, device=dev) if want_status else None)
-    with torch.cuda.device(dev):
+    with _OnDevice(dev):
         rc = _lib.sd_verify_error_feedback(_ptr(target_logits), _ptr(draft_logits), _ptr(draft_tokens), _ptr(uniforms),
                                            float(temperature), B, k, V, code, _ptr(out.accept_len), _ptr(out.tokens),
                                            _ptr(out.loss), _ptr(out.error_grad), _ptr(out.status), None, 0,
@@ -403,7 +422,7 @@ def sd_ensemble_feedback(target_logits: torch.Tensor, draft_logits, temperature:
             status=torch.empty(B, dtype=torch.int32, device=dev) if want_status else None)
     dptr = (ctypes.c_void_p * N)(*[d.data_ptr() for d in draft_logits])
     gptr = (ctypes.c_void_p * N)(*[g.data_ptr() for g in out.grad]) if out.grad is not None else None
-    with torch.cuda.device(dev):
+    with _OnDevice(dev):
         rc = _lib.sd_ensemble_feedback(_ptr(target_logits), dptr, N, float(temperature), float(epsilon), B, k, V, code,
                                        _ptr(cum_loss), _ptr(out.loss), gptr, _ptr(out.round_loss),
                                        _ptr(out.cum_loss), _ptr(out.weights), _ptr(out.status), None, 0,
@@ -432,7 +451,7 @@ def sd_lmhead_grad(grad_logits: torch.Tensor, hidden: torch.Tensor, *, out: Opti
     d = hidden.shape[1]
     if out is None:
         out = torch.empty((V, d), dtype=torch.float32, device=dev)
-    with torch.cuda.device(dev):
+    with _OnDevice(dev):
         rc = _lib.sd_lmhead_grad(_ptr(grad_logits), _ptr(hidden), R, V, d, _ptr(out), _ptr(status), _stream_ptr(stream))
     if rc != 0:
         raise SdVerifyError(rc, "sd_lmhead_grad")
@@ -546,7 +565,7 @@ def sd_verify_feedback_static(target_logits: torch.Tensor, draft_logits: torch.T
     if dev.type != "cuda":
         raise ValueError("device tensors required")
     code = _dtype_code(target_logits)
-    with torch.cuda.device(dev):
+    with _OnDevice(dev):
         rc = _lib.sd_verify_feedback_static(
             _ptr(target_logits), _ptr(draft_logits), _ptr(draft_tokens), _ptr(uniforms), float(temperature),
             B, k, V, code, _ptr(out.accept_len), _ptr(out.tokens), _ptr(out.loss), _ptr(out.grad_draft),
