@@ -412,6 +412,8 @@ int sd_verify_feedback_host(const void* target_logits, const void* draft_logits,
  *                                SD_STATUS_TIMEOUT); the wait also ends after about a second
  *   SD_OPT_PREFETCH              env SD_VERIFY_PREFETCH         default 0    non-zero: while a block is in
  *                                its second pass over a row pair it asks L2 to fetch the next row pair
+ * SD_OPT_CLUSTER, _LAG, _L2_BUDGET_MIB, _WAIT_POLLS and _PREFETCH are options of the cluster kernel: off
+ * their defaults they also keep calls from the two sweeps, which have neither clusters nor waits.
  * sd_set_option returns SD_OK, or SD_ERR_SHAPE for an unknown option; sd_get_option returns the
  * value in force, or -1 for an unknown option.
  */
@@ -429,7 +431,7 @@ long long sd_get_option(int option_id);
 
 /*
  * sd_launch_info -- HOST out-parameters describing how the last successful device call on this
- * thread was launched: path (0 = generic, 1 = stream fast path, 2 = greedy verification, 3 = ensemble feedback, 4 = error-position feedback, 5 = output-layer gradient, 6 = vocabulary-parallel step), cluster size, threads per
+ * thread was launched: path (0 = generic, 1 = fast path (one kernel: cluster kernel, three: the two sweeps), 2 = greedy verification, 3 = ensemble feedback, 4 = error-position feedback, 5 = output-layer gradient, 6 = vocabulary-parallel step), cluster size, threads per
  * block, dynamic shared memory per block, blocks launched, kernels launched.  Any pointer may
  * be NULL.  Diagnostic only.
  */
