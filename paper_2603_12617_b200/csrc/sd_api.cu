@@ -276,7 +276,9 @@ bool use_sweeps(int dtype, double bytes) {
 
 // Rows that are not whole 16-byte vectors: the sweeps take them where draft and gradient start at the same
 // place within a vector and rows are long enough that their ends, which go entry by entry, are the smaller
-// part; the element-wise kernel has the rest.  (16 sequences, 5 tokens, 50 257 bf16 entries: 91.6 us there, 35.9 us here.)
+// part; the element-wise kernel has the rest.  Calls back to back, element-wise / sweeps: 16 sequences,
+// 5 tokens, 50 257 bf16 entries 91.6 / 35.9 us, one sequence, 4 tokens, 32 001 entries 41 / 23 us, one token,
+// 131 351 entries 252 / 23 us; at 8 201 entries and below one launch beats three by 3 to 5 us.
 bool use_ragged_sweeps(const void* D, const void* grad, const void* hint, int V, int dtype) {
     const int vec = vec_elems(dtype);
     return !hint && option(SD_OPT_FORCE_GENERIC) == 0 && V % vec != 0 && V >= 8 * kRegionVecs * vec &&
