@@ -679,21 +679,21 @@ EncodeTiledFn encode_tiled_fn() {
     });
     return fn;
 }
-// Map of a row-major bf16 matrix [rows, cols] (device memory of this GPU) for boxes of
-// box_rows x 64 columns in the 128-byte swizzle; entries outside the matrix read as zero.
-int bf16_matrix_map(CUtensorMap* map, const void* base, int rows, int cols, int box_rows) {
+// Map of a row-major matrix [rows, cols] of bf16 or fp32 (device memory of this GPU) for boxes of
+// box_rows x 128 bytes in the 128-byte swizzle; entries outside the matrix read as zero and are not written.
+int matrix_map(CUtensorMap* map, int dtype, const void* base, int rows, int cols, int box_rows) {
     EncodeTiledFn enc = encode_tiled_fn();
     if (!enc) {
         snprintf(tl_cuda_error, sizeof tl_cuda_error, "cuTensorMapEncodeTiled is not available from this driver");
         return SD_ERR_CUDA;
     }
     const cuuint64_t dims[2] = {(cuuint64_t)cols, (cuuint64_t)rows};
-    const cuuint64_t strides[1] = {(cuuint64_t)cols * 2};
-    const cuuint32_t box[2] = {(cuuint32_t)kGemmChunk, (cuuint32_t)box_rows};
+    const cuuint64_t strides[1] = {(cuuint64_t)cols * elem_bytes(dtype)};
+    const cuuint32_t box[2] = {(cuuint32_t)(128 / elem_bytes(dtype)), (cuuint32_t)box_rows};
     const cuuint32_t estr[2] = {1, 1};
-    const CUresult r = enc(map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, const_cast<void*>(base), dims, strides, box, estr,
-                           CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
-                           CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
+    const CUresult r = enc(map, dtype == SD_DTYPE_F32 ? CU_TENSOR_MAP_DATA_TYPE_FLOAT32 : CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2,
+                           const_cast<void*>(base), dims, strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
+                           CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_128B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
     if (r != CUDA_SUCCESS) {
         snprintf(tl_cuda_error, sizeof tl_cuda_error, "cuTensorMapEncodeTiled failed with code %d", (int)r);
         return SD_ERR_CUDA;
@@ -1296,10 +1296,12 @@ int sd_lmhead_grad(const uint16_t* grad_logits, const uint16_t* hidden, int R, i
     if (!ds->gemm_error) SD_CUDA(cudaMalloc(reinterpret_cast<void**>(&ds->gemm_error), 256));
     uint32_t* err = out_status ? out_status : ds->gemm_error;
     SD_CUDA(cudaMemsetAsync(err, 0, 4, st));
-    CUtensorMap map_g, map_x;
-    rc = bf16_matrix_map(&map_g, grad_logits, R, V, kGemmBK);
+    CUtensorMap map_g, map_x, map_out;
+    rc = matrix_map(&map_g, SD_DTYPE_BF16, grad_logits, R, V, kGemmBK);
     if (rc != SD_OK) return rc;
-    rc = bf16_matrix_map(&map_x, hidden, R, d, kGemmBK);
+    rc = matrix_map(&map_x, SD_DTYPE_BF16, hidden, R, d, kGemmBK);
+    if (rc != SD_OK) return rc;
+    rc = matrix_map(&map_out, SD_DTYPE_F32, out_dW, V, d, kGemmBox);
     if (rc != SD_OK) return rc;
     if (!ds->gemm_attr) {
         SD_CUDA(cudaFuncSetAttribute(sd_lmhead_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kGemmSmem));
@@ -1307,13 +1309,13 @@ int sd_lmhead_grad(const uint16_t* grad_logits, const uint16_t* hidden, int R, i
     }
     GemmParams P;
     P.R = R; P.V = V; P.d = d;
-    P.out = out_dW;
     P.error = err;
     const long long tiles = (long long)((V + kGemmBM - 1) / kGemmBM) * ((d + kGemmBN - 1) / kGemmBN);
-    const unsigned grid = (unsigned)(tiles < ds->sm_count ? tiles : ds->sm_count);
-    sd_lmhead_kernel<<<grid, kGemmThreads, kGemmSmem, st>>>(map_g, map_x, P);
+    const long long pairs = ds->sm_count / 2;
+    const unsigned grid = 2u * (unsigned)(tiles < pairs ? tiles : pairs);
+    sd_lmhead_kernel<<<grid, kGemmThreads, kGemmSmem, st>>>(map_g, map_x, map_out, P);
     SD_CUDA(cudaGetLastError());
-    tl_info[0] = 5; tl_info[1] = 1; tl_info[2] = kGemmThreads; tl_info[3] = kGemmSmem; tl_info[4] = (int)grid; tl_info[5] = 1;
+    tl_info[0] = 5; tl_info[1] = 2; tl_info[2] = kGemmThreads; tl_info[3] = kGemmSmem; tl_info[4] = (int)grid; tl_info[5] = 1;
     return SD_OK;
 }
 

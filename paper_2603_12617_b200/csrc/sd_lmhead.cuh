@@ -5,24 +5,30 @@
 // a dense contraction over the positions of the round: the one place on this path where the
 // tensor cores apply.  sm_100a: operands by TMA (cp.async.bulk.tensor) into 128-byte-swizzled
 // shared memory, tcgen05.mma (bf16 x bf16 -> fp32) with the accumulator in tensor memory,
-// tcgen05.ld for the epilogue.
+// tcgen05.ld and TMA stores for the epilogue.
 //
 // Both operands have the contracted index r as their slow index in memory, so both are "MN-major"
 // operands of the instruction: a tile of g is [64 positions][128 vocabulary entries] with the
-// vocabulary entries contiguous, a tile of X is [64 positions][256 features] likewise.
+// vocabulary entries contiguous, a tile of X is [64 positions][128 features] likewise.
 //
-// One block per SM, persistent over output tiles of 128 x 256; the features run fastest over the
-// tiles, so the blocks that work at the same time share a few tiles of g (each read from HBM once)
-// and all of X (which stays in L2).  Warp roles:
-//   warp 0      producer: one thread issues the TMA loads of a stage (6 boxes of 64 x 64 bf16)
-//   warp 1      one thread issues the MMAs (4 of K = 16 per stage) and the commits
-//   warps 2..5  epilogue: tensor memory -> registers -> a staging block in shared memory -> global
-//               memory in whole 128-byte lines, while the MMAs of the next tile fill the other half
-//               of tensor memory.  (A lane gets 32 consecutive columns of ONE row from tensor memory;
-//               stored from there, every instruction of a warp touches 32 different lines with 16
-//               bytes each, and the result -- 2.1 GB at the full size -- left at 1.4 TB/s.)
+// A pair of blocks (a cluster of two, one block per SM) shares an output tile of 256 x 256 (cta_group::2):
+// block r holds rows 128 r .. 128 r + 127 of the tile, brings their part of g and columns
+// 128 r .. 128 r + 127 of X, and each tensor core reads the other half of X from its neighbour's shared
+// memory.  Persistent over the tiles; the features run fastest, so the pairs that work at the same time
+// share a few tiles of g (each read from HBM once) and all of X (which stays in L2).  Warp roles of a block:
+//   warp 0      producer: one thread issues the TMA loads of the block's share of a stage (4 boxes of 64 x 64
+//               bf16); they complete on the barrier of the pair's first block
+//   warp 1      in the pair's first block one thread issues the MMAs (4 of K = 16 per stage) and the commits,
+//               which free the stage in both blocks
+//   warps 2..5  epilogue: tensor memory -> registers -> 32 x 32 boxes in shared memory -> global memory by TMA
+//               stores, which clip at the ends of dW, while the MMAs of the next tile fill the other half of
+//               tensor memory.
+// What bounds it: for many positions the board's power (1.3 of 1.64 PFLOP/s at 1536 positions, 128 256 x 4096: 1237 us);
+// operands enter an SM at 64 bytes a clock.  One block per tile of 128 x 256 (cta_group::1) needs 96, 27 TB/s of
+// L2 at full rate, and took 1377 us.  For few positions the writing of dW (256 positions 557 us, one block
+// per tile 562; 128 positions 476 and 549).
 // Every wait is bounded; a wait that gives up sets an error word, and the block frees its tensor
-// memory and returns.  No multicast, no cluster.
+// memory and returns.  No multicast of loads.
 #pragma once
 
 #include <cuda.h>
@@ -33,58 +39,83 @@
 
 namespace sdv {
 
-constexpr int kGemmBM = 128;                 // vocabulary entries per tile (rows of dW)
-constexpr int kGemmBN = 256;                 // features per tile (columns of dW)
+constexpr int kGemmBM = 256;                 // vocabulary entries per tile (rows of dW), half of them in each block
+constexpr int kGemmBN = 256;                 // features per tile (columns of dW); each block brings half of them
 constexpr int kGemmBK = 64;                  // positions per stage
-constexpr int kGemmStages = 4;
+constexpr int kGemmStages = 6;
 constexpr int kGemmChunk = 64;               // entries of a 128-byte swizzled row (bf16)
 constexpr int kGemmChunkBytes = kGemmBK * kGemmChunk * 2;            // one TMA box: 8 KiB
-constexpr int kGemmABytes = (kGemmBM / kGemmChunk) * kGemmChunkBytes;   // 16 KiB
-constexpr int kGemmBBytes = (kGemmBN / kGemmChunk) * kGemmChunkBytes;   // 32 KiB
-constexpr int kGemmStageBytes = kGemmABytes + kGemmBBytes;            // 48 KiB
+constexpr int kGemmChunks = 128 / kGemmChunk;                        // boxes of an operand's half tile
+constexpr int kGemmABytes = kGemmChunks * kGemmChunkBytes;           // 16 KiB
+constexpr int kGemmStageBytes = 2 * kGemmABytes;                     // a block's share of a stage: 32 KiB
 constexpr int kGemmThreads = 6 * 32;
 constexpr int kGemmTmemCols = 512;           // two accumulators of 128 lanes x 256 fp32 columns
-constexpr int kGemmStagingStride = 36;       // floats per staged row: 32 + 4, keeps 16-byte accesses conflict-free
-constexpr int kGemmStagingBytes = 32 * kGemmStagingStride * 4;   // per epilogue warp
-constexpr int kGemmSmem = kGemmStages * kGemmStageBytes + 4 * kGemmStagingBytes + 1024 /* alignment */ + 256 /* barriers */;
+constexpr int kGemmBox = 32;                 // rows and columns of a box of the result
+constexpr int kGemmBoxBytes = kGemmBox * kGemmBox * 4;
+constexpr int kGemmBoxes = 2;                // boxes per epilogue warp: one leaves while the next is filled
+constexpr int kGemmSmem = kGemmStages * kGemmStageBytes + 4 * kGemmBoxes * kGemmBoxBytes + 1024 /* alignment */ + 256 /* barriers */;
+static_assert(kGemmSmem <= 227 * 1024, "stages and staging do not fit the shared memory of a block");
+constexpr long long kGemmLeaveCycles = 2000000ll;     // about a millisecond
 constexpr long long kGemmWaitCycles = 4000000000ll;   // about two seconds
 
 struct GemmParams {
     int R, V, d;
-    float* out;              // [V,d]
     uint32_t* error;         // set when a bounded wait gave up
 };
 
 // ---- PTX wrappers --------------------------------------------------------------------------
-__device__ __forceinline__ void tma_load_2d(void* dst_smem, const CUtensorMap* map, int x, int y, uint64_t* bar) {
+// One box into this block's shared memory; its bytes count on `bar` (a shared::cluster address), which may be
+// the other block's of the pair.
+__device__ __forceinline__ void tma_load_2d_pair(void* dst_smem, const CUtensorMap* map, int x, int y, uint32_t bar) {
     asm volatile(
-        "cp.async.bulk.tensor.2d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%3, %4}], [%2];" ::"r"(
+        "cp.async.bulk.tensor.2d.cta_group::2.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%3, %4}], [%2];" ::"r"(
             smem_u32(dst_smem)),
-        "l"(map), "r"(smem_u32(bar)), "r"(x), "r"(y)
+        "l"(map), "r"(bar), "r"(x), "r"(y)
         : "memory");
 }
-__device__ __forceinline__ void tmem_alloc(uint32_t* slot_in_smem, uint32_t cols) {
-    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(slot_in_smem)), "r"(cols)
+// One box of the result out of shared memory; what lies outside the matrix is not written.
+__device__ __forceinline__ void tma_store_2d(const CUtensorMap* map, int x, int y, const void* src_smem) {
+    asm volatile("cp.async.bulk.tensor.2d.global.shared::cta.bulk_group [%0, {%2, %3}], [%1];" ::"l"(map), "r"(smem_u32(src_smem)),
+                 "r"(x), "r"(y)
                  : "memory");
-    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+}
+__device__ __forceinline__ void tma_store_commit() { asm volatile("cp.async.bulk.commit_group;" ::: "memory"); }
+// All but the last `N` boxes of this thread have been read (READ) or written out.
+template <int N, bool READ> __device__ __forceinline__ void tma_store_wait() {
+    if constexpr (READ) asm volatile("cp.async.bulk.wait_group.read %0;" ::"n"(N) : "memory");
+    else                asm volatile("cp.async.bulk.wait_group %0;" ::"n"(N) : "memory");
+}
+// The address of `p` (of this block) in block `rank` of the cluster.
+__device__ __forceinline__ uint32_t cluster_address(const void* p, uint32_t rank) {
+    uint32_t a;
+    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(a) : "r"(smem_u32(p)), "r"(rank));
+    return a;
+}
+__device__ __forceinline__ void tmem_alloc(uint32_t* slot_in_smem, uint32_t cols) {
+    asm volatile("tcgen05.alloc.cta_group::2.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(slot_in_smem)), "r"(cols)
+                 : "memory");
+    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::2.sync.aligned;" ::: "memory");
 }
 __device__ __forceinline__ void tmem_dealloc(uint32_t taddr, uint32_t cols) {
-    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(taddr), "r"(cols) : "memory");
+    asm volatile("tcgen05.dealloc.cta_group::2.sync.aligned.b32 %0, %1;" ::"r"(taddr), "r"(cols) : "memory");
 }
 __device__ __forceinline__ void tc_fence_before() { asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory"); }
 __device__ __forceinline__ void tc_fence_after() { asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory"); }
-// D[tmem] (+)= A[smem] * B[smem]; accumulate = 0 overwrites D.
+// D[tmem] (+)= A[smem] * B[smem] of the pair, each block with its half of the rows; accumulate = 0 overwrites D.
 __device__ __forceinline__ void umma_bf16(uint32_t d_tmem, uint64_t a_desc, uint64_t b_desc, uint32_t idesc, uint32_t accumulate) {
     asm volatile(
         "{\n\t.reg .pred p;\n\t"
         "setp.ne.b32 p, %4, 0;\n\t"
-        "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}" ::"r"(d_tmem),
+        "tcgen05.mma.cta_group::2.kind::f16 [%0], %1, %2, %3, p;\n\t}" ::"r"(d_tmem),
         "l"(a_desc), "l"(b_desc), "r"(idesc), "r"(accumulate)
         : "memory");
 }
-// The barrier gets one arrival when every MMA issued so far by this thread has completed.
+// The barrier gets one arrival in each block of the pair when every MMA issued so far by this thread has completed.
 __device__ __forceinline__ void umma_commit(uint64_t* bar) {
-    asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(smem_u32(bar)) : "memory");
+    asm volatile("tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.multicast::cluster.b64 [%0], %1;" ::"r"(
+                     smem_u32(bar)),
+                 "h"((uint16_t)3)
+                 : "memory");
 }
 // 32 lanes x 32 consecutive fp32 columns of tensor memory: thread i of the warp gets lane i.
 __device__ __forceinline__ void tmem_ld_32x32(uint32_t taddr, uint32_t (&r)[32]) {
@@ -117,7 +148,7 @@ __host__ __device__ constexpr uint32_t umma_idesc_bf16_mn(int M, int N) {
 __device__ __forceinline__ bool gemm_wait(uint64_t* bar, uint32_t parity, volatile int* abort, uint32_t* error) {
     long long t0 = 0;
     for (uint32_t it = 0;; ++it) {
-        if (mbar_try_wait(bar, parity)) return true;
+        if (mbar_try_wait_cluster(bar, parity)) return true;
         if ((it & 255u) == 255u) {
             if (*abort) return false;
             const long long now = clock64();
@@ -131,30 +162,35 @@ __device__ __forceinline__ bool gemm_wait(uint64_t* bar, uint32_t parity, volati
 }
 
 struct GemmShared {
-    uint64_t full[kGemmStages];      // stage filled by TMA                 (1 arrival + bytes)
+    uint64_t full[kGemmStages];      // stage filled by both blocks' TMA    (first block: 1 arrival + bytes)
     uint64_t empty[kGemmStages];     // stage read by the MMAs              (1: commit)
     uint64_t acc_full[2];            // accumulator complete                (1: commit)
-    uint64_t acc_empty[2];           // accumulator read by the epilogue    (4: one per epilogue warp)
+    uint64_t acc_empty[2];           // accumulator read by the epilogues   (first block: 8, one per epilogue warp of the pair)
     uint32_t tmem_base;
     int abort;
 };
 
-__global__ void __launch_bounds__(kGemmThreads, 1)
-sd_lmhead_kernel(const __grid_constant__ CUtensorMap map_g, const __grid_constant__ CUtensorMap map_x, const GemmParams P) {
+__global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kGemmThreads, 1)
+sd_lmhead_kernel(const __grid_constant__ CUtensorMap map_g, const __grid_constant__ CUtensorMap map_x,
+                 const __grid_constant__ CUtensorMap map_out, const GemmParams P) {
     extern __shared__ unsigned char gemm_smem_raw[];
-    unsigned char* smem = reinterpret_cast<unsigned char*>((reinterpret_cast<uintptr_t>(gemm_smem_raw) + 1023) & ~(uintptr_t)1023);
-    float* staging_all = reinterpret_cast<float*>(smem + kGemmStages * kGemmStageBytes);
-    GemmShared& sh = *reinterpret_cast<GemmShared*>(smem + kGemmStages * kGemmStageBytes + 4 * kGemmStagingBytes);
+    // (the same offsets in both blocks: the MMAs take them from one block's descriptors)
+    unsigned char* smem = gemm_smem_raw + ((1024u - (smem_u32(gemm_smem_raw) & 1023u)) & 1023u);
+    unsigned char* boxes = smem + kGemmStages * kGemmStageBytes;
+    GemmShared& sh = *reinterpret_cast<GemmShared*>(boxes + 4 * kGemmBoxes * kGemmBoxBytes);
+    cg::cluster_group cluster = cg::this_cluster();
+    const int rank = (int)cluster.block_rank();
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     volatile int* abort = &sh.abort;
 
     const int tiles_m = (P.V + kGemmBM - 1) / kGemmBM, tiles_n = (P.d + kGemmBN - 1) / kGemmBN;
     const long long tiles = (long long)tiles_m * tiles_n;
     const int kblocks = (P.R + kGemmBK - 1) / kGemmBK;
+    const long long first = blockIdx.x >> 1, step = gridDim.x >> 1;
 
     if (tid == 0) {
         for (int s = 0; s < kGemmStages; ++s) { mbar_init(&sh.full[s], 1); mbar_init(&sh.empty[s], 1); }
-        for (int a = 0; a < 2; ++a) { mbar_init(&sh.acc_full[a], 1); mbar_init(&sh.acc_empty[a], 4); }
+        for (int a = 0; a < 2; ++a) { mbar_init(&sh.acc_full[a], 1); mbar_init(&sh.acc_empty[a], 8); }
         sh.abort = 0;
         fence_barrier_init();
         fence_proxy_async();
@@ -162,6 +198,7 @@ sd_lmhead_kernel(const __grid_constant__ CUtensorMap map_g, const __grid_constan
     if (warp == 1) tmem_alloc(&sh.tmem_base, kGemmTmemCols);     // the whole warp; the same warp frees it
     tc_fence_before();
     __syncthreads();
+    cluster.sync();                            // both blocks' barriers stand before anything arrives on them
     tc_fence_after();
     const uint32_t tmem = sh.tmem_base;
 
@@ -172,45 +209,39 @@ sd_lmhead_kernel(const __grid_constant__ CUtensorMap map_g, const __grid_constan
             uint32_t par = 1;                  // parity of the stage's previous use on empty[]
             long long n = 0;                   // stages issued so far
             bool ok = true;
-            for (long long tile = blockIdx.x; tile < tiles && ok; tile += gridDim.x) {
-                const int m0 = (int)(tile / tiles_n) * kGemmBM, n0 = (int)(tile % tiles_n) * kGemmBN;
+            for (long long tile = first; tile < tiles && ok; tile += step) {
+                const int m0 = (int)(tile / tiles_n) * kGemmBM + rank * 128, n0 = (int)(tile % tiles_n) * kGemmBN + rank * 128;
                 for (int kb = 0; kb < kblocks; ++kb) {
                     if (n >= kGemmStages && !gemm_wait(&sh.empty[stage], par, abort, P.error)) { ok = false; break; }
                     unsigned char* a = smem + (size_t)stage * kGemmStageBytes;
                     unsigned char* b = a + kGemmABytes;
-                    mbar_expect_tx(&sh.full[stage], (uint32_t)kGemmStageBytes);   // boxes out of range still count in full
+                    // the first block's barrier counts the bytes of both (boxes out of range count in full); the
+                    // neighbour's may arrive before it is armed: the phase cannot end without this arrival
+                    if (rank == 0) mbar_expect_tx(&sh.full[stage], 2u * (uint32_t)kGemmStageBytes);
+                    const uint32_t bar = cluster_address(&sh.full[stage], 0);
                     const int r0 = kb * kGemmBK;
 #pragma unroll
-                    for (int c = 0; c < kGemmBM / kGemmChunk; ++c)
-                        tma_load_2d(a + c * kGemmChunkBytes, &map_g, m0 + c * kGemmChunk, r0, &sh.full[stage]);
+                    for (int c = 0; c < kGemmChunks; ++c)
+                        tma_load_2d_pair(a + c * kGemmChunkBytes, &map_g, m0 + c * kGemmChunk, r0, bar);
 #pragma unroll
-                    for (int c = 0; c < kGemmBN / kGemmChunk; ++c)
-                        tma_load_2d(b + c * kGemmChunkBytes, &map_x, n0 + c * kGemmChunk, r0, &sh.full[stage]);
+                    for (int c = 0; c < kGemmChunks; ++c)
+                        tma_load_2d_pair(b + c * kGemmChunkBytes, &map_x, n0 + c * kGemmChunk, r0, bar);
                     ++n;
                     if (++stage == kGemmStages) { stage = 0; par ^= 1u; }
                 }
             }
-            // leaving early: every load issued has landed before the block goes away
-            if (!ok) {
-                const long long t0 = clock64();
-                for (long long i = (n > kGemmStages ? n - kGemmStages : 0); i < n; ++i) {
-                    const uint32_t p = (uint32_t)(i / kGemmStages) & 1u;
-                    while (!mbar_try_wait(&sh.full[i % kGemmStages], p))
-                        if (clock64() - t0 > kGemmWaitCycles) break;
-                }
-            }
         }
     } else if (warp == 1) {
-        // ---- MMA issuer
-        if (lane == 0) {
+        // ---- MMA issuer of the pair
+        if (lane == 0 && rank == 0) {
             constexpr uint32_t idesc = umma_idesc_bf16_mn(kGemmBM, kGemmBN);
             int stage = 0;
             uint32_t par = 0;
-            long long it = 0;                  // tiles of this block so far
+            long long it = 0;                  // tiles of this pair so far
             bool ok = true;
-            for (long long tile = blockIdx.x; tile < tiles && ok; tile += gridDim.x, ++it) {
+            for (long long tile = first; tile < tiles && ok; tile += step, ++it) {
                 const int acc = (int)(it & 1);
-                // the epilogue must have read this accumulator's previous tile
+                // the epilogues must have read this accumulator's previous tile
                 if (it >= 2 && !gemm_wait(&sh.acc_empty[acc], (uint32_t)((it >> 1) - 1) & 1u, abort, P.error)) { ok = false; break; }
                 tc_fence_after();
                 const uint32_t d_tmem = tmem + (uint32_t)acc * kGemmBN;
@@ -233,61 +264,61 @@ sd_lmhead_kernel(const __grid_constant__ CUtensorMap map_g, const __grid_constan
             }
         }
     } else {
-        // ---- epilogue: warp w reads the tensor-memory lanes 32*(w%4) .. +31 (rows of the tile)
+        // ---- epilogue: warp w reads the tensor-memory lanes 32*(w%4) .. +31 (rows of this block's half)
         const int q = warp & 3;
+        unsigned char* const mine = boxes + (size_t)(warp - 2) * kGemmBoxes * kGemmBoxBytes;
         long long it = 0;
+        int box = 0;
         bool ok = true;
-        for (long long tile = blockIdx.x; tile < tiles && ok; tile += gridDim.x, ++it) {
+        for (long long tile = first; tile < tiles && ok; tile += step, ++it) {
             const int acc = (int)(it & 1);
-            const int m0 = (int)(tile / tiles_n) * kGemmBM, n0 = (int)(tile % tiles_n) * kGemmBN;
+            const int m0 = (int)(tile / tiles_n) * kGemmBM + rank * 128, n0 = (int)(tile % tiles_n) * kGemmBN;
             int got = 1;
             if (lane == 0) got = gemm_wait(&sh.acc_full[acc], (uint32_t)(it >> 1) & 1u, abort, P.error) ? 1 : 0;
             got = __shfl_sync(0xffffffffu, got, 0);
             if (!got) { ok = false; break; }
             tc_fence_after();
-            float* stg = staging_all + (size_t)(warp - 2) * (kGemmStagingBytes / 4);
             const int vbase = m0 + q * 32;               // first row of this warp's 32
 #pragma unroll 1
-            for (int c = 0; c < kGemmBN / 32; ++c) {
+            for (int c = 0; c < kGemmBN / kGemmBox; ++c) {
                 uint32_t r[32];
-                tmem_ld_32x32(tmem + ((uint32_t)(q * 32) << 16) + (uint32_t)(acc * kGemmBN + c * 32), r);
+                tmem_ld_32x32(tmem + ((uint32_t)(q * 32) << 16) + (uint32_t)(acc * kGemmBN + c * kGemmBox), r);
                 tmem_ld_wait();
-                // lane = row of the block: 32 columns into the staging block
-#pragma unroll
-                for (int e = 0; e < 32; e += 4)
-                    *reinterpret_cast<float4*>(stg + lane * kGemmStagingStride + e) =
-                        make_float4(__uint_as_float(r[e]), __uint_as_float(r[e + 1]), __uint_as_float(r[e + 2]),
-                                    __uint_as_float(r[e + 3]));
+                // the box that left from here two boxes ago has been read
+                if (lane == 0) tma_store_wait<kGemmBoxes - 1, true>();
                 __syncwarp();
-                // eight lanes per row now: every store instruction writes four whole 128-byte lines
-                const int j0 = n0 + c * 32;
-                const int cr = lane >> 3, cc = (lane & 7) * 4;
+                // lane = row of the box, 128 bytes; 16-byte pieces in the order of the 128-byte swizzle
+                unsigned char* const stg = mine + box * kGemmBoxBytes;
 #pragma unroll
-                for (int i = 0; i < 8; ++i) {
-                    const int rr = i * 4 + cr;
-                    const int v = vbase + rr;
-                    const float4 val = *reinterpret_cast<const float4*>(stg + rr * kGemmStagingStride + cc);
-                    if (v < P.V) {
-                        float* dst = P.out + (size_t)v * P.d + j0 + cc;
-                        if (j0 + cc + 4 <= P.d) {
-                            __stcs(reinterpret_cast<float4*>(dst), val);
-                        } else {
-                            const float t4[4] = {val.x, val.y, val.z, val.w};
-                            for (int e = 0; e < 4; ++e)
-                                if (j0 + cc + e < P.d) dst[e] = t4[e];
-                        }
-                    }
+                for (int e = 0; e < 8; ++e)
+                    *reinterpret_cast<uint4*>(stg + lane * 128 + ((e ^ (lane & 7)) << 4)) =
+                        make_uint4(r[4 * e], r[4 * e + 1], r[4 * e + 2], r[4 * e + 3]);
+                fence_proxy_async();
+                __syncwarp();
+                if (lane == 0) {
+                    if (vbase < P.V && n0 + c * kGemmBox < P.d) tma_store_2d(&map_out, n0 + c * kGemmBox, vbase, stg);
+                    tma_store_commit();
                 }
-                __syncwarp();
+                box = box + 1 == kGemmBoxes ? 0 : box + 1;
             }
             tc_fence_before();
             __syncwarp();
-            if (lane == 0) mbar_arrive(&sh.acc_empty[acc]);
+            if (lane == 0) mbar_arrive_remote(&sh.acc_empty[acc], 0);
         }
+        if (lane == 0) tma_store_wait<0, false>();
     }
+    __syncwarp();
 
+    // leaving early: loads and MMAs in flight, whose barriers may be the neighbour's, have landed before either
+    // block goes away
     tc_fence_before();
     __syncthreads();
+    if (*abort) {
+        const long long t0 = clock64();
+        while (clock64() - t0 < kGemmLeaveCycles) {}
+    }
+    cluster.sync();
+    tc_fence_after();
     if (warp == 1) tmem_dealloc(tmem, kGemmTmemCols);
 }
 
