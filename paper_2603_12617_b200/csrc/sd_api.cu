@@ -10,6 +10,7 @@
 
 #include "sd_kernels.cuh"
 #include "sd_sweep.cuh"
+#include "sd_held.cuh"
 #include "sd_greedy.cuh"
 #include "sd_errpos.cuh"
 #include "sd_lmhead.cuh"
@@ -163,7 +164,10 @@ struct StageSet {
 };
 
 struct DeviceState {
-    DeviceState() { for (auto& row : max_clusters) for (int& v : row) v = -1; }
+    DeviceState() {
+        for (auto& row : max_clusters) for (int& v : row) v = -1;
+        for (auto& t : held_clusters) for (auto& row : t) for (int& v : row) v = -1;
+    }
     std::mutex mu;
     bool probed = false;
     int cc_major = 0;
@@ -186,6 +190,8 @@ struct DeviceState {
     // together they have less than four times the bytes of ws, and the 64th would be larger than the GPU.
     void* ws_retired[64] = {};
     int n_retired = 0;
+    bool held_attr[2][kHeldMaxRegions][4] = {};                   // sd_held_kernel may have large clusters
+    int held_clusters[2][kHeldMaxRegions][kHeldMaxCluster + 1];   // resident clusters of sd_held_kernel, -1 = not asked yet
     bool attr_set[2][4] = {};   // shared-memory / cluster attributes of the fast kernels
     int max_clusters[2][kMaxCluster + 1];   // resident clusters of 1..8 blocks, -1 = not asked yet
     // last launch-shape decision of the fast path
@@ -301,6 +307,94 @@ bool use_ragged_sweeps(const void* D, const void* grad, const void* hint, long l
         return false;
     const long long longer = dtype == SD_DTYPE_BF16 ? 8000 + 60 * units : 5000 + 80 * units;
     return V >= longer || units >= 600 || (units >= 180 && units * V >= 1900000);
+}
+
+// ---- the step with the logits held in registers ------------------------------------------------
+struct HeldShape { int C, N; };
+
+// Launches the kernel in clusters of C blocks, or (resident != null) asks how many such clusters the device holds.
+template <int DT, int N, int MODE>
+int launch_held_of(DeviceState& d, const Params& P, int C, HeldCandidate* cand, cudaStream_t stream, int* resident) {
+    auto kern = sd_held_kernel<DT, N, MODE>;
+    cudaLaunchConfig_t cfg;
+    memset(&cfg, 0, sizeof cfg);
+    const unsigned grid = (unsigned)(resident ? C : (MODE == kHeldEnsemble ? P.B * P.k * P.learners : P.B * (P.k + 1)) * C);
+    cfg.gridDim = dim3(grid, 1, 1);
+    cfg.blockDim = dim3(kHeldThreads, 1, 1);
+    cfg.stream = stream;
+    cudaLaunchAttribute attr[2];
+    attr[0].id = cudaLaunchAttributeClusterDimension;
+    attr[0].val.clusterDim.x = (unsigned)C;
+    attr[0].val.clusterDim.y = 1;
+    attr[0].val.clusterDim.z = 1;
+    attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[1].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = resident ? 1 : 2;
+    if (!d.held_attr[DT][N - 1][MODE]) {
+        SD_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
+        d.held_attr[DT][N - 1][MODE] = true;
+    }
+    if (resident) {
+        if (cudaOccupancyMaxActiveClusters(resident, kern, &cfg) != cudaSuccess) {
+            (void)cudaGetLastError();
+            *resident = 0;
+        }
+        return SD_OK;
+    }
+    SD_CUDA(cudaLaunchKernelEx(&cfg, kern, P, cand));
+    tl_info[0] = 1; tl_info[1] = C; tl_info[2] = kHeldThreads; tl_info[3] = (int)sizeof(HeldShared);
+    tl_info[4] = (int)grid; tl_info[5] = 1;
+    return SD_OK;
+}
+template <int MODE>
+int launch_held(DeviceState& d, const Params& P, const HeldShape& h, int dtype, HeldCandidate* cand, cudaStream_t stream, int* resident = nullptr) {
+    if (dtype == SD_DTYPE_F32) {
+        switch (h.N) {
+            case 1: return launch_held_of<SD_DTYPE_F32, 1, MODE>(d, P, h.C, cand, stream, resident);
+            case 2: return launch_held_of<SD_DTYPE_F32, 2, MODE>(d, P, h.C, cand, stream, resident);
+            case 3: return launch_held_of<SD_DTYPE_F32, 3, MODE>(d, P, h.C, cand, stream, resident);
+            default: return launch_held_of<SD_DTYPE_F32, 4, MODE>(d, P, h.C, cand, stream, resident);
+        }
+    }
+    switch (h.N) {
+        case 1: return launch_held_of<SD_DTYPE_BF16, 1, MODE>(d, P, h.C, cand, stream, resident);
+        case 2: return launch_held_of<SD_DTYPE_BF16, 2, MODE>(d, P, h.C, cand, stream, resident);
+        case 3: return launch_held_of<SD_DTYPE_BF16, 3, MODE>(d, P, h.C, cand, stream, resident);
+        default: return launch_held_of<SD_DTYPE_BF16, 4, MODE>(d, P, h.C, cand, stream, resident);
+    }
+}
+
+// The candidates of sd_held_kernel lie where other kernels have the region masses.
+bool held_room(const WorkspaceLayout& L) { return L.slices > 0 || L.NRmax * sizeof(float) >= sizeof(HeldCandidate); }
+
+// Does a call of `units` rows take sd_held_kernel, and in which shape?  The fewest regions a warp with which every
+// cluster is resident at once (the more SMs, the sooner the rows are there; clusters of more than 11 blocks start
+// and meet late, so they are left to rows that need them); if the clusters need a second round, the most
+// regions a warp, and only where the call would go to the cluster kernel otherwise (`second`).  In us, cluster
+// kernel (start) / here, calls back to back on inputs from HBM:
+//     one round   1 sequence, 4 tokens, 32 000 fp32 16.6 / 9.6;  8, 5, 32 000 bf16 23.0 / 12.3;  1, 4, 128 256 bf16
+//                 20.6 / 12.6, in clusters of 16 with one region a warp 14.8;  4, 5, 128 256 bf16 28.4 / 16.8;
+//                 3, 2, 152 064 fp32 22.9 / 13.2
+//     two rounds  8, 5, 128 256 bf16 35.0 / 29.0;  16, 5, 50 304 bf16 29.1 / 27.6;  32, 4, 32 000 bf16 32.9 / 27.7
+//     three       8, 5, 128 256 fp32 39.1 / 41.2
+// Options that only the cluster kernel has, off their defaults, choose the cluster kernel.
+bool use_held(DeviceState& d, int V, long long units, int dtype, bool second, HeldShape* h) {
+    if (option(SD_OPT_CLUSTER) != 0 || option(SD_OPT_LAG) != -1 || option(SD_OPT_PREFETCH) != 0 ||
+        option(SD_OPT_L2_BUDGET_MIB) != kL2BudgetMiB || option(SD_OPT_WAIT_POLLS) != (long long)kWaitLimit)
+        return false;
+    const int NR = (V / vec_elems(dtype) + kRegionVecs - 1) / kRegionVecs;
+    Params none;
+    memset(&none, 0, sizeof none);
+    for (int N = 1; N <= kHeldMaxRegions; ++N) {
+        const int C = (NR + kHeldWarps * N - 1) / (kHeldWarps * N);
+        if (C > (N < kHeldMaxRegions ? 11 : kHeldMaxCluster)) continue;
+        int& n = d.held_clusters[dtype][N - 1][C];
+        h->C = C; h->N = N;
+        if (n < 0 && launch_held<kHeldStep>(d, none, *h, dtype, nullptr, nullptr, &n) != SD_OK) n = 0;
+        if (units <= n || (second && N == kHeldMaxRegions && units <= 2LL * n)) return true;
+    }
+    return false;
 }
 
 // Launch of a kernel whose blocks come as those of the kernel before it on the stream go.
@@ -519,11 +613,22 @@ int run_device(DeviceState& d, const void* T, const void* D, const int32_t* x, c
                       (!hint || aligned(hint, 16)) && option(SD_OPT_FORCE_GENERIC) == 0;
     const long long units = (long long)B * (k + 1);
     const bool ragged = !fast && L.slices > 0 && use_ragged_sweeps(D, grad, hint, units, V, dtype);
-    const bool sweeps = ragged || (fast && use_sweeps(d, dtype, (double)B * (2 * k + 1) * (double)row_bytes, units, V, L.slices));
-    // (the counters of the sweeps must be zero even if a wait has given up on this scratch)
-    if (!head.zero || (sweeps && head.waited)) {
+    bool sweeps = ragged || (fast && use_sweeps(d, dtype, (double)B * (2 * k + 1) * (double)row_bytes, units, V, L.slices));
+    HeldShape held;
+    const bool holds = fast && held_room(L) && use_held(d, V, units, dtype, !sweeps, &held);
+    if (holds) sweeps = false;
+    // (the counters of the sweeps, and the tickets, must be zero even if a wait has given up on this scratch)
+    if (!head.zero || ((sweeps || holds) && head.waited)) {
         SD_CUDA(cudaMemsetAsync(ws, 0, L.accept, stream));   // tickets, status words, sticky flag, counters
         head.waited = false;
+    }
+    if (holds) {
+        // (the status words are written at the end of a sequence)
+        P.tickets = 2u * (uint32_t)(k + 1);
+        P.RE = kRegionVecs * vec_elems(dtype);
+        P.NR = (V + P.RE - 1) / P.RE;
+        HeldCandidate* cand = reinterpret_cast<HeldCandidate*>(ws + L.region_sums);
+        return hint ? launch_held<kHeldHint>(d, P, held, dtype, cand, stream) : launch_held<kHeldStep>(d, P, held, dtype, cand, stream);
     }
     if (sweeps) {
         // (the status words are cleared by the rows kernel)
@@ -863,14 +968,19 @@ int sd_ensemble_feedback(const void* target_logits, const void* const* draft_log
         P.Dn[n] = draft_logits[n];
         P.Gn[n] = out_grad ? out_grad[n] : nullptr;
     }
-    int G = 0, lag = 0, per = 0;
-    const int C = choose_stream(*d, V, (long long)B * k * n_learners, dtype, &G, &per, &lag);
-    if (C <= 0) return SD_ERR_CUDA;
-    P.blocks_per_unit = C;
-    P.RE = per * vec_elems(dtype);
+    P.RE = kRegionVecs * vec_elems(dtype);
     P.NR = (V + P.RE - 1) / P.RE;
-    rc = dtype == SD_DTYPE_F32 ? launch_stream<SD_DTYPE_F32, true>(*d, P, C, G, lag, st, false, nullptr)
-                               : launch_stream<SD_DTYPE_BF16, true>(*d, P, C, G, lag, st, false, nullptr);
+    HeldShape held;
+    if (use_held(*d, V, (long long)B * k * n_learners, dtype, true, &held)) {
+        rc = launch_held<kHeldEnsemble>(*d, P, held, dtype, nullptr, st);
+    } else {
+        int G = 0, lag = 0, per = 0;
+        const int C = choose_stream(*d, V, (long long)B * k * n_learners, dtype, &G, &per, &lag);
+        if (C <= 0) return SD_ERR_CUDA;
+        P.blocks_per_unit = C;
+        rc = dtype == SD_DTYPE_F32 ? launch_stream<SD_DTYPE_F32, true>(*d, P, C, G, lag, st, false, nullptr)
+                                   : launch_stream<SD_DTYPE_BF16, true>(*d, P, C, G, lag, st, false, nullptr);
+    }
     if (rc != SD_OK) return rc;
     sd_hedge_kernel<<<1, 256, 0, st>>>(out_loss, n_learners, (long long)B * k, (double)epsilon, cum_loss_in,
                                        out_round_loss, out_cum_loss, out_weights, P.sticky, out_status, B);
@@ -930,8 +1040,11 @@ int sd_verify_error_feedback(const void* target_logits, const void* draft_logits
     const long long units = (long long)B * (k + 1);
     P.RE = kRegionVecs * vec_elems(dtype);
     P.NR = (V + P.RE - 1) / P.RE;
-    // (the rule of the full step, so that both give the same bits)
-    if (use_sweeps(*d, dtype, (double)B * (2 * k + 1) * (double)row_bytes, units, V, L.slices)) {
+    // (the rules of the full step, so that both give the same bits)
+    const bool sweeps = use_sweeps(*d, dtype, (double)B * (2 * k + 1) * (double)row_bytes, units, V, L.slices);
+    HeldShape held;
+    const bool holds = held_room(L) && use_held(*d, V, units, dtype, !sweeps, &held);
+    if (sweeps && !holds) {
         Sweep S;
         S.slices = L.slices;
         S.part = reinterpret_cast<PartialStats*>(ws + L.part);
@@ -944,13 +1057,17 @@ int sd_verify_error_feedback(const void* target_logits, const void* draft_logits
         tl_info[0] = 4;
         return SD_OK;
     }
-    if (out_status) SD_CUDA(cudaMemsetAsync(out_status, 0, (size_t)B * 4, st));   // bits are ORed in on the device
-    int G = 0, lag = 0, per = 0;
-    const int C = choose_stream(*d, V, units, dtype, &G, &per, &lag);
-    if (C <= 0) return SD_ERR_CUDA;
-    P.blocks_per_unit = C;
-    rc = dtype == SD_DTYPE_F32 ? launch_stream<SD_DTYPE_F32, false, true>(*d, P, C, G, lag, st, false, nullptr)
-                               : launch_stream<SD_DTYPE_BF16, false, true>(*d, P, C, G, lag, st, false, nullptr);
+    if (holds) {
+        rc = launch_held<kHeldErrors>(*d, P, held, dtype, nullptr, st);      // (clears the status words)
+    } else {
+        if (out_status) SD_CUDA(cudaMemsetAsync(out_status, 0, (size_t)B * 4, st));   // bits are ORed in on the device
+        int G = 0, lag = 0, per = 0;
+        const int C = choose_stream(*d, V, units, dtype, &G, &per, &lag);
+        if (C <= 0) return SD_ERR_CUDA;
+        P.blocks_per_unit = C;
+        rc = dtype == SD_DTYPE_F32 ? launch_stream<SD_DTYPE_F32, false, true>(*d, P, C, G, lag, st, false, nullptr)
+                                   : launch_stream<SD_DTYPE_BF16, false, true>(*d, P, C, G, lag, st, false, nullptr);
+    }
     if (rc != SD_OK) return rc;
     const int slices = (P.NR + kErrSliceRegions - 1) / kErrSliceRegions;
     const unsigned grid = (unsigned)B * (unsigned)slices;

@@ -155,6 +155,11 @@ __device__ __forceinline__ int total_units(const Params& P) {
     return ENS ? P.B * P.k * P.learners : P.B * (P.k + 1);
 }
 
+// Programmatic dependent launch: let the next kernel's blocks come as soon as there is room / wait until
+// the kernel before has finished and its writes are visible.
+__device__ __forceinline__ void launch_dependents() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+__device__ __forceinline__ void await_previous_kernel() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+
 // ------------------------------------------------------------------------------------------
 // element types
 template <int DT> struct Elem;
@@ -446,6 +451,23 @@ __device__ __forceinline__ PartialStats warp_sum_lanes(const LaneSums& ls, float
     r.RT = RT; r.RD = RD;
     r.sT = dT; r.sD = dD; r.w = dW;
     return r;
+}
+
+// The same in fewer exchanges: sT in lanes 0-7, sD in 8-15 and 24-31, w in 16-23.  The three sums are folded into
+// one register pair on the way (a lane keeps what its half of the warp is responsible for): 6 exchanges of a
+// double instead of 15.
+__device__ __forceinline__ double warp_fold_lanes(const LaneSums& ls, int lane) {
+    const double T = (double)ls.sT, W = (double)ls.w;
+    double D = (double)ls.sD;
+    const bool hi = (lane & 16) != 0, odd = (lane & 8) != 0;
+    double a = hi ? W : T;
+    a += shfl_xor_f64(hi ? T : W, 16);       // lanes 0-15: T, lanes 16-31: W
+    D += shfl_xor_f64(D, 16);                // both halves: D
+    double v = odd ? D : a;
+    v += shfl_xor_f64(odd ? a : D, 8);       // lanes 0-7: T, 16-23: W, 8-15 and 24-31: D
+#pragma unroll
+    for (int off = 4; off > 0; off >>= 1) v += shfl_xor_f64(v, off);
+    return v;
 }
 
 // ------------------------------------------------------------------------------------------

@@ -58,25 +58,9 @@ __device__ __forceinline__ uint4 load_l2(const uint4* p, uint64_t policy) {
                  : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "l"(p), "l"(policy));
     return v;
 }
-// Programmatic dependent launch: let the next kernel's blocks come as soon as there is room / wait until
-// the kernel before has finished and its writes are visible.
-__device__ __forceinline__ void launch_dependents() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
-__device__ __forceinline__ void await_previous_kernel() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
-
 // Sums of the lanes of a warp that share the references (RT, RD) into *out, in fp64 and a fixed order.
-// The three sums are folded into one register pair on the way (a lane keeps what its half of the warp is
-// responsible for): 6 exchanges of a double instead of the 15 of warp_sum_lanes.
 __device__ __forceinline__ void warp_post_lanes(const LaneSums& ls, float RT, float RD, int lane, PartialStats* out) {
-    const double T = (double)ls.sT, W = (double)ls.w;
-    double D = (double)ls.sD;
-    const bool hi = (lane & 16) != 0, odd = (lane & 8) != 0;
-    double a = hi ? W : T;
-    a += shfl_xor_f64(hi ? T : W, 16);       // lanes 0-15: T, lanes 16-31: W
-    D += shfl_xor_f64(D, 16);                // both halves: D
-    double v = odd ? D : a;
-    v += shfl_xor_f64(odd ? a : D, 8);       // lanes 0-7: T, 16-23: W, 8-15 and 24-31: D
-#pragma unroll
-    for (int off = 4; off > 0; off >>= 1) v += shfl_xor_f64(v, off);
+    const double v = warp_fold_lanes(ls, lane);
     if (lane == 0) { out->RT = RT; out->RD = RD; out->sT = v; }
     if (lane == 8) out->sD = v;
     if (lane == 16) out->w = v;
