@@ -415,8 +415,7 @@ cudaError_t launch_following(K kern, dim3 grid, int threads, cudaStream_t stream
 
 template <int DT, int MODE, bool RAGGED = false>
 int launch_sweeps_of(const Params& P, const Sweep& S, long long units, bool all, cudaStream_t stream) {
-    sd_sweep_stats_kernel<DT, RAGGED><<<dim3((unsigned)units, (unsigned)S.slices), kSweepThreads, 0, stream>>>(P, S);
-    SD_CUDA(cudaGetLastError());
+    SD_CUDA(launch_following(sd_sweep_stats_kernel<DT, RAGGED>, dim3((unsigned)units, (unsigned)S.slices), kSweepThreads, stream, P, S));
     SD_CUDA(launch_following(sd_sweep_rows_kernel<DT>, dim3((unsigned)P.B), kSweepThreads, stream, P, S));
     // the rows that are drawn from, then (if anything of them is wanted) all rows
     const unsigned second = (unsigned)S.draw_blocks + (all ? (unsigned)(units * S.slices) : 0u);
@@ -1071,9 +1070,8 @@ int sd_verify_error_feedback(const void* target_logits, const void* draft_logits
     if (rc != SD_OK) return rc;
     const int slices = (P.NR + kErrSliceRegions - 1) / kErrSliceRegions;
     const unsigned grid = (unsigned)B * (unsigned)slices;
-    if (dtype == SD_DTYPE_F32) sd_errpos_kernel<SD_DTYPE_F32><<<grid, kErrThreads, 0, st>>>(P, slices);
-    else                       sd_errpos_kernel<SD_DTYPE_BF16><<<grid, kErrThreads, 0, st>>>(P, slices);
-    SD_CUDA(cudaGetLastError());
+    SD_CUDA(dtype == SD_DTYPE_F32 ? launch_following(sd_errpos_kernel<SD_DTYPE_F32>, dim3(grid), kErrThreads, st, P, slices)
+                                  : launch_following(sd_errpos_kernel<SD_DTYPE_BF16>, dim3(grid), kErrThreads, st, P, slices));
     tl_info[0] = 4; tl_info[5] = 2;
     return SD_OK;
 }
@@ -1135,9 +1133,8 @@ int sd_verify_greedy(const void* target_logits, const int32_t* draft_tokens, int
     if (per_sm < 1 || per_sm > 8) per_sm = 4;
     const long long cap = (long long)d->sm_count * per_sm;
     const unsigned grid = (unsigned)(items < cap ? items : cap);
-    if (dtype == SD_DTYPE_F32) sd_greedy_kernel<SD_DTYPE_F32><<<grid, kGreedyThreads, 0, st>>>(P);
-    else                       sd_greedy_kernel<SD_DTYPE_BF16><<<grid, kGreedyThreads, 0, st>>>(P);
-    SD_CUDA(cudaGetLastError());
+    SD_CUDA(dtype == SD_DTYPE_F32 ? launch_following(sd_greedy_kernel<SD_DTYPE_F32>, dim3(grid), kGreedyThreads, st, P)
+                                  : launch_following(sd_greedy_kernel<SD_DTYPE_BF16>, dim3(grid), kGreedyThreads, st, P));
     if (!workspace) keep_scratch(d, known, head);
     tl_info[0] = 2; tl_info[1] = 1; tl_info[2] = kGreedyThreads; tl_info[3] = 0;
     tl_info[4] = (int)grid; tl_info[5] = 1;
@@ -1322,9 +1319,8 @@ int sd_vp_partial(const void* target_shard, const void* draft_shard, const int32
     P.records = static_cast<VpRecord*>(out_records);
     const unsigned units = (unsigned)B * (unsigned)(k + 1);
     cudaStream_t st = static_cast<cudaStream_t>(stream);
-    if (dtype == SD_DTYPE_F32) sd_vp_stats_kernel<SD_DTYPE_F32><<<units, kVpThreads, 0, st>>>(P);
-    else                       sd_vp_stats_kernel<SD_DTYPE_BF16><<<units, kVpThreads, 0, st>>>(P);
-    SD_CUDA(cudaGetLastError());
+    SD_CUDA(dtype == SD_DTYPE_F32 ? launch_following(sd_vp_stats_kernel<SD_DTYPE_F32>, dim3(units), kVpThreads, st, P)
+                                  : launch_following(sd_vp_stats_kernel<SD_DTYPE_BF16>, dim3(units), kVpThreads, st, P));
     tl_info[0] = 6; tl_info[1] = 1; tl_info[2] = kVpThreads; tl_info[3] = 0; tl_info[4] = (int)units; tl_info[5] = 1;
     return SD_OK;
 }
@@ -1356,10 +1352,9 @@ int sd_vp_finish(const void* target_shard, const void* draft_shard, const int32_
     P.status = out_status;
     P.local_mass = out_local_mass;
     cudaStream_t st = static_cast<cudaStream_t>(stream);
-    sd_vp_rows_kernel<<<(unsigned)B, 96, 0, st>>>(P);
+    SD_CUDA(launch_following(sd_vp_rows_kernel, dim3((unsigned)B), 96, st, P));
     const int slices = (P.NR + kVpSliceRegions - 1) / kVpSliceRegions;
     const unsigned grid = (unsigned)B * (unsigned)(k + 1) * (unsigned)slices;
-    SD_CUDA(cudaGetLastError());
     SD_CUDA(dtype == SD_DTYPE_F32 ? launch_following(sd_vp_grad_kernel<SD_DTYPE_F32>, dim3(grid), kVpThreads, st, P, slices)
                                   : launch_following(sd_vp_grad_kernel<SD_DTYPE_BF16>, dim3(grid), kVpThreads, st, P, slices));
     SD_CUDA(launch_following(sd_vp_mass_kernel, dim3((unsigned)B), 32, st, P));
@@ -1389,9 +1384,8 @@ int sd_vp_draw(const void* target_shard, const void* draft_shard, const int32_t*
     P.tokens = out_tokens;
     P.status = out_status;
     cudaStream_t st = static_cast<cudaStream_t>(stream);
-    if (dtype == SD_DTYPE_F32) sd_vp_draw_kernel<SD_DTYPE_F32><<<(unsigned)B, 32, 0, st>>>(P);
-    else                       sd_vp_draw_kernel<SD_DTYPE_BF16><<<(unsigned)B, 32, 0, st>>>(P);
-    SD_CUDA(cudaGetLastError());
+    SD_CUDA(dtype == SD_DTYPE_F32 ? launch_following(sd_vp_draw_kernel<SD_DTYPE_F32>, dim3((unsigned)B), 32, st, P)
+                                  : launch_following(sd_vp_draw_kernel<SD_DTYPE_BF16>, dim3((unsigned)B), 32, st, P));
     tl_info[0] = 6; tl_info[5] = 1;
     return SD_OK;
 }

@@ -29,6 +29,8 @@ __global__ void __launch_bounds__(kErrThreads, 4) sd_errpos_kernel(const __grid_
     constexpr int kGroups = kRegionRows;            // a region is kRegionRows x 32 vectors, as in the streaming kernel
     __shared__ int is_last;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    await_previous_kernel();
+    launch_dependents();
     const int b = (int)blockIdx.x / slices, sl = (int)blockIdx.x - b * slices;
     const int k = P.k;
 

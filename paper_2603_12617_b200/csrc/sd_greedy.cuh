@@ -96,6 +96,8 @@ __global__ void __launch_bounds__(kGreedyThreads, 4) sd_greedy_kernel(const Gree
     constexpr int VEC = E::VEC;
     __shared__ int is_last;
     __shared__ int am_sh[kGreedyTailRows], x_sh[kGreedyTailRows];
+    await_previous_kernel();
+    launch_dependents();
     const int tid = threadIdx.x, lane = tid & 31;
     const int K1 = P.k + 1;
     const long long items = (long long)P.B * K1 * P.items_per_row;

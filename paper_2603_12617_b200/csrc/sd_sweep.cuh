@@ -295,6 +295,7 @@ sd_sweep_stats_kernel(const __grid_constant__ Params P, const __grid_constant__ 
     using ET = typename E::type;
     __shared__ PartialStats wpart[kSweepWarps];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    await_previous_kernel();                         // (first: the rows kernel reads inputs before its own wait)
     launch_dependents();
     const int unit = blockIdx.x, slice = blockIdx.y;
     const UnitRef ur = unit_ref<false>(P, unit);
@@ -436,6 +437,7 @@ sd_sweep_grad_kernel(const __grid_constant__ Params P, const __grid_constant__ S
         b = unit / (P.k + 1);
     }
     await_previous_kernel();
+    launch_dependents();
 
     if (!SD_IN(b, P.B, 22)) return;
     // the first rejected position of the sequence

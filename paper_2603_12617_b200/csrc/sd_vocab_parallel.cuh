@@ -84,6 +84,8 @@ __global__ void __launch_bounds__(kVpThreads, 4) sd_vp_stats_kernel(const VpPara
     using ET = typename E::type;
     constexpr int VEC = E::VEC;
     __shared__ PartialStats warp_part[kVpWarps];
+    await_previous_kernel();
+    launch_dependents();
     const int unit = blockIdx.x;
     const int K1 = P.k + 1;
     const int b = unit / K1, i = unit - b * K1;
@@ -131,6 +133,7 @@ __global__ void __launch_bounds__(kVpThreads, 4) sd_vp_stats_kernel(const VpPara
 __global__ void __launch_bounds__(96) sd_vp_rows_kernel(const VpParams P) {
     __shared__ int accepted[SD_MAX_K + 1];
     __shared__ uint32_t flags_sh;
+    await_previous_kernel();
     launch_dependents();
     const int b = blockIdx.x, i = threadIdx.x;
     const int K1 = P.k + 1;
@@ -271,6 +274,7 @@ __global__ void __launch_bounds__(32) sd_vp_mass_kernel(const VpParams P) {
     const int per = (P.NR + 31) / 32;
     const int j0 = min(P.NR, lane * per), j1 = min(P.NR, j0 + per);
     await_previous_kernel();
+    launch_dependents();
     for (int which = 0; which < 2; ++which) {
         const float* rs = P.region_sums + ((size_t)b * 2 + which) * P.NR;
         double mine = 0.0;
@@ -288,6 +292,8 @@ __global__ void __launch_bounds__(32) sd_vp_draw_kernel(const VpParams P) {
     constexpr int PER = kRegionVecs * Elem<DT>::VEC / 32;
     const int b = blockIdx.x, lane = threadIdx.x;
     const int k = P.k, K1 = k + 1;
+    await_previous_kernel();
+    launch_dependents();
     const int n = P.accept_len[b];
     const bool bonus = (n == k);
     uint32_t flags = 0;
