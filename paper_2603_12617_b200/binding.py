@@ -1,13 +1,19 @@
-"""Thin ctypes binding of the C ABI in ``include/sd_verify.h``.
+"""Thin binding of the C ABI in ``include/sd_verify.h``.
 
 Argument marshalling only: every step of the verify-and-feedback path runs in the CUDA library.
 torch is used for device memory, streams and nothing else.  The functions have the names of the
-C entry points.  If the shared library is missing or cannot be loaded the import of this module
+C entry points.  If a shared library is missing or cannot be loaded the import of this module
 fails: there is no fallback.
+
+A call goes through ctypes; the hot entry points first ask ``csrc/sd_native.cpp``, which does the
+same for plain tensors on the current device without the interpreter in between and answers None to
+everything else.
 """
 from __future__ import annotations
 
 import ctypes
+import importlib.machinery
+import importlib.util
 import os
 from dataclasses import dataclass
 from typing import Optional
@@ -106,6 +112,23 @@ def _load() -> ctypes.CDLL:
 
 
 _lib = _load()
+
+
+def _load_native():
+    path = os.path.join(_HERE, "lib", "sd_native.so")
+    if not os.path.exists(path):
+        raise ImportError(f"{path} is missing: build it with `python -c 'import __graft_entry__ as g; g.build()'`")
+    loader = importlib.machinery.ExtensionFileLoader("sd_native", path)
+    module = importlib.util.module_from_spec(importlib.util.spec_from_file_location("sd_native", path, loader=loader))
+    loader.exec_module(module)
+    # the entry points of the library that was loaded above, in the order of its struct Library
+    module.bind(*[ctypes.cast(fn, ctypes.c_void_p).value for fn in (
+        _lib.sd_verify_feedback, _lib.sd_verify_feedback_bf16, _lib.sd_verify_greedy, _lib.sd_verify_error_feedback,
+        _lib.sd_verify_feedback_hint, _lib.sd_ensemble_feedback, _lib.sd_lmhead_grad, _lib.sd_vp_partial, _lib.sd_vp_finish, _lib.sd_vp_draw)])
+    return module
+
+
+_native = _load_native()
 
 
 @dataclass
@@ -228,6 +251,12 @@ def sd_verify_feedback(target_logits: torch.Tensor, draft_logits: torch.Tensor,
                        out: Optional[StepOutputs] = None,
                        stream: Optional[torch.cuda.Stream] = None) -> StepOutputs:
     """``sd_verify_feedback`` / ``sd_verify_feedback_bf16`` on device tensors (library scratch)."""
+    if out is None and stream is None:
+        r = _native.step(target_logits, draft_logits, draft_tokens, uniforms, temperature, bool(want_loss), bool(want_grad))
+        if r is not None:
+            if r[0] != 0:
+                raise SdVerifyError(r[0], "sd_verify_feedback")
+            return StepOutputs(r[1], r[2], r[3], r[4])
     B, k, V = _shapes(target_logits, draft_logits, draft_tokens, uniforms)
     dev = target_logits.device
     if dev.type != "cuda":
@@ -290,6 +319,12 @@ def sd_verify_feedback_hint(target_logits: torch.Tensor, draft_logits: torch.Ten
                             stream: Optional[torch.cuda.Stream] = None) -> StepOutputs:
     """``sd_verify_feedback_hint``: the step plus sum_v (hint - gradient)^2 per position.  ``grad_out``
     may be ``hint`` itself (the gradient then replaces the hint in place)."""
+    if grad_out is None and workspace is not None and stream is None:
+        r = _native.hint(target_logits, draft_logits, draft_tokens, uniforms, temperature, hint, workspace)
+        if r is not None:
+            if r[0] != 0:
+                raise SdVerifyError(r[0], "sd_verify_feedback_hint")
+            return StepOutputs(r[1], r[2], r[3], r[4], status=r[5], hint_err=r[6])
     B, k, V = _shapes(target_logits, draft_logits, draft_tokens, uniforms)
     if tuple(hint.shape) != (B, k, V) or hint.dtype != draft_logits.dtype or not hint.is_contiguous():
         raise ValueError("hint must be a contiguous [B,k,V] tensor of the logits' dtype")
@@ -330,6 +365,12 @@ def sd_verify_greedy(target_logits: torch.Tensor, draft_tokens: torch.Tensor, *,
                      workspace: Optional[torch.Tensor] = None, out: Optional[GreedyOutputs] = None,
                      stream: Optional[torch.cuda.Stream] = None) -> GreedyOutputs:
     """``sd_verify_greedy`` on device tensors: accept iff the draft token is the target's argmax."""
+    if out is None and workspace is None and stream is None:
+        r = _native.greedy(target_logits, draft_tokens, bool(want_argmax))
+        if r is not None:
+            if r[0] != 0:
+                raise SdVerifyError(r[0], "sd_verify_greedy")
+            return GreedyOutputs(r[1], r[2], r[3])
     if target_logits.dim() != 3 or not target_logits.is_contiguous():
         raise ValueError("target logits must be contiguous [B,k+1,V]")
     B, k1, V = target_logits.shape
@@ -369,6 +410,13 @@ def sd_verify_error_feedback(target_logits: torch.Tensor, draft_logits: torch.Te
                              out: Optional[ErrorFeedbackOutputs] = None,
                              stream: Optional[torch.cuda.Stream] = None) -> ErrorFeedbackOutputs:
     """``sd_verify_error_feedback`` on device tensors (library scratch)."""
+    if out is None and stream is None:
+        r = _native.errors(target_logits, draft_logits, draft_tokens, uniforms, temperature, bool(want_loss), bool(want_grad),
+                           bool(want_status))
+        if r is not None:
+            if r[0] != 0:
+                raise SdVerifyError(r[0], "sd_verify_error_feedback")
+            return ErrorFeedbackOutputs(r[1], r[2], r[3], r[4], r[5])
     B, k, V = _shapes(target_logits, draft_logits, draft_tokens, uniforms)
     dev = target_logits.device
     if dev.type != "cuda":
@@ -406,6 +454,12 @@ def sd_ensemble_feedback(target_logits: torch.Tensor, draft_logits, temperature:
                          want_status: bool = False, out: Optional[EnsembleOutputs] = None,
                          stream: Optional[torch.cuda.Stream] = None) -> EnsembleOutputs:
     """``sd_ensemble_feedback`` on device tensors: N draft logit sets against one target."""
+    if out is None and stream is None:
+        r = _native.ensemble(target_logits, draft_logits, temperature, epsilon, cum_loss, bool(want_grad), bool(want_status))
+        if r is not None:
+            if r[0] != 0:
+                raise SdVerifyError(r[0], "sd_ensemble_feedback")
+            return EnsembleOutputs(r[1], r[2], r[3], r[4], r[5], r[6])
     if target_logits.dim() != 3 or not target_logits.is_contiguous():
         raise ValueError("target logits must be contiguous [B,k+1,V]")
     B, k1, V = target_logits.shape
@@ -444,6 +498,12 @@ def sd_lmhead_grad(grad_logits: torch.Tensor, hidden: torch.Tensor, *, out: Opti
                    status: Optional[torch.Tensor] = None, stream: Optional[torch.cuda.Stream] = None) -> torch.Tensor:
     """``sd_lmhead_grad``: dW = g^T X for g [R,V] (or [B,k,V]) and X [R,d], both bfloat16 on the device;
     returns dW [V,d] float32."""
+    if out is None and status is None and stream is None:
+        r = _native.lmhead(grad_logits, hidden)
+        if r is not None:
+            if r[0] != 0:
+                raise SdVerifyError(r[0], "sd_lmhead_grad")
+            return r[1]
     if grad_logits.dim() == 3:
         grad_logits = grad_logits.reshape(-1, grad_logits.shape[-1])
     if grad_logits.dim() != 2 or hidden.dim() != 2 or grad_logits.shape[0] != hidden.shape[0]:
@@ -495,6 +555,12 @@ def sd_vp_partial(target_shard: torch.Tensor, draft_shard: torch.Tensor, draft_t
                   temperature: float, v_offset: int, V_total: int, workspace: torch.Tensor, *,
                   out_records: Optional[torch.Tensor] = None, stream: Optional[torch.cuda.Stream] = None) -> torch.Tensor:
     """Phase 1 of the vocabulary-parallel step: this shard's record of every row, [B*(k+1), 48] bytes."""
+    if stream is None:
+        r = _native.vp_partial(target_shard, draft_shard, draft_tokens, temperature, v_offset, V_total, workspace, out_records)
+        if r is not None:
+            if r[0] != 0:
+                raise SdVerifyError(r[0], "sd_vp_partial")
+            return r[1] if out_records is None else out_records
     B, k, Vs = _vp_shapes(target_shard, draft_shard, draft_tokens)
     if out_records is None:
         out_records = torch.empty((B * (k + 1), SD_VP_RECORD_BYTES), dtype=torch.uint8, device=target_shard.device)
@@ -520,6 +586,13 @@ def sd_vp_finish(target_shard: torch.Tensor, draft_shard: torch.Tensor, draft_to
                  n_ranks: int, rank: int, workspace: torch.Tensor, *, want_loss: bool = True, want_grad: bool = True,
                  stream: Optional[torch.cuda.Stream] = None) -> VpFinishOutputs:
     """Phase 2: ``all_records`` is the rank-ordered gather [n_ranks, B*(k+1), 48] of phase 1's records."""
+    if stream is None:
+        r = _native.vp_finish(target_shard, draft_shard, draft_tokens, uniforms, temperature, v_offset, V_total, all_records,
+                              n_ranks, rank, workspace, bool(want_loss), bool(want_grad))
+        if r is not None:
+            if r[0] != 0:
+                raise SdVerifyError(r[0], "sd_vp_finish")
+            return VpFinishOutputs(r[1], r[2], r[3], r[4], r[5])
     B, k, Vs = _vp_shapes(target_shard, draft_shard, draft_tokens)
     if all_records.numel() * all_records.element_size() != n_ranks * B * (k + 1) * SD_VP_RECORD_BYTES:
         raise ValueError("all_records must hold n_ranks * B * (k+1) records")
@@ -544,6 +617,13 @@ def sd_vp_draw(target_shard: torch.Tensor, draft_shard: torch.Tensor, draft_toke
                stream: Optional[torch.cuda.Stream] = None) -> torch.Tensor:
     """Phase 3: ``all_masses`` is the rank-ordered gather [n_ranks, B, 2] of phase 2's shares.  Returns
     tokens [B,k+1] with -1 where another rank's shard holds the extra token."""
+    if stream is None:
+        r = _native.vp_draw(target_shard, draft_shard, draft_tokens, uniforms, temperature, v_offset, V_total, accept_len,
+                            all_masses, n_ranks, rank, status, workspace)
+        if r is not None:
+            if r[0] != 0:
+                raise SdVerifyError(r[0], "sd_vp_draw")
+            return r[1]
     B, k, Vs = _vp_shapes(target_shard, draft_shard, draft_tokens)
     if all_masses.dtype != torch.float64 or all_masses.numel() != n_ranks * B * 2:
         raise ValueError("all_masses must be float64 [n_ranks, B, 2]")
