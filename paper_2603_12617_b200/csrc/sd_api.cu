@@ -981,9 +981,8 @@ int sd_ensemble_feedback(const void* target_logits, const void* const* draft_log
                                    : launch_stream<SD_DTYPE_BF16, true>(*d, P, C, G, lag, st, false, nullptr);
     }
     if (rc != SD_OK) return rc;
-    sd_hedge_kernel<<<1, 256, 0, st>>>(out_loss, n_learners, (long long)B * k, (double)epsilon, cum_loss_in,
-                                       out_round_loss, out_cum_loss, out_weights, P.sticky, out_status, B);
-    SD_CUDA(cudaGetLastError());
+    SD_CUDA(launch_following(sd_hedge_kernel, dim3(1), kHedgeThreads, st, (const float*)out_loss, n_learners, (long long)B * k, (double)epsilon,
+                             cum_loss_in, out_round_loss, out_cum_loss, out_weights, (const uint32_t*)P.sticky, out_status, B));
     tl_info[0] = 3; tl_info[5] = 2;
     return SD_OK;
 }

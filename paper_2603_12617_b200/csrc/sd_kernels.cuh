@@ -1012,42 +1012,52 @@ __global__ void __launch_bounds__(kGenericThreads) sd_generic_kernel(const __gri
 }
 
 // ---- online ensemble ---------------------------------------------------------------------
-// Mean loss of the round per learner (fixed summation order), cumulative losses, Hedge weights.
-__global__ void __launch_bounds__(256) sd_hedge_kernel(const float* loss, int N, long long per, double eps,
-                                                       const double* cum_in, double* round_loss, double* cum_out,
-                                                       float* weights, const uint32_t* sticky, uint32_t* status,
-                                                       int B) {
-    __shared__ double part[256];
-    __shared__ double mean[kMaxLearners];
-    const int tid = threadIdx.x;
-    for (int n = 0; n < N; ++n) {
+// Mean loss of the round per learner (fixed summation order), cumulative losses, Hedge weights.  One block, four
+// warps to a learner with eight loads in flight each, then a lane to a learner: round trips and fp64 exponentials
+// are all it consists of.
+constexpr int kHedgeThreads = kMaxLearners * 4 * 32;
+__global__ void __launch_bounds__(kHedgeThreads) sd_hedge_kernel(const float* loss, int N, long long per, double eps,
+                                                                 const double* cum_in, double* round_loss, double* cum_out,
+                                                                 float* weights, const uint32_t* sticky, uint32_t* status,
+                                                                 int B) {
+    __shared__ double part[kMaxLearners][4];
+    const int tid = threadIdx.x, lane = tid & 31, n = tid >> 7, q = (tid >> 5) & 3;
+    await_previous_kernel();
+    launch_dependents();
+    if (n < N) {
+        const float* const l = loss + (size_t)n * per;
         double s = 0.0;
-        for (long long j = tid; j < per; j += 256) s += (double)loss[(size_t)n * per + j];
-        part[tid] = s;
-        __syncthreads();
-        for (int w = 128; w > 0; w >>= 1) {
-            if (tid < w) part[tid] += part[tid + w];
-            __syncthreads();
+        for (long long j = q * 32 + lane; j < per; j += 8 * 128) {
+            float v[8];
+#pragma unroll
+            for (int z = 0; z < 8; ++z) v[z] = j + z * 128 < per ? l[j + z * 128] : 0.f;
+#pragma unroll
+            for (int z = 0; z < 8; ++z) s += (double)v[z];
         }
-        if (tid == 0) mean[n] = part[0] / (double)per;
-        __syncthreads();
+        s = warp_sum(s);
+        if (lane == 0) part[n][q] = s;
     }
-    if (tid == 0) {
-        double cum[kMaxLearners], lowest = INFINITY, Z = 0.0;
-        for (int n = 0; n < N; ++n) {
-            cum[n] = (cum_in ? cum_in[n] : 0.0) + mean[n];
-            if (cum[n] < lowest) lowest = cum[n];
+    __syncthreads();
+    if (tid < 32) {
+        const int i = min(lane, N - 1);
+        const double mean = ((part[i][0] + part[i][1]) + (part[i][2] + part[i][3])) / (double)per;
+        const double cum = (cum_in ? cum_in[i] : 0.0) + mean;
+        double lowest = INFINITY, Z = 0.0;
+        for (int m = 0; m < N; ++m) {
+            const double c = __shfl_sync(0xffffffffu, cum, m);
+            if (c < lowest) lowest = c;
         }
-        for (int n = 0; n < N; ++n) Z += exp(-eps * (cum[n] - lowest));
-        for (int n = 0; n < N; ++n) {
-            round_loss[n] = mean[n];
-            cum_out[n] = cum[n];
-            weights[n] = (float)(exp(-eps * (cum[n] - lowest)) / Z);
+        const double e = exp(-eps * (cum - lowest));
+        for (int m = 0; m < N; ++m) Z += __shfl_sync(0xffffffffu, e, m);
+        if (lane < N) {
+            round_loss[lane] = mean;
+            cum_out[lane] = cum;
+            weights[lane] = (float)(e / Z);
         }
     }
     // a bounded wait gave up somewhere in the feedback kernel: nothing of this round is valid
     if (status && *sticky != 0)
-        for (int b = tid; b < B; b += 256) atomicOr(status + b, kStatusTimeout);
+        for (int b = tid; b < B; b += kHedgeThreads) atomicOr(status + b, kStatusTimeout);
 }
 
 }  // namespace sdv
