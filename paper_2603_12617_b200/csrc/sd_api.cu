@@ -433,7 +433,20 @@ int launch_sweeps(const Params& P, Sweep& S, long long units, int dtype, cudaStr
     // 74.8).
     const bool all = MODE != kSweepErrors && (P.grad || MODE == kSweepHint || S.all_rows);
     S.kept = all ? (80u << 20) / (unsigned)(S.regions * kRegionVecs * 32) : 0u;
-    S.draw_blocks = P.B * S.slices;
+    // Where the second sweep is the drawn rows alone, its items are as small as leaves every block resident at
+    // once: the time of such a sweep is a chain of round trips, one for each region of a warp.
+    S.draw_regions = S.regions;
+    S.draw_slices = S.slices;
+    if (!all) {
+        for (int r = kSweepWarps; r < S.regions; r += kSweepWarps) {
+            const int s = (P.NR + r - 1) / r;
+            if ((long long)P.B * s > (RAGGED ? 592 : 888)) continue;
+            S.draw_regions = r;
+            S.draw_slices = s;
+            break;
+        }
+    }
+    S.draw_blocks = P.B * S.draw_slices;
     const int rc = dtype == SD_DTYPE_F32 ? launch_sweeps_of<SD_DTYPE_F32, MODE, RAGGED>(P, S, units, all, stream)
                                          : launch_sweeps_of<SD_DTYPE_BF16, MODE, RAGGED>(P, S, units, all, stream);
     if (rc != SD_OK) return rc;

@@ -506,8 +506,8 @@ __device__ __forceinline__ AcceptOperands load_accept_operands(const Params& P, 
 }
 
 // End of a (sequence, row) unit, by one thread: row constants to the workspace, the KL loss and
-// the rejection test of the row's draft token.
-__device__ inline void finish_row(const Params& P, int b, int i, const PartialStats& st, const RowConst& rc,
+// the rejection test of the row's draft token, whose outcome it returns.
+__device__ inline bool finish_row(const Params& P, int b, int i, const PartialStats& st, const RowConst& rc,
                                   const AcceptOperands& op) {
     const bool bonus = (i == P.k);
     const int unit = b * (P.k + 1) + i;
@@ -516,6 +516,7 @@ __device__ inline void finish_row(const Params& P, int b, int i, const PartialSt
     const bool okD = bonus || ((st.sD > 0.0) && isfinite(st.sD));
     if (!okT || !okD) flags |= SD_STATUS_BAD_ROW;
     if (SD_IN(unit, P.B * (P.k + 1), 20)) P.rowc[unit] = rc;
+    bool acc = false;
     if (!bonus) {
         // log2 p_v = aT_v - log2 S_T and log2 q_v = aD_v - log2 S_D, so
         // KL(p||q) = ln2 * [ E_p(aT - aD) - log2 S_T + log2 S_D ]
@@ -525,7 +526,6 @@ __device__ inline void finish_row(const Params& P, int b, int i, const PartialSt
             P.loss[b * P.k + i] = (float)kl;
         }
         // rejection test for draft token x[b,i] with ratio p(x)/q(x) in fp64
-        bool acc = false;
         if (!op.valid) {
             flags |= SD_STATUS_BAD_TOKEN;
         } else if (okT && okD) {
@@ -544,6 +544,7 @@ __device__ inline void finish_row(const Params& P, int b, int i, const PartialSt
         if (SD_IN(b * P.k + i, P.B * P.k, 22)) P.accept[b * P.k + i] = acc ? 1 : 0;
     }
     if (flags) atomicOr(&P.wstatus[b], flags);
+    return acc;
 }
 
 // End of a (sequence, row, learner) unit of the ensemble feedback, by one thread: the learner's loss.

@@ -46,7 +46,9 @@ struct Sweep {
     uint32_t* arrived;       // workspace [units], zero on entry and zero again on exit
     unsigned kept;           // items, from the last one backwards, that L2 is asked to keep between the sweeps
     int all_rows;            // second sweep: masses of every row wanted (acceptance probabilities)
-    int draw_blocks;         // second sweep: its first blocks, those of the rows that are drawn from
+    int draw_blocks;         // second sweep: its first blocks, those of the rows that are drawn from,
+    int draw_slices;         // ... the items of such a row
+    int draw_regions;        // ... and their sampling regions
 };
 
 // What the second sweep is for.
@@ -329,12 +331,14 @@ sd_sweep_stats_kernel(const __grid_constant__ Params P, const __grid_constant__ 
     }
 }
 
-// A block per sequence, a warp per row.
+// A block per sequence, a warp per row.  Leaves the sequence's first rejected position (k if there is none) in
+// P.accept[b * k].
 template <int DT>
 __global__ void __launch_bounds__(kSweepThreads)
 sd_sweep_rows_kernel(const __grid_constant__ Params P, const __grid_constant__ Sweep S) {
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int b = blockIdx.x;
+    __shared__ uint8_t accepted[SD_MAX_K];
     launch_dependents();
     for (int i = warp; i <= P.k; i += kSweepWarps) {
         const int unit = b * (P.k + 1) + i;
@@ -346,9 +350,18 @@ sd_sweep_rows_kernel(const __grid_constant__ Params P, const __grid_constant__ S
         const PartialStats row = warp_merge_lanes(mine ? load_partial_cg(S.part + (size_t)unit * S.slices + lane) : empty_partial());
         if (lane == 0) {
             if (P.status && i == 0 && SD_IN(b, P.B, 21)) P.status[b] = 0;      // the words are ORed in by the second sweep
-            finish_row(P, b, i, row, row_constants(P, i == P.k, row), aop);
+            const bool acc = finish_row(P, b, i, row, row_constants(P, i == P.k, row), aop);
+            if (i < P.k) accepted[i] = acc;
         }
     }
+    __syncthreads();
+    if (warp != 0) return;
+    int n = P.k;
+    for (int i0 = 0; i0 < P.k; i0 += 32) {
+        const unsigned m = __ballot_sync(0xffffffffu, i0 + lane < P.k && !accepted[i0 + lane]);
+        if (m) { n = i0 + __ffs(m) - 1; break; }
+    }
+    if (lane == 0 && SD_IN(b * P.k, P.B * P.k, 22)) P.accept[b * P.k] = (uint8_t)n;
 }
 
 // Pass 2 of a warp's regions of an item.
@@ -425,10 +438,10 @@ sd_sweep_grad_kernel(const __grid_constant__ Params P, const __grid_constant__ S
     __shared__ int is_last;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const bool draws = (int)blockIdx.x < S.draw_blocks;
-    int unit, slice, b, n = P.k;
+    int unit, slice, b;
     if (draws) {
-        b = (int)blockIdx.x / S.slices;
-        slice = (int)blockIdx.x - b * S.slices;
+        b = (int)blockIdx.x / S.draw_slices;
+        slice = (int)blockIdx.x - b * S.draw_slices;
         unit = 0;
     } else {
         const int units = total_units<false>(P), id = (int)(gridDim.x - 1u - blockIdx.x);
@@ -439,25 +452,28 @@ sd_sweep_grad_kernel(const __grid_constant__ Params P, const __grid_constant__ S
     await_previous_kernel();
     launch_dependents();
 
-    if (!SD_IN(b, P.B, 22)) return;
-    // the first rejected position of the sequence
-    for (int i0 = 0; i0 < P.k; i0 += 32) {
-        const unsigned m = __ballot_sync(0xffffffffu, i0 + lane < P.k && P.accept[b * P.k + i0 + lane] == 0);
-        if (m) { n = i0 + __ffs(m) - 1; break; }
+    if (!SD_IN(b, P.B, 22) || !SD_IN(unit, total_units<false>(P), 20)) return;
+    const int regions = draws ? S.draw_regions : S.regions, slices = draws ? S.draw_slices : S.slices;
+    if (!SD_IN(slice, slices, 20)) return;
+    // (both loads under way together: of a block's chain of round trips this is one less)
+    RowConst rc = P.rowc[unit];
+    const int n = P.accept[b * P.k];
+    if (draws) {
+        unit = b * (P.k + 1) + n;
+        if (!SD_IN(unit, total_units<false>(P), 20)) return;
+        rc = P.rowc[unit];
+    } else if (unit - b * (P.k + 1) == n) {
+        return;                                       // the first blocks have it
     }
-    if (draws) unit = b * (P.k + 1) + n;
-    else if (unit - b * (P.k + 1) == n) return;      // the first blocks have it
     const UnitRef ur = unit_ref<false>(P, unit);
     if (!draws && ur.bonus) return;
-    if (!SD_IN(unit, total_units<false>(P), 20) || !SD_IN(slice, S.slices, 20)) return;
-    const RowConst rc = P.rowc[unit];
-    const int v0 = (slice * S.regions + warp) * kRegionVecs;
+    const int v0 = (slice * regions + warp) * kRegionVecs;
     float herr = 0.f;
-    float* const rsum = P.region_sums + (size_t)unit * P.NR + slice * S.regions + warp;
+    float* const rsum = P.region_sums + (size_t)unit * P.NR + slice * regions + warp;
     const bool masses = draws || HINT || S.all_rows;
     if constexpr (RAGGED) {
         const RowFrame<DT> f = row_frame<DT>(P, ur);
-        int v1 = min((slice + 1) * S.regions, P.NR) * kRegionVecs;
+        int v1 = min((slice + 1) * regions, P.NR) * kRegionVecs;
         if (!SD_IN(ur.t_row, (long long)P.B * (P.k + 1), 12) || !SD_IN(ur.d_row, (long long)P.B * P.k, 12)) v1 = 0;
         if (v0 < v1 && !SD_IN(v0 / kRegionVecs + (v1 - 1 - v0) / kSweepStep * kSweepWarps, P.NR, 13)) v1 = 0;
         ET* const grow = (P.grad && !ur.bonus) ? reinterpret_cast<ET*>(P.grad) + ur.d_row * P.V : nullptr;
@@ -465,7 +481,7 @@ sd_sweep_grad_kernel(const __grid_constant__ Params P, const __grid_constant__ S
         else if (masses) ragged_pass2<DT, false, true>(f, P.V, v0, v1, grow, rsum, lane, P.c, rc);
         else             ragged_pass2<DT, false, false>(f, P.V, v0, v1, grow, nullptr, lane, P.c, rc);
     } else {
-        int nvec = min((slice + 1) * S.regions * kRegionVecs, P.V / E::VEC) - v0;
+        int nvec = min((slice + 1) * regions * kRegionVecs, P.V / E::VEC) - v0;
         if (nvec > 0 && !SD_IN((long long)(v0 + nvec) * E::VEC - 1, P.V, 12)) nvec = 0;
         if (!SD_IN(ur.t_row, (long long)P.B * (P.k + 1), 12) || !SD_IN(ur.d_row, (long long)P.B * P.k, 12)) nvec = 0;
         if (nvec > 0 && !SD_IN(v0 / kRegionVecs + (nvec - 1) / kSweepStep * kSweepWarps, P.NR, 13)) nvec = 0;
@@ -509,7 +525,7 @@ sd_sweep_grad_kernel(const __grid_constant__ Params P, const __grid_constant__ S
             if (SD_IN(slice, P.hint_stride, 27)) P.hint_part[(size_t)unit * P.hint_stride + slice] = e;
         }
         __threadfence();
-        is_last = SD_IN(unit, total_units<false>(P), 28) && atomicAdd(S.arrived + unit, 1u) == (uint32_t)S.slices - 1u;
+        is_last = SD_IN(unit, total_units<false>(P), 28) && atomicAdd(S.arrived + unit, 1u) == (uint32_t)slices - 1u;
         if (is_last) {
             __threadfence();
             S.arrived[unit] = 0;
