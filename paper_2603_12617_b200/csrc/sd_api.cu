@@ -200,7 +200,7 @@ struct DeviceState {
     double dec_l2 = 0.0;
     // output-layer gradient
     uint32_t* gemm_error = nullptr;
-    bool gemm_attr = false;
+    bool gemm_attr[2] = {};
     // host-memory entry point
     StageSet stage[2];
     cudaStream_t s_h2d = nullptr, s_comp = nullptr, s_d2h = nullptr;
@@ -1426,9 +1426,11 @@ int sd_lmhead_grad(const uint16_t* grad_logits, const uint16_t* hidden, int R, i
     if (rc != SD_OK) return rc;
     rc = matrix_map(&map_out, SD_DTYPE_F32, out_dW, V, d, kGemmBox);
     if (rc != SD_OK) return rc;
-    if (!ds->gemm_attr) {
-        SD_CUDA(cudaFuncSetAttribute(sd_lmhead_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kGemmSmem));
-        ds->gemm_attr = true;
+    const bool few = R <= kGemmFewPositions;
+    const int smem = few ? GemmShape<true>::kSmem : GemmShape<false>::kSmem, threads = few ? GemmShape<true>::kThreads : GemmShape<false>::kThreads;
+    if (!ds->gemm_attr[few]) {
+        SD_CUDA(cudaFuncSetAttribute(few ? sd_lmhead_kernel<true> : sd_lmhead_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
+        ds->gemm_attr[few] = true;
     }
     GemmParams P;
     P.R = R; P.V = V; P.d = d;
@@ -1436,9 +1438,10 @@ int sd_lmhead_grad(const uint16_t* grad_logits, const uint16_t* hidden, int R, i
     const long long tiles = (long long)((V + kGemmBM - 1) / kGemmBM) * ((d + kGemmBN - 1) / kGemmBN);
     const long long pairs = ds->sm_count / 2;
     const unsigned grid = 2u * (unsigned)(tiles < pairs ? tiles : pairs);
-    sd_lmhead_kernel<<<grid, kGemmThreads, kGemmSmem, st>>>(map_g, map_x, map_out, P);
+    if (few) sd_lmhead_kernel<true><<<grid, threads, smem, st>>>(map_g, map_x, map_out, P);
+    else     sd_lmhead_kernel<false><<<grid, threads, smem, st>>>(map_g, map_x, map_out, P);
     SD_CUDA(cudaGetLastError());
-    tl_info[0] = 5; tl_info[1] = 2; tl_info[2] = kGemmThreads; tl_info[3] = kGemmSmem; tl_info[4] = (int)grid; tl_info[5] = 1;
+    tl_info[0] = 5; tl_info[1] = 2; tl_info[2] = threads; tl_info[3] = smem; tl_info[4] = (int)grid; tl_info[5] = 1;
     return SD_OK;
 }
 

@@ -20,13 +20,14 @@
 //               bf16); they complete on the barrier of the pair's first block
 //   warp 1      in the pair's first block one thread issues the MMAs (4 of K = 16 per stage) and the commits,
 //               which free the stage in both blocks
-//   warps 2..5  epilogue: tensor memory -> registers -> 32 x 32 boxes in shared memory -> global memory by TMA
+//   from warp 2 epilogue: tensor memory -> registers -> 32 x 32 boxes in shared memory -> global memory by TMA
 //               stores, which clip at the ends of dW, while the MMAs of the next tile fill the other half of
 //               tensor memory.
 // What bounds it: for many positions the board's power (1.3 of 1.64 PFLOP/s at 1536 positions, 128 256 x 4096: 1237 us);
 // operands enter an SM at 64 bytes a clock.  One block per tile of 128 x 256 (cta_group::1) needs 96, 27 TB/s of
-// L2 at full rate, and took 1377 us.  For few positions the writing of dW (256 positions 557 us, one block
-// per tile 562; 128 positions 476 and 549).
+// L2 at full rate, and took 1377 us.  For few positions the writing of dW, which wants more boxes under way than
+// loads (GemmShape): 256 positions 437 us (4.8 TB/s out), with four epilogue warps 494, one block per tile 562;
+// 128 positions 390, 415 and 549.
 // Every wait is bounded; a wait that gives up sets an error word, and the block frees its tensor
 // memory and returns.  No multicast of loads.
 #pragma once
@@ -42,19 +43,27 @@ namespace sdv {
 constexpr int kGemmBM = 256;                 // vocabulary entries per tile (rows of dW), half of them in each block
 constexpr int kGemmBN = 256;                 // features per tile (columns of dW); each block brings half of them
 constexpr int kGemmBK = 64;                  // positions per stage
-constexpr int kGemmStages = 6;
 constexpr int kGemmChunk = 64;               // entries of a 128-byte swizzled row (bf16)
 constexpr int kGemmChunkBytes = kGemmBK * kGemmChunk * 2;            // one TMA box: 8 KiB
 constexpr int kGemmChunks = 128 / kGemmChunk;                        // boxes of an operand's half tile
 constexpr int kGemmABytes = kGemmChunks * kGemmChunkBytes;           // 16 KiB
 constexpr int kGemmStageBytes = 2 * kGemmABytes;                     // a block's share of a stage: 32 KiB
-constexpr int kGemmThreads = 6 * 32;
 constexpr int kGemmTmemCols = 512;           // two accumulators of 128 lanes x 256 fp32 columns
 constexpr int kGemmBox = 32;                 // rows and columns of a box of the result
 constexpr int kGemmBoxBytes = kGemmBox * kGemmBox * 4;
 constexpr int kGemmBoxes = 2;                // boxes per epilogue warp: one leaves while the next is filled
-constexpr int kGemmSmem = kGemmStages * kGemmStageBytes + 4 * kGemmBoxes * kGemmBoxBytes + 1024 /* alignment */ + 256 /* barriers */;
-static_assert(kGemmSmem <= 227 * 1024, "stages and staging do not fit the shared memory of a block");
+// The two shapes of the kernel (both fill the shared memory of a block).  Few positions: eight epilogue warps, two to
+// a quarter of the tensor-memory lanes; many: six stages.  512 positions 581 us in the second, 599 in the first;
+// 1536 positions 1219 and 1280; 256 positions 494 and 437 (128 256 x 4096).
+template <bool FEW> struct GemmShape {
+    static constexpr int kStages = FEW ? 5 : 6;
+    static constexpr int kEpilogueWarps = FEW ? 8 : 4;
+    static constexpr int kThreads = (2 + kEpilogueWarps) * 32;
+    static constexpr int kColumns = kGemmBN * 4 / kEpilogueWarps;        // of the accumulator, per epilogue warp
+    static constexpr int kSmem = kStages * kGemmStageBytes + kEpilogueWarps * kGemmBoxes * kGemmBoxBytes + 1024 /* alignment */ + 256 /* barriers */;
+    static_assert(kSmem <= 227 * 1024, "stages and staging do not fit the shared memory of a block");
+};
+constexpr int kGemmFewPositions = 384;
 constexpr long long kGemmLeaveCycles = 2000000ll;     // about a millisecond
 constexpr long long kGemmWaitCycles = 4000000000ll;   // about two seconds
 
@@ -161,23 +170,27 @@ __device__ __forceinline__ bool gemm_wait(uint64_t* bar, uint32_t parity, volati
     return false;
 }
 
-struct GemmShared {
+template <bool FEW> struct GemmShared {
+    static constexpr int kGemmStages = GemmShape<FEW>::kStages;
     uint64_t full[kGemmStages];      // stage filled by both blocks' TMA    (first block: 1 arrival + bytes)
     uint64_t empty[kGemmStages];     // stage read by the MMAs              (1: commit)
     uint64_t acc_full[2];            // accumulator complete                (1: commit)
-    uint64_t acc_empty[2];           // accumulator read by the epilogues   (first block: 8, one per epilogue warp of the pair)
+    uint64_t acc_empty[2];           // accumulator read by the epilogues   (first block: one per epilogue warp of the pair)
     uint32_t tmem_base;
     int abort;
 };
 
-__global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kGemmThreads, 1)
+template <bool FEW>
+__global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(GemmShape<FEW>::kThreads, 1)
 sd_lmhead_kernel(const __grid_constant__ CUtensorMap map_g, const __grid_constant__ CUtensorMap map_x,
                  const __grid_constant__ CUtensorMap map_out, const GemmParams P) {
+    using Shape = GemmShape<FEW>;
+    constexpr int kGemmStages = Shape::kStages;
     extern __shared__ unsigned char gemm_smem_raw[];
     // (the same offsets in both blocks: the MMAs take them from one block's descriptors)
     unsigned char* smem = gemm_smem_raw + ((1024u - (smem_u32(gemm_smem_raw) & 1023u)) & 1023u);
     unsigned char* boxes = smem + kGemmStages * kGemmStageBytes;
-    GemmShared& sh = *reinterpret_cast<GemmShared*>(boxes + 4 * kGemmBoxes * kGemmBoxBytes);
+    GemmShared<FEW>& sh = *reinterpret_cast<GemmShared<FEW>*>(boxes + Shape::kEpilogueWarps * kGemmBoxes * kGemmBoxBytes);
     cg::cluster_group cluster = cg::this_cluster();
     const int rank = (int)cluster.block_rank();
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
@@ -190,7 +203,7 @@ sd_lmhead_kernel(const __grid_constant__ CUtensorMap map_g, const __grid_constan
 
     if (tid == 0) {
         for (int s = 0; s < kGemmStages; ++s) { mbar_init(&sh.full[s], 1); mbar_init(&sh.empty[s], 1); }
-        for (int a = 0; a < 2; ++a) { mbar_init(&sh.acc_full[a], 1); mbar_init(&sh.acc_empty[a], 8); }
+        for (int a = 0; a < 2; ++a) { mbar_init(&sh.acc_full[a], 1); mbar_init(&sh.acc_empty[a], 2 * Shape::kEpilogueWarps); }
         sh.abort = 0;
         fence_barrier_init();
         fence_proxy_async();
@@ -265,7 +278,7 @@ sd_lmhead_kernel(const __grid_constant__ CUtensorMap map_g, const __grid_constan
         }
     } else {
         // ---- epilogue: warp w reads the tensor-memory lanes 32*(w%4) .. +31 (rows of this block's half)
-        const int q = warp & 3;
+        const int q = warp & 3, c0 = ((warp - 2) >> 2) * (Shape::kColumns / kGemmBox);
         unsigned char* const mine = boxes + (size_t)(warp - 2) * kGemmBoxes * kGemmBoxBytes;
         long long it = 0;
         int box = 0;
@@ -280,7 +293,7 @@ sd_lmhead_kernel(const __grid_constant__ CUtensorMap map_g, const __grid_constan
             tc_fence_after();
             const int vbase = m0 + q * 32;               // first row of this warp's 32
 #pragma unroll 1
-            for (int c = 0; c < kGemmBN / kGemmBox; ++c) {
+            for (int c = c0; c < c0 + Shape::kColumns / kGemmBox; ++c) {
                 uint32_t r[32];
                 tmem_ld_32x32(tmem + ((uint32_t)(q * 32) << 16) + (uint32_t)(acc * kGemmBN + c * kGemmBox), r);
                 tmem_ld_wait();
