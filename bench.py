@@ -278,10 +278,12 @@ def rotating_sets(host_tensors, dev):
 
 
 def kernel_names(path, info) -> str:
-    """The kernels a step launched: what the path is named after, or the two sweeps or the element-wise kernel where
-    the library took those (sd_launch_info)."""
+    """The kernels a step launched: what the path is named after, or the two sweeps, the kernel that holds the logits
+    or the element-wise kernel where the library took those (sd_launch_info)."""
     if info["path"] == 0:
         return "sd_generic_kernel"
+    if info["path"] in (1, 3, 4) and info["threads"] == 512:
+        return path.kernel.replace("sd_stream_kernel", "sd_held_kernel")
     if info["path"] in (1, 4) and info["kernels"] == 3:
         return "sd_sweep_stats_kernel + sd_sweep_rows_kernel + sd_sweep_grad_kernel"
     return path.kernel
@@ -409,7 +411,7 @@ class VocabParallelPath(SamplePath):
     """One rank of the vocabulary-parallel step on this GPU: the workload's logits cut into --shards column
     shards, this rank's three local calls timed on its own shard with the other ranks' records and masses
     already in place (the gathers of a real deployment are not part of the timed region: one GPU here)."""
-    name, kernel, traffic_path = "vp", "sd_vp_stats_kernel + sd_vp_rows_kernel + sd_vp_grad_kernel + sd_vp_mass_kernel + sd_vp_draw_kernel", "vp"
+    name, kernel, traffic_path = "vp", "sd_vp_stats_kernel + sd_vp_rows_kernel + sd_vp_grad_kernel + sd_vp_draw_kernel", "vp"
 
     def __init__(self, args, cfg, dev, rank, binding):
         import torch
@@ -451,7 +453,7 @@ class VocabParallelPath(SamplePath):
         self.dtype = "f32" if cfg.dtype == "f32" else "f32 (bf16 storage)"
         self.extra = {"shards": G, "timed": f"the three local calls of rank 0 (columns 0..{Vs - 1}); the two gathers and the "
                                            "token maximum of a real deployment are not in the timed region",
-                      "kernels_per_step": 5}
+                      "kernels_per_step": 4}
         self.e2e_entry = "sd_vp_partial + sd_vp_finish + sd_vp_draw of one rank between pinned-memory copies of its shard"
 
     def step(self, i):

@@ -265,13 +265,15 @@ int launch_stream(DeviceState& d, const Params& P, int C, int G, int lag, cudaSt
     cfg.blockDim = dim3(kStreamThreads, 1, 1);
     cfg.dynamicSmemBytes = (size_t)stream_smem<DT>();
     cfg.stream = stream;
-    cudaLaunchAttribute attr[1];
+    cudaLaunchAttribute attr[2];
     attr[0].id = cudaLaunchAttributeClusterDimension;
     attr[0].val.clusterDim.x = (unsigned)C;
     attr[0].val.clusterDim.y = 1;
     attr[0].val.clusterDim.z = 1;
+    attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[1].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr;
-    cfg.numAttrs = 1;
+    cfg.numAttrs = query_only ? 1 : 2;
     if (query_only) {
         int n = 0;
         cudaError_t e = cudaOccupancyMaxActiveClusters(&n, kern, &cfg);
@@ -399,24 +401,32 @@ bool use_held(DeviceState& d, int V, long long units, int dtype, bool second, He
 
 // Launch of a kernel whose blocks come as those of the kernel before it on the stream go.
 template <class K, class... A>
-cudaError_t launch_following(K kern, dim3 grid, int threads, cudaStream_t stream, const A&... args) {
+cudaError_t launch_following_clusters(K kern, dim3 grid, int threads, unsigned cluster, cudaStream_t stream, const A&... args) {
     cudaLaunchConfig_t cfg;
     memset(&cfg, 0, sizeof cfg);
     cfg.gridDim = grid;
     cfg.blockDim = dim3((unsigned)threads, 1, 1);
     cfg.stream = stream;
-    cudaLaunchAttribute attr[1];
+    cudaLaunchAttribute attr[2];
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     attr[0].val.programmaticStreamSerializationAllowed = 1;
+    attr[1].id = cudaLaunchAttributeClusterDimension;
+    attr[1].val.clusterDim.x = cluster;
+    attr[1].val.clusterDim.y = 1;
+    attr[1].val.clusterDim.z = 1;
     cfg.attrs = attr;
-    cfg.numAttrs = 1;
+    cfg.numAttrs = cluster > 1 ? 2 : 1;
     return cudaLaunchKernelEx(&cfg, kern, args...);
+}
+template <class K, class... A>
+cudaError_t launch_following(K kern, dim3 grid, int threads, cudaStream_t stream, const A&... args) {
+    return launch_following_clusters(kern, grid, threads, 1u, stream, args...);
 }
 
 template <int DT, int MODE, bool RAGGED = false>
 int launch_sweeps_of(const Params& P, const Sweep& S, long long units, bool all, cudaStream_t stream) {
     SD_CUDA(launch_following(sd_sweep_stats_kernel<DT, RAGGED>, dim3((unsigned)units, (unsigned)S.slices), kSweepThreads, stream, P, S));
-    SD_CUDA(launch_following(sd_sweep_rows_kernel<DT>, dim3((unsigned)P.B), kSweepThreads, stream, P, S));
+    SD_CUDA(launch_following(sd_sweep_rows_kernel<DT>, dim3((unsigned)P.B), 32 * (P.k + 1 < kRowsMaxWarps ? P.k + 1 : kRowsMaxWarps), stream, P, S));
     // the rows that are drawn from, then (if anything of them is wanted) all rows
     const unsigned second = (unsigned)S.draw_blocks + (all ? (unsigned)(units * S.slices) : 0u);
     SD_CUDA(launch_following(sd_sweep_grad_kernel<DT, MODE, RAGGED>, dim3(second), kSweepThreads, stream, P, S));
@@ -433,11 +443,13 @@ int launch_sweeps(const Params& P, Sweep& S, long long units, int dtype, cudaStr
     // 74.8).
     const bool all = MODE != kSweepErrors && (P.grad || MODE == kSweepHint || S.all_rows);
     S.kept = all ? (80u << 20) / (unsigned)(S.regions * kRegionVecs * 32) : 0u;
-    // Where the second sweep is the drawn rows alone, its items are as small as leaves every block resident at
-    // once: the time of such a sweep is a chain of round trips, one for each region of a warp.
+    // The items of the drawn rows are as small as leaves all their blocks resident at once, where the second sweep is
+    // the drawn rows alone or not much more than a round of blocks: a draw is a chain of round trips, one for each
+    // region of a warp, and its end is the call's (16 sequences, 4 tokens, 151 936 bf16 entries 31.0 -> 28.3 us; 32,
+    // 8, 128 256, 2304 items, 59.5 -> 60.4).  (The hint error is summed by items of one size.)
     S.draw_regions = S.regions;
     S.draw_slices = S.slices;
-    if (!all) {
+    if (MODE != kSweepHint && (!all || units * S.slices <= 1332)) {
         for (int r = kSweepWarps; r < S.regions; r += kSweepWarps) {
             const int s = (P.NR + r - 1) / r;
             if ((long long)P.B * s > (RAGGED ? 592 : 888)) continue;
@@ -458,8 +470,7 @@ int launch_sweeps(const Params& P, Sweep& S, long long units, int dtype, cudaStr
 template <int DT>
 int launch_generic(const Params& P, cudaStream_t stream) {
     const long long units = (long long)P.B * (P.k + 1);
-    sd_generic_kernel<DT><<<(unsigned)units, kGenericThreads, 0, stream>>>(P);
-    SD_CUDA(cudaGetLastError());
+    SD_CUDA(launch_following(sd_generic_kernel<DT>, dim3((unsigned)units), kGenericThreads, stream, P));
     tl_info[0] = 0; tl_info[1] = 1; tl_info[2] = kGenericThreads; tl_info[3] = 0;
     tl_info[4] = (int)units; tl_info[5] = 1;
     return SD_OK;
@@ -1331,9 +1342,15 @@ int sd_vp_partial(const void* target_shard, const void* draft_shard, const int32
     P.records = static_cast<VpRecord*>(out_records);
     const unsigned units = (unsigned)B * (unsigned)(k + 1);
     cudaStream_t st = static_cast<cudaStream_t>(stream);
-    SD_CUDA(dtype == SD_DTYPE_F32 ? launch_following(sd_vp_stats_kernel<SD_DTYPE_F32>, dim3(units), kVpThreads, st, P)
-                                  : launch_following(sd_vp_stats_kernel<SD_DTYPE_BF16>, dim3(units), kVpThreads, st, P));
-    tl_info[0] = 6; tl_info[1] = 1; tl_info[2] = kVpThreads; tl_info[3] = 0; tl_info[4] = (int)units; tl_info[5] = 1;
+    // blocks of a row: all blocks resident (eight of 128 threads to an SM), and a region for every warp
+    const int NR = vp_layout(B, k, V_shard, dtype).NR;
+    unsigned C = (unsigned)ds->sm_count * 8u / units;
+    if (C > (unsigned)((NR + kVpStatsWarps - 1) / kVpStatsWarps)) C = (unsigned)((NR + kVpStatsWarps - 1) / kVpStatsWarps);
+    if (C > (unsigned)kVpMaxCluster) C = kVpMaxCluster;
+    if (C < 1) C = 1;
+    SD_CUDA(dtype == SD_DTYPE_F32 ? launch_following_clusters(sd_vp_stats_kernel<SD_DTYPE_F32>, dim3(units * C), kVpStatsThreads, C, st, P)
+                                  : launch_following_clusters(sd_vp_stats_kernel<SD_DTYPE_BF16>, dim3(units * C), kVpStatsThreads, C, st, P));
+    tl_info[0] = 6; tl_info[1] = (int)C; tl_info[2] = kVpStatsThreads; tl_info[3] = 0; tl_info[4] = (int)(units * C); tl_info[5] = 1;
     return SD_OK;
 }
 
@@ -1364,13 +1381,12 @@ int sd_vp_finish(const void* target_shard, const void* draft_shard, const int32_
     P.status = out_status;
     P.local_mass = out_local_mass;
     cudaStream_t st = static_cast<cudaStream_t>(stream);
-    SD_CUDA(launch_following(sd_vp_rows_kernel, dim3((unsigned)B), 96, st, P));
+    SD_CUDA(launch_following(sd_vp_rows_kernel, dim3((unsigned)B), 32 * (k + 1 < kRowsMaxWarps ? k + 1 : kRowsMaxWarps), st, P));
     const int slices = (P.NR + kVpSliceRegions - 1) / kVpSliceRegions;
     const unsigned grid = (unsigned)B * (unsigned)(k + 1) * (unsigned)slices;
     SD_CUDA(dtype == SD_DTYPE_F32 ? launch_following(sd_vp_grad_kernel<SD_DTYPE_F32>, dim3(grid), kVpThreads, st, P, slices)
                                   : launch_following(sd_vp_grad_kernel<SD_DTYPE_BF16>, dim3(grid), kVpThreads, st, P, slices));
-    SD_CUDA(launch_following(sd_vp_mass_kernel, dim3((unsigned)B), 32, st, P));
-    tl_info[0] = 6; tl_info[1] = 1; tl_info[2] = kVpThreads; tl_info[3] = 0; tl_info[4] = (int)grid; tl_info[5] = 3;
+    tl_info[0] = 6; tl_info[1] = 1; tl_info[2] = kVpThreads; tl_info[3] = 0; tl_info[4] = (int)grid; tl_info[5] = 2;
     return SD_OK;
 }
 

@@ -505,10 +505,19 @@ __device__ __forceinline__ AcceptOperands load_accept_operands(const Params& P, 
     return a;
 }
 
+// Logarithms of a row's denominators.  Those are a thousand cycles of fp64 one after the other; a warp's lanes
+// take them side by side.
+struct RowLogs { double T, D; };
+__device__ __forceinline__ RowLogs row_logs(const PartialStats& st) { return RowLogs{log2(st.sT), log2(st.sD)}; }
+__device__ __forceinline__ RowLogs warp_row_logs(const PartialStats& st) {
+    const double l = log2((threadIdx.x & 1) ? st.sD : st.sT);
+    return RowLogs{__shfl_sync(0xffffffffu, l, 0), __shfl_sync(0xffffffffu, l, 1)};
+}
+
 // End of a (sequence, row) unit, by one thread: row constants to the workspace, the KL loss and
 // the rejection test of the row's draft token, whose outcome it returns.
 __device__ inline bool finish_row(const Params& P, int b, int i, const PartialStats& st, const RowConst& rc,
-                                  const AcceptOperands& op) {
+                                  const AcceptOperands& op, const RowLogs& logs) {
     const bool bonus = (i == P.k);
     const int unit = b * (P.k + 1) + i;
     uint32_t flags = 0;
@@ -520,7 +529,7 @@ __device__ inline bool finish_row(const Params& P, int b, int i, const PartialSt
     if (!bonus) {
         // log2 p_v = aT_v - log2 S_T and log2 q_v = aD_v - log2 S_D, so
         // KL(p||q) = ln2 * [ E_p(aT - aD) - log2 S_T + log2 S_D ]
-        const double l2ST = log2(st.sT), l2SD = log2(st.sD);
+        const double l2ST = logs.T, l2SD = logs.D;
         if (P.loss && SD_IN(b * P.k + i, P.B * P.k, 21)) {
             const double kl = 0.6931471805599453 * (st.w / st.sT - l2ST + l2SD);
             P.loss[b * P.k + i] = (float)kl;

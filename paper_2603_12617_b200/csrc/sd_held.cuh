@@ -49,8 +49,6 @@ __device__ __forceinline__ void held_load(uint4& v, const uint4* p, bool in, uin
                  "@p ld.global.L1::no_allocate.L2::cache_hint.v4.u32 {%0,%1,%2,%3}, [%4], %6;\n\t}"
                  : "+r"(v.x), "+r"(v.y), "+r"(v.z), "+r"(v.w) : "l"(p), "r"((int)in), "l"(policy));
 }
-__device__ __forceinline__ void cluster_arrive() { asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory"); }
-__device__ __forceinline__ void cluster_wait() { asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory"); }
 
 // Merge of `n` partials in shared memory by one warp.  Every lane gets the same bits.
 __device__ __forceinline__ PartialStats held_merge(const PartialStats* part, int n, int lane) {
@@ -74,20 +72,24 @@ __device__ __forceinline__ PartialStats held_merge(const PartialStats* part, int
     return r;
 }
 
-// End of a sequence, by the warp that took its last ticket.
+// End of a sequence, by the warp that took its last ticket.  Of up to 32 rows a lane each asks for everything that may
+// be wanted, so that one round trip does.
 __device__ __forceinline__ void held_finish(const Params& P, const HeldCandidate* cand, int b, int lane) {
     const int k = P.k;
     const int32_t x_first = (lane < k) ? P.x[b * k + lane] : -1;
     const uint32_t word = __ldcg(P.wstatus + b);
+    int2 c = make_int2(0, 0);
+    if (lane <= k && SD_IN(b * (k + 1) + lane, P.B * (k + 1), 20)) c = __ldcg(reinterpret_cast<const int2*>(cand + b * (k + 1) + lane));
     int n = k;
     for (int i0 = 0; i0 < k; i0 += 32) {
         const int i = i0 + lane;
         const unsigned m = __ballot_sync(0xffffffffu, i < k && __ldcg(P.accept + b * k + i) == 0);
         if (m) { n = i0 + __ffs(m) - 1; break; }
     }
-    const int unit = b * (k + 1) + n;
-    if (!SD_IN(unit, P.B * (k + 1), 23) || !SD_IN(n, k + 1, 23)) return;
-    const int2 c = __ldcg(reinterpret_cast<const int2*>(cand + unit));
+    if (!SD_IN(n, k + 1, 23)) return;
+    c.x = __shfl_sync(0xffffffffu, c.x, n & 31);
+    c.y = __shfl_sync(0xffffffffu, c.y, n & 31);
+    if (n >= 32) c = __ldcg(reinterpret_cast<const int2*>(cand + b * (k + 1) + n));
     if (lane == 0) {
         P.accept_len[b] = n;
         if (P.status) P.status[b] = word | (uint32_t)c.y;
@@ -173,6 +175,9 @@ sd_held_kernel(const __grid_constant__ Params P, HeldCandidate* const cand) {
     const uint4* const gT = reinterpret_cast<const uint4*>(reinterpret_cast<const ET*>(P.T) + ur.t_row * P.V);
     const uint4* const gD = reinterpret_cast<const uint4*>(reinterpret_cast<const ET*>(ENS ? P.Dn[ur.n] : P.D) + offD);
 
+    // (asked for before anything else: wanted at the end of the chain)
+    float uk = 0.f;
+    if (!STATS && !ENS) asm volatile("ld.global.nc.f32 %0, [%1];" : "=f"(uk) : "l"(P.u + (size_t)ur.b * (P.k + 1) + P.k));
     uint4 rt[N][kRegionRows], rd[N][kRegionRows];
     const uint64_t policy = STATS || ENS ? policy_normal() : policy_discard();     // (somebody else reads them too)
 #pragma unroll
@@ -201,14 +206,8 @@ sd_held_kernel(const __grid_constant__ Params P, HeldCandidate* const cand) {
         float mT = -INFINITY, mD = -INFINITY;
 #pragma unroll
         for (int j = 0; j < N; ++j) {
-#pragma unroll
-            for (int g = 0; g < kRegionRows; ++g) {
-                float v[VEC];
-                E::unpack(rt[j][g], v);
-                mT = fmaxf(mT, tree_max<VEC>(v));
-                E::unpack(rd[j][g], v);
-                mD = fmaxf(mD, tree_max<VEC>(v));
-            }
+            mT = fmaxf(mT, region_max<DT>(rt[j]));
+            mD = fmaxf(mD, region_max<DT>(rd[j]));
         }
         RT = warp_max_ref(ref_of(mT, P.c));
         RD = warp_max_ref(ref_of(mD, P.c));
@@ -248,7 +247,7 @@ sd_held_kernel(const __grid_constant__ Params P, HeldCandidate* const cand) {
     if constexpr (STATS) {
         if (reports && lane == 0) {
             if (P.status && ur.i == 0 && SD_IN(ur.b, P.B, 21)) P.status[ur.b] = 0;      // the next kernel ORs its bits in
-            finish_row(P, ur.b, ur.i, sh.row, rc, aop);
+            finish_row(P, ur.b, ur.i, sh.row, rc, aop, row_logs(sh.row));
         }
         return;
     } else {
@@ -299,7 +298,7 @@ sd_held_kernel(const __grid_constant__ Params P, HeldCandidate* const cand) {
             if (lane < C) *cluster.map_shared_rank(&mass[slot], lane) = make_double2(total, (double)herr);
             __syncwarp();
             cluster_arrive();
-            if (reports && round == 0 && lane == 0) finish_row(P, ur.b, ur.i, sh.row, rc, aop);
+            if (reports && round == 0 && lane == 0) finish_row(P, ur.b, ur.i, sh.row, rc, aop, row_logs(sh.row));
             __syncwarp();
             cluster_wait();
 
@@ -335,7 +334,7 @@ sd_held_kernel(const __grid_constant__ Params P, HeldCandidate* const cand) {
                 if (ur.bonus) flags |= SD_STATUS_BAD_ROW;
                 mine = slot == 0;
             } else {
-                const double t = (double)P.u[ur.b * (P.k + 1) + P.k] * all;
+                const double t = (double)uk * all;
                 int owner = 0x7fffffff, last = -1;
                 double run = incl - held, prefix = 0.0;
                 for (int s = s0; s < s1; ++s) {

@@ -102,6 +102,9 @@ __device__ __forceinline__ void st_async_remote(void* dst, uint64_t a, uint64_t 
         "r"(smem_u32(bar)), "l"(a), "l"(b), "r"(rank)
         : "memory");
 }
+// The hardware barrier of a cluster, in two halves (all threads of all its blocks).
+__device__ __forceinline__ void cluster_arrive() { asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory"); }
+__device__ __forceinline__ void cluster_wait() { asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory"); }
 // Non-blocking: has the phase of that parity completed?  (try_wait may suspend the thread for a while.)
 __device__ __forceinline__ bool mbar_test(uint64_t* bar, uint32_t parity) {
     uint32_t ok;
@@ -242,25 +245,40 @@ struct Pass1State {
     LaneSums ls;
 };
 
+// Largest entry of a lane's part of a region (NaN entries don't count); bf16 pairs are compared as they lie.
+template <int DT>
+__device__ __forceinline__ float region_max(const uint4 (&r)[kRegionRows]) {
+    using E = Elem<DT>;
+    if constexpr (DT == SD_DTYPE_BF16) {
+        const auto max2 = [](uint32_t a, uint32_t b) {
+            uint32_t m;
+            asm("max.bf16x2 %0, %1, %2;" : "=r"(m) : "r"(a), "r"(b));
+            return m;
+        };
+        uint32_t m[kRegionRows];
+#pragma unroll
+        for (int g = 0; g < kRegionRows; ++g) m[g] = max2(max2(r[g].x, r[g].y), max2(r[g].z, r[g].w));
+#pragma unroll
+        for (int g = 1; g < kRegionRows; ++g) m[0] = max2(m[0], m[g]);
+        return fmaxf(__uint_as_float(m[0] << 16), __uint_as_float(m[0] & 0xffff0000u));
+    } else {
+        float m[kRegionRows];
+#pragma unroll
+        for (int g = 0; g < kRegionRows; ++g) {
+            float v[E::VEC];
+            E::unpack(r[g], v);
+            m[g] = tree_max<E::VEC>(v);
+        }
+        return tree_max<kRegionRows>(m);
+    }
+}
+
 // The region's maxima raise the references; the running sums follow.
 template <int DT, bool BONUS>
 __device__ __forceinline__ void raise_references(const uint4 (&rt)[kRegionRows], const uint4 (&rd)[kRegionRows],
                                                  float c, Pass1State& s) {
-    using E = Elem<DT>;
-    constexpr int VEC = E::VEC;
-    float mT[kRegionRows], mD[kRegionRows];
-#pragma unroll
-    for (int g = 0; g < kRegionRows; ++g) {
-        float v[VEC];
-        E::unpack(rt[g], v);
-        mT[g] = tree_max<VEC>(v);
-        if (!BONUS) {
-            E::unpack(rd[g], v);
-            mD[g] = tree_max<VEC>(v);
-        }
-    }
-    const float nT = fmaxf(s.RT, warp_max_ref(ref_of(tree_max<kRegionRows>(mT), c)));
-    const float nD = BONUS ? kEmptyRef : fmaxf(s.RD, warp_max_ref(ref_of(tree_max<kRegionRows>(mD), c)));
+    const float nT = fmaxf(s.RT, warp_max_ref(ref_of(region_max<DT>(rt), c)));
+    const float nD = BONUS ? kEmptyRef : fmaxf(s.RD, warp_max_ref(ref_of(region_max<DT>(rd), c)));
     s.ls.rescale(nT - s.RT, nD - s.RD);
     s.RT = nT;
     s.RD = nD;
@@ -567,6 +585,8 @@ sd_stream_kernel(const __grid_constant__ Params P, const int lag_stages, const i
     }
     // every block of the cluster has initialised its barriers before anyone arrives on them
     cluster.sync();
+    await_previous_kernel();
+    launch_dependents();
 
     if (warp == kStatsWarp) {
         // ---- statistics: block partial -> cluster exchange -> row constants
@@ -632,7 +652,7 @@ sd_stream_kernel(const __grid_constant__ Params P, const int lag_stages, const i
             if (reports && lane == 0 && !bonus) aop = load_accept_operands<DT>(P, b, i);
             // the row report needs pass 1 only: it runs while the consumers are in pass 2
             if (!mbar_wait_sleepy<200>(&sh.row_pub[dslot], dph, wc)) break;
-            if (reports && lane == 0) finish_row(P, b, i, sh.row[dslot], sh.rc_done[dslot], aop);
+            if (reports && lane == 0) finish_row(P, b, i, sh.row[dslot], sh.rc_done[dslot], aop, row_logs(sh.row[dslot]));
             if (!mbar_wait_sleepy<200>(&sh.s2_done[dslot], dph, wc)) break;
             __syncwarp();
             if constexpr (STATS) {
@@ -907,6 +927,8 @@ template <int DT>
 __global__ void __launch_bounds__(kGenericThreads) sd_generic_kernel(const __grid_constant__ Params P) {
     using E = Elem<DT>;
     __shared__ GenericShared sh;
+    await_previous_kernel();
+    launch_dependents();
 
     const int unit = blockIdx.x;
     const int b = unit / (P.k + 1), i = unit % (P.k + 1);
@@ -958,7 +980,7 @@ __global__ void __launch_bounds__(kGenericThreads) sd_generic_kernel(const __gri
             AcceptOperands aop;
             aop.valid = false;
             if (!bonus) aop = load_accept_operands<DT>(P, b, i);
-            finish_row(P, b, i, row, rcw, aop);
+            finish_row(P, b, i, row, rcw, aop, row_logs(row));
         }
     }
     __syncthreads();

@@ -60,6 +60,14 @@ __device__ __forceinline__ uint4 load_l2(const uint4* p, uint64_t policy) {
                  : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "l"(p), "l"(policy));
     return v;
 }
+// The same for vectors that the neighbouring lane reads too (kept in L1).
+__device__ __forceinline__ uint4 load_l2_shared(const uint4* p, uint64_t policy) {
+    uint4 v;
+    asm volatile("ld.global.L2::cache_hint.v4.u32 {%0,%1,%2,%3}, [%4], %5;"
+                 : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "l"(p), "l"(policy));
+    return v;
+}
+
 // Sums of the lanes of a warp that share the references (RT, RD) into *out, in fp64 and a fixed order.
 __device__ __forceinline__ void warp_post_lanes(const LaneSums& ls, float RT, float RD, int lane, PartialStats* out) {
     const double v = warp_fold_lanes(ls, lane);
@@ -72,20 +80,7 @@ __device__ __forceinline__ void warp_post_lanes(const LaneSums& ls, float RT, fl
 // references (the same references and sums).
 template <int DT, bool BONUS>
 __device__ __forceinline__ void follow_references(const uint4 (&rt)[kRegionRows], const uint4 (&rd)[kRegionRows], float c, Pass1State& s) {
-    using E = Elem<DT>;
-    constexpr int VEC = E::VEC;
-    float mT[kRegionRows], mD[kRegionRows];
-#pragma unroll
-    for (int g = 0; g < kRegionRows; ++g) {
-        float v[VEC];
-        E::unpack(rt[g], v);
-        mT[g] = tree_max<VEC>(v);
-        if (!BONUS) {
-            E::unpack(rd[g], v);
-            mD[g] = tree_max<VEC>(v);
-        }
-    }
-    const float t = tree_max<kRegionRows>(mT), d = BONUS ? 0.f : tree_max<kRegionRows>(mD);
+    const float t = region_max<DT>(rt), d = BONUS ? 0.f : region_max<DT>(rd);
     if (!__any_sync(0xffffffffu, __fmul_rn(t, c) > s.RT || (!BONUS && __fmul_rn(d, c) > s.RD))) return;
     const float nT = fmaxf(s.RT, warp_max_ref(ref_of(t, c)));
     const float nD = BONUS ? kEmptyRef : fmaxf(s.RD, warp_max_ref(ref_of(d, c)));
@@ -164,15 +159,19 @@ __device__ __forceinline__ bool inner_in_bounds(const RowFrame<DT>& f, int V, in
 }
 // An inner region.
 template <int DT, bool BONUS>
-__device__ __forceinline__ void load_inner(const RowFrame<DT>& f, int v, int lane, uint4 (&rt)[kRegionRows], uint4 (&rd)[kRegionRows]) {
+__device__ __forceinline__ void load_inner(const RowFrame<DT>& f, int v, int lane, uint64_t policy, uint4 (&rt)[kRegionRows],
+                                           uint4 (&rd)[kRegionRows]) {
+    uint4 next[kRegionRows];
+    const bool shifted = !BONUS && f.shift;
 #pragma unroll
     for (int g = 0; g < kRegionRows; ++g) {
-        rt[g] = __ldg(f.T16 + v + g * 32 + lane);
-        if (!BONUS) rd[g] = __ldg(f.D16 + v + g * 32 + lane);
+        rt[g] = load_l2_shared(f.T16 + v + g * 32 + lane, policy);
+        if (!BONUS) rd[g] = load_l2(f.D16 + v + g * 32 + lane, policy);
+        if (shifted) next[g] = load_l2_shared(f.T16 + v + g * 32 + lane + 1, policy);
     }
-    if (!BONUS && f.shift) {
+    if (shifted) {
 #pragma unroll
-        for (int g = 0; g < kRegionRows; ++g) rt[g] = funnel<DT>(rt[g], __ldg(f.T16 + v + g * 32 + lane + 1), f.shift);
+        for (int g = 0; g < kRegionRows; ++g) rt[g] = funnel<DT>(rt[g], next[g], f.shift);
     }
 }
 // Any region, entry by entry; what is not in the row reads as -inf.
@@ -196,14 +195,15 @@ __device__ __noinline__ void load_edge(const RowFrame<DT>& f, int V, int v, int 
 }
 
 template <int DT, bool BONUS>
-__device__ __forceinline__ void ragged_pass1(const RowFrame<DT>& f, int V, int v0, int v1, int lane, float c, Pass1State& s) {
+__device__ __forceinline__ void ragged_pass1(const RowFrame<DT>& f, int V, int v0, int v1, int lane, float c, uint64_t policy,
+                                             Pass1State& s) {
     for (int v = v0; v < v1; v += kSweepStep) {
         uint4 rt[kRegionRows], rd[kRegionRows];
         const bool inner = inner_region<DT>(f, V, v);
         if (inner && !inner_in_bounds<DT, BONUS>(f, V, v)) continue;
-        if (inner) load_inner<DT, BONUS>(f, v, lane, rt, rd);
+        if (inner) load_inner<DT, BONUS>(f, v, lane, policy, rt, rd);
         else       load_edge<DT, BONUS>(f, V, v, lane, rt, rd);
-        raise_references<DT, BONUS>(rt, rd, c, s);      // (every region, as the element-wise kernel does)
+        follow_references<DT, BONUS>(rt, rd, c, s);     // (every region, as the element-wise kernel does)
         float sT = 0.f, sD = 0.f, sW = 0.f;
         if (inner) region_sums_of<DT, BONUS, false>(rt, rd, c, s.RT, s.RD, sT, sD, sW);
         // masked target entries (a NaN) or a row's end: with the test for them
@@ -229,7 +229,7 @@ __device__ __forceinline__ void ragged_pass2(const RowFrame<DT>& f, int V, int v
             if (!MASS) break;
         } else if (inner_region<DT>(f, V, v)) {
             if (!inner_in_bounds<DT, BONUS>(f, V, v)) continue;       // (the gradient lies where the draft does)
-            load_inner<DT, BONUS>(f, v, lane, rt, rd);
+            load_inner<DT, BONUS>(f, v, lane, policy_discard(), rt, rd);
             mass = pass2_region_impl<DT, BONUS, false, MASS>(rt, rd, kRegionVecs, lane, c, rc,
                                                              grow ? grow + (size_t)v * VEC - f.lead : nullptr, rt, unused);
         } else {
@@ -256,17 +256,17 @@ __device__ __forceinline__ void ragged_pass2(const RowFrame<DT>& f, int V, int v
 }
 
 // Pass 1 of a warp's regions of an item: gT and gD lead to the first of them, `nvec` vectors of the item lie
-// from there on.  (Fetching the next region while this one is worked on was measured as well: no faster,
+// from there on, the next region `step` vectors further.  (Fetching the next region while this one is worked on was measured as well: no faster,
 // the other warps of the SM hide the loads.)
 // The references come from the warp's first region, which costs least, but an entry far above them has an
 // exponent as large, rounded as coarsely.  RAISE: every region raises them, so that no exponent is above 0,
 // for callers with few warps, hence few references, to a row.
 template <int DT, bool BONUS, bool RAISE = false>
-__device__ __forceinline__ void sweep_pass1(const uint4* gT, const uint4* gD, int nvec, int lane, float c, uint64_t policy,
+__device__ __forceinline__ void sweep_pass1(const uint4* gT, const uint4* gD, int nvec, int step, int lane, float c, uint64_t policy,
                                             Pass1State& s) {
     constexpr float kTooLarge = 1.152921504606846976e18f;   // 2^60
     bool first = true;
-    for (; nvec >= kRegionVecs; gT += kSweepStep, gD += kSweepStep, nvec -= kSweepStep, first = false) {
+    for (; nvec >= kRegionVecs; gT += step, gD += step, nvec -= step, first = false) {
         uint4 rt[kRegionRows], rd[kRegionRows];
 #pragma unroll
         for (int g = 0; g < kRegionRows; ++g) {
@@ -305,22 +305,22 @@ sd_sweep_stats_kernel(const __grid_constant__ Params P, const __grid_constant__ 
     Pass1State ps;
     ps.RT = ps.RD = kEmptyRef;
     ps.ls.init();
+    const unsigned from_end = (gridDim.y - 1u - blockIdx.y) * gridDim.x + (gridDim.x - 1u - blockIdx.x);
+    const uint64_t policy = from_end < S.kept ? policy_keep() : policy_discard();
     if constexpr (RAGGED) {
         const RowFrame<DT> f = row_frame<DT>(P, ur);
         int v1 = min((slice + 1) * S.regions * kRegionVecs, f.nvec);
         if (!SD_IN(ur.t_row, (long long)P.B * (P.k + 1), 10) || !SD_IN(ur.d_row, (long long)P.B * P.k, 11)) v1 = 0;
-        if (ur.bonus) ragged_pass1<DT, true>(f, P.V, v0, v1, lane, P.c, ps);
-        else          ragged_pass1<DT, false>(f, P.V, v0, v1, lane, P.c, ps);
+        if (ur.bonus) ragged_pass1<DT, true>(f, P.V, v0, v1, lane, P.c, policy, ps);
+        else          ragged_pass1<DT, false>(f, P.V, v0, v1, lane, P.c, policy, ps);
     } else {
         int nvec = min((slice + 1) * S.regions * kRegionVecs, P.V / E::VEC) - v0;
         if (nvec > 0 && !SD_IN((long long)(v0 + nvec) * E::VEC - 1, P.V, 10)) nvec = 0;
         if (!SD_IN(ur.t_row, (long long)P.B * (P.k + 1), 10) || !SD_IN(ur.d_row, (long long)P.B * P.k, 11)) nvec = 0;
         const uint4* const gT = reinterpret_cast<const uint4*>(reinterpret_cast<const ET*>(P.T) + ur.t_row * P.V) + v0;
         const uint4* const gD = reinterpret_cast<const uint4*>(reinterpret_cast<const ET*>(P.D) + ur.d_row * P.V) + v0;
-        const unsigned from_end = (gridDim.y - 1u - blockIdx.y) * gridDim.x + (gridDim.x - 1u - blockIdx.x);
-        const uint64_t policy = from_end < S.kept ? policy_keep() : policy_discard();
-        if (ur.bonus) sweep_pass1<DT, true>(gT, gD, nvec, lane, P.c, policy, ps);
-        else          sweep_pass1<DT, false>(gT, gD, nvec, lane, P.c, policy, ps);
+        if (ur.bonus) sweep_pass1<DT, true>(gT, gD, nvec, kSweepStep, lane, P.c, policy, ps);
+        else          sweep_pass1<DT, false>(gT, gD, nvec, kSweepStep, lane, P.c, policy, ps);
     }
     warp_post_lanes(ps.ls, ps.RT, ps.RD, lane, &wpart[warp]);
     __syncthreads();
@@ -331,16 +331,17 @@ sd_sweep_stats_kernel(const __grid_constant__ Params P, const __grid_constant__ 
     }
 }
 
-// A block per sequence, a warp per row.  Leaves the sequence's first rejected position (k if there is none) in
-// P.accept[b * k].
+// A block per sequence, a warp per row (up to kRowsMaxWarps of them at a time).  Leaves the sequence's first rejected
+// position (k if there is none) in P.accept[b * k].
+constexpr int kRowsMaxWarps = 16;
 template <int DT>
-__global__ void __launch_bounds__(kSweepThreads)
+__global__ void __launch_bounds__(kRowsMaxWarps * 32)
 sd_sweep_rows_kernel(const __grid_constant__ Params P, const __grid_constant__ Sweep S) {
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, warps = (int)blockDim.x >> 5;
     const int b = blockIdx.x;
     __shared__ uint8_t accepted[SD_MAX_K];
     launch_dependents();
-    for (int i = warp; i <= P.k; i += kSweepWarps) {
+    for (int i = warp; i <= P.k; i += warps) {
         const int unit = b * (P.k + 1) + i;
         AcceptOperands aop;
         aop.valid = false;
@@ -348,9 +349,10 @@ sd_sweep_rows_kernel(const __grid_constant__ Params P, const __grid_constant__ S
         await_previous_kernel();
         const bool mine = lane < S.slices && SD_IN((long long)unit * S.slices + lane, (long long)total_units<false>(P) * S.slices, 26);
         const PartialStats row = warp_merge_lanes(mine ? load_partial_cg(S.part + (size_t)unit * S.slices + lane) : empty_partial());
+        const RowLogs logs = warp_row_logs(row);
         if (lane == 0) {
             if (P.status && i == 0 && SD_IN(b, P.B, 21)) P.status[b] = 0;      // the words are ORed in by the second sweep
-            const bool acc = finish_row(P, b, i, row, row_constants(P, i == P.k, row), aop);
+            const bool acc = finish_row(P, b, i, row, row_constants(P, i == P.k, row), aop, logs);
             if (i < P.k) accepted[i] = acc;
         }
     }

@@ -70,28 +70,33 @@ struct VpParams {
 };
 
 // ---- phase 1 -------------------------------------------------------------------------------
-// A block per row, its warps take the row's regions in turn, with the loop of the single-GPU first sweep (a
-// maximum for every two vectors and a test for masked entries took 18.0 us on 320 rows of 37 984 bf16 entries).
-// Every region raises the references: with those of a warp's first region alone (15.7 us) the error of fp32
-// gradients against 64 bits doubled.  With a vote whether any entry is above them that costs nothing there (15.7;
-// 1792 rows of 32 064 entries 42.0 -> 44.0; raised without looking 16.4 and 45.0), with 64 registers (48: 16.5).
-// The kernels of phase 2 follow one another without a gap; rows that are not drawn from skip their masses.
-// The three calls of one rank, 64 sequences, 4 tokens, a quarter of 151 936 bf16 entries: 69 us, now 53 us, most
-// of it the calling thread's.
+// A cluster of C blocks per row (as many as leave all of them resident: a warp's time is a chain of round trips, one
+// per region), its warps take the row's regions in turn, with the loop of the single-GPU first sweep (a
+// maximum for every two vectors and a test for masked entries took 18.0 us on 320 rows of 37 984 bf16 entries,
+// one block of eight warps per row 15.7).
+// Every region raises the references: with those of a warp's first region alone the error of fp32
+// gradients against 64 bits doubled.  With a vote whether any entry is above them that costs nothing there
+// (1792 rows of 32 064 entries 42.0 -> 44.0; raised without looking 45.0).
+constexpr int kVpStatsWarps = 4;
+constexpr int kVpStatsThreads = kVpStatsWarps * 32;
+constexpr int kVpMaxCluster = 8;
 template <int DT>
-__global__ void __launch_bounds__(kVpThreads, 4) sd_vp_stats_kernel(const VpParams P) {
+__global__ void __launch_bounds__(kVpStatsThreads, 8) sd_vp_stats_kernel(const VpParams P) {
     using E = Elem<DT>;
     using ET = typename E::type;
     constexpr int VEC = E::VEC;
-    __shared__ PartialStats warp_part[kVpWarps];
+    __shared__ PartialStats part[kVpMaxCluster * kVpStatsWarps];     // of the cluster's first block: every warp's
+    cg::cluster_group cluster = cg::this_cluster();
+    const int C = (int)cluster.num_blocks(), rank = (int)cluster.block_rank();
+    if (C > 1) cluster_arrive();                                     // (waited for before the first remote store)
     await_previous_kernel();
     launch_dependents();
-    const int unit = blockIdx.x;
+    const int unit = (int)blockIdx.x / C;
     const int K1 = P.k + 1;
     const int b = unit / K1, i = unit - b * K1;
     const bool bonus = (i == P.k);
-    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    if (!SD_IN(unit, P.B * K1, 60)) return;
+    const int tid = threadIdx.x, lane = tid & 31, slot = rank * kVpStatsWarps + (tid >> 5), slots = C * kVpStatsWarps;
+    const bool reports = rank == 0 && tid == 0;
     const uint4* Trow = reinterpret_cast<const uint4*>(reinterpret_cast<const ET*>(P.T) + (size_t)unit * P.Vs);
     const uint4* Drow = reinterpret_cast<const uint4*>(reinterpret_cast<const ET*>(P.D) + (size_t)(b * P.k + (bonus ? 0 : i)) * P.Vs);
     const int NV = P.Vs / VEC;
@@ -99,7 +104,7 @@ __global__ void __launch_bounds__(kVpThreads, 4) sd_vp_stats_kernel(const VpPara
     // (the drafted token's logits are asked for first: two dependent reads that the sweep hides)
     float tx = 0.f, dx = 0.f;
     uint32_t has_token = 0;
-    if (tid == 0 && !bonus) {
+    if (reports && !bonus) {
         const int xg = P.x[b * P.k + i] - P.v_offset;
         if (xg >= 0 && xg < P.Vs) {
             has_token = 1;
@@ -110,55 +115,84 @@ __global__ void __launch_bounds__(kVpThreads, 4) sd_vp_stats_kernel(const VpPara
     Pass1State ps;
     ps.RT = ps.RD = kEmptyRef;
     ps.ls.init();
-    const int w0 = warp * kRegionVecs;
+    const int w0 = slot * kRegionVecs;
     const uint64_t policy = policy_normal();     // what fits stays in L2 for the second sweep
-    if (bonus) sweep_pass1<DT, true, true>(Trow + w0, Drow + w0, NV - w0, lane, P.c, policy, ps);
-    else       sweep_pass1<DT, false, true>(Trow + w0, Drow + w0, NV - w0, lane, P.c, policy, ps);
-    warp_post_lanes(ps.ls, ps.RT, ps.RD, lane, &warp_part[warp]);
-    __syncthreads();
-    if (tid == 0) {
+    const int nvec = SD_IN(unit, P.B * K1, 60) ? NV - w0 : 0;
+    if (bonus) sweep_pass1<DT, true, true>(Trow + w0, Drow + w0, nvec, slots * kRegionVecs, lane, P.c, policy, ps);
+    else       sweep_pass1<DT, false, true>(Trow + w0, Drow + w0, nvec, slots * kRegionVecs, lane, P.c, policy, ps);
+    __syncwarp();
+    if (C > 1) {
+        cluster_wait();
+        warp_post_lanes(ps.ls, ps.RT, ps.RD, lane, cluster.map_shared_rank(&part[slot], 0));
+        __syncwarp();
+        cluster_arrive();
+        cluster_wait();
+    } else {
+        warp_post_lanes(ps.ls, ps.RT, ps.RD, lane, &part[slot]);
+        __syncthreads();
+    }
+    if (rank == 0 && tid < 32) {
         VpRecord r;
-        r.st = merge_partials_serial(warp_part, kVpWarps);
+        r.st = warp_merge_lanes(lane < slots ? part[lane] : empty_partial());
         r.tx = tx;
         r.dx = dx;
         r.has_token = has_token;
         r.pad = 0;
-        P.records[unit] = r;
+        if (lane == 0 && SD_IN(unit, P.B * K1, 60)) P.records[unit] = r;
     }
 }
 
 // ---- phase 2 -------------------------------------------------------------------------------
-// One block per sequence, one thread per row: merge of the G records of the row in rank order,
-// row constants, loss, rejection test; then the accept length.  Every rank computes the same bits.
-__global__ void __launch_bounds__(96) sd_vp_rows_kernel(const VpParams P) {
-    __shared__ int accepted[SD_MAX_K + 1];
+// One block per sequence, one warp per row (up to kRowsMaxWarps of them at a time), one lane per rank: merge of the G
+// records of the row in a fixed order, row constants, loss, rejection test; then the accept length.  Every rank
+// computes the same bits.
+__global__ void __launch_bounds__(kRowsMaxWarps * 32) sd_vp_rows_kernel(const VpParams P) {
+    __shared__ uint8_t accepted[SD_MAX_K + 1];
     __shared__ uint32_t flags_sh;
     await_previous_kernel();
     launch_dependents();
-    const int b = blockIdx.x, i = threadIdx.x;
+    const int b = blockIdx.x, lane = threadIdx.x & 31, warp = threadIdx.x >> 5, warps = (int)blockDim.x >> 5;
     const int K1 = P.k + 1;
-    if (i == 0) flags_sh = 0;
+    if (threadIdx.x == 0) flags_sh = 0;
     __syncthreads();
-    if (i < K1) {
+    for (int i = warp; i < K1; i += warps) {
         const int unit = b * K1 + i;
         const bool bonus = (i == P.k);
         const size_t rows = (size_t)P.B * K1;
-        float RT = kEmptyRef, RD = kEmptyRef;
-        for (int g = 0; g < P.G; ++g) {
-            RT = fmaxf(RT, P.all[(size_t)g * rows + unit].st.RT);
-            RD = fmaxf(RD, P.all[(size_t)g * rows + unit].st.RD);
-        }
-        PartialStats st;
-        st.RT = RT; st.RD = RD;
-        st.sT = st.sD = st.w = 0.0;
+        const int xg = bonus ? 0 : P.x[b * P.k + i];
+        const float u = P.u[b * K1 + i];
+        PartialStats st = empty_partial();
         float tx = 0.f, dx = 0.f;
         bool have = false;
-        for (int g = 0; g < P.G; ++g) {
-            const VpRecord r = P.all[(size_t)g * rows + unit];
-            const PartialStats q = rescaled(r.st, RT, RD);
-            st.sT += q.sT; st.sD += q.sD; st.w += q.w;
-            if (r.has_token && !have) { have = true; tx = r.tx; dx = r.dx; }
+        for (int g0 = 0; g0 < P.G; g0 += 32) {
+            PartialStats part = empty_partial();
+            bool has = false;
+            float t = 0.f, d = 0.f;
+            if (g0 + lane < P.G) {
+                const VpRecord r = P.all[(size_t)(g0 + lane) * rows + unit];
+                part = r.st;
+                has = r.has_token != 0;
+                t = r.tx;
+                d = r.dx;
+            }
+            part = warp_merge_lanes(part);
+            if (g0 == 0) {
+                st = part;
+            } else {
+                const float RT = fmaxf(st.RT, part.RT), RD = fmaxf(st.RD, part.RD);
+                const PartialStats a = rescaled(st, RT, RD), c = rescaled(part, RT, RD);
+                st.RT = RT; st.RD = RD;
+                st.sT = a.sT + c.sT; st.sD = a.sD + c.sD; st.w = a.w + c.w;
+            }
+            const unsigned m = __ballot_sync(0xffffffffu, has);
+            if (m && !have) {
+                have = true;
+                tx = __shfl_sync(0xffffffffu, t, __ffs(m) - 1);
+                dx = __shfl_sync(0xffffffffu, d, __ffs(m) - 1);
+            }
         }
+        const RowLogs logs = warp_row_logs(st);
+        if (lane != 0) continue;
         const RowConst rc = row_constants_of(P.inv_tau, bonus, st);
         P.rowc[unit] = rc;
         uint32_t flags = 0;
@@ -167,10 +201,9 @@ __global__ void __launch_bounds__(96) sd_vp_rows_kernel(const VpParams P) {
         if (!okT || !okD) flags |= SD_STATUS_BAD_ROW;
         bool acc = true;
         if (!bonus) {
-            const double l2ST = log2(st.sT), l2SD = log2(st.sD);
+            const double l2ST = logs.T, l2SD = logs.D;
             if (P.loss) P.loss[b * P.k + i] = (float)(0.6931471805599453 * (st.w / st.sT - l2ST + l2SD));
             acc = false;
-            const int xg = P.x[b * P.k + i];
             if (xg < 0 || xg >= P.V_total || !have) {
                 flags |= SD_STATUS_BAD_TOKEN;
             } else if (okT && okD) {
@@ -183,24 +216,31 @@ __global__ void __launch_bounds__(96) sd_vp_rows_kernel(const VpParams P) {
                     const double l2q = (ddx * (double)P.c - (double)st.RD) - l2SD;
                     rho = exp2(l2p - l2q);
                 }
-                acc = (double)P.u[b * K1 + i] < (rho < 1.0 ? rho : 1.0);
+                acc = (double)u < (rho < 1.0 ? rho : 1.0);
             }
         }
         accepted[i] = acc ? 1 : 0;
         if (flags) atomicOr(&flags_sh, flags);
     }
     __syncthreads();
-    if (i == 0) {
-        int n = P.k;
-        for (int j = 0; j < P.k; ++j)
-            if (!accepted[j]) { n = j; break; }
+    if (warp != 0) return;
+    int n = P.k;
+    for (int i0 = 0; i0 < P.k; i0 += 32) {
+        const unsigned m = __ballot_sync(0xffffffffu, i0 + lane < P.k && !accepted[i0 + lane]);
+        if (m) { n = i0 + __ffs(m) - 1; break; }
+    }
+    if (lane == 0) {
         P.accept_len[b] = n;
         if (P.status) P.status[b] = flags_sh;
+        // until the gradient kernel has the masses, their place counts the blocks that have written theirs
+        *reinterpret_cast<uint32_t*>(P.local_mass + (size_t)b * 2) = 0;
     }
 }
 
 // Second sweep over the shard: one block per (row, slice of sampling regions).  Gradient of every
-// pair row; masses of the regions of row n_b of every sequence (the bonus row when n_b = k).
+// pair row; masses of the regions of row n_b of every sequence (the bonus row when n_b = k); and, by the block that
+// brings that row's last slice, this shard's share of the row's mass (fixed order, fp64).  Rows that are not drawn
+// from skip their masses.
 constexpr int kVpSliceRegions = 32;
 template <int DT>
 __global__ void __launch_bounds__(kVpThreads, 6) sd_vp_grad_kernel(const VpParams P, const int slices) {
@@ -266,22 +306,23 @@ __global__ void __launch_bounds__(kVpThreads, 6) sd_vp_grad_kernel(const VpParam
             if (lane == 0) { rsum[r] = mass; rsum[P.NR + r] = pm; }
         }
     }
-}
-
-// This shard's share of the mass of the row the extra token is drawn from (fixed order, fp64).
-__global__ void __launch_bounds__(32) sd_vp_mass_kernel(const VpParams P) {
-    const int b = blockIdx.x, lane = threadIdx.x;
+    __shared__ int is_last;
+    __syncthreads();
+    if (tid == 0) {
+        __threadfence();
+        is_last = atomicAdd(reinterpret_cast<uint32_t*>(P.local_mass + (size_t)b * 2), 1u) == (uint32_t)slices - 1u;
+        if (is_last) __threadfence();
+    }
+    __syncthreads();
+    if (!is_last || warp > 1) return;
+    // (one warp to each of the two masses)
     const int per = (P.NR + 31) / 32;
     const int j0 = min(P.NR, lane * per), j1 = min(P.NR, j0 + per);
-    await_previous_kernel();
-    launch_dependents();
-    for (int which = 0; which < 2; ++which) {
-        const float* rs = P.region_sums + ((size_t)b * 2 + which) * P.NR;
-        double mine = 0.0;
-        for (int j = j0; j < j1; ++j) mine += (double)rs[j];
-        const double incl = warp_inclusive_scan(mine);
-        if (lane == 31) P.local_mass[b * 2 + which] = incl;
-    }
+    const float* const rs = rsum + (size_t)warp * P.NR;
+    double mine = 0.0;
+    for (int j = j0; j < j1; ++j) mine += (double)__ldcg(rs + j);
+    const double incl = warp_inclusive_scan(mine);
+    if (lane == 31) P.local_mass[(size_t)b * 2 + warp] = incl;
 }
 
 // ---- phase 3 -------------------------------------------------------------------------------
@@ -294,26 +335,49 @@ __global__ void __launch_bounds__(32) sd_vp_draw_kernel(const VpParams P) {
     const int k = P.k, K1 = k + 1;
     await_previous_kernel();
     launch_dependents();
+    // everything that does not depend on where the draw falls is asked for at once: the warp's time is round trips
     const int n = P.accept_len[b];
+    const float uk = P.u[b * K1 + k];
+    const int32_t x_first = lane < k ? P.x[b * k + lane] : -1;
+    double2 mass = make_double2(0.0, 0.0);
+    if (lane < P.G) {
+        const double* const m = P.all_mass + ((size_t)lane * P.B + b) * 2;
+        mass = make_double2(m[0], m[1]);
+    }
+    const int per = (P.NR + 31) / 32;
+    const int j0 = min(P.NR, lane * per), j1 = min(P.NR, j0 + per);
+    constexpr int kHeld = 8;
+    float held[kHeld];
+#pragma unroll
+    for (int q = 0; q < kHeld; ++q) held[q] = j0 + q < j1 ? P.region_sums[(size_t)b * 2 * P.NR + j0 + q] : 0.f;
     const bool bonus = (n == k);
+    const int unit = b * K1 + n;
+    const RowConst rc = P.rowc[unit];
+    // rank g's shares
+    const auto share = [&](int g, int which) {
+        if (P.G > 32) return P.all_mass[((size_t)g * P.B + b) * 2 + which];
+        return __shfl_sync(0xffffffffu, which ? mass.y : mass.x, g);
+    };
     uint32_t flags = 0;
     int which = 0;
     double total = 0.0;
-    for (int g = 0; g < P.G; ++g) total += P.all_mass[((size_t)g * P.B + b) * 2];
+    for (int g = 0; g < P.G; ++g) total += share(g, 0);
     if (!bonus && !(total > 0.0)) {
         // a rejection whose residual has no mass on any rank (q = p and a forced rejection): the extra
         // token comes from p_n, and the status says so
         flags |= SD_STATUS_ZERO_RESIDUAL;
         which = 1;
         total = 0.0;
-        for (int g = 0; g < P.G; ++g) total += P.all_mass[((size_t)g * P.B + b) * 2 + 1];
+        for (int g = 0; g < P.G; ++g) total += share(g, 1);
+#pragma unroll
+        for (int q = 0; q < kHeld; ++q) held[q] = j0 + q < j1 ? P.region_sums[((size_t)b * 2 + 1) * P.NR + j0 + q] : 0.f;
     }
     const int mode = bonus ? 1 : (which ? 2 : 0);
-    const double t = (double)P.u[b * K1 + k] * total;
+    const double t = (double)uk * total;
     int owner = -1, last_with_mass = -1;
     double before = 0.0, run = 0.0;
     for (int g = 0; g < P.G; ++g) {
-        const double m = P.all_mass[((size_t)g * P.B + b) * 2 + which];
+        const double m = share(g, which);
         if (m > 0.0) last_with_mass = g;
         if (owner < 0 && run + m > t) { owner = g; before = run; }
         run += m;
@@ -331,23 +395,30 @@ __global__ void __launch_bounds__(32) sd_vp_draw_kernel(const VpParams P) {
         Params Q;
         memset(&Q, 0, sizeof Q);
         Q.T = P.T; Q.D = P.D; Q.V = P.Vs; Q.c = P.c;
-        const int unit = b * K1 + n;
-        const RowConst rc = P.rowc[unit];
         const size_t offT = (size_t)unit * P.Vs, offD = (size_t)(b * k + (bonus ? 0 : n)) * P.Vs;
         const float* rs = P.region_sums + ((size_t)b * 2 + which) * P.NR;
-        const int per = (P.NR + 31) / 32;
-        const int j0 = min(P.NR, lane * per), j1 = min(P.NR, j0 + per);
+        const auto sum_of = [&](int j) { return (double)rs[j]; };
         double mine = 0.0;
-        for (int j = j0; j < j1; ++j) mine += (double)rs[j];
+#pragma unroll
+        for (int q = 0; q < kHeld; ++q) mine += (double)held[q];
+        for (int j = j0 + kHeld; j < j1; ++j) mine += sum_of(j);
         const double incl = warp_inclusive_scan(mine);
         int cand = 0x7fffffff;
         double cand_prefix = 0.0;
         if (!past_end) {
             double r2 = before + (incl - mine);
-            for (int j = j0; j < j1; ++j) {
-                const double next = r2 + (double)rs[j];
-                if (next > t) { cand = j; cand_prefix = r2; break; }
-                r2 = next;
+#pragma unroll
+            for (int q = 0; q < kHeld; ++q) {
+                if (cand == 0x7fffffff && j0 + q < j1) {
+                    const double next = r2 + (double)held[q];
+                    if (next > t) { cand = j0 + q; cand_prefix = r2; }
+                    else r2 = next;
+                }
+            }
+            for (int j = j0 + kHeld; j < j1 && cand == 0x7fffffff; ++j) {
+                const double next = r2 + sum_of(j);
+                if (next > t) { cand = j; cand_prefix = r2; }
+                else r2 = next;
             }
         }
         const unsigned has = __ballot_sync(0xffffffffu, cand != 0x7fffffff);
@@ -377,7 +448,7 @@ __global__ void __launch_bounds__(32) sd_vp_draw_kernel(const VpParams P) {
     }
     if (lane == 0 && flags && P.status) atomicOr(P.status + b, flags);
     for (int i = lane; i <= k; i += 32)
-        P.tokens[b * K1 + i] = (i < n) ? P.x[b * k + i] : (i == n ? y : -1);
+        P.tokens[b * K1 + i] = (i < n) ? (i == lane ? x_first : P.x[b * k + i]) : (i == n ? y : -1);
 }
 
 }  // namespace sdv
