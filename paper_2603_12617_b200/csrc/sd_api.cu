@@ -372,14 +372,16 @@ bool held_room(const WorkspaceLayout& L) { return L.slices > 0 || L.NRmax * size
 
 // Does a call of `units` rows take sd_held_kernel, and in which shape?  The fewest regions a warp with which every
 // cluster is resident at once (the more SMs, the sooner the rows are there; clusters of more than 11 blocks start
-// and meet late, so they are left to rows that need them); if the clusters need a second round, the most
-// regions a warp, and only where the call would go to the cluster kernel otherwise (`second`).  In us, cluster
-// kernel (start) / here, calls back to back on inputs from HBM:
-//     one round   1 sequence, 4 tokens, 32 000 fp32 16.6 / 9.6;  8, 5, 32 000 bf16 23.0 / 12.3;  1, 4, 128 256 bf16
-//                 20.6 / 12.6, in clusters of 16 with one region a warp 14.8;  4, 5, 128 256 bf16 28.4 / 16.8;
-//                 3, 2, 152 064 fp32 22.9 / 13.2
-//     two rounds  8, 5, 128 256 bf16 35.0 / 29.0;  16, 5, 50 304 bf16 29.1 / 27.6;  32, 4, 32 000 bf16 32.9 / 27.7
-//     three       8, 5, 128 256 fp32 39.1 / 41.2
+// and meet late, so they are left to rows that need them).  In us, cluster kernel (start) / sweeps / here, calls
+// back to back on inputs from HBM:
+//     1 sequence, 4 tokens, 32 000 fp32 16.6 / - / 8.8;  8, 5, 32 000 bf16 23.0 / - / 10.9;  1, 4, 128 256 bf16
+//     20.6 / - / 12.6, in clusters of 16 with one region a warp 14.8;  3, 2, 152 064 fp32 22.9 / - / 13.2;
+//     15 rows of 128 256 fp32 - / 18.6 / 13.5;  33 of 128 256 bf16 - / 21.4 / 15.8;  147 of 32 000 bf16 - / 22.4 / 16.3
+// Of clusters whose size is no power of two, one fewer than the device says is resident has its SMs at once: 45 rows of
+// 65 536 bf16 (clusters of 3, all of them resident by that count) 19.3, 42 rows 14.4; 12 of 152 064 fp32
+// (clusters of 10) 19.2, 9 rows 12.6.
+// A second round costs as much as the first.  Where there are sweeps they are faster then (42 rows of 100 000 bf16 23.7,
+// sweeps 21.2; 48 of 128 256 27.7 and 22.4); the cluster kernel is not (35.0).  `second`: two rounds are allowed.
 // Options that only the cluster kernel has, off their defaults, choose the cluster kernel.
 bool use_held(DeviceState& d, int V, long long units, int dtype, bool second, HeldShape* h) {
     if (option(SD_OPT_CLUSTER) != 0 || option(SD_OPT_LAG) != -1 || option(SD_OPT_PREFETCH) != 0 ||
@@ -394,7 +396,7 @@ bool use_held(DeviceState& d, int V, long long units, int dtype, bool second, He
         int& n = d.held_clusters[dtype][N - 1][C];
         h->C = C; h->N = N;
         if (n < 0 && launch_held<kHeldStep>(d, none, *h, dtype, nullptr, nullptr, &n) != SD_OK) n = 0;
-        if (units <= n || (second && N == kHeldMaxRegions && units <= 2LL * n)) return true;
+        if (units <= ((C & (C - 1)) ? n - 1 : n) || (second && N == kHeldMaxRegions && units <= 2LL * n)) return true;
     }
     return false;
 }
@@ -558,8 +560,10 @@ int choose_stream(DeviceState& d, int V, long long units, int dtype, int* G_out,
 //           375 MB (7) 144 / 148;  100 352: 318 MB (6) 122 / 122, 372 MB (7) 137 / 143;
 //           24 000: 256 MB (10) 101 / 100, 307 MB (12) 116 / 119;  20 000: 191 MB (9) 81.6 / 79.3, 213 MB (10) 85.5 / 87.8;
 //           16 384 and below: faster at every size, 440 MB 179 / 170 (the cluster kernel's stages fit such rows badly)
-// At the small end the two launches more cost the calling thread 5 us, which a caller that issues rounds
-// back to back pays instead of the GPU.
+// The smallest calls go to sd_held_kernel first (use_held); of the others the sweeps are the faster ones however small
+// they are (us, cluster kernel / sweeps as they are now): 100 sequences, 2 tokens, 8 192 bf16 entries, 8 MB 19.6 / 19.5;
+// 64, 8, 1 000 fp32, 4 MB 23.1 / 16.2; 64, 4, 8 192 fp32, 19 MB 24.0 / 19.8; 8, 5, 128 256 bf16, 23 MB 35.0 / 22.4;
+// 16, 5, 50 304 fp32, 35 MB 28.2 / 23.2; 8, 5, 128 256 fp32, 45 MB 35.4 / 26.1.
 // The ensemble stays with the cluster kernel, whose units share a target row: 3 learners on 32 sequences,
 // 8 tokens, bf16 151 / 151; on 16 sequences, 4 tokens, fp32 67.7 / 72.3.
 // Options that only the cluster kernel has, off their defaults, choose the cluster kernel.
@@ -569,8 +573,8 @@ bool use_sweeps(DeviceState& d, int dtype, double bytes, long long units, int V,
     if (option(SD_OPT_CLUSTER) != 0 || option(SD_OPT_LAG) != -1 || option(SD_OPT_PREFETCH) != 0 ||
         option(SD_OPT_L2_BUDGET_MIB) != kL2BudgetMiB || option(SD_OPT_WAIT_POLLS) != (long long)kWaitLimit)
         return false;
-    if (dtype == SD_DTYPE_BF16) return bytes >= 32e6;
-    if (bytes < 48e6 || bytes > 450e6) return false;
+    if (dtype == SD_DTYPE_BF16) return true;
+    if (bytes > 450e6) return false;
     if (V < 18000) return true;
     int G = 0, per = 0, lag = 0;                // row pairs of a round = clusters
     if (choose_stream(d, V, units, dtype, &G, &per, &lag) <= 0) return true;

@@ -155,6 +155,17 @@ __device__ __forceinline__ int total_units(const Params& P) {
     return ENS ? P.B * P.k * P.learners : P.B * (P.k + 1);
 }
 
+// Adds to a counter of the whole GPU and says whether that made it `all`.  What this thread has written, or has seen
+// written by its block at a barrier, is visible to whoever brings the last share; and that one sees what all of
+// them had.  (A release on the way up and an acquire for the last one only: less to wait for than __threadfence,
+// which asks for an order of all writes of all threads, on both sides of a plain atomic.)
+__device__ __forceinline__ bool count_up(uint32_t* p, uint32_t n, uint32_t all) {
+    uint32_t old;
+    asm volatile("atom.add.release.gpu.global.u32 %0, [%1], %2;" : "=r"(old) : "l"(p), "r"(n) : "memory");
+    if (old + n != all) return false;
+    asm volatile("fence.acq_rel.gpu;" ::: "memory");
+    return true;
+}
 // Programmatic dependent launch: let the next kernel's blocks come as soon as there is room / wait until
 // the kernel before has finished and its writes are visible.
 __device__ __forceinline__ void launch_dependents() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
@@ -865,11 +876,7 @@ __device__ __noinline__ void resolve_sequence(const Params& P, int b, int known_
 // Tickets of one block for sequence b: `n` of the sequence's tickets at once, by one thread, after everything the tickets stand for has been ordered before
 // this thread.  True if these were the last tickets of the sequence.
 __device__ __forceinline__ bool take_tickets(const Params& P, int b, uint32_t n) {
-    __threadfence();
-    const uint32_t old = atomicAdd(P.ticket + b, n);
-    const bool last = (old + n == P.tickets);
-    if (last) __threadfence();
-    return last;
+    return count_up(P.ticket + b, n, P.tickets);
 }
 
 }  // namespace sdv

@@ -79,13 +79,8 @@ __global__ void __launch_bounds__(kErrThreads, 4) sd_errpos_kernel(const __grid_
     }
 
     // the block's masses are out before its ticket is; the last ticket of the sequence draws
-    __threadfence();
     __syncthreads();
-    if (tid == 0) {
-        const uint32_t old = atomicAdd(P.ticket + b, 1u);
-        is_last = (old == (uint32_t)slices - 1u);
-        if (is_last) __threadfence();
-    }
+    if (tid == 0) is_last = count_up(P.ticket + b, 1u, (uint32_t)slices);
     __syncthreads();
     if (is_last && warp == 0) resolve_sequence<DT, true>(P, b);   // also sets ticket and status words back to zero
 }

@@ -150,13 +150,8 @@ __global__ void __launch_bounds__(kGreedyThreads, 4) sd_greedy_kernel(const Gree
     }
 
     // this block's keys are out before its ticket is
-    __threadfence();
     __syncthreads();
-    if (tid == 0) {
-        const uint32_t old = atomicAdd(P.ticket, 1u);
-        is_last = (old == gridDim.x - 1);
-        if (is_last) __threadfence();
-    }
+    if (tid == 0) is_last = count_up(P.ticket, 1u, gridDim.x);
     __syncthreads();
     if (!is_last) return;
 

@@ -389,6 +389,7 @@ sd_held_kernel(const __grid_constant__ Params P, HeldCandidate* const cand) {
                 int got = 0;
                 if (lane == 0) got = take_tickets(P, ur.b, tickets) ? 1 : 0;
                 last_ticket = __shfl_sync(0xffffffffu, got, 0) != 0;
+                __syncwarp();
             }
             break;
         }

@@ -671,6 +671,7 @@ sd_stream_kernel(const __grid_constant__ Params P, const int lag_stages, const i
                 int last = 0;
                 if (lane == 0) last = take_tickets(P, b, (uint32_t)seg) ? 1 : 0;
                 last = __shfl_sync(0xffffffffu, last, 0);
+                __syncwarp();
                 if (last) resolve_sequence<DT, true>(P, b);
                 seg = 0;
                 __syncwarp();

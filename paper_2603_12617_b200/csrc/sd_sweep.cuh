@@ -526,12 +526,8 @@ sd_sweep_grad_kernel(const __grid_constant__ Params P, const __grid_constant__ S
             for (int w = 0; w < kSweepWarps; ++w) e += (double)hpart[w];
             if (SD_IN(slice, P.hint_stride, 27)) P.hint_part[(size_t)unit * P.hint_stride + slice] = e;
         }
-        __threadfence();
-        is_last = SD_IN(unit, total_units<false>(P), 28) && atomicAdd(S.arrived + unit, 1u) == (uint32_t)slices - 1u;
-        if (is_last) {
-            __threadfence();
-            S.arrived[unit] = 0;
-        }
+        is_last = SD_IN(unit, total_units<false>(P), 28) && count_up(S.arrived + unit, 1u, (uint32_t)slices);
+        if (is_last) S.arrived[unit] = 0;
     }
     __syncwarp();
     if (is_last) sweep_row_done<DT, HINT, RAGGED>(P, S, unit, n, rc);

@@ -308,11 +308,7 @@ __global__ void __launch_bounds__(kVpThreads, 6) sd_vp_grad_kernel(const VpParam
     }
     __shared__ int is_last;
     __syncthreads();
-    if (tid == 0) {
-        __threadfence();
-        is_last = atomicAdd(reinterpret_cast<uint32_t*>(P.local_mass + (size_t)b * 2), 1u) == (uint32_t)slices - 1u;
-        if (is_last) __threadfence();
-    }
+    if (tid == 0) is_last = count_up(reinterpret_cast<uint32_t*>(P.local_mass + (size_t)b * 2), 1u, (uint32_t)slices);
     __syncthreads();
     if (!is_last || warp > 1) return;
     // (one warp to each of the two masses)
