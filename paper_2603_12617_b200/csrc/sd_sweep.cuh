@@ -103,8 +103,10 @@ __device__ __forceinline__ PartialStats load_partial_cg(const PartialStats* p) {
 // place), the target's entries are moved into place: two neighbouring vectors and a funnel shift that is
 // the same for the whole row, 15 instructions for 8 bf16 pairs.  A bonus row is laid out on itself.
 // Regions at the ends of a row, where a vector would reach into another row or out of the tensor, are read
-// and written entry by entry.  16 sequences, 5 tokens, 50 257 bf16 entries: 34.9 us, against 91.6 us for the
-// element-wise kernel, whose one block per row reads two bytes a lane.
+// and written entry by entry, out of line and with registers of their own: with one set for both, filled by a
+// function for the ends, every region went through local memory (13 sequences, 8 tokens, 110 593 fp32 entries 67.3 us,
+// 43.9 since; 122, 4, 119 177 302 and 213; 64, 4, 100 001 bf16 84.9 and 62.8).  16 sequences, 5 tokens, 50 257 bf16
+// entries: 27.2 us, against 91.6 us for the element-wise kernel, whose one block per row reads two bytes a lane.
 template <int DT> struct RowFrame {
     const typename Elem<DT>::type *rowT, *rowD;
     const uint4 *T16, *D16;      // vector 0 of the regions, aligned: up to a vector before the row
@@ -176,7 +178,7 @@ __device__ __forceinline__ void load_inner(const RowFrame<DT>& f, int v, int lan
 }
 // Any region, entry by entry; what is not in the row reads as -inf.
 template <int DT, bool BONUS>
-__device__ __noinline__ void load_edge(const RowFrame<DT>& f, int V, int v, int lane, uint4 (&rt)[kRegionRows], uint4 (&rd)[kRegionRows]) {
+__device__ __forceinline__ void load_edge(const RowFrame<DT>& f, int V, int v, int lane, uint4 (&rt)[kRegionRows], uint4 (&rd)[kRegionRows]) {
     using E = Elem<DT>;
     constexpr int VEC = E::VEC;
 #pragma unroll
@@ -193,22 +195,59 @@ __device__ __noinline__ void load_edge(const RowFrame<DT>& f, int V, int v, int 
         rd[g] = E::pack(d);
     }
 }
+// Both passes over a region at an end of the row, out of line: all of its vectors' registers are these functions' own,
+// and the loops over inner regions keep to theirs.
+template <int DT, bool BONUS>
+__device__ __noinline__ Pass1State edge_pass1(const RowFrame<DT> f, int V, int v, int lane, float c, Pass1State s) {
+    uint4 rt[kRegionRows], rd[kRegionRows];
+    load_edge<DT, BONUS>(f, V, v, lane, rt, rd);
+    follow_references<DT, BONUS>(rt, rd, c, s);
+    float sT, sD, sW;
+    region_sums_of<DT, BONUS, true>(rt, rd, c, s.RT, s.RD, sT, sD, sW);
+    s.ls.sT += sT;
+    s.ls.sD += sD;
+    s.ls.w += sW;
+    return s;
+}
+template <int DT, bool BONUS, bool MASS>
+__device__ __noinline__ float edge_pass2(const RowFrame<DT> f, int V, int v, typename Elem<DT>::type* grow, int lane, float c, const RowConst rc) {
+    using E = Elem<DT>;
+    constexpr int VEC = E::VEC;
+    uint4 rt[kRegionRows], rd[kRegionRows];
+    float unused = 0.f;
+    load_edge<DT, BONUS>(f, V, v, lane, rt, rd);
+    const float mass = pass2_region_impl<DT, BONUS, false, MASS>(rt, rd, kRegionVecs, lane, c, rc, nullptr, rt, unused);
+    if (!BONUS && grow) {
+#pragma unroll
+        for (int g = 0; g < kRegionRows; ++g) {
+            float t[VEC], d[VEC];
+            E::unpack(rt[g], t);
+            E::unpack(rd[g], d);
+            const int e0 = (v + g * 32 + lane) * VEC - f.lead;
+#pragma unroll
+            for (int z = 0; z < VEC; ++z)
+                if (e0 + z >= 0 && e0 + z < V && SD_IN(e0 + z, V, 18)) E::store(grow, e0 + z, grad_elem(t[z], d[z], c, rc));
+        }
+    }
+    return mass;
+}
 
 template <int DT, bool BONUS>
 __device__ __forceinline__ void ragged_pass1(const RowFrame<DT>& f, int V, int v0, int v1, int lane, float c, uint64_t policy,
                                              Pass1State& s) {
     for (int v = v0; v < v1; v += kSweepStep) {
+        if (!inner_region<DT>(f, V, v)) {
+            s = edge_pass1<DT, BONUS>(f, V, v, lane, c, s);
+            continue;
+        }
         uint4 rt[kRegionRows], rd[kRegionRows];
-        const bool inner = inner_region<DT>(f, V, v);
-        if (inner && !inner_in_bounds<DT, BONUS>(f, V, v)) continue;
-        if (inner) load_inner<DT, BONUS>(f, v, lane, policy, rt, rd);
-        else       load_edge<DT, BONUS>(f, V, v, lane, rt, rd);
+        if (!inner_in_bounds<DT, BONUS>(f, V, v)) continue;
+        load_inner<DT, BONUS>(f, v, lane, policy, rt, rd);
         follow_references<DT, BONUS>(rt, rd, c, s);     // (every region, as the element-wise kernel does)
         float sT = 0.f, sD = 0.f, sW = 0.f;
-        if (inner) region_sums_of<DT, BONUS, false>(rt, rd, c, s.RT, s.RD, sT, sD, sW);
-        // masked target entries (a NaN) or a row's end: with the test for them
-        if (!inner || __any_sync(0xffffffffu, sW != sW))
-            region_sums_of<DT, BONUS, true>(rt, rd, c, s.RT, s.RD, sT, sD, sW);
+        region_sums_of<DT, BONUS, false>(rt, rd, c, s.RT, s.RD, sT, sD, sW);
+        // masked target entries (a NaN): with the test for them
+        if (__any_sync(0xffffffffu, sW != sW)) region_sums_of<DT, BONUS, true>(rt, rd, c, s.RT, s.RD, sT, sD, sW);
         s.ls.sT += sT;
         s.ls.sD += sD;
         s.ls.w += sW;
@@ -220,33 +259,19 @@ __device__ __forceinline__ void ragged_pass1(const RowFrame<DT>& f, int V, int v
 template <int DT, bool BONUS, bool MASS>
 __device__ __forceinline__ void ragged_pass2(const RowFrame<DT>& f, int V, int v0, int v1, typename Elem<DT>::type* grow, float* rsum,
                                              int lane, float c, const RowConst& rc) {
-    using E = Elem<DT>;
-    constexpr int VEC = E::VEC;
+    constexpr int VEC = Elem<DT>::VEC;
     for (int v = v0; v < v1; v += kSweepStep) {
-        uint4 rt[kRegionRows], rd[kRegionRows];
         float mass = 0.f, unused = 0.f;
         if (v >= f.nvec) {
             if (!MASS) break;
         } else if (inner_region<DT>(f, V, v)) {
+            uint4 rt[kRegionRows], rd[kRegionRows];
             if (!inner_in_bounds<DT, BONUS>(f, V, v)) continue;       // (the gradient lies where the draft does)
             load_inner<DT, BONUS>(f, v, lane, policy_discard(), rt, rd);
             mass = pass2_region_impl<DT, BONUS, false, MASS>(rt, rd, kRegionVecs, lane, c, rc,
                                                              grow ? grow + (size_t)v * VEC - f.lead : nullptr, rt, unused);
         } else {
-            load_edge<DT, BONUS>(f, V, v, lane, rt, rd);
-            mass = pass2_region_impl<DT, BONUS, false, MASS>(rt, rd, kRegionVecs, lane, c, rc, nullptr, rt, unused);
-            if (!BONUS && grow) {
-#pragma unroll
-                for (int g = 0; g < kRegionRows; ++g) {
-                    float t[VEC], d[VEC];
-                    E::unpack(rt[g], t);
-                    E::unpack(rd[g], d);
-                    const int e0 = (v + g * 32 + lane) * VEC - f.lead;
-#pragma unroll
-                    for (int z = 0; z < VEC; ++z)
-                        if (e0 + z >= 0 && e0 + z < V && SD_IN(e0 + z, V, 18)) E::store(grow, e0 + z, grad_elem(t[z], d[z], c, rc));
-                }
-            }
+            mass = edge_pass2<DT, BONUS, MASS>(f, V, v, grow, lane, c, rc);
         }
         if constexpr (MASS) {
             if (lane == 0) *rsum = mass;
@@ -291,7 +316,7 @@ __device__ __forceinline__ void sweep_pass1(const uint4* gT, const uint4* gD, in
 
 // One block per item: blockIdx.x = unit, blockIdx.y = slice.
 template <int DT, bool RAGGED>
-__global__ void __launch_bounds__(kSweepThreads, RAGGED ? 4 : 6)
+__global__ void __launch_bounds__(kSweepThreads, !RAGGED ? 6 : DT == SD_DTYPE_F32 ? 6 : 5)
 sd_sweep_stats_kernel(const __grid_constant__ Params P, const __grid_constant__ Sweep S) {
     using E = Elem<DT>;
     using ET = typename E::type;
