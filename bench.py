@@ -282,7 +282,9 @@ def kernel_names(path, info) -> str:
     or the element-wise kernel where the library took those (sd_launch_info)."""
     if info["path"] == 0:
         return "sd_generic_kernel"
-    if info["path"] in (1, 3, 4) and info["threads"] == 512:
+    if info["path"] == 4 and info.get("threads") == 512:
+        return "sd_held_kernel<pass 1 only> + sd_held_kernel<drawn rows>"
+    if info["path"] in (1, 3) and info.get("threads") == 512:
         return path.kernel.replace("sd_stream_kernel", "sd_held_kernel")
     if info["path"] in (1, 4) and info["kernels"] == 3:
         return "sd_sweep_stats_kernel + sd_sweep_rows_kernel + sd_sweep_grad_kernel"

@@ -1,0 +1,95 @@
+"""The calling thread's part in C++ (csrc/sd_native.cpp): what it takes it answers as the general way does, and it
+leaves everything else to that way."""
+import types
+
+import pytest
+import torch
+
+from paper_2603_12617_b200 import binding, shard
+
+NONE = types.SimpleNamespace(**{n: (lambda *a: None) for n in ("step", "hint", "greedy", "errors", "ensemble", "lmhead", "vp_partial",
+                                                               "vp_finish", "vp_draw")})
+
+
+def test_anything_but_device_tensors_is_left_to_the_general_way():
+    T, D = torch.zeros(1, 3, 8), torch.zeros(1, 2, 8)
+    x, u = torch.zeros(1, 2, dtype=torch.int32), torch.zeros(1, 3)
+    n = binding._native
+    assert n.step(T, D, x, u, 1.0, True, True) is None
+    assert n.step(T, D, x, u, 1.0) is None and n.step(None, 1, "x", [], {}, True, True) is None
+    assert n.greedy(T, x, True) is None and n.errors(T, D, x, u, 1.0, True, True, True) is None
+    assert n.hint(T, D, x, u, 1.0, D, T) is None and n.ensemble(T, [D], 1.0, 1.0, None, True, False) is None
+    assert n.lmhead(D[0], D[0]) is None and n.vp_partial(T, D, x, 1.0, 0, 8, T, None) is None
+    assert n.vp_finish(T, D, x, u, 1.0, 0, 8, T, 1, 0, T, True, True) is None
+    assert n.vp_draw(T, D, x, u, 1.0, 0, 8, x, T, 1, 0, x, T) is None
+    with pytest.raises(ValueError):
+        binding.sd_verify_feedback(T, D, x, u, 1.0)
+    with pytest.raises(TypeError):
+        n.bind(1, 2)
+
+
+def flat(o):
+    if isinstance(o, torch.Tensor) or o is None:
+        return [o]
+    if isinstance(o, (list, tuple)):
+        return [t for v in o for t in flat(v)]
+    return [t for v in vars(o).values() for t in flat(v)]
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("dtype", [torch.float32, torch.bfloat16])
+def test_same_answers_as_the_general_way(dtype, monkeypatch):
+    B, k, V = 3, 2, 4096
+    g = torch.Generator(device="cuda").manual_seed(3)
+    T = torch.randn(B, k + 1, V, device="cuda", generator=g).to(dtype)
+    D = torch.randn(B, k, V, device="cuda", generator=g).to(dtype)
+    x = torch.randint(0, V, (B, k), device="cuda", dtype=torch.int32, generator=g)
+    u = torch.rand(B, k + 1, device="cuda", generator=g)
+    code = binding._dtype_code(T)
+    cum = torch.rand(2, device="cuda", dtype=torch.float64, generator=g)
+    ws = torch.empty(binding.sd_hint_workspace_bytes(B, k, V, code), dtype=torch.uint8, device="cuda")
+    vws = torch.empty(binding.sd_vp_workspace_bytes(B, k, V, code), dtype=torch.uint8, device="cuda")
+    calls = {
+        "step": lambda T=T, x=x, tau=0.8: binding.sd_verify_feedback(T, D, x, u, tau),
+        "step without": lambda: binding.sd_verify_feedback(T, D, x, u, 1, want_loss=False, want_grad=False),
+        "greedy": lambda T=T: binding.sd_verify_greedy(T, x),
+        "greedy without": lambda: binding.sd_verify_greedy(T, x, want_argmax=False),
+        "errors": lambda: binding.sd_verify_error_feedback(T, D, x, u, 0.8),
+        "errors without": lambda: binding.sd_verify_error_feedback(T, D, x, u, 0.8, want_loss=False, want_grad=False, want_status=False),
+        "hint": lambda: binding.sd_verify_feedback_hint(T, D, x, u, 0.8, D, workspace=ws),
+        "ensemble": lambda: binding.sd_ensemble_feedback(T, [D, D], 0.8, 10.0, cum_loss=cum, want_status=True),
+        "ensemble without": lambda: binding.sd_ensemble_feedback(T, (D,), 0.8, 10, want_grad=False),
+        "lmhead": lambda: binding.sd_lmhead_grad(D.bfloat16().view(B * k, V), T[0, :1, :64].bfloat16().expand(B * k, 64).contiguous()),
+    }
+
+    def vp():
+        rec = binding.sd_vp_partial(T, D, x, 0.8, 0, V, vws)
+        f = binding.sd_vp_finish(T, D, x, u, 0.8, 0, V, rec, 1, 0, vws)
+        return rec, f, binding.sd_vp_draw(T, D, x, u, 0.8, 0, V, f.accept_len, f.local_mass, 1, 0, f.status, vws)
+    calls["vp"] = vp
+    native = binding._native
+    for name, call in calls.items():
+        with monkeypatch.context() as m:
+            m.setattr(binding, "_native", NONE)
+            want = flat(call())
+        got = flat(call())
+        torch.cuda.synchronize()
+        assert len(got) == len(want), name
+        for a, b in zip(got, want):
+            assert (a is None) == (b is None), name
+            if a is not None:
+                assert (a.dtype, a.shape, a.stride(), a.device) == (b.dtype, b.shape, b.stride(), b.device), name
+                assert torch.equal(a.contiguous().view(torch.uint8), b.contiguous().view(torch.uint8)), name
+    # taken only as they are: no views of other layouts, no subclasses, nothing that raises the general way
+    class Mine(torch.Tensor):
+        pass
+    assert native.step(T, D, x, u, 0.8, True, True) is not None
+    for bad in ((T.transpose(0, 1).contiguous().transpose(0, 1), x), (T, x.long()), (T.as_subclass(Mine), x), (T[:, :2], x)):
+        assert native.step(bad[0], D, bad[1], u, 0.8, True, True) is None
+        assert native.greedy(bad[0], bad[1], True) is None or bad[0].shape[1] == 2
+    assert native.step(T, D, x, u, "1", True, True) is None
+    with pytest.raises(ValueError):
+        binding.sd_verify_feedback(T, D, x.long(), u, 0.8)
+    with pytest.raises(binding.SdVerifyError):
+        binding.sd_verify_feedback(T, D, x, u, 0.0)
+    assert shard.vocab_cuts(V, 1, T.element_size())[0] == (0, V)
