@@ -27,10 +27,11 @@
  *   - Unless an argument is documented as HOST, every pointer is a DEVICE pointer owned by the
  *     caller.  The library never frees or reallocates caller memory.
  *   - Tensors are dense, row-major, contiguous.  Logit rows may start at any element-aligned
- *     address.  Rows whose byte length and base address are multiples of 16 take one persistent
- *     kernel (bulk copies, clusters) or, in batches for which that is faster, two sweeps of small
- *     blocks.  Rows of other lengths take the two sweeps as well where they are long or many enough
- *     and the gradient starts at the same place within 16 bytes as the draft logits (up to 1.7 times the
+ *     address.  Rows whose byte length and base address are multiples of 16 are held in registers by
+ *     clusters of blocks where all rows of the call are on the chip at once; other such calls take two
+ *     sweeps of small blocks or, large batches of fp32 logits, one persistent kernel (bulk copies,
+ *     clusters).  Rows of other lengths take the two sweeps as well where they are long or many enough
+ *     and the gradient starts at the same place within 16 bytes as the draft logits (up to 1.5 times the
  *     time of padded rows); everything else takes an element-wise kernel (two to six times).  All give
  *     the same results but for the order of sums: pad the vocabulary to a multiple of 8 entries if you can.
  *   - Work is enqueued on `stream` (a cudaStream_t passed as void*, NULL = the legacy default
@@ -270,8 +271,9 @@ size_t sd_greedy_workspace_bytes(int B, int k);
  *                                      bytes, or NULL for the library's own
  *   stream                        in   cudaStream_t
  * Rows must be whole 16-byte vectors and every tensor 16-byte aligned (SD_ERR_ALIGN otherwise:
- * there is no element-wise path for this entry point).  Two kernels are enqueued: the streaming
- * kernel of sd_verify_feedback over (sequence, row, learner) units, then a one-block reduction.
+ * there is no element-wise path for this entry point).  Two kernels are enqueued: one of the kernels
+ * of sd_verify_feedback over (sequence, row, learner) units (the persistent one, or that which holds
+ * the rows), then a one-block reduction.
  */
 int sd_ensemble_feedback(const void* target_logits, const void* const* draft_logits, int n_learners,
                          float temperature, float epsilon, int B, int k, int V, int dtype,
@@ -424,7 +426,8 @@ int sd_verify_feedback_host(const void* target_logits, const void* draft_logits,
  *   SD_OPT_PREFETCH              env SD_VERIFY_PREFETCH         default 0    non-zero: while a block is in
  *                                its second pass over a row pair it asks L2 to fetch the next row pair
  * SD_OPT_CLUSTER, _LAG, _L2_BUDGET_MIB, _WAIT_POLLS and _PREFETCH are options of the cluster kernel: off
- * their defaults they also keep calls from the two sweeps, which have neither clusters nor waits.
+ * their defaults they also keep calls from the two sweeps and from the kernel that holds the rows, which
+ * have no such options and no waits that could give up.
  * sd_set_option returns SD_OK, or SD_ERR_SHAPE for an unknown option; sd_get_option returns the
  * value in force, or -1 for an unknown option.
  */
@@ -442,8 +445,8 @@ long long sd_get_option(int option_id);
 
 /*
  * sd_launch_info -- HOST out-parameters describing how the last successful device call on this
- * thread was launched: path (0 = generic, 1 = fast path (one kernel: cluster kernel, three: the two sweeps),
- * 2 = greedy verification, 3 = ensemble feedback, 4 = error-position feedback, 5 = output-layer gradient,
+ * thread was launched: path (0 = generic, 1 = fast path (one kernel: cluster kernel or, with 512 threads a
+ * block, held rows; three: the two sweeps), 2 = greedy verification, 3 = ensemble feedback, 4 = error-position feedback, 5 = output-layer gradient,
  * 6 = vocabulary-parallel step), cluster size, threads per block, dynamic shared memory per block, blocks
  * launched, kernels launched (sd_verify_feedback_host: of all its slices).  Any pointer may be NULL.
  * Diagnostic only.

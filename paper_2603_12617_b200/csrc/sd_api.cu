@@ -190,7 +190,7 @@ struct DeviceState {
     // together they have less than four times the bytes of ws, and the 64th would be larger than the GPU.
     void* ws_retired[64] = {};
     int n_retired = 0;
-    bool held_attr[2][kHeldMaxRegions][4] = {};                   // sd_held_kernel may have large clusters
+    bool held_attr[2][kHeldMaxRegions][kHeldModes] = {};                   // sd_held_kernel may have large clusters
     int held_clusters[2][kHeldMaxRegions][kHeldMaxCluster + 1];   // resident clusters of sd_held_kernel, -1 = not asked yet
     bool attr_set[2][4] = {};   // shared-memory / cluster attributes of the fast kernels
     int max_clusters[2][kMaxCluster + 1];   // resident clusters of 1..8 blocks, -1 = not asked yet
@@ -320,7 +320,7 @@ int launch_held_of(DeviceState& d, const Params& P, int C, HeldCandidate* cand, 
     auto kern = sd_held_kernel<DT, N, MODE>;
     cudaLaunchConfig_t cfg;
     memset(&cfg, 0, sizeof cfg);
-    const unsigned grid = (unsigned)(resident ? C : (MODE == kHeldEnsemble ? P.B * P.k * P.learners : P.B * (P.k + 1)) * C);
+    const unsigned grid = (unsigned)(resident ? C : (MODE == kHeldDraw ? P.B : MODE == kHeldEnsemble ? P.B * P.k * P.learners : P.B * (P.k + 1)) * C);
     cfg.gridDim = dim3(grid, 1, 1);
     cfg.blockDim = dim3(kHeldThreads, 1, 1);
     cfg.stream = stream;
@@ -372,7 +372,7 @@ bool held_room(const WorkspaceLayout& L) { return L.slices > 0 || L.NRmax * size
 
 // Does a call of `units` rows take sd_held_kernel, and in which shape?  The fewest regions a warp with which every
 // cluster is resident at once (the more SMs, the sooner the rows are there; clusters of more than 11 blocks start
-// and meet late, so they are left to rows that need them).  In us, cluster kernel (start) / sweeps / here, calls
+// and meet late, so they are left to rows that need them).  In us, cluster kernel / sweeps / here, calls
 // back to back on inputs from HBM:
 //     1 sequence, 4 tokens, 32 000 fp32 16.6 / - / 8.8;  8, 5, 32 000 bf16 23.0 / - / 10.9;  1, 4, 128 256 bf16
 //     20.6 / - / 12.6, in clusters of 16 with one region a warp 14.8;  3, 2, 152 064 fp32 22.9 / - / 13.2;
@@ -425,10 +425,15 @@ cudaError_t launch_following(K kern, dim3 grid, int threads, cudaStream_t stream
     return launch_following_clusters(kern, grid, threads, 1u, stream, args...);
 }
 
+// A warp for every row of a sequence, up to sixteen, but no fewer than eight: the blocks of the second sweep come in
+// behind those of the rows kernel while the first sweep still runs, and the smaller these are the more of them
+// (hint error, one draft token, 46 sequences of 129 216 bf16 entries, blocks of two warps 35.0 us, of eight 33.1).
+int rows_threads(int k) { return 32 * (k < 8 ? 8 : k + 1 < kRowsMaxWarps ? k + 1 : kRowsMaxWarps); }
+
 template <int DT, int MODE, bool RAGGED = false>
 int launch_sweeps_of(const Params& P, const Sweep& S, long long units, bool all, cudaStream_t stream) {
     SD_CUDA(launch_following(sd_sweep_stats_kernel<DT, RAGGED>, dim3((unsigned)units, (unsigned)S.slices), kSweepThreads, stream, P, S));
-    SD_CUDA(launch_following(sd_sweep_rows_kernel<DT>, dim3((unsigned)P.B), 32 * (P.k + 1 < kRowsMaxWarps ? P.k + 1 : kRowsMaxWarps), stream, P, S));
+    SD_CUDA(launch_following(sd_sweep_rows_kernel<DT>, dim3((unsigned)P.B), rows_threads(P.k), stream, P, S));
     // the rows that are drawn from, then (if anything of them is wanted) all rows
     const unsigned second = (unsigned)S.draw_blocks + (all ? (unsigned)(units * S.slices) : 0u);
     SD_CUDA(launch_following(sd_sweep_grad_kernel<DT, MODE, RAGGED>, dim3(second), kSweepThreads, stream, P, S));
@@ -1084,7 +1089,13 @@ int sd_verify_error_feedback(const void* target_logits, const void* draft_logits
         return SD_OK;
     }
     if (holds) {
-        rc = launch_held<kHeldErrors>(*d, P, held, dtype, nullptr, st);      // (clears the status words)
+        rc = launch_held<kHeldErrors>(*d, P, held, dtype, nullptr, st);
+        // (fewer rows: more SMs for each)
+        if (rc == SD_OK && use_held(*d, V, B, dtype, false, &held)) rc = launch_held<kHeldDraw>(*d, P, held, dtype, nullptr, st);
+        if (rc != SD_OK) return rc;
+        if (!workspace) keep_scratch(d, L.accept, head);
+        tl_info[0] = 4; tl_info[5] = 2;
+        return SD_OK;
     } else {
         if (out_status) SD_CUDA(cudaMemsetAsync(out_status, 0, (size_t)B * 4, st));   // bits are ORed in on the device
         int G = 0, lag = 0, per = 0;

@@ -72,11 +72,27 @@ __device__ __forceinline__ PartialStats held_merge(const PartialStats* part, int
     return r;
 }
 
+// What a sequence puts out, by one warp: accept length n, token y after it, status.  first: the lane's own draft token
+// (of the first 32), asked for beforehand.
+__device__ __forceinline__ void held_emit(const Params& P, int b, int n, int y, uint32_t status, int32_t first, int lane) {
+    const int k = P.k;
+    if (lane == 0) {
+        P.accept_len[b] = n;
+        if (P.status) P.status[b] = status;
+        P.wstatus[b] = 0;               // ready for the next call
+        P.ticket[b] = 0;
+    }
+    for (int i = lane; i <= k; i += 32) {
+        const int32_t xi = i >= n ? -1 : i == lane ? first : P.x[b * k + i];
+        if (SD_IN(b * (k + 1) + i, P.B * (k + 1), 25)) P.tokens[b * (k + 1) + i] = i == n ? y : xi;
+    }
+}
+
 // End of a sequence, by the warp that took its last ticket.  Of up to 32 rows a lane each asks for everything that may
 // be wanted, so that one round trip does.
 __device__ __forceinline__ void held_finish(const Params& P, const HeldCandidate* cand, int b, int lane) {
     const int k = P.k;
-    const int32_t x_first = (lane < k) ? P.x[b * k + lane] : -1;
+    const int32_t first = lane < k ? P.x[b * k + lane] : -1;
     const uint32_t word = __ldcg(P.wstatus + b);
     int2 c = make_int2(0, 0);
     if (lane <= k && SD_IN(b * (k + 1) + lane, P.B * (k + 1), 20)) c = __ldcg(reinterpret_cast<const int2*>(cand + b * (k + 1) + lane));
@@ -90,16 +106,7 @@ __device__ __forceinline__ void held_finish(const Params& P, const HeldCandidate
     c.x = __shfl_sync(0xffffffffu, c.x, n & 31);
     c.y = __shfl_sync(0xffffffffu, c.y, n & 31);
     if (n >= 32) c = __ldcg(reinterpret_cast<const int2*>(cand + b * (k + 1) + n));
-    if (lane == 0) {
-        P.accept_len[b] = n;
-        if (P.status) P.status[b] = word | (uint32_t)c.y;
-        P.wstatus[b] = 0;               // ready for the next call
-        P.ticket[b] = 0;
-    }
-    for (int i = lane; i <= k; i += 32) {
-        const int32_t xi = (i == lane) ? x_first : ((i < k) ? P.x[b * k + i] : -1);
-        if (SD_IN(b * (k + 1) + i, P.B * (k + 1), 25)) P.tokens[b * (k + 1) + i] = (i < n) ? xi : (i == n ? c.x : -1);
-    }
+    held_emit(P, b, n, c.x, word | (uint32_t)c.y, first, lane);
 }
 
 // Inverse-CDF search inside a region held in registers: `prefix` = mass before it, `t` = target.  The vocabulary
@@ -141,11 +148,11 @@ __device__ __forceinline__ int held_search(const uint4 (&rt)[kRegionRows], const
     return last || first == 0x7fffffff ? lastm : first;
 }
 
-// What the kernel is for.  Errors: first pass only -- row constants, losses and rejection tests (the error-position
-// feedback finishes the one row it needs in a kernel of its own).  Hint: the second pass also sums the squared
+// What the kernel is for.  Errors: first pass only -- row constants, losses and rejection tests; then Draw: the second
+// pass over the one row of every sequence that the error-position feedback wants, a cluster to a sequence.  Hint: the second pass also sums the squared
 // distance to the hint.  Ensemble: the units are those of the ensemble feedback (see UnitRef); nothing is verified
 // or drawn.
-enum HeldMode { kHeldStep = 0, kHeldErrors = 1, kHeldHint = 2, kHeldEnsemble = 3 };
+enum HeldMode { kHeldStep = 0, kHeldErrors = 1, kHeldHint = 2, kHeldEnsemble = 3, kHeldDraw = 4, kHeldModes = 5 };
 
 // cand: workspace [B*(k+1)] (step and hint).
 template <int DT, int N, int MODE>
@@ -154,7 +161,7 @@ sd_held_kernel(const __grid_constant__ Params P, HeldCandidate* const cand) {
     using E = Elem<DT>;
     using ET = typename E::type;
     constexpr int VEC = E::VEC;
-    constexpr bool STATS = MODE == kHeldErrors, HINT = MODE == kHeldHint, ENS = MODE == kHeldEnsemble;
+    constexpr bool STATS = MODE == kHeldErrors, HINT = MODE == kHeldHint, ENS = MODE == kHeldEnsemble, DRAW = MODE == kHeldDraw;
     __shared__ HeldShared sh;
     await_previous_kernel();
     launch_dependents();
@@ -163,7 +170,16 @@ sd_held_kernel(const __grid_constant__ Params P, HeldCandidate* const cand) {
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     cluster_arrive();                                      // (waited for before the first remote store)
 
-    const int unit = (int)blockIdx.x / C;
+    int unit = (int)blockIdx.x / C;
+    if constexpr (DRAW) {
+        // of the sequence, the first rejected row (the bonus row if there is none)
+        const int b = unit;
+        unit = b * (P.k + 1) + P.k;
+        for (int i0 = 0; i0 < P.k; i0 += 32) {
+            const unsigned m = __ballot_sync(0xffffffffu, i0 + lane < P.k && P.accept[b * P.k + i0 + lane] == 0);
+            if (m) { unit = b * (P.k + 1) + i0 + __ffs(m) - 1; break; }
+        }
+    }
     const UnitRef ur = unit_ref<ENS>(P, unit);
     const int slots = C * kHeldWarps, slot = rank * kHeldWarps + warp;
     // this warp's regions [r0, r0 + n)
@@ -193,57 +209,69 @@ sd_held_kernel(const __grid_constant__ Params P, HeldCandidate* const cand) {
             held_load(rd[j][g], gD + vi, in && !ur.bonus, policy);
         }
     }
-    const bool reports = rank == 0 && warp == 0;
+    const bool reports = !DRAW && rank == 0 && warp == 0;
+    RowConst rc;
+    int32_t first = -1;
+    uint32_t word = 0;
+    if constexpr (DRAW) {
+        rc = P.rowc[unit];
+        if (lane < P.k) first = P.x[ur.b * P.k + lane];
+        word = P.wstatus[ur.b];
+    }
     AcceptOperands aop;
     aop.valid = false;
     if (!ENS && reports && lane == 0 && !ur.bonus) aop = load_accept_operands<DT>(P, ur.b, ur.i);
 
     // ---- first pass: references from the maxima of all the warp holds
-    LaneSums ls;
-    ls.init();
-    float RT = kEmptyRef, RD = kEmptyRef;
-    {
-        float mT = -INFINITY, mD = -INFINITY;
+    if constexpr (!DRAW) {
+        LaneSums ls;
+        ls.init();
+        float RT = kEmptyRef, RD = kEmptyRef;
+        {
+            float mT = -INFINITY, mD = -INFINITY;
+#pragma unroll
+            for (int j = 0; j < N; ++j) {
+                mT = fmaxf(mT, region_max<DT>(rt[j]));
+                mD = fmaxf(mD, region_max<DT>(rd[j]));
+            }
+            RT = warp_max_ref(ref_of(mT, P.c));
+            RD = warp_max_ref(ref_of(mD, P.c));
+        }
 #pragma unroll
         for (int j = 0; j < N; ++j) {
-            mT = fmaxf(mT, region_max<DT>(rt[j]));
-            mD = fmaxf(mD, region_max<DT>(rd[j]));
+            if (j < n) {
+                float sT, sD, sW;
+                region_sums_of<DT, false, false>(rt[j], rd[j], P.c, RT, RD, sT, sD, sW);
+                // masked target entries make a NaN: with the test for them
+                if (__any_sync(0xffffffffu, sW != sW)) region_sums_of<DT, false, true>(rt[j], rd[j], P.c, RT, RD, sT, sD, sW);
+                ls.sT += sT;
+                ls.sD += sD;
+                ls.w += sW;
+            }
         }
-        RT = warp_max_ref(ref_of(mT, P.c));
-        RD = warp_max_ref(ref_of(mD, P.c));
-    }
-#pragma unroll
-    for (int j = 0; j < N; ++j) {
-        if (j < n) {
-            float sT, sD, sW;
-            region_sums_of<DT, false, false>(rt[j], rd[j], P.c, RT, RD, sT, sD, sW);
-            // masked target entries make a NaN: with the test for them
-            if (__any_sync(0xffffffffu, sW != sW)) region_sums_of<DT, false, true>(rt[j], rd[j], P.c, RT, RD, sT, sD, sW);
-            ls.sT += sT;
-            ls.sD += sD;
-            ls.w += sW;
+        {
+            // the warp's partial to every block of the cluster
+            const double v = warp_fold_lanes(ls, lane);
+            PartialStats mine;
+            mine.RT = RT; mine.RD = RD;
+            mine.sT = __shfl_sync(0xffffffffu, v, 0);
+            mine.sD = __shfl_sync(0xffffffffu, v, 8);
+            mine.w = __shfl_sync(0xffffffffu, v, 16);
+            cluster_wait();
+            if (lane < C) *cluster.map_shared_rank(&sh.part[slot], lane) = mine;
+            __syncwarp();
         }
-    }
-    {
-        // the warp's partial to every block of the cluster
-        const double v = warp_fold_lanes(ls, lane);
-        PartialStats mine;
-        mine.RT = RT; mine.RD = RD;
-        mine.sT = __shfl_sync(0xffffffffu, v, 0);
-        mine.sD = __shfl_sync(0xffffffffu, v, 8);
-        mine.w = __shfl_sync(0xffffffffu, v, 16);
+        cluster_arrive();
         cluster_wait();
-        if (lane < C) *cluster.map_shared_rank(&sh.part[slot], lane) = mine;
-        __syncwarp();
+        if (warp == 0) {
+            const PartialStats row = held_merge(sh.part, slots, lane);
+            if (lane == 0) { sh.row = row; sh.rc = row_constants(P, ur.bonus, row); }
+        }
+        __syncthreads();
+        rc = sh.rc;
+    } else {
+        cluster_wait();
     }
-    cluster_arrive();
-    cluster_wait();
-    if (warp == 0) {
-        const PartialStats row = held_merge(sh.part, slots, lane);
-        if (lane == 0) { sh.row = row; sh.rc = row_constants(P, ur.bonus, row); }
-    }
-    __syncthreads();
-    RowConst rc = sh.rc;
     if constexpr (STATS) {
         if (reports && lane == 0) {
             if (P.status && ur.i == 0 && SD_IN(ur.b, P.B, 21)) P.status[ur.b] = 0;      // the next kernel ORs its bits in
@@ -253,7 +281,12 @@ sd_held_kernel(const __grid_constant__ Params P, HeldCandidate* const cand) {
     } else {
         // ---- second pass, and a third one, of p_n's masses, if max(0, p - q) has none
         void* const gbase = ENS ? P.Gn[ur.n] : P.grad;
-        ET* gdst = (gbase && !ur.bonus) ? reinterpret_cast<ET*>(gbase) + offD : nullptr;
+        ET* gdst = (gbase && !ur.bonus) ? reinterpret_cast<ET*>(gbase) + (DRAW ? (size_t)ur.b * P.V : offD) : nullptr;
+        if (DRAW && gbase && ur.bonus) {
+            // no error position: a zero row
+            uint4* const z = reinterpret_cast<uint4*>(reinterpret_cast<ET*>(gbase) + (size_t)ur.b * P.V);
+            for (int vi = r0 * kRegionVecs + lane; vi < min(NV, (r0 + n) * kRegionVecs); vi += 32) __stcs(z + vi, make_uint4(0u, 0u, 0u, 0u));
+        }
         const uint4* const gH = HINT ? reinterpret_cast<const uint4*>(reinterpret_cast<const ET*>(P.hint) + offD) : nullptr;
         if constexpr (ENS) {
             if (reports && lane == 0) finish_row_ensemble(P, ur, sh.row);
@@ -377,6 +410,10 @@ sd_held_kernel(const __grid_constant__ Params P, HeldCandidate* const cand) {
                     y = held_search<DT>(ft, fd, (r0 + max(at, 0)) * kRegionVecs * VEC, lane, P.c, rc, before, t, to_last);
                     if (y < 0) y = 0;
                 }
+            }
+            if constexpr (DRAW) {
+                if (mine) held_emit(P, ur.b, ur.i, y, word | flags, first, lane);
+                return;
             }
             // two tickets of a unit: its row report, its candidate
             uint32_t tickets = reports ? 1u : 0u;
