@@ -1090,8 +1090,10 @@ int sd_verify_error_feedback(const void* target_logits, const void* draft_logits
     }
     if (holds) {
         rc = launch_held<kHeldErrors>(*d, P, held, dtype, nullptr, st);
-        // (fewer rows: more SMs for each)
-        if (rc == SD_OK && use_held(*d, V, B, dtype, false, &held)) rc = launch_held<kHeldDraw>(*d, P, held, dtype, nullptr, st);
+        // (fewer rows: more SMs for each, where that shape fits; else the one that has just been launched)
+        HeldShape draw;
+        if (!use_held(*d, V, B, dtype, false, &draw)) draw = held;
+        if (rc == SD_OK) rc = launch_held<kHeldDraw>(*d, P, draw, dtype, nullptr, st);
         if (rc != SD_OK) return rc;
         if (!workspace) keep_scratch(d, L.accept, head);
         tl_info[0] = 4; tl_info[5] = 2;

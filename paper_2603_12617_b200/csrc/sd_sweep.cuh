@@ -19,9 +19,9 @@
 // sd_stream_kernel reads every logit from HBM once, but its 28 consumer warps share one ring and all blocks
 // read at the same time and compute at the same time, so at bf16, where the exponentials take as long as
 // the reads, it moves 2.9 TB/s.  Step on 32 sequences, 8 draft tokens, 128 256 bf16 entries: 71.1 us there,
-// 61.6 us here (first sweep 31, rows 3, second 28); 64 sequences, 4 tokens, 151 936: 93.4 and 74.7 us; one
-// sequence, 4 tokens, 32 000 fp32: 16.5 and 14.5 us.  The rule which of the two a call takes is use_sweeps
-// (host).
+// 58 us here (61.6 before the first kernel was launched programmatically and the maxima taken of packed bf16; first
+// sweep 29, rows 3, second 28); 64 sequences, 4 tokens, 151 936: 93.4 and 72 us; 8, 5, 128 256: 35.0 and 22.
+// The rule which of the two a call takes is use_sweeps (host).
 //
 // Tried and dropped, on the first of these: one persistent kernel whose warps take both passes of an item
 // from per-warp rings of bulk copies (82 us: many 1 KiB copies in flight slow each other down) or of
