@@ -36,18 +36,29 @@ struct HeldShared {
     PartialStats row;
 };
 
-// An entry that adds nothing to any sum and makes no NaN either (its logarithms stay finite).
-template <int DT> __device__ __forceinline__ uint4 held_nothing() {
-    return DT == SD_DTYPE_F32 ? make_uint4(0xf149f2cau, 0xf149f2cau, 0xf149f2cau, 0xf149f2cau)     // -1e30
-                              : make_uint4(0xf149f149u, 0xf149f149u, 0xf149f149u, 0xf149f149u);
-}
-
 // A vector that nothing else will read, or `v` as it is.
 __device__ __forceinline__ void held_load(uint4& v, const uint4* p, bool in, uint64_t policy) {
     asm volatile("{\n\t.reg .pred p;\n\t"
                  "setp.ne.b32 p, %5, 0;\n\t"
                  "@p ld.global.L1::no_allocate.L2::cache_hint.v4.u32 {%0,%1,%2,%3}, [%4], %6;\n\t}"
                  : "+r"(v.x), "+r"(v.y), "+r"(v.z), "+r"(v.w) : "l"(p), "r"((int)in), "l"(policy));
+}
+
+// Softmax sums of a lane's part of a region of which `nv` vectors are in the row (those behind it hold -inf, for which
+// the arithmetic has no test: they are left out by their place).
+template <int DT, bool MASKED>
+__device__ __forceinline__ void held_sums(const uint4 (&rt)[kRegionRows], const uint4 (&rd)[kRegionRows], int nv, int lane, float c,
+                                          float RT, float RD, float& sT, float& sD, float& sW) {
+    using E = Elem<DT>;
+    sT = sD = sW = 0.f;
+#pragma unroll
+    for (int g = 0; g < kRegionRows; ++g) {
+        float tv[E::VEC], dv[E::VEC], pT, pD, pW;
+        E::unpack(rt[g], tv);
+        E::unpack(rd[g], dv);
+        LaneSums::vector_pair<E::VEC, MASKED>(tv, dv, c, -RT, -RD, pT, pD, pW);
+        if (g * 32 + lane < nv) { sT += pT; sD += pD; sW += pW; }
+    }
 }
 
 // Merge of `n` partials in shared memory by one warp.  Every lane gets the same bits.
@@ -202,9 +213,9 @@ sd_held_kernel(const __grid_constant__ Params P, HeldCandidate* const cand) {
         for (int g = 0; g < kRegionRows; ++g) {
             const int vi = (r0 + j) * kRegionVecs + g * 32 + lane;
             const bool in = j < n && vi < NV && SD_IN((long long)vi * VEC + VEC - 1, P.V, 10);
-            rt[j][g] = held_nothing<DT>();
+            rt[j][g] = E::masked();
             // (a bonus row goes the same way with draft logits of 0, whose sums nobody looks at, and kD = 0)
-            rd[j][g] = ur.bonus ? make_uint4(0u, 0u, 0u, 0u) : held_nothing<DT>();
+            rd[j][g] = ur.bonus ? make_uint4(0u, 0u, 0u, 0u) : E::masked();
             held_load(rt[j][g], gT + vi, in, policy);
             held_load(rd[j][g], gD + vi, in && !ur.bonus, policy);
         }
@@ -241,9 +252,10 @@ sd_held_kernel(const __grid_constant__ Params P, HeldCandidate* const cand) {
         for (int j = 0; j < N; ++j) {
             if (j < n) {
                 float sT, sD, sW;
-                region_sums_of<DT, false, false>(rt[j], rd[j], P.c, RT, RD, sT, sD, sW);
+                const int nv = NV - (r0 + j) * kRegionVecs;
+                held_sums<DT, false>(rt[j], rd[j], nv, lane, P.c, RT, RD, sT, sD, sW);
                 // masked target entries make a NaN: with the test for them
-                if (__any_sync(0xffffffffu, sW != sW)) region_sums_of<DT, false, true>(rt[j], rd[j], P.c, RT, RD, sT, sD, sW);
+                if (__any_sync(0xffffffffu, sW != sW)) held_sums<DT, true>(rt[j], rd[j], nv, lane, P.c, RT, RD, sT, sD, sW);
                 ls.sT += sT;
                 ls.sD += sD;
                 ls.w += sW;

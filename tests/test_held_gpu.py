@@ -107,3 +107,26 @@ def test_special_rows(binding, k, V, dtype):
         assert 0 <= n[b] <= k and 0 <= tok[b, n[b]] < V and (tok[b, n[b] + 1:] == -1).all()
     err, rows = alike(binding, Td, Dd, xd, ud, inp.tau, out)
     assert torch.equal(err.loss[good], out.loss[good]) and torch.equal(err.error_grad[good], rows[good])
+
+
+@pytest.mark.parametrize("V,dtype", [(520, "f32"), (256 * 17 - 4, "f32"), (256 * 16 * 4, "f32"), (520, "bf16"), (32000, "bf16")])
+@pytest.mark.parametrize("tau", [2e29, 1e30, 1e33])
+def test_nothing_behind_the_end_of_a_row_takes_part(binding, V, dtype, tau):
+    """So hot that every probability is 1/V to fp32 (logits over the temperature are far below 2^-24): a draw with uniform u is
+    entry u V, off by one at most for the rounding of fp32 sums of equal terms, whether it comes from a bonus row or
+    from a rejection without residual mass; whatever lies behind the row's last entry must have no share in it."""
+    B, k = 24, 2
+    inp = synth.make_inputs(synth.custom_config(B=B, k=k, V=V, dtype=dtype, tau=1.0, index=132))
+    inp.uniforms[:, k] = (np.arange(B) + 0.5).astype(np.float32) / B
+    inp.draft_tokens[1::2, 1] = V                  # every second sequence: rejected there
+    T, D, x, u = to_device(inp)
+    ex = binding.sd_verify_feedback_ex(T, D, x, u, tau)
+    assert binding.sd_launch_info()["threads"] == 512
+    alike(binding, T, D, x, u, tau, ex)
+    hint = binding.sd_verify_feedback_hint(T, D, x, u, tau, torch.zeros_like(D))
+    torch.cuda.synchronize()
+    want = torch.tensor([k, 1] * (B // 2), dtype=torch.int32, device="cuda")
+    for o in (ex, hint):
+        assert torch.equal(o.accept_len, want)
+        assert (o.tokens.gather(1, want[:, None].long()).squeeze(1) - u[:, k] * V).abs().max() <= 1
+        assert (o.loss.abs() <= 1e-6).all() and (o.grad_draft.float().abs() * tau * V <= 1e-6).all()
