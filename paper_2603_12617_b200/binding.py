@@ -545,10 +545,18 @@ def _vp_shapes(target_shard, draft_shard, draft_tokens):
         raise ValueError("shape mismatch between the shards and the draft tokens")
     if target_shard.dtype != draft_shard.dtype:
         raise TypeError("target and draft shards must have the same dtype")
+    if draft_tokens.dtype != torch.int32:
+        raise ValueError("draft_tokens must be int32 [B,k]")
     for t in (target_shard, draft_shard, draft_tokens):
         if not t.is_cuda or not t.is_contiguous():
             raise ValueError("device-resident contiguous tensors expected")
     return B, k, Vs
+
+
+def _vp_holds(name: str, t: torch.Tensor, count: int, *dtypes: torch.dtype) -> None:
+    """The kernels read or write ``count`` entries from the tensor's first on."""
+    if t.dtype not in dtypes or t.numel() < count or not t.is_contiguous():
+        raise ValueError(f"{name} must be a contiguous {dtypes[0]} tensor of {count} entries")
 
 
 def sd_vp_partial(target_shard: torch.Tensor, draft_shard: torch.Tensor, draft_tokens: torch.Tensor,
@@ -564,6 +572,8 @@ def sd_vp_partial(target_shard: torch.Tensor, draft_shard: torch.Tensor, draft_t
     B, k, Vs = _vp_shapes(target_shard, draft_shard, draft_tokens)
     if out_records is None:
         out_records = torch.empty((B * (k + 1), SD_VP_RECORD_BYTES), dtype=torch.uint8, device=target_shard.device)
+    elif not out_records.is_contiguous() or out_records.numel() * out_records.element_size() < B * (k + 1) * SD_VP_RECORD_BYTES:
+        raise ValueError("out_records must be contiguous, with room for B * (k+1) records")
     rc = _lib.sd_vp_partial(_ptr(target_shard), _ptr(draft_shard), _ptr(draft_tokens), float(temperature), B, k, Vs,
                             int(v_offset), int(V_total), _dtype_code(target_shard), _ptr(out_records), _ptr(workspace),
                             workspace.numel() * workspace.element_size(), _stream_ptr(stream))
@@ -594,7 +604,8 @@ def sd_vp_finish(target_shard: torch.Tensor, draft_shard: torch.Tensor, draft_to
                 raise SdVerifyError(r[0], "sd_vp_finish")
             return VpFinishOutputs(r[1], r[2], r[3], r[4], r[5])
     B, k, Vs = _vp_shapes(target_shard, draft_shard, draft_tokens)
-    if all_records.numel() * all_records.element_size() != n_ranks * B * (k + 1) * SD_VP_RECORD_BYTES:
+    _vp_holds("uniforms", uniforms, B * (k + 1), torch.float32)
+    if all_records.numel() * all_records.element_size() != n_ranks * B * (k + 1) * SD_VP_RECORD_BYTES or not all_records.is_contiguous():
         raise ValueError("all_records must hold n_ranks * B * (k+1) records")
     dev = target_shard.device
     accept_len = torch.empty((B,), dtype=torch.int32, device=dev)
@@ -625,7 +636,11 @@ def sd_vp_draw(target_shard: torch.Tensor, draft_shard: torch.Tensor, draft_toke
                 raise SdVerifyError(r[0], "sd_vp_draw")
             return r[1]
     B, k, Vs = _vp_shapes(target_shard, draft_shard, draft_tokens)
-    if all_masses.dtype != torch.float64 or all_masses.numel() != n_ranks * B * 2:
+    _vp_holds("uniforms", uniforms, B * (k + 1), torch.float32)
+    _vp_holds("accept_len", accept_len, B, torch.int32)
+    if status is not None:
+        _vp_holds("status", status, B, torch.int32, torch.uint32)
+    if all_masses.dtype != torch.float64 or all_masses.numel() != n_ranks * B * 2 or not all_masses.is_contiguous():
         raise ValueError("all_masses must be float64 [n_ranks, B, 2]")
     tokens = torch.empty((B, k + 1), dtype=torch.int32, device=target_shard.device)
     rc = _lib.sd_vp_draw(_ptr(target_shard), _ptr(draft_shard), _ptr(draft_tokens), _ptr(uniforms), float(temperature),

@@ -319,7 +319,7 @@ PyObject* vp_partial(PyObject*, PyObject* const* a, Py_ssize_t n) {
     at::Tensor rec;
     if (a[7] != Py_None) {
         const at::Tensor* r = plain(a[7], s.dev);
-        if (!r) return none();
+        if (!r || bytes_of(*r) < (size_t)s.B * (s.k + 1) * kVpRecordBytes) return none();
         rec = *r;
     } else {
         rec = s.make({(int64_t)s.B * (s.k + 1), kVpRecordBytes}, at::kByte);
@@ -372,7 +372,9 @@ PyObject* vp_draw(PyObject*, PyObject* const* a, Py_ssize_t n) {
         return none();
     const at::Tensor *u = s.uniforms(a[3]), *len = u ? plain(a[7], s.dev) : nullptr, *mass = len ? plain(a[8], s.dev) : nullptr;
     const at::Tensor *status = mass ? plain(a[11], s.dev) : nullptr, *ws = status ? plain(a[12], s.dev) : nullptr;
-    if (!ws || ranks < 1 || mass->scalar_type() != at::kDouble || mass->numel() != (int64_t)ranks * s.B * 2) return none();
+    if (!ws || ranks < 1 || mass->scalar_type() != at::kDouble || mass->numel() != (int64_t)ranks * s.B * 2 ||
+        len->scalar_type() != at::kInt || len->numel() < s.B || status->scalar_type() != at::kInt || status->numel() < s.B)
+        return none();
     const at::Tensor tokens = s.make({s.B, s.k + 1}, at::kInt);
     void* const st = s.stream();
     const int rc = unlocked([&] {

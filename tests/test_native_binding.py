@@ -93,3 +93,45 @@ def test_same_answers_as_the_general_way(dtype, monkeypatch):
     with pytest.raises(binding.SdVerifyError):
         binding.sd_verify_feedback(T, D, x, u, 0.0)
     assert shard.vocab_cuts(V, 1, T.element_size())[0] == (0, V)
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("way", ["C++", "general"])
+def test_buffers_of_the_vocabulary_parallel_step_that_are_too_small_or_of_another_type(way, monkeypatch):
+    """What the kernels would read or write from a tensor's first entry on has to be there; more room is fine."""
+    B, k, V = 3, 2, 4096
+    g = torch.Generator(device="cuda").manual_seed(5)
+    T, D = torch.randn(B, k + 1, V, device="cuda", generator=g), torch.randn(B, k, V, device="cuda", generator=g)
+    x = torch.randint(0, V, (B, k), device="cuda", dtype=torch.int32, generator=g)
+    u = torch.rand(B, k + 1, device="cuda", generator=g)
+    ws = torch.empty(binding.sd_vp_workspace_bytes(B, k, V, binding.SD_DTYPE_F32), dtype=torch.uint8, device="cuda")
+    if way == "general":
+        monkeypatch.setattr(binding, "_native", NONE)
+    rows = B * (k + 1)
+    records = binding.sd_vp_partial(T, D, x, 0.8, 0, V, ws)
+    room = torch.full((rows + 2, 48), 7, dtype=torch.uint8, device="cuda")
+    assert binding.sd_vp_partial(T, D, x, 0.8, 0, V, ws, out_records=room) is room
+    assert torch.equal(room[:rows], records) and (room[rows:] == 7).all()
+    for bad in (records[:-1], torch.empty(rows, 96, dtype=torch.uint8, device="cuda")[:, :48], torch.empty(0, dtype=torch.uint8, device="cuda")):
+        with pytest.raises(ValueError):
+            binding.sd_vp_partial(T, D, x, 0.8, 0, V, ws, out_records=bad)
+    with pytest.raises(ValueError):
+        binding.sd_vp_partial(T, D, x.long(), 0.8, 0, V, ws)
+    f = binding.sd_vp_finish(T, D, x, u, 0.8, 0, V, records, 1, 0, ws)
+    for bad in (u.double(), u[:, :k].contiguous(), u.t()):
+        with pytest.raises(ValueError):
+            binding.sd_vp_finish(T, D, x, bad, 0.8, 0, V, records, 1, 0, ws)
+        with pytest.raises(ValueError):
+            binding.sd_vp_draw(T, D, x, bad, 0.8, 0, V, f.accept_len, f.local_mass, 1, 0, f.status, ws)
+    with pytest.raises(ValueError):
+        binding.sd_vp_finish(T, D, x, u, 0.8, 0, V, records.expand(1, rows, 48)[:, :1].expand(1, rows, 48), 1, 0, ws)
+    n, st = f.accept_len, f.status
+    want = binding.sd_vp_draw(T, D, x, u, 0.8, 0, V, n, f.local_mass, 1, 0, st, ws)
+    for good in ((n, None), (n, st.view(torch.uint32)), (torch.cat([n, n]), torch.cat([st, st]))):
+        assert torch.equal(binding.sd_vp_draw(T, D, x, u, 0.8, 0, V, good[0], f.local_mass, 1, 0, good[1], ws), want)
+    for bad in ((n.long(), st), (n[:-1], st), (n.float(), st), (n, st.long()), (n, st[:-1]), (n, st.float())):
+        with pytest.raises(ValueError):
+            binding.sd_vp_draw(T, D, x, u, 0.8, 0, V, bad[0], f.local_mass, 1, 0, bad[1], ws)
+    with pytest.raises(ValueError):
+        binding.sd_vp_draw(T, D, x, u, 0.8, 0, V, n, f.local_mass[:1].expand(B, 2), 1, 0, st, ws)
+    torch.cuda.synchronize()
