@@ -332,7 +332,8 @@ __global__ void __launch_bounds__(32) sd_vp_draw_kernel(const VpParams P) {
     await_previous_kernel();
     launch_dependents();
     // everything that does not depend on where the draw falls is asked for at once: the warp's time is round trips
-    const int n = P.accept_len[b];
+    // (the caller's memory: a length that phase 2 cannot have written leads to no row but the sequence's own)
+    const int n = min(max(P.accept_len[b], 0), k);
     const float uk = P.u[b * K1 + k];
     const int32_t x_first = lane < k ? P.x[b * k + lane] : -1;
     double2 mass = make_double2(0.0, 0.0);

@@ -220,3 +220,24 @@ def test_two_late_large_entries_are_no_less_exact_than_early_ones(binding):
     p = p.gather(2, at[:, :k])
     bound = p * (1 - p) * 2 * (2.0 ** -22 + 2.0 ** -23 * np.log(2)) + 3 * 2.0 ** -24 * p
     assert (err <= bound).all(), (err / bound).max()
+
+
+@pytest.mark.parametrize("G", [1, 3])
+def test_accept_lengths_out_of_range_are_taken_as_the_nearest_in_it(binding, G):
+    """accept_len is the caller's memory: whatever it holds, no rank reads another row than the sequence's own."""
+    B, k, V = 6, 3, 4096
+    inp = synth.make_inputs(synth.custom_config(B=B, k=k, V=V, dtype="f32", index=76))
+    T, D, x, u = to_device(inp)
+    cuts = shard.vocab_cuts(V, G, 4)
+    Ts, Ds = [T[:, :, a:b].contiguous() for a, b in cuts], [D[:, :, a:b].contiguous() for a, b in cuts]
+    ws = [torch.empty(max(256, binding.sd_vp_workspace_bytes(B, k, b - a, binding.SD_DTYPE_F32)), dtype=torch.uint8, device="cuda") for a, b in cuts]
+    recs = torch.stack([binding.sd_vp_partial(Ts[g], Ds[g], x, inp.tau, cuts[g][0], V, ws[g]) for g in range(G)])
+    fins = [binding.sd_vp_finish(Ts[g], Ds[g], x, u, inp.tau, cuts[g][0], V, recs, G, g, ws[g]) for g in range(G)]
+    masses = torch.stack([f.local_mass for f in fins])
+    lens = torch.tensor([-1, k + 1, -2 ** 31, 2 ** 31 - 1, 0, k], dtype=torch.int32, device="cuda")
+    for g in range(G):
+        got, want = (binding.sd_vp_draw(Ts[g], Ds[g], x, u, inp.tau, cuts[g][0], V, n, masses, G, g, None, ws[g]) for n in (lens, lens.clamp(0, k)))
+        torch.cuda.synchronize()
+        assert torch.equal(got, want)
+        n = lens.clamp(0, k).tolist()
+        assert all(got[b, :n[b]].tolist() == x[b, :n[b]].tolist() and (got[b, n[b] + 1:] == -1).all() for b in range(B))
