@@ -119,13 +119,21 @@ template <class... A> PyObject* answer(int rc, const A&... outs) {
     for (Py_ssize_t i = 0; i < n; ++i) PyTuple_SET_ITEM(r, i, items[i]);
     return r;
 }
-// The library's functions run without the interpreter's lock, as ctypes runs them.
-template <class F> int unlocked(F&& f) {
-    int rc;
-    Py_BEGIN_ALLOW_THREADS
-    rc = f();
-    Py_END_ALLOW_THREADS
-    return rc;
+// Calls `f` without the interpreter's lock, as ctypes does.  Its arguments are evaluated before the lock is given up: a
+// tensor's address may have to be made (a lazy copy) or be refused with an exception.  And whatever leaves here leaves
+// with the lock.
+class Unlocked {
+    PyThreadState* const state = PyEval_SaveThread();
+
+public:
+    Unlocked() = default;
+    Unlocked(const Unlocked&) = delete;
+    Unlocked& operator=(const Unlocked&) = delete;
+    ~Unlocked() { PyEval_RestoreThread(state); }
+};
+template <class... P, class... A> int unlocked(int (*f)(P...), A... args) {
+    const Unlocked guard;
+    return f(args...);
 }
 
 // step(T, D, x, u, temperature, want_loss, want_grad) -> rc, accept_len, tokens, loss, grad
@@ -142,13 +150,12 @@ PyObject* step(PyObject*, PyObject* const* a, Py_ssize_t n) {
     float* const lp = loss ? (float*)ptr(l) : nullptr;
     void* const gp = grad ? ptr(g) : nullptr;
     void* const st = s.stream();
-    const int rc = unlocked([&] {
-        return s.code == SD_DTYPE_F32
-                   ? lib.step_f32((const float*)ptr(*s.T), (const float*)ptr(*s.D), (const int32_t*)ptr(*s.x), (const float*)ptr(*u), tau,
-                                  s.B, s.k, s.V, (int32_t*)ptr(len), (int32_t*)ptr(tokens), lp, (float*)gp, st)
-                   : lib.step_bf16((const uint16_t*)ptr(*s.T), (const uint16_t*)ptr(*s.D), (const int32_t*)ptr(*s.x), (const float*)ptr(*u),
-                                   tau, s.B, s.k, s.V, (int32_t*)ptr(len), (int32_t*)ptr(tokens), lp, (uint16_t*)gp, st);
-    });
+    const int rc = s.code == SD_DTYPE_F32
+                       ? unlocked(lib.step_f32, (const float*)ptr(*s.T), (const float*)ptr(*s.D), (const int32_t*)ptr(*s.x),
+                            (const float*)ptr(*u),
+                                  tau, s.B, s.k, s.V, (int32_t*)ptr(len), (int32_t*)ptr(tokens), lp, (float*)gp, st)
+                       : unlocked(lib.step_bf16, (const uint16_t*)ptr(*s.T), (const uint16_t*)ptr(*s.D), (const int32_t*)ptr(*s.x),
+                                  (const float*)ptr(*u), tau, s.B, s.k, s.V, (int32_t*)ptr(len), (int32_t*)ptr(tokens), lp, (uint16_t*)gp, st);
     return answer(rc, len, tokens, l, g);
     END_HANDLE_TH_ERRORS
 }
@@ -164,11 +171,10 @@ PyObject* hint(PyObject*, PyObject* const* a, Py_ssize_t n) {
     const at::Tensor len = s.make({s.B}, at::kInt), tokens = s.make({s.B, s.k + 1}, at::kInt), l = s.make({s.B, s.k}, at::kFloat);
     const at::Tensor g = at::empty_like(*s.D), status = s.make({s.B}, at::kInt), err = s.make({s.B, s.k}, at::kFloat);
     void* const st = s.stream();
-    const int rc = unlocked([&] {
-        return lib.hint(ptr(*s.T), ptr(*s.D), (const int32_t*)ptr(*s.x), (const float*)ptr(*u), tau, s.B, s.k, s.V, s.code, ptr(*h),
-                        (int32_t*)ptr(len), (int32_t*)ptr(tokens), (float*)ptr(l), ptr(g), (float*)ptr(err), (uint32_t*)ptr(status),
-                        ptr(*ws), bytes_of(*ws), st);
-    });
+    const int rc = unlocked(lib.hint, ptr(*s.T), ptr(*s.D), (const int32_t*)ptr(*s.x), (const float*)ptr(*u), tau, s.B, s.k, s.V, s.code,
+                            ptr(*h),
+                            (int32_t*)ptr(len), (int32_t*)ptr(tokens), (float*)ptr(l), ptr(g), (float*)ptr(err), (uint32_t*)ptr(status),
+                            ptr(*ws), bytes_of(*ws), st);
     return answer(rc, len, tokens, l, g, status, err);
     END_HANDLE_TH_ERRORS
 }
@@ -189,10 +195,9 @@ PyObject* greedy(PyObject*, PyObject* const* a, Py_ssize_t n) {
     const at::Tensor best = a[2] == Py_True ? s.make({B, k1}, at::kInt) : at::Tensor();
     int32_t* const bp = best.defined() ? (int32_t*)ptr(best) : nullptr;
     void* const st = s.stream();
-    const int rc = unlocked([&] {
-        return lib.greedy(ptr(*T), (const int32_t*)ptr(*x), (int)B, (int)k1 - 1, (int)V, code, (int32_t*)ptr(len), (int32_t*)ptr(tokens), bp,
-                          nullptr, 0, st);
-    });
+    const int rc = unlocked(lib.greedy, ptr(*T), (const int32_t*)ptr(*x), (int)B, (int)k1 - 1, (int)V, code, (int32_t*)ptr(len),
+                            (int32_t*)ptr(tokens), bp,
+                            nullptr, 0, st);
     return answer(rc, len, tokens, best);
     END_HANDLE_TH_ERRORS
 }
@@ -213,10 +218,8 @@ PyObject* errors(PyObject*, PyObject* const* a, Py_ssize_t n) {
     void* const gp = g.defined() ? ptr(g) : nullptr;
     uint32_t* const sp = status.defined() ? (uint32_t*)ptr(status) : nullptr;
     void* const st = s.stream();
-    const int rc = unlocked([&] {
-        return lib.errors(ptr(*s.T), ptr(*s.D), (const int32_t*)ptr(*s.x), (const float*)ptr(*u), tau, s.B, s.k, s.V, s.code,
-                          (int32_t*)ptr(len), (int32_t*)ptr(tokens), lp, gp, sp, nullptr, 0, st);
-    });
+    const int rc = unlocked(lib.errors, ptr(*s.T), ptr(*s.D), (const int32_t*)ptr(*s.x), (const float*)ptr(*u), tau, s.B, s.k, s.V, s.code,
+                            (int32_t*)ptr(len), (int32_t*)ptr(tokens), lp, gp, sp, nullptr, 0, st);
     return answer(rc, len, tokens, l, g, status);
     END_HANDLE_TH_ERRORS
 }
@@ -259,10 +262,9 @@ PyObject* ensemble(PyObject*, PyObject* const* a, Py_ssize_t n) {
     }
     uint32_t* const sp = status.defined() ? (uint32_t*)ptr(status) : nullptr;
     void* const st = s.stream();
-    const int rc = unlocked([&] {
-        return lib.ensemble(ptr(*T), D, (int)N, tau, eps, (int)B, (int)k, (int)V, code, cum_in, (float*)ptr(loss), grad ? G : nullptr,
+    const int rc = unlocked(lib.ensemble, ptr(*T), D, (int)N, tau, eps, (int)B, (int)k, (int)V, code, cum_in, (float*)ptr(loss),
+                            grad ? G : nullptr,
                             (double*)ptr(mean), (double*)ptr(cum), (float*)ptr(weights), sp, nullptr, 0, st);
-    });
     PyObject* grads = Py_None;
     if (grad) {
         grads = PyList_New(N);
@@ -299,10 +301,8 @@ PyObject* lmhead(PyObject*, PyObject* const* a, Py_ssize_t n) {
         return none();
     const at::Tensor out = s.make({g->size(1), x->size(1)}, at::kFloat);
     void* const st = s.stream();
-    const int rc = unlocked([&] {
-        return lib.lmhead((const uint16_t*)ptr(*g), (const uint16_t*)ptr(*x), (int)g->size(0), (int)g->size(1), (int)x->size(1),
-                          (float*)ptr(out), nullptr, st);
-    });
+    const int rc = unlocked(lib.lmhead, (const uint16_t*)ptr(*g), (const uint16_t*)ptr(*x), (int)g->size(0), (int)g->size(1), (int)x->size(1),
+                            (float*)ptr(out), nullptr, st);
     return answer(rc, out);
     END_HANDLE_TH_ERRORS
 }
@@ -325,10 +325,9 @@ PyObject* vp_partial(PyObject*, PyObject* const* a, Py_ssize_t n) {
         rec = s.make({(int64_t)s.B * (s.k + 1), kVpRecordBytes}, at::kByte);
     }
     void* const st = s.stream();
-    const int rc = unlocked([&] {
-        return lib.vp_partial(ptr(*s.T), ptr(*s.D), (const int32_t*)ptr(*s.x), tau, s.B, s.k, s.V, off, total, s.code, ptr(rec), ptr(*ws),
-                              bytes_of(*ws), st);
-    });
+    const int rc = unlocked(lib.vp_partial, ptr(*s.T), ptr(*s.D), (const int32_t*)ptr(*s.x), tau, s.B, s.k, s.V, off, total, s.code,
+                            ptr(rec), ptr(*ws),
+                            bytes_of(*ws), st);
     return answer(rc, rec);
     END_HANDLE_TH_ERRORS
 }
@@ -352,11 +351,10 @@ PyObject* vp_finish(PyObject*, PyObject* const* a, Py_ssize_t n) {
     float* const lp = l.defined() ? (float*)ptr(l) : nullptr;
     void* const gp = g.defined() ? ptr(g) : nullptr;
     void* const st = s.stream();
-    const int rc = unlocked([&] {
-        return lib.vp_finish(ptr(*s.T), ptr(*s.D), (const int32_t*)ptr(*s.x), (const float*)ptr(*u), tau, s.B, s.k, s.V, off, total, s.code,
-                             ptr(*all), ranks, rank, (int32_t*)ptr(len), lp, gp, (double*)ptr(mass), (uint32_t*)ptr(status), ptr(*ws),
-                             bytes_of(*ws), st);
-    });
+    const int rc = unlocked(lib.vp_finish, ptr(*s.T), ptr(*s.D), (const int32_t*)ptr(*s.x), (const float*)ptr(*u), tau, s.B, s.k, s.V, off,
+                            total, s.code,
+                            ptr(*all), ranks, rank, (int32_t*)ptr(len), lp, gp, (double*)ptr(mass), (uint32_t*)ptr(status), ptr(*ws),
+                            bytes_of(*ws), st);
     return answer(rc, len, l, g, mass, status);
     END_HANDLE_TH_ERRORS
 }
@@ -377,11 +375,10 @@ PyObject* vp_draw(PyObject*, PyObject* const* a, Py_ssize_t n) {
         return none();
     const at::Tensor tokens = s.make({s.B, s.k + 1}, at::kInt);
     void* const st = s.stream();
-    const int rc = unlocked([&] {
-        return lib.vp_draw(ptr(*s.T), ptr(*s.D), (const int32_t*)ptr(*s.x), (const float*)ptr(*u), tau, s.B, s.k, s.V, off, total, s.code,
-                           (const int32_t*)ptr(*len), (const double*)ptr(*mass), ranks, rank, (int32_t*)ptr(tokens), (uint32_t*)ptr(*status),
-                           ptr(*ws), bytes_of(*ws), st);
-    });
+    const int rc = unlocked(lib.vp_draw, ptr(*s.T), ptr(*s.D), (const int32_t*)ptr(*s.x), (const float*)ptr(*u), tau, s.B, s.k, s.V, off,
+                            total, s.code,
+                            (const int32_t*)ptr(*len), (const double*)ptr(*mass), ranks, rank, (int32_t*)ptr(tokens), (uint32_t*)ptr(*status),
+                            ptr(*ws), bytes_of(*ws), st);
     return answer(rc, tokens);
     END_HANDLE_TH_ERRORS
 }

@@ -1,5 +1,8 @@
 """The calling thread's part in C++ (csrc/sd_native.cpp): what it takes it answers as the general way does, and it
 leaves everything else to that way."""
+import os
+import subprocess
+import sys
 import types
 
 import pytest
@@ -135,3 +138,50 @@ def test_buffers_of_the_vocabulary_parallel_step_that_are_too_small_or_of_anothe
     with pytest.raises(ValueError):
         binding.sd_vp_draw(T, D, x, u, 0.8, 0, V, n, f.local_mass[:1].expand(B, 2), 1, 0, st, ws)
     torch.cuda.synchronize()
+
+
+# A process of its own: an exception that gets out without the interpreter's lock takes the interpreter with it.
+REFUSING = """
+import threading, torch
+from paper_2603_12617_b200 import binding as b
+T, D = torch.zeros(2, 3, 4096, device="cuda"), torch.zeros(2, 2, 4096, device="cuda")
+x, u = torch.zeros(2, 2, dtype=torch.int32, device="cuda"), torch.zeros(2, 3, device="cuda")
+G, X = torch.zeros(4, 64, dtype=torch.bfloat16, device="cuda"), torch.zeros(4, 64, dtype=torch.bfloat16, device="cuda")
+ws = torch.empty(1 << 20, dtype=torch.uint8, device="cuda")
+rec = b.sd_vp_partial(T, D, x, 1.0, 0, 4096, ws)
+f = b.sd_vp_finish(T, D, x, u, 1.0, 0, 4096, rec, 1, 0, ws)
+bad = lambda t: (torch._C._set_throw_on_mutable_data_ptr(t), t)[1]
+calls = [lambda v: b.sd_verify_feedback(T, D, x, v, 1.0), lambda v: b.sd_verify_feedback(T.bfloat16(), D.bfloat16(), x, v, 1.0),
+         lambda v: b.sd_verify_feedback_hint(T, D, x, v, 1.0, D, workspace=ws), lambda v: b.sd_verify_error_feedback(T, D, x, v, 1.0),
+         lambda v: b.sd_vp_finish(T, D, x, v, 1.0, 0, 4096, rec, 1, 0, ws),
+         lambda v: b.sd_vp_draw(T, D, x, v, 1.0, 0, 4096, f.accept_len, f.local_mass, 1, 0, f.status, ws)]
+with_x = [lambda v: b.sd_verify_greedy(T, v), lambda v: b.sd_vp_partial(T, D, v, 1.0, 0, 4096, ws)]
+with_D = [lambda v: b.sd_ensemble_feedback(T, [D, v], 1.0, 10.0)]
+with_X = [lambda v: b.sd_lmhead_grad(G, v)]
+done = 0
+for group, t in ((calls, u), (with_x, x), (with_D, D), (with_X, X)):
+    for call in group:
+        call(t)
+        try:
+            call(bad(t.clone()))
+        except RuntimeError as e:
+            assert "data pointer" in str(e), e
+            done += 1
+        ran = []
+        th = threading.Thread(target=lambda: ran.append(1))      # the lock is where it belongs
+        th.start()
+        th.join()
+        assert ran
+        call(t)
+torch.cuda.synchronize()
+print("refused", done)
+"""
+
+
+@pytest.mark.gpu
+def test_tensors_that_refuse_their_address_raise():
+    """The address of a tensor is asked for while the interpreter's lock is held: a refusal is an exception like any other."""
+    root = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
+    env = dict(os.environ, PYTHONPATH=os.pathsep.join([root, os.environ.get("PYTHONPATH", "")]))
+    r = subprocess.run([sys.executable, "-c", REFUSING], env=env, cwd=root, capture_output=True, text=True, timeout=300)
+    assert r.returncode == 0 and "refused 10" in r.stdout, r.stdout + r.stderr
