@@ -20,6 +20,8 @@ from typing import Optional
 
 import torch
 
+from . import native_library
+
 SD_DTYPE_F32 = 0
 SD_DTYPE_BF16 = 1
 
@@ -115,7 +117,7 @@ _lib = _load()
 
 
 def _load_native():
-    path = os.path.join(_HERE, "lib", "sd_native.so")
+    path = os.path.join(_HERE, "lib", native_library())
     if not os.path.exists(path):
         raise ImportError(f"{path} is missing: build it with `python -c 'import __graft_entry__ as g; g.build()'`")
     loader = importlib.machinery.ExtensionFileLoader("sd_native", path)

@@ -31,6 +31,24 @@ def test_anything_but_device_tensors_is_left_to_the_general_way():
         n.bind(1, 2)
 
 
+def test_a_build_against_another_torch_is_not_loaded(monkeypatch):
+    monkeypatch.setattr(torch, "__version__", "0.0.1")
+    with pytest.raises(ImportError, match="0.0.1"):
+        binding._load_native()
+
+
+def test_the_build_makes_one_for_the_torch_that_runs(monkeypatch):
+    import __graft_entry__ as entry
+    entry.build()
+    ran = []
+    monkeypatch.setattr(entry.subprocess, "Popen", lambda c: types.SimpleNamespace(wait=lambda: ran.append(c) or 0, returncode=0))
+    entry.build()
+    assert ran == []                                             # everything is there
+    monkeypatch.setattr(torch, "__version__", "0.0.1")
+    entry.build()
+    assert len(ran) == 1 and ran[0][0] == "g++" and "0.0.1" in ran[0][ran[0].index("-o") + 1]
+
+
 def flat(o):
     if isinstance(o, torch.Tensor) or o is None:
         return [o]
