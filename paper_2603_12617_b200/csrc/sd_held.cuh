@@ -182,29 +182,34 @@ sd_held_kernel(const __grid_constant__ Params P, HeldCandidate* const cand) {
     cluster_arrive();                                      // (waited for before the first remote store)
 
     int unit = (int)blockIdx.x / C;
+    bool ok = true;                                        // (range checks; all threads go on to the cluster's barriers)
     if constexpr (DRAW) {
         // of the sequence, the first rejected row (the bonus row if there is none)
         const int b = unit;
+        ok = SD_IN(b, P.B, 22);
         unit = b * (P.k + 1) + P.k;
-        for (int i0 = 0; i0 < P.k; i0 += 32) {
+        for (int i0 = 0; ok && i0 < P.k; i0 += 32) {
             const unsigned m = __ballot_sync(0xffffffffu, i0 + lane < P.k && P.accept[b * P.k + i0 + lane] == 0);
             if (m) { unit = b * (P.k + 1) + i0 + __ffs(m) - 1; break; }
         }
     }
+    ok = ok && SD_IN(unit, total_units<ENS>(P), 20);
     const UnitRef ur = unit_ref<ENS>(P, unit);
     const int slots = C * kHeldWarps, slot = rank * kHeldWarps + warp;
     // this warp's regions [r0, r0 + n)
     const int NV = P.V / VEC, NR = P.NR, base = NR / slots, rem = NR - base * slots;
     const int r0 = slot * base + min(slot, rem);
     int n = base + (slot < rem ? 1 : 0);
-    if (!SD_IN(ur.t_row, (long long)P.B * (P.k + 1), 10) || !SD_IN(ur.d_row, (long long)P.B * P.k, 11)) n = 0;
+    // (without regions a warp neither loads nor stores: what is read of a row is where its gradient and its hint lie, too)
+    if (!ok || !SD_IN(ur.t_row, (long long)P.B * (P.k + 1), 10) || !SD_IN(ur.d_row, (long long)P.B * P.k, 11)) n = 0;
+    if (n > 0 && !SD_IN((long long)min(NV, (r0 + n) * kRegionVecs) * VEC - 1, P.V, 12)) n = 0;
     const size_t offD = ur.d_row * P.V;
     const uint4* const gT = reinterpret_cast<const uint4*>(reinterpret_cast<const ET*>(P.T) + ur.t_row * P.V);
     const uint4* const gD = reinterpret_cast<const uint4*>(reinterpret_cast<const ET*>(ENS ? P.Dn[ur.n] : P.D) + offD);
 
     // (asked for before anything else: wanted at the end of the chain)
     float uk = 0.f;
-    if (!STATS && !ENS) asm volatile("ld.global.nc.f32 %0, [%1];" : "=f"(uk) : "l"(P.u + (size_t)ur.b * (P.k + 1) + P.k));
+    if (!STATS && !ENS && ok) asm volatile("ld.global.nc.f32 %0, [%1];" : "=f"(uk) : "l"(P.u + (size_t)ur.b * (P.k + 1) + P.k));
     uint4 rt[N][kRegionRows], rd[N][kRegionRows];
     const uint64_t policy = STATS || ENS ? policy_normal() : policy_discard();     // (somebody else reads them too)
 #pragma unroll
@@ -212,7 +217,7 @@ sd_held_kernel(const __grid_constant__ Params P, HeldCandidate* const cand) {
 #pragma unroll
         for (int g = 0; g < kRegionRows; ++g) {
             const int vi = (r0 + j) * kRegionVecs + g * 32 + lane;
-            const bool in = j < n && vi < NV && SD_IN((long long)vi * VEC + VEC - 1, P.V, 10);
+            const bool in = j < n && vi < NV;
             rt[j][g] = E::masked();
             // (a bonus row goes the same way with draft logits of 0, whose sums nobody looks at, and kD = 0)
             rd[j][g] = ur.bonus ? make_uint4(0u, 0u, 0u, 0u) : E::masked();
@@ -225,13 +230,15 @@ sd_held_kernel(const __grid_constant__ Params P, HeldCandidate* const cand) {
     int32_t first = -1;
     uint32_t word = 0;
     if constexpr (DRAW) {
-        rc = P.rowc[unit];
-        if (lane < P.k) first = P.x[ur.b * P.k + lane];
-        word = P.wstatus[ur.b];
+        if (ok) {
+            rc = P.rowc[unit];
+            if (lane < P.k) first = P.x[ur.b * P.k + lane];
+            word = P.wstatus[ur.b];
+        }
     }
     AcceptOperands aop;
     aop.valid = false;
-    if (!ENS && reports && lane == 0 && !ur.bonus) aop = load_accept_operands<DT>(P, ur.b, ur.i);
+    if (!ENS && ok && reports && lane == 0 && !ur.bonus) aop = load_accept_operands<DT>(P, ur.b, ur.i);
 
     // ---- first pass: references from the maxima of all the warp holds
     if constexpr (!DRAW) {
@@ -424,17 +431,17 @@ sd_held_kernel(const __grid_constant__ Params P, HeldCandidate* const cand) {
                 }
             }
             if constexpr (DRAW) {
-                if (mine) held_emit(P, ur.b, ur.i, y, word | flags, first, lane);
+                if (mine && ok) held_emit(P, ur.b, ur.i, y, word | flags, first, lane);
                 return;
             }
             // two tickets of a unit: its row report, its candidate
             uint32_t tickets = reports ? 1u : 0u;
             if (mine) {
                 ++tickets;
-                if (lane == 0 && SD_IN(unit, total_units<false>(P), 20))
+                if (lane == 0 && ok)
                     *reinterpret_cast<int2*>(cand + unit) = make_int2(y, (int)flags);
             }
-            if (tickets) {
+            if (tickets && ok) {
                 int got = 0;
                 if (lane == 0) got = take_tickets(P, ur.b, tickets) ? 1 : 0;
                 last_ticket = __shfl_sync(0xffffffffu, got, 0) != 0;

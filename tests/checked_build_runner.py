@@ -1,5 +1,5 @@
-"""Runs every entry point on tiny, ragged and multi-stage shapes, and the two sweeps on the smallest that take them, through whichever build of the library
-SD_VERIFY_LIBRARY names, compares with the CPU oracle, and prints what sd_bounds_report counted.
+"""Runs every entry point on tiny, ragged and multi-stage shapes, on every kernel that it may take, through whichever build of the
+library SD_VERIFY_LIBRARY names, compares with the CPU oracle, and prints what sd_bounds_report counted.
 Started as a child process by test_bounds_checked_gpu.py (the library is chosen at import)."""
 import json
 import sys
@@ -20,6 +20,19 @@ def shifted(t, lead):
     return v
 
 
+# Which kernel a call took, by its threads a block; the error-position feedback's second one has 256 in any case.
+KERNEL = {1024: "cluster", 512: "held", 256: "sweeps"}
+SEEN = set()
+
+
+def took(entry):
+    info = b.sd_launch_info()
+    kernel = "element-wise" if info["path"] == 0 else KERNEL[info["threads"]]
+    assert info["kernels"] == {"sweeps": 3}.get(kernel, 2 if entry in ("errors", "ensemble") else 1), (entry, info)
+    SEEN.add((entry, kernel))
+    return kernel
+
+
 def main():
     assert b.sd_bounds_report() is not None, "this build of the library has no range checks"
     shapes = [(2, 2, 5, "f32"), (3, 1, 17, "bf16"), (2, 3, 1023, "f32"), (4, 2, 1024, "bf16"), (5, 3, 7168 + 256, "f32"),
@@ -29,22 +42,33 @@ def main():
         inp = synth.make_inputs(cfg)
         T, D, x, u = to_device(inp)
         ref = oracle_of(inp)
+        es = T.element_size()
+        whole = (V * es) % 16 == 0
         for cluster in (0, 3, 8):
             b.sd_set_option(b.SD_OPT_CLUSTER, cluster)
-            check(inp, b.sd_verify_feedback_ex(T, D, x, u, inp.tau), ref, max_band_frac=1.0)
+            ex = b.sd_verify_feedback_ex(T, D, x, u, inp.tau)
+            kernel = took("step")
+            assert not whole or (kernel == "cluster") == (cluster != 0)
+            check(inp, ex, ref, max_band_frac=1.0)
+            h = b.sd_verify_feedback_hint(T, D, x, u, inp.tau, torch.zeros_like(D))
+            assert took("hint") == kernel or not whole
+            check(inp, h, ref, max_band_frac=1.0)
+            if whole:
+                e = b.sd_verify_error_feedback(T, D, x, u, inp.tau)
+                assert took("errors") == kernel
+                assert torch.equal(e.accept_len, h.accept_len)
+                n = e.accept_len.long()
+                rows = torch.where((n < k)[:, None], ex.grad_draft[torch.arange(B, device="cuda"), n.clamp(max=k - 1)], 0)
+                assert torch.equal(e.error_grad, rows)
+                m = b.sd_ensemble_feedback(T, [D, D.clone()], inp.tau, 10.0)
+                took("ensemble")
+                assert (m.loss - ex.loss).abs().max() <= 1e-4 * ex.loss.abs().max() + 4e-7 and torch.equal(m.loss[0], m.loss[1])
         b.sd_set_option(b.SD_OPT_CLUSTER, 0)
         check(inp, b.sd_verify_feedback(T, D, x, u, inp.tau), ref, max_band_frac=1.0)
-        h = b.sd_verify_feedback_hint(T, D, x, u, inp.tau, torch.zeros_like(D))
-        check(inp, h, ref, max_band_frac=1.0)
-        es = T.element_size()
-        if (V * es) % 16 == 0:
-            e = b.sd_verify_error_feedback(T, D, x, u, inp.tau)
-            assert torch.equal(e.accept_len, h.accept_len)
         g = b.sd_verify_greedy(T, x)
         gref = sd_oracle.verify_greedy(inp.target_logits, inp.draft_tokens)
         assert (g.accept_len.cpu().numpy() == gref.accept_len).all() and (g.tokens.cpu().numpy() == gref.tokens).all()
-        if (V * es) % 16 == 0:
-            b.sd_ensemble_feedback(T, [D, D.clone()], inp.tau, 10.0)
+        if whole:
             if V // (16 // es) >= 2:
                 code = b.SD_DTYPE_F32 if dt == "f32" else b.SD_DTYPE_BF16
                 cuts = shard.vocab_cuts(V, 2, es)
@@ -59,7 +83,7 @@ def main():
                     b.sd_vp_draw(Ts[r], Ds[r], x, u, inp.tau, cuts[r][0], V, fins[r].accept_len, m, 2, r, fins[r].status, ws[r])
         torch.cuda.synchronize()
 
-    # the two sweeps: whole-vector rows from 32 MB of bf16 and 48 MB of fp32 logits, odd rows wherever they start
+    # the two sweeps: whole-vector rows of more than fit the chip at once, odd rows wherever they start
     for (B, k, V, dt, leadT, leadD) in [(40, 3, 58000, "bf16", 0, 0), (24, 3, 72004, "f32", 0, 0), (1300, 2, 4104, "bf16", 0, 0),
                                         (200, 2, 4097, "bf16", 1, 6), (150, 3, 2051, "f32", 2, 1), (3, 2, 50257, "bf16", 0, 0),
                                         (2, 2, 512 * 65 - 1, "bf16", 3, 0), (3, 2, 40003, "f32", 3, 3)]:
@@ -72,17 +96,20 @@ def main():
                             loss=torch.empty((B, k), device="cuda"), grad_draft=shifted(torch.zeros_like(D), leadD),
                             acc_prob=torch.empty((B, k), device="cuda"), status=torch.empty(B, dtype=torch.int32, device="cuda"))
         b.sd_verify_feedback_ex(T, D, x, u, inp.tau, out=out)
-        assert b.sd_launch_info()["kernels"] == 3
+        assert took("step") == "sweeps"
         check(inp, out, oracle_of(inp), max_band_frac=1.0)
         only = b.sd_verify_feedback(T, D, x, u, inp.tau, want_loss=False, want_grad=False)
         assert torch.equal(only.tokens, out.tokens)
         if V * T.element_size() % 16 == 0:
             e = b.sd_verify_error_feedback(T, D, x, u, inp.tau)
-            assert b.sd_launch_info()["kernels"] == 3
+            assert took("errors") == "sweeps"
             h = b.sd_verify_feedback_hint(T, D, x, u, inp.tau, torch.zeros_like(D))
-            assert b.sd_launch_info()["kernels"] == 3
+            assert took("hint") == "sweeps"
             assert torch.equal(e.tokens, out.tokens) and torch.equal(h.tokens, out.tokens)
         torch.cuda.synchronize()
+    # a later rule may not take a kernel out of this run
+    assert SEEN == {(e, n) for e in ("step", "hint", "errors", "ensemble") for n in ("cluster", "held", "sweeps")
+                    if (e, n) != ("ensemble", "sweeps")} | {("step", "element-wise"), ("hint", "element-wise")}, SEEN
     print("REPORT " + json.dumps(b.sd_bounds_report()))
 
 
