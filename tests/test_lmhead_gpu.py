@@ -66,6 +66,27 @@ def test_small_shapes_every_entry(binding, R, V, d):
     assert binding.sd_launch_info()["path"] == 5
 
 
+@pytest.mark.parametrize("R,V,d", [(65, 256 * 150 + 8, 256 + 72), (384, 256 * 9 + 8, 256 * 8 + 80),
+                                   (385, 256 * 9 + 8, 256 * 8 + 80), (449, 256 * 150 + 8, 256 + 72)])
+def test_more_tiles_than_pairs_of_blocks_every_entry(binding, R, V, d):
+    """What a pair of blocks carries from tile to tile -- stages, both accumulators, the boxes of the result -- in either shape of
+    the kernel (up to 384 positions, and more): 90 tiles, so that some of 74 pairs have two, and 302, so that some have five and
+    every barrier of an accumulator goes through both parities; every dimension ends off the tile."""
+    gb, Xb = operands(R, V, d, seed=R + V)
+    status = torch.zeros(1, dtype=torch.int32, device="cuda")
+    guard = torch.full((V * d + 128,), -7.0, dtype=torch.float32, device="cuda")
+    out = guard[64:64 + V * d].view(V, d)
+    binding.sd_lmhead_grad(dev_bf16(gb), dev_bf16(Xb), out=out, status=status)
+    info = binding.sd_launch_info()
+    assert (info["threads"], info["blocks"]) == (320 if R <= 384 else 192, 2 * (torch.cuda.get_device_properties(0).multi_processor_count // 2))
+    torch.cuda.synchronize()
+    assert status.item() == 0
+    assert (guard[:64] == -7).all() and (guard[-64:] == -7).all(), "written outside dW"
+    bound = TOL * (np.abs(synth.bf16_bits_to_f32(gb).astype(np.float64)).T @ np.abs(synth.bf16_bits_to_f32(Xb).astype(np.float64))) + 1e-30
+    err = np.abs(out.cpu().numpy().astype(np.float64) - sd_oracle.lmhead_grad(gb, Xb))
+    assert (err <= bound).all(), f"worst ratio {np.max(err / bound):.3g} at {np.unravel_index(np.argmax(err / bound), err.shape)}"
+
+
 def test_full_size_sampled(binding):
     """The shape the benchmark times (R = 256*6 positions, V = 128256, d = 4096): entries sampled over
     the whole of dW, including the corners of tiles, each computed by the oracle on its own."""
