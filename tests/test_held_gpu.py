@@ -130,3 +130,59 @@ def test_nothing_behind_the_end_of_a_row_takes_part(binding, V, dtype, tau):
         assert torch.equal(o.accept_len, want)
         assert (o.tokens.gather(1, want[:, None].long()).squeeze(1) - u[:, k] * V).abs().max() <= 1
         assert (o.loss.abs() <= 1e-6).all() and (o.grad_draft.float().abs() * tau * V <= 1e-6).all()
+
+
+def small_workspace(binding, T, k, hint=False):
+    """Without room for the two sweeps: two rounds of held rows are the faster way then."""
+    B, V = T.shape[0], T.shape[2]
+    size = (binding.sd_hint_workspace_bytes if hint else binding.sd_workspace_bytes)(B, k, V, binding._dtype_code(T))
+    return torch.full((size - 256,), 0xA5, dtype=torch.uint8, device="cuda")
+
+
+def errors_in(binding, T, D, x, u, tau, ws):
+    B, k = x.shape
+    o = binding.ErrorFeedbackOutputs(torch.empty(B, dtype=torch.int32, device="cuda"), torch.empty(B, k + 1, dtype=torch.int32, device="cuda"),
+                                     torch.empty(B, k, device="cuda"), torch.empty_like(D[:, 0]), torch.empty(B, dtype=torch.int32, device="cuda"))
+    p = [t.data_ptr() for t in (T, D, x, u)]
+    rc = binding._lib.sd_verify_error_feedback(*p, tau, B, k, T.shape[2], binding._dtype_code(T), o.accept_len.data_ptr(), o.tokens.data_ptr(),
+                                               o.loss.data_ptr(), o.error_grad.data_ptr(), o.status.data_ptr(), ws.data_ptr(), ws.numel(),
+                                               torch.cuda.current_stream().cuda_stream)
+    assert rc == 0
+    return o
+
+
+# Clusters of 1, 3 and 4 blocks.  B = 0: as many sequences as clusters of three are resident, with one draft token two rounds exactly,
+# in which the drawn rows fit no shape of one round of their own (one cluster of such a size is held back) and take that of the first pass.
+@pytest.mark.parametrize("B,k,V,dtype", [(60, 3, 512 * 64 - 8, "bf16"), (50, 4, 256 * 64, "f32"), (15, 4, 512 * 180 + 8, "bf16"),
+                                         (0, 1, 512 * 180 - 8, "bf16"), (12, 4, 256 * 256 - 4, "f32")])
+def test_two_rounds(binding, B, k, V, dtype):
+    dt = torch.bfloat16 if dtype == "bf16" else torch.float32
+    for n in range(74, 37, -1) if B == 0 else []:
+        Z = torch.zeros(n, k + 1, V, dtype=dt, device="cuda")
+        binding.sd_verify_feedback_ex(Z, Z[:, :k].contiguous(), torch.zeros(n, k, dtype=torch.int32, device="cuda"),
+                                      torch.zeros(n, k + 1, device="cuda"), 1.0, workspace=small_workspace(binding, Z, k))
+        if binding.sd_launch_info()["threads"] == 512:
+            B = n
+            break
+    inp = synth.make_inputs(synth.custom_config(B=B, k=k, V=V, dtype=dtype, tau=0.9, index=133))
+    T, D, x, u = to_device(inp)
+    C = -(-V // (512 if dtype == "bf16" else 256) // 64)
+    resident = torch.cuda.get_device_properties(0).multi_processor_count // C
+    assert resident < B * (k + 1) <= 2 * resident
+    ex = binding.sd_verify_feedback_ex(T, D, x, u, inp.tau, workspace=small_workspace(binding, T, k))
+    info = binding.sd_launch_info()
+    assert (info["path"], info["kernels"], info["threads"], info["cluster_size"], info["blocks"]) == (1, 1, 512, C, C * B * (k + 1))
+    check(inp, ex, oracle_of(inp), max_band_frac=1.0)
+    err = errors_in(binding, T, D, x, u, inp.tau, small_workspace(binding, T, k))
+    info = binding.sd_launch_info()
+    assert (info["path"], info["kernels"], info["threads"]) == (4, 2, 512) and (k > 1 or (info["cluster_size"], info["blocks"]) == (C, C * B))
+    hint = binding.sd_verify_feedback_hint(T, D, x, u, inp.tau, torch.zeros_like(D), workspace=small_workspace(binding, T, k, hint=True))
+    assert binding.sd_launch_info()["blocks"] == C * B * (k + 1)
+    ens = binding.sd_ensemble_feedback(T, [D], inp.tau, 10.0)
+    torch.cuda.synchronize()
+    for o in (err, hint):
+        assert torch.equal(o.accept_len, ex.accept_len) and torch.equal(o.tokens, ex.tokens) and torch.equal(o.loss, ex.loss)
+        assert torch.equal(o.status, ex.status)
+    n = ex.accept_len.long()
+    assert torch.equal(err.error_grad, torch.where((n < k)[:, None], ex.grad_draft[torch.arange(B, device="cuda"), n.clamp(max=k - 1)], 0))
+    assert torch.equal(hint.grad_draft, ex.grad_draft) and torch.equal(ens.loss[0], ex.loss) and torch.equal(ens.grad[0], ex.grad_draft)
