@@ -328,7 +328,8 @@ int sd_verify_error_feedback(const void* target_logits, const void* draft_logits
  *                   extra token is drawn from (residual of row n_b, or the bonus row), and of the mass of
  *                   p_{n_b} (what a residual without mass falls back to).
  *   exchange        all-gather the shares: all_masses [G][B][2], in rank order.
- *   sd_vp_draw      phase 3: out_tokens [B,k+1]: the accepted draft tokens, then the extra token if this
+ *   sd_vp_draw      phase 3 (accept_len as phase 2 wrote it; values outside [0,k] are taken as the nearest in
+ *                   it): out_tokens [B,k+1]: the accepted draft tokens, then the extra token if this
  *                   rank's shard holds it (global index) and -1 otherwise, then -1 padding.
  *   exchange        element-wise maximum of out_tokens over the ranks.
  *

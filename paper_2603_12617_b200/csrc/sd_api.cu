@@ -99,7 +99,7 @@ long long sweep_row_regions(int V, int dtype) {
 }
 
 // Sampling regions per item of the two sweeps: four per warp where that leaves enough items for every SM
-// (nominally 888 blocks at a time), down to one per warp for the smallest calls, and so many that a row
+// (nominally 888 blocks at a time, six on each of 148), down to one per warp for the smallest calls, and so many that a row
 // never falls into more than kMaxSlices items.  Measured on 288 rows of 128 256 bf16 entries: three per
 // warp 63.4 us, four 61.6 us, five 63.7 us (more items cost more prologues and merges, fewer leave the last
 // wave of blocks emptier).
@@ -297,11 +297,14 @@ int launch_stream(DeviceState& d, const Params& P, int C, int G, int lag, cudaSt
 // row: as long as every row has an SM to itself its time depends on the row's length alone, while that of
 // the sweeps grows with the rows; with more rows than that its time steps up.  So the length from which the
 // sweeps are faster grows with the rows, up to about 180 of them; from there a call's entries decide.
-// Calls back to back, element-wise / sweeps in us (4 tokens, i.e. 5 rows a sequence):
-//     bf16  8 201 entries 5 rows 18.8 / 19.7, 100 rows 20.8 / 22.9, 200 24.8 / 26.9, 320 39.1 / 30.5;
-//           12 001: 20 rows 22.7 / 20.1, 145 22.8 / 26.4, 200 29.9 / 28.6;  32 001: 5 rows 40.2 / 19.7, 320 130 / 47.4
-//     fp32  4 097: 5 rows 14.6 / 14.7, 320 22.8 / 24.2, 640 33.5 / 30.4;  8 201: 40 rows 18.7 / 17.1, 145 18.7 / 22.8,
-//           320 33.8 / 29.0;  16 385: 145 rows 28.8 / 28.6, 320 52.4 / 38.9;  32 001: 5 rows 47.5 / 16.2
+// The line was drawn with sweeps a quarter slower than the present ones.  Calls back to back as the kernels are now,
+// element-wise / sweeps in us (4 tokens, i.e. 5 rows a sequence; * = calls to which the line gives the slower kernel):
+//     bf16  4 097 entries 80 rows 18.6 / 19.7, 320 28.1 / 22.0 *, 500 30.6 / 24.7;  8 201: 5 rows 21.2 / 18.3 *,
+//           100 21.9 / 21.0 *, 200 25.6 / 22.1 *, 320 39.2 / 24.2;  12 001: 20 rows 24.3 / 19.1, 145 28.6 / 22.4 *,
+//           200 34.1 / 23.0;  16 385: 145 34.7 / 22.6 *;  32 001: 5 rows 41.7 / 18.0, 320 119 / 33.4
+//     fp32  4 097: 5 rows 14.5 / 14.0 *, 180 16.5 / 16.7, 320 22.3 / 18.3 *, 640 30.7 / 21.5;  8 201: 40 rows 18.0 / 15.4,
+//           145 20.0 / 17.3 *, 320 30.2 / 21.2;  16 385: 145 rows 27.3 / 19.7 *, 320 47.8 / 25.5;  32 001: 5 rows 46.2 / 14.2
+// So the sweeps would now do from about 5 000 entries on whatever the rows, and below that from some 200 rows.
 bool use_ragged_sweeps(const void* D, const void* grad, const void* hint, long long units, int V, int dtype) {
     const int vec = vec_elems(dtype);
     if (hint || option(SD_OPT_FORCE_GENERIC) != 0 || V % vec == 0 || V < 8 * kRegionVecs * vec ||
@@ -451,9 +454,10 @@ int launch_sweeps(const Params& P, Sweep& S, long long units, int dtype, cudaStr
     const bool all = MODE != kSweepErrors && (P.grad || MODE == kSweepHint || S.all_rows);
     S.kept = all ? (80u << 20) / (unsigned)(S.regions * kRegionVecs * 32) : 0u;
     // The items of the drawn rows are as small as leaves all their blocks resident at once, where the second sweep is
-    // the drawn rows alone or not much more than a round of blocks: a draw is a chain of round trips, one for each
-    // region of a warp, and its end is the call's (16 sequences, 4 tokens, 151 936 bf16 entries 31.0 -> 28.3 us; 32,
-    // 8, 128 256, 2304 items, 59.5 -> 60.4).  (The hint error is summed by items of one size.)
+    // the drawn rows alone or not much more than a round of blocks (888 at a time, 592 of odd rows: six and four on each
+    // of 148 SMs): a draw is a chain of round trips, one for each
+    // region of a warp, and its end is the call's (16 sequences, 4 tokens, 151 936 bf16 entries, 800 items, 31.0 -> 28.3 us;
+    // 32, 8, 128 256, 2304 items, 59.5 -> 60.4; the line lies at a round and a half).  (The hint error is summed by items of one size.)
     S.draw_regions = S.regions;
     S.draw_slices = S.slices;
     if (MODE != kSweepHint && (!all || units * S.slices <= 1332)) {
@@ -570,7 +574,8 @@ int choose_stream(DeviceState& d, int V, long long units, int dtype, int* G_out,
 // 64, 8, 1 000 fp32, 4 MB 23.1 / 16.2; 64, 4, 8 192 fp32, 19 MB 24.0 / 19.8; 8, 5, 128 256 bf16, 23 MB 35.0 / 22.4;
 // 16, 5, 50 304 fp32, 35 MB 28.2 / 23.2; 8, 5, 128 256 fp32, 45 MB 35.4 / 26.1.
 // The ensemble stays with the cluster kernel, whose units share a target row: 3 learners on 32 sequences,
-// 8 tokens, bf16 151 / 151; on 16 sequences, 4 tokens, fp32 67.7 / 72.3.
+// 8 tokens, bf16 151 / 151; on 16 sequences, 4 tokens, fp32 67.7 / 72.3 (against sweeps over its units that were not kept,
+// launched one after the other and with maxima of unpacked entries).
 // Options that only the cluster kernel has, off their defaults, choose the cluster kernel.
 // (Nor can the second sweep have more blocks than a grid: a billion rows of one vector.)
 bool use_sweeps(DeviceState& d, int dtype, double bytes, long long units, int V, int slices) {
@@ -1071,7 +1076,8 @@ int sd_verify_error_feedback(const void* target_logits, const void* draft_logits
     const long long units = (long long)B * (k + 1);
     P.RE = kRegionVecs * vec_elems(dtype);
     P.NR = (V + P.RE - 1) / P.RE;
-    // (the rules of the full step, so that both give the same bits)
+    // (the rules of the full step: the same row sums, hence the same losses, tests and gradient to the last bit.  So
+    // is the draw on the sweeps; on held rows its totals are sums of another grouping, in fp64)
     const bool sweeps = use_sweeps(*d, dtype, (double)B * (2 * k + 1) * (double)row_bytes, units, V, L.slices);
     HeldShape held;
     const bool holds = held_room(L) && use_held(*d, V, units, dtype, !sweeps, &held);

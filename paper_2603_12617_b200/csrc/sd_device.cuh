@@ -873,8 +873,8 @@ __device__ __noinline__ void resolve_sequence(const Params& P, int b, int known_
     }
 }
 
-// Tickets of one block for sequence b: `n` of the sequence's tickets at once, by one thread, after everything the tickets stand for has been ordered before
-// this thread.  True if these were the last tickets of the sequence.
+// Tickets of one block for sequence b: `n` of the sequence's tickets at once, by one thread, after everything the
+// tickets stand for has been ordered before this thread.  True if these were the last tickets of the sequence.
 __device__ __forceinline__ bool take_tickets(const Params& P, int b, uint32_t n) {
     return count_up(P.ticket + b, n, P.tickets);
 }

@@ -17,7 +17,7 @@
 //                      address before them, their two ends entry by entry.
 //
 // 288 rows of 128 256 bf16 entries: 22.5 us with one row's item after another and a reduction for each, and a
-// last block that read one key after the other; 16.6 us as it is (18.6 before it was launched
+// last block that read one key after the other; 16.8 us as it is (18.6 before it was launched
 // programmatically and took its ticket with one release; 74 MB: 11.3 us at the copy bandwidth, the rest
 // is launch, ramp and the last block).
 #pragma once

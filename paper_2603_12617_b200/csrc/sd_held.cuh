@@ -7,9 +7,10 @@
 // and tokens.  The only waits are hardware barriers of a cluster.
 //
 // For calls whose rows are all on the chip at once (up to 19 MB of logits, 128 KiB an SM): what bounds them is the
-// chain of dependent steps.  1 sequence, 4 tokens, 32 000 fp32 entries, 9.6 us a call, calls back to back: the launch
-// 1.0 (2.2 if the next call could not come in while this one goes out), loads 2, sums and exchange 2, gradient,
-// masses and exchange 2, search 1.5, tickets and the end of the sequence 1.8.  sd_stream_kernel took 16.6: it
+// chain of dependent steps.  1 sequence, 4 tokens, 32 000 fp32 entries, 8.8 us a call, calls back to back (11 if the next
+// call could not come in while this one goes out).  Clock stamps in one unit add up to 8.7: loads and maxima 1.4, sums 0.15,
+// their exchange and merge 1.35, gradient and masses 0.55, their exchange 1.9, whose the draw is 0.6, search 0.7,
+// the last ticket 1.35, the end of the sequence 0.7.  sd_stream_kernel took 16.6: it
 // fills a ring that is read twice, hands sums from warp to warp, and draws by one warp at the end, from
 // memory.  With more rows than fit, clusters come in rounds of 13 us that nothing overlaps, and kernels that
 // stream are the faster ones (rule and figures: use_held, host).
@@ -24,7 +25,6 @@ constexpr int kHeldThreads = kHeldWarps * 32;
 constexpr int kHeldMaxCluster = 16;
 constexpr int kHeldMaxRegions = 4;                        // regions of a warp
 constexpr int kHeldSlots = kHeldMaxCluster * kHeldWarps;  // warps of a cluster
-constexpr int kHeldPerLane = kHeldSlots / 32;
 
 // What a unit leaves for the end of its sequence: the token it would emit, and status bits that count if it does.
 struct HeldCandidate { int32_t token; uint32_t flags; };
@@ -160,9 +160,10 @@ __device__ __forceinline__ int held_search(const uint4 (&rt)[kRegionRows], const
 }
 
 // What the kernel is for.  Errors: first pass only -- row constants, losses and rejection tests; then Draw: the second
-// pass over the one row of every sequence that the error-position feedback wants, a cluster to a sequence.  Hint: the second pass also sums the squared
-// distance to the hint.  Ensemble: the units are those of the ensemble feedback (see UnitRef); nothing is verified
-// or drawn.
+// pass over the one row of every sequence that the error-position feedback wants, a cluster to a sequence (of another
+// shape than the first pass had, so that a total may round otherwise in fp64).  Hint: the second pass also sums the
+// squared distance to the hint.  Ensemble: the units are those of the ensemble feedback (see UnitRef); nothing is
+// verified or drawn.
 enum HeldMode { kHeldStep = 0, kHeldErrors = 1, kHeldHint = 2, kHeldEnsemble = 3, kHeldDraw = 4, kHeldModes = 5 };
 
 // cand: workspace [B*(k+1)] (step and hint).
@@ -292,10 +293,8 @@ sd_held_kernel(const __grid_constant__ Params P, HeldCandidate* const cand) {
         cluster_wait();
     }
     if constexpr (STATS) {
-        if (reports && lane == 0) {
-            if (P.status && ur.i == 0 && SD_IN(ur.b, P.B, 21)) P.status[ur.b] = 0;      // the next kernel ORs its bits in
-            finish_row(P, ur.b, ur.i, sh.row, rc, aop, row_logs(sh.row));
-        }
+        // (the status words are written by the kernel of the drawn rows)
+        if (reports && lane == 0) finish_row(P, ur.b, ur.i, sh.row, rc, aop, row_logs(sh.row));
         return;
     } else {
         // ---- second pass, and a third one, of p_n's masses, if max(0, p - q) has none

@@ -23,11 +23,12 @@
 //   from warp 2 epilogue: tensor memory -> registers -> 32 x 32 boxes in shared memory -> global memory by TMA
 //               stores, which clip at the ends of dW, while the MMAs of the next tile fill the other half of
 //               tensor memory.
-// What bounds it: for many positions the board's power (1.3 of 1.64 PFLOP/s at 1536 positions, 128 256 x 4096: 1237 us);
+// What bounds it: for many positions the board's power (1536 positions, 128 256 x 4096: 1240 us = 1.3 PFLOP/s for 20 calls
+// on a cool board, 1450 = 1.12 after seconds of it, of 1.64 and 1.39 measured with cuBLAS);
 // operands enter an SM at 64 bytes a clock.  One block per tile of 128 x 256 (cta_group::1) needs 96, 27 TB/s of
 // L2 at full rate, and took 1377 us.  For few positions the writing of dW, which wants more boxes under way than
-// loads (GemmShape): 256 positions 437 us (4.8 TB/s out), with four epilogue warps 494, one block per tile 562;
-// 128 positions 390, 415 and 549.
+// loads (GemmShape): 256 positions 470 us (4.5 TB/s out), with four epilogue warps 512; 128 positions 397 and 413
+// (one block per tile: 562 and 549).
 // Every wait is bounded; a wait that gives up sets an error word, and the block frees its tensor
 // memory and returns.  No multicast of loads.
 #pragma once
@@ -53,8 +54,11 @@ constexpr int kGemmBox = 32;                 // rows and columns of a box of the
 constexpr int kGemmBoxBytes = kGemmBox * kGemmBox * 4;
 constexpr int kGemmBoxes = 2;                // boxes per epilogue warp: one leaves while the next is filled
 // The two shapes of the kernel (both fill the shared memory of a block).  Few positions: eight epilogue warps, two to
-// a quarter of the tensor-memory lanes; many: six stages.  512 positions 581 us in the second, 599 in the first;
-// 1536 positions 1219 and 1280; 256 positions 494 and 437 (128 256 x 4096).
+// a quarter of the tensor-memory lanes; many: six stages.  us, six stages / eight warps, calls back to back on a warm board:
+//     128 256 x 4096   128 positions 413 / 397, 256 512 / 470, 384 564 / 583, 512 654 / 723, 1536 from cold 1240 / 1317
+//     128 256 x 1024   256 152 / 137, 384 161 / 153, 512 167 / 186      151 936 x 2048   256 322 / 289, 384 360 / 368, 512 407 / 433
+//      32 000 x 4096   256 160 / 122, 384 146 / 140, 512 158 / 174       32 000 x 1024   256 47 / 48, 384 51 / 47, 768 54 / 60
+// So they meet near 384 positions, whatever the other two sizes.
 template <bool FEW> struct GemmShape {
     static constexpr int kStages = FEW ? 5 : 6;
     static constexpr int kEpilogueWarps = FEW ? 8 : 4;

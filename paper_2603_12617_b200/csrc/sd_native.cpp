@@ -405,8 +405,8 @@ PyObject* bind(PyObject*, PyObject* const* a, Py_ssize_t n) {
 }
 
 #define SD_METHOD(name) {#name, reinterpret_cast<PyCFunction>(reinterpret_cast<void (*)()>(&name)), METH_FASTCALL, nullptr}
-PyMethodDef methods[] = {SD_METHOD(bind),       SD_METHOD(step),      SD_METHOD(hint),    SD_METHOD(greedy), SD_METHOD(errors),
-                         SD_METHOD(ensemble),   SD_METHOD(lmhead),    SD_METHOD(vp_partial), SD_METHOD(vp_finish), SD_METHOD(vp_draw), {nullptr, nullptr, 0, nullptr}};
+PyMethodDef methods[] = {SD_METHOD(bind),   SD_METHOD(step),       SD_METHOD(hint),      SD_METHOD(greedy),  SD_METHOD(errors), SD_METHOD(ensemble),
+                         SD_METHOD(lmhead), SD_METHOD(vp_partial), SD_METHOD(vp_finish), SD_METHOD(vp_draw), {nullptr, nullptr, 0, nullptr}};
 PyModuleDef module = {PyModuleDef_HEAD_INIT, "sd_native", nullptr, -1, methods, nullptr, nullptr, nullptr, nullptr};
 
 }  // namespace

@@ -19,8 +19,8 @@
 // sd_stream_kernel reads every logit from HBM once, but its 28 consumer warps share one ring and all blocks
 // read at the same time and compute at the same time, so at bf16, where the exponentials take as long as
 // the reads, it moves 2.9 TB/s.  Step on 32 sequences, 8 draft tokens, 128 256 bf16 entries: 71.1 us there,
-// 58 us here (61.6 before the first kernel was launched programmatically and the maxima taken of packed bf16; first
-// sweep 29, rows 3, second 28); 64 sequences, 4 tokens, 151 936: 93.4 and 72 us; 8, 5, 128 256: 35.0 and 22.
+// 58.7 us here (61.6 before the first kernel was launched programmatically and the maxima taken of packed bf16);
+// 64 sequences, 4 tokens, 151 936: 93.4 and 72.9 us; 8, 5, 128 256: 35.0 and 22.
 // The rule which of the two a call takes is use_sweeps (host).
 //
 // Tried and dropped, on the first of these: one persistent kernel whose warps take both passes of an item
@@ -105,8 +105,8 @@ __device__ __forceinline__ PartialStats load_partial_cg(const PartialStats* p) {
 // Regions at the ends of a row, where a vector would reach into another row or out of the tensor, are read
 // and written entry by entry, out of line and with registers of their own: with one set for both, filled by a
 // function for the ends, every region went through local memory (13 sequences, 8 tokens, 110 593 fp32 entries 67.3 us,
-// 43.9 since; 122, 4, 119 177 302 and 213; 64, 4, 100 001 bf16 84.9 and 62.8).  16 sequences, 5 tokens, 50 257 bf16
-// entries: 27.2 us, against 91.6 us for the element-wise kernel, whose one block per row reads two bytes a lane.
+// 42 since; 122, 4, 119 177 302 and 206; 64, 4, 100 001 bf16 84.9 and 64).  16 sequences, 5 tokens, 50 257 bf16
+// entries: 25.3 us, against 91.6 us for the element-wise kernel, whose one block per row reads two bytes a lane.
 template <int DT> struct RowFrame {
     const typename Elem<DT>::type *rowT, *rowD;
     const uint4 *T16, *D16;      // vector 0 of the regions, aligned: up to a vector before the row
@@ -281,8 +281,8 @@ __device__ __forceinline__ void ragged_pass2(const RowFrame<DT>& f, int V, int v
 }
 
 // Pass 1 of a warp's regions of an item: gT and gD lead to the first of them, `nvec` vectors of the item lie
-// from there on, the next region `step` vectors further.  (Fetching the next region while this one is worked on was measured as well: no faster,
-// the other warps of the SM hide the loads.)
+// from there on, the next region `step` vectors further.  (Fetching the next region while this one is worked on was
+// measured as well: no faster, the other warps of the SM hide the loads.)
 // The references come from the warp's first region, which costs least, but an entry far above them has an
 // exponent as large, rounded as coarsely.  RAISE: every region raises them, so that no exponent is above 0,
 // for callers with few warps, hence few references, to a row.

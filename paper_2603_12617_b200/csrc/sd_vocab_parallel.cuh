@@ -12,8 +12,8 @@
 //                                 row constants, KL loss, rejection tests, accept length
 //            sd_vp_grad_kernel    second sweep over the shard: the gradient's columns of every
 //                                 row, and the masses of the sampling regions of the one row per
-//                                 sequence that the extra token is drawn from
-//            sd_vp_mass_kernel    per sequence: this shard's share of that row's mass, and of the mass
+//                                 sequence that the extra token is drawn from; the last block of
+//                                 that row: this shard's share of its mass, and of the mass
 //                                 of p_n (the fallback of a residual without mass)        -> 16 bytes
 //   exchange all-gather of the shares
 //   phase 3  sd_vp_draw_kernel    per sequence: exclusive scan of the shares in rank order; the rank
