@@ -438,7 +438,7 @@ int launch_sweeps_of(const Params& P, const Sweep& S, long long units, bool all,
     SD_CUDA(launch_following(sd_sweep_stats_kernel<DT, RAGGED>, dim3((unsigned)units, (unsigned)S.slices), kSweepThreads, stream, P, S));
     SD_CUDA(launch_following(sd_sweep_rows_kernel<DT>, dim3((unsigned)P.B), rows_threads(P.k), stream, P, S));
     // the rows that are drawn from, then (if anything of them is wanted) all rows
-    const unsigned second = (unsigned)S.draw_blocks + (all ? (unsigned)(units * S.slices) : 0u);
+    const unsigned second = (unsigned)S.draw_blocks + (all ? (unsigned)P.B * (unsigned)P.k * (unsigned)S.slices : 0u);
     SD_CUDA(launch_following(sd_sweep_grad_kernel<DT, MODE, RAGGED>, dim3(second), kSweepThreads, stream, P, S));
     return SD_OK;
 }

@@ -592,8 +592,7 @@ __device__ __forceinline__ float mass_of(float t, float d, float c, const RowCon
 // every load in flight before the first is used: the warp that draws is on the critical path of
 // its sequence, and one round trip to L2 is all it should pay per region.  VECTOR: rows are whole
 // 16-byte vectors and PER is a multiple of the entries of a vector (fast path); otherwise element
-// loads.  Entries before the start (v0 < 0: rows whose regions are laid out from an aligned address before
-// them) or past the end of the row have mass 0.
+// loads.  Entries past the end of the row have mass 0.
 template <int DT, int PER, bool VECTOR>
 __device__ __forceinline__ void lane_masses(const Params& P, const RowConst& rc, int mode, size_t offT, size_t offD,
                                             int v0, float (&m)[PER]) {
@@ -623,25 +622,24 @@ __device__ __forceinline__ void lane_masses(const Params& P, const RowConst& rc,
     } else {
 #pragma unroll
         for (int e = 0; e < PER; ++e) {
-            const bool in = v0 + e >= 0 && v0 + e < P.V;
+            const bool in = v0 + e < P.V;
             t[e] = in ? E::load(P.T, offT + v0 + e) : -INFINITY;
             d[e] = (in && mode == 0) ? E::load(P.D, offD + v0 + e) : -INFINITY;
         }
     }
 #pragma unroll
-    for (int e = 0; e < PER; ++e) m[e] = (v0 + e >= 0 && v0 + e < P.V) ? mass_of(t[e], d[e], P.c, rc, mode) : 0.f;
+    for (int e = 0; e < PER; ++e) m[e] = (v0 + e < P.V) ? mass_of(t[e], d[e], P.c, rc, mode) : 0.f;
 }
 
 // Inverse-CDF search inside one sampling region.  prefix = mass before the region, t = target.
 // last_with_mass: ignore t and return the last entry of the region that has mass.
-// Every lane takes a contiguous run of PER = RE/32 entries; region 0 starts `lead` entries before the row.  Returns (in every lane) the
+// Every lane takes a contiguous run of PER = RE/32 entries.  Returns (in every lane) the
 // vocabulary index, or -1 if the region has no qualifying entry.
 template <int DT, int PER, bool VECTOR>
 __device__ int search_region(const Params& P, const RowConst& rc, int mode, size_t offT, size_t offD,
-                             int region, double prefix, double t, bool last_with_mass, double* region_total,
-                             int lead = 0) {
+                             int region, double prefix, double t, bool last_with_mass, double* region_total) {
     const int lane = threadIdx.x & 31;
-    const int v0 = region * (32 * PER) + lane * PER - lead;
+    const int v0 = region * (32 * PER) + lane * PER;
     float m[PER];
     lane_masses<DT, PER, VECTOR>(P, rc, mode, offT, offD, v0, m);
     double loc = 0.0;
@@ -677,10 +675,10 @@ __device__ int search_region(const Params& P, const RowConst& rc, int mode, size
 // rejection leaves no residual mass in fp32, which exact arithmetic rules out.
 template <int DT, int PER, bool VECTOR>
 __device__ int draw_row_slow(const Params& P, const RowConst& rc, int mode, size_t offT,
-                             size_t offD, double u, int lead = 0) {
+                             size_t offD, double u) {
     double total = 0.0, rtot;
     for (int j = 0; j < P.NR; ++j) {
-        search_region<DT, PER, VECTOR>(P, rc, mode, offT, offD, j, 0.0, 0.0, true, &rtot, lead);
+        search_region<DT, PER, VECTOR>(P, rc, mode, offT, offD, j, 0.0, 0.0, true, &rtot);
         total += rtot;
     }
     if (!(total > 0.0) || !isfinite(total)) return 0;
@@ -688,24 +686,20 @@ __device__ int draw_row_slow(const Params& P, const RowConst& rc, int mode, size
     double prefix = 0.0;
     int last_mass = -1;
     for (int j = 0; j < P.NR; ++j) {
-        const int y = search_region<DT, PER, VECTOR>(P, rc, mode, offT, offD, j, prefix, t, false, &rtot, lead);
+        const int y = search_region<DT, PER, VECTOR>(P, rc, mode, offT, offD, j, prefix, t, false, &rtot);
         if (y >= 0) return y;
         if (rtot > 0.0) last_mass = j;
         prefix += rtot;
     }
     if (last_mass < 0) return 0;
-    const int y = search_region<DT, PER, VECTOR>(P, rc, mode, offT, offD, last_mass, 0.0, 0.0, true, &rtot, lead);
+    const int y = search_region<DT, PER, VECTOR>(P, rc, mode, offT, offD, last_mass, 0.0, 0.0, true, &rtot);
     return y < 0 ? 0 : y;
 }
 
 // FAST: the regions are those of the fast path (kRegionVecs vectors, rows of whole vectors);
 // otherwise those of the generic path (kGenericRegionElems entries, any alignment).
-// KNOWN: the accept length and the constants of its row are the caller's (and the sums over whole rows for
-// hint error and acceptance probability somebody else's business).
-// RAGGED: regions of the fast path's size, but the row's regions start `lead` entries before it.
-template <int DT, bool FAST, bool KNOWN = false, bool RAGGED = false>
-__device__ __noinline__ void resolve_sequence(const Params& P, int b, int known_n = 0, RowConst known_rc = RowConst{},
-                                              int lead = 0) {
+template <int DT, bool FAST>
+__device__ __noinline__ void resolve_sequence(const Params& P, int b) {
     constexpr int PER = FAST ? kRegionVecs * Elem<DT>::VEC / 32 : kGenericRegionElems / 32;
     const int lane = threadIdx.x & 31;
     const int k = P.k, NR = P.NR;
@@ -722,8 +716,8 @@ __device__ __noinline__ void resolve_sequence(const Params& P, int b, int known_
     }
 
     // accept length: first rejected position
-    int n = KNOWN ? known_n : k;
-    for (int i0 = 0; !KNOWN && i0 < k; i0 += 32) {
+    int n = k;
+    for (int i0 = 0; i0 < k; i0 += 32) {
         const int i = i0 + lane;
         const bool rej = (i < k) && (__ldcg(P.accept + b * k + i) == 0);
         const unsigned m = __ballot_sync(0xffffffffu, rej);
@@ -732,7 +726,7 @@ __device__ __noinline__ void resolve_sequence(const Params& P, int b, int known_
     uint32_t flags = 0;
 
     // hint error per position: the shares of the blocks that worked on the row, in their order
-    if (!KNOWN && P.hint_err) {
+    if (P.hint_err) {
         for (int i = lane; i < k; i += 32) {
             const double* hp = P.hint_part + (size_t)(b * (k + 1) + i) * P.hint_stride;
             double e = 0.0;
@@ -742,7 +736,7 @@ __device__ __noinline__ void resolve_sequence(const Params& P, int b, int known_
     }
 
     // diagnostic: acceptance probability 1 - sum max(0,p-q) per position (Eq. 1)
-    if (!KNOWN && P.acc_prob) {
+    if (P.acc_prob) {
         for (int i = 0; i < k; ++i) {
             const float* rsi = P.region_sums + (size_t)(b * (k + 1) + i) * NR;
             double part = 0.0;
@@ -762,11 +756,8 @@ __device__ __noinline__ void resolve_sequence(const Params& P, int b, int known_
     const int unit = b * (k + 1) + n;
     if (!SD_IN(unit, P.B * (k + 1), 23) || !SD_IN(n, k + 1, 23)) return;
     const float* rs = P.region_sums + (size_t)unit * NR;
-    RowConst rc = known_rc;
-    if constexpr (!KNOWN) {
-        const float4 rcv = __ldcg(reinterpret_cast<const float4*>(P.rowc + unit));
-        rc = RowConst{rcv.x, rcv.y, rcv.z, rcv.w};
-    }
+    const float4 rcv = __ldcg(reinterpret_cast<const float4*>(P.rowc + unit));
+    const RowConst rc{rcv.x, rcv.y, rcv.z, rcv.w};
     const size_t offT = (size_t)unit * P.V;
     const size_t offD = (size_t)(b * k + (bonus ? 0 : n)) * P.V;
     const double uk = (double)uk_f;
@@ -801,7 +792,7 @@ __device__ __noinline__ void resolve_sequence(const Params& P, int b, int known_
             flags |= SD_STATUS_BAD_ROW;
         } else {
             flags |= SD_STATUS_ZERO_RESIDUAL;   // draw from p_n instead
-            y = draw_row_slow<DT, PER, FAST && !RAGGED>(P, rc, 2, offT, offD, uk, lead);
+            y = draw_row_slow<DT, PER, FAST>(P, rc, 2, offT, offD, uk);
         }
     } else {
         // first region whose running sum exceeds t, and the mass before it
@@ -851,9 +842,9 @@ __device__ __noinline__ void resolve_sequence(const Params& P, int b, int known_
         }
         if (region >= 0 && SD_IN(region, NR, 24)) {
             double rtot;
-            y = search_region<DT, PER, FAST && !RAGGED>(P, rc, bonus ? 1 : 0, offT, offD, region, prefix, t, past_end, &rtot, lead);
+            y = search_region<DT, PER, FAST>(P, rc, bonus ? 1 : 0, offT, offD, region, prefix, t, past_end, &rtot);
             // region sum and re-summed entries may disagree in the last bits: last entry with mass
-            if (y < 0) y = search_region<DT, PER, FAST && !RAGGED>(P, rc, bonus ? 1 : 0, offT, offD, region, 0.0, 0.0, true, &rtot, lead);
+            if (y < 0) y = search_region<DT, PER, FAST>(P, rc, bonus ? 1 : 0, offT, offD, region, 0.0, 0.0, true, &rtot);
             if (y < 0) y = 0;
         }
     }

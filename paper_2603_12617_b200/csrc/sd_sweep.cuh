@@ -371,9 +371,10 @@ sd_sweep_rows_kernel(const __grid_constant__ Params P, const __grid_constant__ S
         AcceptOperands aop;
         aop.valid = false;
         if (lane == 0 && i < P.k) aop = load_accept_operands<DT>(P, b, i);   // (inputs of the call)
-        await_previous_kernel();
         const bool mine = lane < S.slices && SD_IN((long long)unit * S.slices + lane, (long long)total_units<false>(P) * S.slices, 26);
-        const PartialStats row = warp_merge_lanes(mine ? load_partial_cg(S.part + (size_t)unit * S.slices + lane) : empty_partial());
+        const PartialStats* const part = S.part + (size_t)unit * S.slices + lane;
+        await_previous_kernel();
+        const PartialStats row = warp_merge_lanes(mine ? load_partial_cg(part) : empty_partial());
         const RowLogs logs = warp_row_logs(row);
         if (lane == 0) {
             if (P.status && i == 0 && SD_IN(b, P.B, 21)) P.status[b] = 0;      // the words are ORed in by the second sweep
@@ -427,34 +428,181 @@ __device__ __forceinline__ void sweep_pass2(const uint4* gT, const uint4* gD, co
     }
 }
 
-// A row of the second sweep whose sums over the whole row are wanted, by the warp of the block that brought
-// its last item: hint error, acceptance probability, the draw.
-template <int DT, bool HINT, bool RAGGED>
-__device__ __noinline__ void sweep_row_done(const Params& P, const Sweep& S, int unit, int n, const RowConst rc) {
+// ---- the draw -----------------------------------------------------------------------------------
+// Sums of the threads of a block before a thread's own, and of all of them, in a fixed order.  All threads; `sums` is
+// free again after the next barrier.
+__device__ __noinline__ double block_sums_before(double mine, double* sums, double* all) {
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const double incl = warp_inclusive_scan(mine);
+    if (lane == 31) sums[warp] = incl;
+    __syncthreads();
+    double before = 0.0, total = 0.0;
+#pragma unroll 1
+    for (int w = 0; w < kSweepWarps; ++w) {
+        if (w == warp) before = total;
+        total += sums[w];
+    }
+    *all = total;
+    return before + (incl - mine);
+}
+
+// The extra token of a sequence, and what the sequence puts out, by the block that brought the last item of the row that
+// it is drawn from, `unit`, once that row's region masses are all there.  Its end is the call's where the sweep is short, and what it consists of is
+// round trips and sums that wait for one another; so a block does it, a region or two to a thread and then an entry or
+// two of the region.  `lead`: entries of region 0 before the row.  From the last item to the end of the call 4 us, by one
+// warp with sixteen regions and entries to a lane, one after the other, 7.5: 16 sequences, 5 tokens, 50 257 bf16 entries
+// 25.4 -> 20.2 us, 16, 5, 65 536 21.0 -> 19.2, 12, 4, 128 256 fp32 27.9 -> 26.2; error feedback 64, 4, 151 936 bf16
+// 52.0 -> 50.6.  (Run once beforehand by blocks that wait anyway, so that its instructions are there: slower, 52.6.)
+template <int DT>
+__device__ __noinline__ void sweep_draw(const Params& P, int unit, int lead) {
+    using E = Elem<DT>;
+    constexpr int kEntries = kRegionVecs * E::VEC, PER = kEntries / kSweepThreads;
+    static_assert(SD_MAX_K < kSweepThreads, "a thread for every token");
+    __shared__ double sums[2][kSweepWarps];
+    __shared__ double prefix_sh;
+    __shared__ int owner[2], found, last_mass;
+    const int tid = threadIdx.x, k = P.k, NR = P.NR;
+    const int b = unit / (k + 1), n = unit - b * (k + 1);
+    const bool bonus = n == k;
+    if (!SD_IN(unit, P.B * (k + 1), 23)) return;
+    float* const rs = P.region_sums + (size_t)unit * NR;
+    const size_t offT = (size_t)unit * P.V, offD = (size_t)(b * k + (bonus ? 0 : n)) * P.V;
+    // (everything that depends on nothing, at once)
+    const float4 rcv = __ldcg(reinterpret_cast<const float4*>(P.rowc + unit));
+    const RowConst rc{rcv.x, rcv.y, rcv.z, rcv.w};
+    const double uk = (double)P.u[b * (k + 1) + k];
+    const int32_t x = tid < n ? P.x[b * k + tid] : -1;
+    uint32_t word = 0, flags = 0;
+    if (tid == 0) {
+        word = __ldcg(P.wstatus + b) | (__ldcg(P.sticky) != 0 ? kStatusTimeout : 0u);
+        owner[0] = owner[1] = found = 0x7fffffff;
+        last_mass = -1;
+    }
+    const int per = (NR + kSweepThreads - 1) / kSweepThreads, j0 = tid * per, j1 = min(NR, j0 + per);
+    int mode = bonus ? 1 : 0, y = 0;
+    double all, t;
+    for (;;) {
+        // (the first two regions of a thread stay in registers: rows of up to 512 regions)
+        float held[2];
+#pragma unroll
+        for (int q = 0; q < 2; ++q) held[q] = j0 + q < j1 ? __ldcg(rs + j0 + q) : 0.f;
+        double mine = (double)held[0] + (double)held[1];
+        for (int j = j0 + 2; j < j1; ++j) mine += (double)__ldcg(rs + j);
+        const double before = block_sums_before(mine, sums[0], &all);
+        t = uk * all;
+        if (!(all > 0.0) || !isfinite(all)) {                      // (the same for every thread)
+            if (mode != 0) {
+                if (bonus) flags |= SD_STATUS_BAD_ROW;
+                break;
+            }
+            // a rejection whose residual has no mass: the masses of p_n in their place
+            flags |= SD_STATUS_ZERO_RESIDUAL;
+            mode = 2;
+            const int lane = tid & 31;
+            for (int j = tid >> 5; j < NR; j += kSweepWarps) {
+                float m = 0.f;
+                for (int e = lane; e < kEntries; e += 32) {
+                    const int v = j * kEntries + e - lead;
+                    if (v >= 0 && v < P.V) m += prob_elem(E::load(P.T, offT + v), P.c, rc);
+                }
+#pragma unroll
+                for (int off = 16; off > 0; off >>= 1) m += __shfl_xor_sync(0xffffffffu, m, off);
+                if (lane == 0) rs[j] = m;
+            }
+            __syncthreads();
+            continue;
+        }
+        // the first region whose running sum exceeds t, or (rounding pushed u * R to the total) the last with mass
+        if (mine > 0.0 && before + mine > t) atomicMin(&owner[0], tid);
+        if (mine > 0.0) atomicMax(&last_mass, tid);
+        __syncthreads();
+        const bool past_end = owner[0] == 0x7fffffff;
+        if (tid == (past_end ? last_mass : owner[0])) {
+            int at = -1;
+            double run = before;
+            for (int j = j0; j < j1; ++j) {
+                const double m = j == j0 ? (double)held[0] : j == j0 + 1 ? (double)held[1] : (double)__ldcg(rs + j);
+                if (!(m > 0.0)) continue;
+                at = j;
+                if (!past_end && run + m > t) break;
+                run += m;
+            }
+            found = max(at, 0);
+            prefix_sh = run;
+        }
+        __syncthreads();
+        const int region = found;
+        const double prefix = past_end ? 0.0 : prefix_sh;
+        if (tid == 0) last_mass = -1;
+        // the same among the region's entries, recomputed as they were
+        float m[PER];
+        const int v0 = region * kEntries + tid * PER - lead;
+        mine = 0.0;
+#pragma unroll
+        for (int e = 0; e < PER; ++e) {
+            const bool in = v0 + e >= 0 && v0 + e < P.V && SD_IN(region, NR, 24);
+            const float tl = in ? E::load(P.T, offT + v0 + e) : -INFINITY, dl = in && mode == 0 ? E::load(P.D, offD + v0 + e) : -INFINITY;
+            m[e] = in ? mass_of(tl, dl, P.c, rc, mode) : 0.f;
+            mine += (double)m[e];
+        }
+        double region_all;
+        const double inside = prefix + block_sums_before(mine, sums[1], &region_all);
+        if (!past_end && mine > 0.0 && inside + mine > t) atomicMin(&owner[1], tid);
+        if (mine > 0.0) atomicMax(&last_mass, tid);
+        __syncthreads();
+        // (region sum and re-summed entries may disagree in the last bits: the last entry with mass then, too)
+        const bool to_last = owner[1] == 0x7fffffff;
+        if (tid == (to_last ? last_mass : owner[1])) {
+            int at = -1;
+            double run = inside;
+#pragma unroll
+            for (int e = 0; e < PER; ++e) {
+                if (m[e] > 0.f && (to_last || at < 0 || !(run > t))) at = v0 + e;     // (the first behind which the sum exceeds t)
+                run += (double)m[e];
+            }
+            found = max(at, 0);
+        }
+        if (tid == 0 && last_mass < 0) found = 0;
+        __syncthreads();
+        y = found;
+        break;
+    }
+    if (tid == 0) {
+        P.accept_len[b] = n;
+        const uint32_t st = word | flags;
+        if (P.status && st) atomicOr(P.status + b, st);
+        P.wstatus[b] = 0;               // ready for the next call
+    }
+    if (tid <= k && SD_IN(b * (k + 1) + tid, P.B * (k + 1), 25)) P.tokens[b * (k + 1) + tid] = tid == n ? y : x;
+}
+
+// Sums over a whole row of the second sweep, by one warp of the block that brought the row's last item: hint error,
+// acceptance probability.
+template <bool HINT>
+__device__ __noinline__ void sweep_row_sums(const Params& P, const Sweep& S, int unit, size_t d_row) {
     const int lane = threadIdx.x & 31;
-    const UnitRef ur = unit_ref<false>(P, unit);
-    if (!SD_IN(unit, total_units<false>(P), 23) || (!ur.bonus && !SD_IN(ur.d_row, (long long)P.B * P.k, 21))) return;
-    if (HINT && !ur.bonus) {
+    if (!SD_IN(unit, total_units<false>(P), 23) || !SD_IN(d_row, (long long)P.B * P.k, 21)) return;
+    if (HINT) {
         // the items' shares in their order
         double e = 0.0;
         const double* hp = P.hint_part + (size_t)unit * P.hint_stride;
         for (int i = 0; i < S.slices; ++i) e += __ldcg(hp + i);
-        if (lane == 0) P.hint_err[ur.d_row] = (float)e;
+        if (lane == 0) P.hint_err[d_row] = (float)e;
     }
-    if (S.all_rows && !ur.bonus) {
+    if (S.all_rows) {
         // diagnostic: acceptance probability 1 - sum max(0,p-q) of the position
         const float* rs = P.region_sums + (size_t)unit * P.NR;
         double part = 0.0;
         for (int j = lane; j < P.NR; j += 32) part += (double)__ldcg(rs + j);
         const double R = warp_sum(part) * (double)P.tau;
-        if (lane == 0) P.acc_prob[ur.d_row] = (float)(1.0 - R);
+        if (lane == 0) P.acc_prob[d_row] = (float)(1.0 - R);
     }
-    if (ur.i == n) resolve_sequence<DT, true, true, RAGGED>(P, ur.b, n, rc, RAGGED ? row_frame<DT>(P, ur).lead : 0);
 }
 
 // One block per item.  The first S.draw_blocks blocks take the rows that are drawn from (so that the draws,
 // chains of dependent reads, are over long before the sweep is); the rest all other pair rows, from the
-// last item of the first sweep backwards.
+// last item of the first sweep backwards.  (Blocks for bonus rows, which would only find nothing to do: 32 sequences, 8
+// tokens, 128 256 bf16 entries 57.7 us, without 57.4.)
 template <int DT, int MODE, bool RAGGED>
 __global__ void __launch_bounds__(kSweepThreads, MODE == kSweepHint || RAGGED ? 4 : 6)
 sd_sweep_grad_kernel(const __grid_constant__ Params P, const __grid_constant__ Sweep S) {
@@ -471,10 +619,10 @@ sd_sweep_grad_kernel(const __grid_constant__ Params P, const __grid_constant__ S
         slice = (int)blockIdx.x - b * S.draw_slices;
         unit = 0;
     } else {
-        const int units = total_units<false>(P), id = (int)(gridDim.x - 1u - blockIdx.x);
-        slice = id / units;
-        unit = id - slice * units;
-        b = unit / (P.k + 1);
+        const int rows = P.B * P.k, id = (int)(gridDim.x - 1u - blockIdx.x);
+        slice = id / rows;
+        b = (id - slice * rows) / P.k;
+        unit = id - slice * rows + b;
     }
     await_previous_kernel();
     launch_dependents();
@@ -493,7 +641,6 @@ sd_sweep_grad_kernel(const __grid_constant__ Params P, const __grid_constant__ S
         return;                                       // the first blocks have it
     }
     const UnitRef ur = unit_ref<false>(P, unit);
-    if (!draws && ur.bonus) return;
     const int v0 = (slice * regions + warp) * kRegionVecs;
     float herr = 0.f;
     float* const rsum = P.region_sums + (size_t)unit * P.NR + slice * regions + warp;
@@ -543,8 +690,8 @@ sd_sweep_grad_kernel(const __grid_constant__ Params P, const __grid_constant__ S
         if (lane == 0) hpart[warp] = herr;
     }
     __syncthreads();
-    if (warp != 0) return;
-    if (lane == 0) {
+    if (!draws && warp != 0) return;                  // (of the drawn rows, the block that brings the last item draws)
+    if (tid == 0) {
         if (HINT && !ur.bonus) {
             // this item's share of the row's hint error: the warps' shares in their order, in fp64
             double e = 0.0;
@@ -554,8 +701,13 @@ sd_sweep_grad_kernel(const __grid_constant__ Params P, const __grid_constant__ S
         is_last = SD_IN(unit, total_units<false>(P), 28) && count_up(S.arrived + unit, 1u, (uint32_t)slices);
         if (is_last) S.arrived[unit] = 0;
     }
-    __syncwarp();
-    if (is_last) sweep_row_done<DT, HINT, RAGGED>(P, S, unit, n, rc);
+    if (draws) __syncthreads();
+    else __syncwarp();
+    if (!is_last) return;
+    if ((HINT || S.all_rows) && !ur.bonus && warp == 0) sweep_row_sums<HINT>(P, S, unit, ur.d_row);
+    if (!draws) return;
+    if (S.all_rows) __syncthreads();                  // (the draw may put other masses in place of the row's)
+    sweep_draw<DT>(P, unit, RAGGED ? row_frame<DT>(P, ur).lead : 0);
 }
 
 }  // namespace sdv
