@@ -286,6 +286,8 @@ def kernel_names(path, info) -> str:
         return "sd_held_kernel<pass 1 only> + sd_held_kernel<drawn rows>"
     if info["path"] in (1, 3) and info.get("threads") == 512:
         return path.kernel.replace("sd_stream_kernel", "sd_held_kernel")
+    if info["path"] == 3 and info.get("threads") == 256:
+        return "sd_ensemble_stats_kernel + sd_ensemble_rows_kernel + sd_ensemble_grad_kernel"
     if info["path"] in (1, 4) and info["kernels"] == 3:
         return "sd_sweep_stats_kernel + sd_sweep_rows_kernel + sd_sweep_grad_kernel"
     return path.kernel

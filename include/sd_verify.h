@@ -268,7 +268,9 @@ size_t sd_greedy_workspace_bytes(int B, int k);
  *   out_weights     [N] float     out  device, sums to 1
  *   out_status      [B] uint32    out  device SD_STATUS_BAD_ROW / SD_STATUS_TIMEOUT bits, or NULL
  *   workspace                     in   device scratch of SD_ENSEMBLE_SCRATCH_BYTES, aligned to 256
- *                                      bytes, or NULL for the library's own
+ *                                      bytes, or NULL for the library's own (of which bf16 calls that are
+ *                                      not held on the chip take 16 bytes and up to 1 KiB a row and learner,
+ *                                      for the two sweeps; with a workspace the cluster kernel serves them)
  *   stream                        in   cudaStream_t
  * Rows must be whole 16-byte vectors and every tensor 16-byte aligned (SD_ERR_ALIGN otherwise:
  * there is no element-wise path for this entry point).  Two kernels are enqueued: one of the kernels

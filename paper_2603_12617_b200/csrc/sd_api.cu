@@ -10,6 +10,7 @@
 
 #include "sd_kernels.cuh"
 #include "sd_sweep.cuh"
+#include "sd_ensemble.cuh"
 #include "sd_held.cuh"
 #include "sd_greedy.cuh"
 #include "sd_errpos.cuh"
@@ -573,9 +574,6 @@ int choose_stream(DeviceState& d, int V, long long units, int dtype, int* G_out,
 // they are (us, cluster kernel / sweeps as they are now): 100 sequences, 2 tokens, 8 192 bf16 entries, 8 MB 19.6 / 19.5;
 // 64, 8, 1 000 fp32, 4 MB 23.1 / 16.2; 64, 4, 8 192 fp32, 19 MB 24.0 / 19.8; 8, 5, 128 256 bf16, 23 MB 35.0 / 22.4;
 // 16, 5, 50 304 fp32, 35 MB 28.2 / 23.2; 8, 5, 128 256 fp32, 45 MB 35.4 / 26.1.
-// The ensemble stays with the cluster kernel, whose units share a target row: 3 learners on 32 sequences,
-// 8 tokens, bf16 151 / 151; on 16 sequences, 4 tokens, fp32 67.7 / 72.3 (against sweeps over its units that were not kept,
-// launched one after the other and with maxima of unpacked entries).
 // Options that only the cluster kernel has, off their defaults, choose the cluster kernel.
 // (Nor can the second sweep have more blocks than a grid: a billion rows of one vector.)
 bool use_sweeps(DeviceState& d, int dtype, double bytes, long long units, int V, int slices) {
@@ -589,6 +587,18 @@ bool use_sweeps(DeviceState& d, int dtype, double bytes, long long units, int V,
     int G = 0, per = 0, lag = 0;                // row pairs of a round = clusters
     if (choose_stream(d, V, units, dtype, &G, &per, &lag) <= 0) return true;
     return (double)units < (V < 26000 ? 9.5 : 6.5) * G;
+}
+
+// Does an ensemble whose rows are not held take two sweeps that share the target among the learners (sd_ensemble.cuh; else
+// the cluster kernel, whose learners follow one another)?  bf16 rows do at every size measured, in us, cluster kernel / sweeps:
+// 3 learners, 256 positions of 128 256 entries 145 / 122, 144 of 32 000 35.0 / 22.1, 32 of 65 536 24.2 / 24.2, 768 of 151 936
+// 479 / 418; 2 learners, 256 of 128 256 103 / 87; 4 learners 167 / 155.  fp32 rows stay: they have half as many exponentials
+// to the byte, and reading once wins or nearly does (3 learners, 576 positions of 32 000 122 / 133, 192 of 128 256 170 / 171,
+// 128 of them 123 / 116, 512 354 / 445).  Options that only the cluster kernel has, off their defaults, choose it.
+bool use_ensemble_sweeps(int dtype, long long positions, int slices) {
+    if (dtype != SD_DTYPE_BF16 || positions * slices >= INT_MAX) return false;
+    return option(SD_OPT_CLUSTER) == 0 && option(SD_OPT_LAG) == -1 && option(SD_OPT_PREFETCH) == 0 &&
+           option(SD_OPT_L2_BUDGET_MIB) == kL2BudgetMiB && option(SD_OPT_WAIT_POLLS) == (long long)kWaitLimit;
 }
 
 uint32_t wait_polls() {
@@ -951,6 +961,69 @@ int sd_verify_feedback_static(const void* target_logits, const void* draft_logit
 }
 
 // ---- online ensemble -------------------------------------------------------------------------
+}  // extern "C"
+namespace {
+// Scratch of the ensemble's two sweeps, which begins where the cluster kernel's flag word is.
+struct EnsembleLayout { size_t rowc, part, total; int slices; };
+EnsembleLayout ensemble_layout(int B, int k, int V, int dtype, int n_learners) {
+    EnsembleLayout L;
+    const size_t rows = (size_t)B * k * n_learners;
+    const long long R = sweep_row_regions(V, dtype), positions = (long long)B * k;
+    // Four regions to a warp where that leaves a block for every SM's four (592), down to one in small calls.  3 learners,
+    // regions an item 8 / 16 / 24 / 32 / 40 / 64, us: 256 positions of 128 256 bf16 entries 139 / 126 / 123 / 122 / 125 / 125;
+    // 768 of 151 936 491 / 435 / 425 / 418 / 413 / 410; 144 of 32 000 23.8 / 22.1 / 25.5 / 27.9 / 27.5 / 29.7.
+    long long ri = (positions * R / 592 + kSweepWarps - 1) / kSweepWarps * kSweepWarps;
+    ri = ri < kSweepWarps ? kSweepWarps : ri > 4 * kSweepWarps ? 4 * kSweepWarps : ri;
+    const long long s = (R + ri - 1) / ri;
+    L.slices = (int)(s > kMaxSlices ? kMaxSlices : s);
+    L.rowc = kAlign;
+    L.part = align_up(L.rowc + rows * sizeof(RowConst), kAlign);
+    L.total = align_up(L.part + rows * L.slices * sizeof(PartialStats), kAlign);
+    return L;
+}
+
+template <int DT, int NL>
+int launch_ensemble_group(const Params& P, const EnsembleSweep& S, const HedgeArgs& H, bool second, cudaStream_t stream) {
+    const long long positions = (long long)P.B * P.k;
+    if (!second) {
+        SD_CUDA(launch_following(sd_ensemble_stats_kernel<DT, NL>, dim3((unsigned)positions, (unsigned)S.slices), kSweepThreads, stream, P, S));
+        return SD_OK;
+    }
+    bool wanted = false;
+    for (int n = 0; n < NL; ++n) wanted = wanted || P.Gn[S.n0 + n] != nullptr;
+    if (!wanted && S.n0 != 0) return SD_OK;
+    SD_CUDA(launch_following(sd_ensemble_grad_kernel<DT, NL>, dim3(1u + (wanted ? (unsigned)(positions * S.slices) : 0u)), kSweepThreads, stream, P, S, H));
+    return SD_OK;
+}
+
+template <int DT>
+int launch_ensemble_sweeps(const Params& P, EnsembleSweep S, const HedgeArgs& H, cudaStream_t stream) {
+    // groups of learners of the same size or one less
+    const int groups = (P.learners + kEnsembleGroup - 1) / kEnsembleGroup;
+    S.kept = (80u << 20) / (unsigned)(S.regions * kRegionVecs * 16 * ((P.learners + groups - 1) / groups + 1));
+    for (int second = 0; second < 2; ++second) {
+        for (int g = 0; g < groups; ++g) {
+            S.n0 = P.learners * g / groups;
+            int rc = SD_OK;
+            switch (P.learners * (g + 1) / groups - S.n0) {
+                case 1: rc = launch_ensemble_group<DT, 1>(P, S, H, second != 0, stream); break;
+                case 2: rc = launch_ensemble_group<DT, 2>(P, S, H, second != 0, stream); break;
+                case 3: rc = launch_ensemble_group<DT, 3>(P, S, H, second != 0, stream); break;
+                default: rc = launch_ensemble_group<DT, 4>(P, S, H, second != 0, stream); break;
+            }
+            if (rc != SD_OK) return rc;
+        }
+        if (!second) {
+            const long long rows = (long long)P.B * P.k * P.learners;
+            SD_CUDA(launch_following(sd_ensemble_rows_kernel, dim3((unsigned)((rows + kSweepWarps - 1) / kSweepWarps)), kSweepThreads, stream, P, S));
+        }
+    }
+    tl_info[1] = 1; tl_info[2] = kSweepThreads; tl_info[3] = 0;
+    tl_info[4] = (int)(P.B * P.k * S.slices); tl_info[5] = 2 * groups + 1;
+    return SD_OK;
+}
+}  // namespace
+extern "C" {
 int sd_ensemble_feedback(const void* target_logits, const void* const* draft_logits, int n_learners,
                          float temperature, float epsilon, int B, int k, int V, int dtype,
                          const double* cum_loss_in, float* out_loss, void* const* out_grad,
@@ -980,14 +1053,22 @@ int sd_ensemble_feedback(const void* target_logits, const void* const* draft_log
     std::lock_guard<std::mutex> lock(d->mu);
     cudaStream_t st = static_cast<cudaStream_t>(stream);
     unsigned char* ws = static_cast<unsigned char*>(workspace);
+    HeldShape held;
+    const bool holds = use_held(*d, V, (long long)B * k * n_learners, dtype, true, &held);
+    const EnsembleLayout L = ensemble_layout(B, k, V, dtype, n_learners);
+    // (the sweeps' scratch is the library's: what a caller brings is a flag word)
+    const bool sweeps = !holds && !ws && use_ensemble_sweeps(dtype, (long long)B * k, L.slices) && (d->ws_bytes >= L.total || !capturing(st));
     if (!ws) {
         Head head;                 // (cleared below; the flag word sits where other entry points expect zeros)
-        rc = own_scratch(d, SD_ENSEMBLE_SCRATCH_BYTES, SD_ENSEMBLE_SCRATCH_BYTES, st, &head);
+        const size_t need = sweeps ? L.total : SD_ENSEMBLE_SCRATCH_BYTES;
+        rc = own_scratch(d, need, need, st, &head);
         if (rc != SD_OK) return rc;
         ws = static_cast<unsigned char*>(d->ws);
     }
-    SD_CUDA(cudaMemsetAsync(ws, 0, SD_ENSEMBLE_SCRATCH_BYTES, st));
-    if (out_status) SD_CUDA(cudaMemsetAsync(out_status, 0, (size_t)B * 4, st));
+    if (!sweeps) {
+        SD_CUDA(cudaMemsetAsync(ws, 0, SD_ENSEMBLE_SCRATCH_BYTES, st));
+        if (out_status) SD_CUDA(cudaMemsetAsync(out_status, 0, (size_t)B * 4, st));
+    }
 
     Params P;
     memset(&P, 0, sizeof P);
@@ -1007,8 +1088,19 @@ int sd_ensemble_feedback(const void* target_logits, const void* const* draft_log
     }
     P.RE = kRegionVecs * vec_elems(dtype);
     P.NR = (V + P.RE - 1) / P.RE;
-    HeldShape held;
-    if (use_held(*d, V, (long long)B * k * n_learners, dtype, true, &held)) {
+    if (sweeps) {
+        EnsembleSweep S;
+        S.slices = L.slices;
+        S.regions = (P.NR + L.slices - 1) / L.slices;
+        S.n0 = 0;
+        S.part = reinterpret_cast<PartialStats*>(ws + L.part);
+        S.rowc = reinterpret_cast<RowConst*>(ws + L.rowc);
+        const HedgeArgs H{(double)epsilon, cum_loss_in, out_round_loss, out_cum_loss, out_weights};
+        rc = launch_ensemble_sweeps<SD_DTYPE_BF16>(P, S, H, st);
+        tl_info[0] = 3;
+        return rc;
+    }
+    if (holds) {
         rc = launch_held<kHeldEnsemble>(*d, P, held, dtype, nullptr, st);
     } else {
         int G = 0, lag = 0, per = 0;

@@ -1035,6 +1035,38 @@ __global__ void __launch_bounds__(kGenericThreads) sd_generic_kernel(const __gri
 }
 
 // ---- online ensemble ---------------------------------------------------------------------
+// A warp's share of a learner's losses, in every lane's turn `step` of them apart and eight loads in flight.
+__device__ __forceinline__ void hedge_sum(const float* l, long long per, long long first, int step, double& out) {
+    double s = 0.0;
+    for (long long j = first; j < per; j += 8 * step) {
+        float v[8];
+#pragma unroll
+        for (int z = 0; z < 8; ++z) v[z] = j + z * step < per ? l[j + z * step] : 0.f;
+#pragma unroll
+        for (int z = 0; z < 8; ++z) s += (double)v[z];
+    }
+    s = warp_sum(s);
+    if ((threadIdx.x & 31) == 0) out = s;
+}
+// Cumulative losses and Hedge weights from the means of N learners, a lane to a learner (the lanes behind them hold the
+// last one's), by one warp.
+__device__ __forceinline__ void hedge_weights(int N, double mean, double eps, const double* cum_in, double* round_loss, double* cum_out,
+                                              float* weights) {
+    const int lane = threadIdx.x & 31;
+    const double cum = (cum_in ? cum_in[min(lane, N - 1)] : 0.0) + mean;
+    double lowest = INFINITY, Z = 0.0;
+    for (int m = 0; m < N; ++m) {
+        const double c = __shfl_sync(0xffffffffu, cum, m);
+        if (c < lowest) lowest = c;
+    }
+    const double e = exp(-eps * (cum - lowest));
+    for (int m = 0; m < N; ++m) Z += __shfl_sync(0xffffffffu, e, m);
+    if (lane < N) {
+        round_loss[lane] = mean;
+        cum_out[lane] = cum;
+        weights[lane] = (float)(e / Z);
+    }
+}
 // Mean loss of the round per learner (fixed summation order), cumulative losses, Hedge weights.  One block, four
 // warps to a learner with eight loads in flight each, then a lane to a learner: round trips and fp64 exponentials
 // are all it consists of.
@@ -1047,36 +1079,11 @@ __global__ void __launch_bounds__(kHedgeThreads) sd_hedge_kernel(const float* lo
     const int tid = threadIdx.x, lane = tid & 31, n = tid >> 7, q = (tid >> 5) & 3;
     await_previous_kernel();
     launch_dependents();
-    if (n < N) {
-        const float* const l = loss + (size_t)n * per;
-        double s = 0.0;
-        for (long long j = q * 32 + lane; j < per; j += 8 * 128) {
-            float v[8];
-#pragma unroll
-            for (int z = 0; z < 8; ++z) v[z] = j + z * 128 < per ? l[j + z * 128] : 0.f;
-#pragma unroll
-            for (int z = 0; z < 8; ++z) s += (double)v[z];
-        }
-        s = warp_sum(s);
-        if (lane == 0) part[n][q] = s;
-    }
+    if (n < N) hedge_sum(loss + (size_t)n * per, per, q * 32 + lane, 128, part[n][q]);
     __syncthreads();
     if (tid < 32) {
         const int i = min(lane, N - 1);
-        const double mean = ((part[i][0] + part[i][1]) + (part[i][2] + part[i][3])) / (double)per;
-        const double cum = (cum_in ? cum_in[i] : 0.0) + mean;
-        double lowest = INFINITY, Z = 0.0;
-        for (int m = 0; m < N; ++m) {
-            const double c = __shfl_sync(0xffffffffu, cum, m);
-            if (c < lowest) lowest = c;
-        }
-        const double e = exp(-eps * (cum - lowest));
-        for (int m = 0; m < N; ++m) Z += __shfl_sync(0xffffffffu, e, m);
-        if (lane < N) {
-            round_loss[lane] = mean;
-            cum_out[lane] = cum;
-            weights[lane] = (float)(e / Z);
-        }
+        hedge_weights(N, ((part[i][0] + part[i][1]) + (part[i][2] + part[i][3])) / (double)per, eps, cum_in, round_loss, cum_out, weights);
     }
     // a bounded wait gave up somewhere in the feedback kernel: nothing of this round is valid
     if (status && *sticky != 0)

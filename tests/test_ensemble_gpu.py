@@ -241,3 +241,85 @@ def test_gradients_of_some_learners_can_be_left_out(binding):
     assert rc == 0
     assert torch.equal(out.loss, full.loss) and torch.equal(out.weights, full.weights)
     assert torch.equal(g2, full.grad[2]) and (g0 == 7.0).all()
+
+
+# Two sweeps that share the target among the learners (csrc/sd_ensemble.cuh): bf16 rows of more than the chip holds twice.
+@pytest.mark.parametrize("B,k,V,N", [(200, 3, 4104, 1), (1200, 2, 504, 3), (100, 3, 512 * 32 + 8, 2), (100, 3, 512 * 32 - 8, 2), (40, 3, 512 * 64 + 8, 3),
+                                     (40, 4, 20000, 5), (30, 3, 30000, 8), (2, 64, 30000, 4), (2, 2, 5500008, 2)])
+def test_two_sweeps(binding, options, B, k, V, N):
+    """Rows shorter than a region, of a region more or less than an item, of the most items; one to four learners to a
+    group, and groups of two sizes; with and without gradients; the cluster kernel, which one of its options selects."""
+    cfg = synth.custom_config(B, k, V, dtype="bf16", tau=0.9)
+    inp, Ds, out, ref = run(binding, cfg, N=N, cum_in=np.linspace(0.3, 0.1, N))
+    info = binding.sd_launch_info()
+    assert (info["path"], info["threads"], info["kernels"]) == (3, 256, 3 if N <= 4 else 5)
+    T, dDs = dev(inp.target_logits), [dev(d) for d in Ds]
+    cum = torch.from_numpy(np.linspace(0.3, 0.1, N)).cuda()
+    only = binding.sd_ensemble_feedback(T, dDs, inp.tau, EPS, cum_loss=cum, want_grad=False)
+    torch.cuda.synchronize()
+    assert torch.equal(only.loss, out.loss) and torch.equal(only.weights, out.weights)
+    options(binding.SD_OPT_CLUSTER, 2)
+    other = binding.sd_ensemble_feedback(T, dDs, inp.tau, EPS, cum_loss=cum)
+    assert binding.sd_launch_info()["threads"] == 1024
+    torch.cuda.synchronize()
+    compare(inp, Ds, other, ref, np.linspace(0.3, 0.1, N))
+
+
+def test_two_sweeps_special_rows(binding):
+    """Masked regions, entries far above all before them (target, one learner, both), identical models, a draft entry far
+    below all others; and rows without a finite entry, which the status names."""
+    B, k, V, N = 60, 3, 20000, 3
+    inp = synth.make_inputs(synth.custom_config(B, k, V, dtype="bf16", tau=0.9, index=130))
+    Ds = synth.ensemble_drafts(inp, N)
+    T = inp.target_logits
+
+    def value(v):
+        return synth.f32_to_bf16_bits(np.array([v], np.float32))[0]
+    ninf = np.uint16(0xFF80)
+    T[0:2, :, 100:9000] = ninf
+    for D in Ds:
+        D[0:2, :, 100:6000] = ninf
+    T[2, 0, 18000] = value(300)
+    Ds[1][3, 1, 15000] = value(300)
+    T[4, 1, 12000], Ds[2][4, 1, V - 3] = value(300), value(300)
+    Ds[0][5] = T[5, :k]
+    T[6, :, :V - 1] = ninf
+    Ds[1][7, 2, 5] = value(-1e30)
+    ref = sd_oracle.ensemble_feedback(T, Ds, inp.tau, EPS, nthreads=min(8, sd_oracle.max_threads()))
+    out = binding.sd_ensemble_feedback(dev(T), [dev(d) for d in Ds], inp.tau, EPS, want_status=True)
+    assert binding.sd_launch_info()["threads"] == 256
+    torch.cuda.synchronize()
+    assert (out.status.cpu().numpy() == 0).all()
+    assert np.isfinite(ref.loss).all()
+    compare(inp, Ds, out, ref)
+    T[8, 1], Ds[2][9, 0] = ninf, ninf
+    bad = binding.sd_ensemble_feedback(dev(T), [dev(d) for d in Ds], inp.tau, EPS, want_status=True)
+    torch.cuda.synchronize()
+    want = np.zeros(B)
+    want[8:10] = binding.SD_STATUS_BAD_ROW
+    assert (bad.status.cpu().numpy() == want).all()
+    keep = [b for b in range(B) if b not in (8, 9)]
+    assert torch.equal(bad.loss[:, keep], out.loss[:, keep])
+
+
+def test_two_sweeps_in_a_graph(binding):
+    """A replay and eager calls on the library's scratch, one after the other."""
+    cfg = synth.custom_config(60, 3, 20000, dtype="bf16", tau=0.9, index=131)
+    inp = synth.make_inputs(cfg)
+    Ds = synth.ensemble_drafts(inp, 3)
+    T, dDs = dev(inp.target_logits), [dev(d) for d in Ds]
+    x, u = torch.from_numpy(inp.draft_tokens).cuda(), torch.from_numpy(inp.uniforms).cuda()
+    want = binding.sd_ensemble_feedback(T, dDs, inp.tau, EPS)
+    step = binding.sd_verify_feedback(T, dDs[0], x, u, inp.tau)
+    torch.cuda.synchronize()
+    g = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(g):
+        out = binding.sd_ensemble_feedback(T, dDs, inp.tau, EPS)
+        assert binding.sd_launch_info()["threads"] == 256
+    for _ in range(2):
+        g.replay()
+        again = binding.sd_verify_feedback(T, dDs[0], x, u, inp.tau)
+        torch.cuda.synchronize()
+        assert torch.equal(again.tokens, step.tokens) and torch.equal(again.grad_draft, step.grad_draft)
+        assert torch.equal(out.loss, want.loss) and torch.equal(out.weights, want.weights)
+        assert all(torch.equal(a, b) for a, b in zip(out.grad, want.grad))
