@@ -434,13 +434,17 @@ cudaError_t launch_following(K kern, dim3 grid, int threads, cudaStream_t stream
 // (hint error, one draft token, 46 sequences of 129 216 bf16 entries, blocks of two warps 35.0 us, of eight 33.1).
 int rows_threads(int k) { return 32 * (k < 8 ? 8 : k + 1 < kRowsMaxWarps ? k + 1 : kRowsMaxWarps); }
 
-template <int DT, int MODE, bool RAGGED = false>
+template <int DT, int MODE, bool RAGGED, bool FINE>
 int launch_sweeps_of(const Params& P, const Sweep& S, long long units, bool all, cudaStream_t stream) {
-    SD_CUDA(launch_following(sd_sweep_stats_kernel<DT, RAGGED>, dim3((unsigned)units, (unsigned)S.slices), kSweepThreads, stream, P, S));
+    const dim3 first = FINE ? dim3((unsigned)((units - S.fine_units) * S.slices + (long long)S.fine_units * S.fine_slices))
+                            : dim3((unsigned)units, (unsigned)S.slices);
+    SD_CUDA(launch_following(sd_sweep_stats_kernel<DT, RAGGED, FINE>, first, kSweepThreads, stream, P, S));
     SD_CUDA(launch_following(sd_sweep_rows_kernel<DT>, dim3((unsigned)P.B), rows_threads(P.k), stream, P, S));
-    // the rows that are drawn from, then (if anything of them is wanted) all rows
-    const unsigned second = (unsigned)S.draw_blocks + (all ? (unsigned)P.B * (unsigned)P.k * (unsigned)S.slices : 0u);
-    SD_CUDA(launch_following(sd_sweep_grad_kernel<DT, MODE, RAGGED>, dim3(second), kSweepThreads, stream, P, S));
+    // the rows that are drawn from, then (if anything of them is wanted) all pair rows; the hint error is summed by items of one size
+    constexpr bool FINE2 = FINE && MODE != kSweepHint;
+    const long long rows = (long long)P.B * P.k, fine = FINE2 ? S.fine_rows : 0;
+    const unsigned second = (unsigned)S.draw_blocks + (all ? (unsigned)((rows - fine) * S.slices + fine * S.fine_slices) : 0u);
+    SD_CUDA(launch_following(sd_sweep_grad_kernel<DT, MODE, RAGGED, FINE2>, dim3(second), kSweepThreads, stream, P, S));
     return SD_OK;
 }
 
@@ -454,6 +458,25 @@ int launch_sweeps(const Params& P, Sweep& S, long long units, int dtype, cudaStr
     // 74.8).
     const bool all = MODE != kSweepErrors && (P.grad || MODE == kSweepHint || S.all_rows);
     S.kept = all ? (80u << 20) / (unsigned)(S.regions * kRegionVecs * 32) : 0u;
+    // Items of more than two regions a warp become smaller towards the end of a sweep, so that its blocks end together: the
+    // last 300 (a third of a round of 888) of the first sweep, and as many of the second, have two.  Step, in us, items of one size /
+    // small ones 225 / 300 / 450 / 600: 32 sequences, 8 tokens, 128 256 bf16 entries 57.2 / 56.0 / 55.8 / 55.6 / 55.9; 48, 4, 128 256
+    // 47.3 / 45.8 / 45.7 / 46.0 / 46.5; 16, 6, 128 256 28.7 / 27.6 / 27.6 / 27.9 / 28.1; 100, 8, 152 064 200.7 / 199.6 / 199.4 / 199.3 / 199.3;
+    // 90, 4, 32 000 29.4 / 28.1 / 28.1 / 28.3 / 28.6.  As kernels of their own (smaller
+    // calls keep the shorter way to their items): 32, 8, 128 256 57.4 -> 56.1; 64, 4, 151 936 70.9 -> 69.7; error feedback there 51.1 -> 50.7.
+    // bf16 only: fp32 44, 4, 128 256 77.4 / 76.8 / 76.6, 24, 4 45.1 / 45.1 / 45.3, and the hint's first sweep, which has to add up as
+    // the step's does, 32, 6, 128 256 103.9 -> 104.3.
+    S.fine_units = S.fine_rows = 0;
+    S.fine_slices = S.slices;
+    S.fine_regions = S.regions;
+    S.part_stride = S.slices;
+    const int fine_slices = (P.NR + 2 * kSweepWarps - 1) / (2 * kSweepWarps);
+    if (!RAGGED && dtype == SD_DTYPE_BF16 && S.regions > 2 * kSweepWarps && fine_slices <= kMaxSlices) {
+        S.fine_slices = S.part_stride = fine_slices;      // (a unit has room for NR / 8 partials, those of a region's mass each)
+        S.fine_regions = 2 * kSweepWarps;
+        S.fine_units = (int)(units < 300 / fine_slices ? units : 300 / fine_slices);
+        S.fine_rows = P.B * P.k < 300 / fine_slices ? P.B * P.k : 300 / fine_slices;
+    }
     // The items of the drawn rows are as small as leaves all their blocks resident at once, where the second sweep is
     // the drawn rows alone or not much more than a round of blocks (888 at a time, 592 of odd rows: six and four on each
     // of 148 SMs): a draw is a chain of round trips, one for each
@@ -471,8 +494,12 @@ int launch_sweeps(const Params& P, Sweep& S, long long units, int dtype, cudaStr
         }
     }
     S.draw_blocks = P.B * S.draw_slices;
-    const int rc = dtype == SD_DTYPE_F32 ? launch_sweeps_of<SD_DTYPE_F32, MODE, RAGGED>(P, S, units, all, stream)
-                                         : launch_sweeps_of<SD_DTYPE_BF16, MODE, RAGGED>(P, S, units, all, stream);
+    int rc;
+    if (!RAGGED && S.fine_units > 0)
+        rc = launch_sweeps_of<SD_DTYPE_BF16, MODE, false, true>(P, S, units, all, stream);
+    else
+        rc = dtype == SD_DTYPE_F32 ? launch_sweeps_of<SD_DTYPE_F32, MODE, RAGGED, false>(P, S, units, all, stream)
+                                   : launch_sweeps_of<SD_DTYPE_BF16, MODE, RAGGED, false>(P, S, units, all, stream);
     if (rc != SD_OK) return rc;
     tl_info[0] = 1; tl_info[1] = 1; tl_info[2] = kSweepThreads; tl_info[3] = 0;
     tl_info[4] = (int)(units * S.slices); tl_info[5] = 3;

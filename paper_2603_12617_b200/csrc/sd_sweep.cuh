@@ -42,7 +42,11 @@ constexpr int kSweepStep = kSweepWarps * kRegionVecs;   // vectors from a warp's
 struct Sweep {
     int slices;              // items per unit (1..kMaxSlices)
     int regions;             // sampling regions per item (the last item of a unit may have fewer)
-    PartialStats* part;      // workspace [units][slices]; its memory is region_sums' from the second sweep on
+    int fine_units;          // units from the last one backwards whose items are smaller in the first sweep,
+    int fine_rows;           // pair rows from the first one on whose items are smaller in the second:
+    int fine_slices, fine_regions;   // so many of so many regions (slices and regions where there are none)
+    int part_stride;         // room for a unit's partials
+    PartialStats* part;      // workspace [units][part_stride]; its memory is region_sums' from the second sweep on
     uint32_t* arrived;       // workspace [units], zero on entry and zero again on exit
     unsigned kept;           // items, from the last one backwards, that L2 is asked to keep between the sweeps
     int all_rows;            // second sweep: masses of every row wanted (acceptance probabilities)
@@ -314,8 +318,9 @@ __device__ __forceinline__ void sweep_pass1(const uint4* gT, const uint4* gD, in
     if (nvec > 0) s = pass1_region_again<DT, BONUS>(gT, gD, nvec, lane, c, s);   // cut short by the end of the row
 }
 
-// One block per item: blockIdx.x = unit, blockIdx.y = slice.
-template <int DT, bool RAGGED>
+// One block per item: blockIdx.x = unit, blockIdx.y = slice.  FINE (a grid of one dimension): the units with large items like
+// that, then those with small ones.
+template <int DT, bool RAGGED, bool FINE>
 __global__ void __launch_bounds__(kSweepThreads, !RAGGED ? 6 : DT == SD_DTYPE_F32 ? 6 : 5)
 sd_sweep_stats_kernel(const __grid_constant__ Params P, const __grid_constant__ Sweep S) {
     using E = Elem<DT>;
@@ -324,22 +329,37 @@ sd_sweep_stats_kernel(const __grid_constant__ Params P, const __grid_constant__ 
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     await_previous_kernel();                         // (first: the rows kernel reads inputs before its own wait)
     launch_dependents();
-    const int unit = blockIdx.x, slice = blockIdx.y;
+    int unit = blockIdx.x, slice = blockIdx.y, regions = S.regions;
+    unsigned behind = (gridDim.y - 1u - blockIdx.y) * gridDim.x + (gridDim.x - 1u - blockIdx.x);     // items
+    if constexpr (FINE) {
+        int units = total_units<false>(P) - S.fine_units;
+        const int large = units * S.slices;
+        if (unit < large) {
+            slice = unit / units;
+            unit -= slice * units;
+            behind -= S.fine_units * S.fine_slices / 2;           // (of about half as many regions each)
+        } else {
+            slice = (unit - large) / S.fine_units;
+            unit = unit - large - slice * S.fine_units + units;
+            regions = S.fine_regions;
+            behind /= 2;
+        }
+    }
+    const uint64_t policy = behind < S.kept ? policy_keep() : policy_discard();
+    const int at = unit * S.part_stride + slice;
     const UnitRef ur = unit_ref<false>(P, unit);
-    const int v0 = (slice * S.regions + warp) * kRegionVecs;
+    const int v0 = (slice * regions + warp) * kRegionVecs;
     Pass1State ps;
     ps.RT = ps.RD = kEmptyRef;
     ps.ls.init();
-    const unsigned from_end = (gridDim.y - 1u - blockIdx.y) * gridDim.x + (gridDim.x - 1u - blockIdx.x);
-    const uint64_t policy = from_end < S.kept ? policy_keep() : policy_discard();
     if constexpr (RAGGED) {
         const RowFrame<DT> f = row_frame<DT>(P, ur);
-        int v1 = min((slice + 1) * S.regions * kRegionVecs, f.nvec);
+        int v1 = min((slice + 1) * regions * kRegionVecs, f.nvec);
         if (!SD_IN(ur.t_row, (long long)P.B * (P.k + 1), 10) || !SD_IN(ur.d_row, (long long)P.B * P.k, 11)) v1 = 0;
         if (ur.bonus) ragged_pass1<DT, true>(f, P.V, v0, v1, lane, P.c, policy, ps);
         else          ragged_pass1<DT, false>(f, P.V, v0, v1, lane, P.c, policy, ps);
     } else {
-        int nvec = min((slice + 1) * S.regions * kRegionVecs, P.V / E::VEC) - v0;
+        int nvec = min((slice + 1) * regions * kRegionVecs, P.V / E::VEC) - v0;
         if (nvec > 0 && !SD_IN((long long)(v0 + nvec) * E::VEC - 1, P.V, 10)) nvec = 0;
         if (!SD_IN(ur.t_row, (long long)P.B * (P.k + 1), 10) || !SD_IN(ur.d_row, (long long)P.B * P.k, 11)) nvec = 0;
         const uint4* const gT = reinterpret_cast<const uint4*>(reinterpret_cast<const ET*>(P.T) + ur.t_row * P.V) + v0;
@@ -351,8 +371,7 @@ sd_sweep_stats_kernel(const __grid_constant__ Params P, const __grid_constant__ 
     __syncthreads();
     if (warp == 0) {
         const PartialStats item = warp_merge_lanes(lane < kSweepWarps ? wpart[lane] : empty_partial());
-        if (lane == 0 && SD_IN((long long)unit * S.slices + slice, (long long)total_units<false>(P) * S.slices, 26))
-            S.part[(size_t)unit * S.slices + slice] = item;
+        if (lane == 0 && SD_IN(at, (long long)total_units<false>(P) * S.part_stride, 26)) S.part[at] = item;
     }
 }
 
@@ -371,8 +390,9 @@ sd_sweep_rows_kernel(const __grid_constant__ Params P, const __grid_constant__ S
         AcceptOperands aop;
         aop.valid = false;
         if (lane == 0 && i < P.k) aop = load_accept_operands<DT>(P, b, i);   // (inputs of the call)
-        const bool mine = lane < S.slices && SD_IN((long long)unit * S.slices + lane, (long long)total_units<false>(P) * S.slices, 26);
-        const PartialStats* const part = S.part + (size_t)unit * S.slices + lane;
+        const int slices = unit < total_units<false>(P) - S.fine_units ? S.slices : S.fine_slices;
+        const bool mine = lane < slices && SD_IN(unit, total_units<false>(P), 26);
+        const PartialStats* const part = S.part + (size_t)unit * S.part_stride + lane;
         await_previous_kernel();
         const PartialStats row = warp_merge_lanes(mine ? load_partial_cg(part) : empty_partial());
         const RowLogs logs = warp_row_logs(row);
@@ -603,7 +623,7 @@ __device__ __noinline__ void sweep_row_sums(const Params& P, const Sweep& S, int
 // chains of dependent reads, are over long before the sweep is); the rest all other pair rows, from the
 // last item of the first sweep backwards.  (Blocks for bonus rows, which would only find nothing to do: 32 sequences, 8
 // tokens, 128 256 bf16 entries 57.7 us, without 57.4.)
-template <int DT, int MODE, bool RAGGED>
+template <int DT, int MODE, bool RAGGED, bool FINE>
 __global__ void __launch_bounds__(kSweepThreads, MODE == kSweepHint || RAGGED ? 4 : 6)
 sd_sweep_grad_kernel(const __grid_constant__ Params P, const __grid_constant__ Sweep S) {
     using E = Elem<DT>;
@@ -613,22 +633,36 @@ sd_sweep_grad_kernel(const __grid_constant__ Params P, const __grid_constant__ S
     __shared__ int is_last;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const bool draws = (int)blockIdx.x < S.draw_blocks;
-    int unit, slice, b;
+    int unit, slice, b, regions = S.draw_regions, slices = S.draw_slices;
     if (draws) {
         b = (int)blockIdx.x / S.draw_slices;
         slice = (int)blockIdx.x - b * S.draw_slices;
         unit = 0;
     } else {
-        const int rows = P.B * P.k, id = (int)(gridDim.x - 1u - blockIdx.x);
+        // FINE: of the last rows the large items, then of the first ones the small
+        int id = (int)(gridDim.x - 1u - blockIdx.x), from = 0, rows = P.B * P.k;
+        regions = S.regions;
+        slices = S.slices;
+        if constexpr (FINE) {
+            if (id < S.fine_rows * S.fine_slices) {
+                rows = S.fine_rows;
+                regions = S.fine_regions;
+                slices = S.fine_slices;
+            } else {
+                from = S.fine_rows;
+                id -= from * S.fine_slices;
+                rows -= from;
+            }
+        }
         slice = id / rows;
-        b = (id - slice * rows) / P.k;
-        unit = id - slice * rows + b;
+        const int row = from + id - slice * rows;
+        b = row / P.k;
+        unit = row + b;
     }
     await_previous_kernel();
     launch_dependents();
 
     if (!SD_IN(b, P.B, 22) || !SD_IN(unit, total_units<false>(P), 20)) return;
-    const int regions = draws ? S.draw_regions : S.regions, slices = draws ? S.draw_slices : S.slices;
     if (!SD_IN(slice, slices, 20)) return;
     // (both loads under way together: of a block's chain of round trips this is one less)
     RowConst rc = P.rowc[unit];
