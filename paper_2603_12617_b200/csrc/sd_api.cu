@@ -1524,10 +1524,15 @@ int sd_vp_finish(const void* target_shard, const void* draft_shard, const int32_
     P.local_mass = out_local_mass;
     cudaStream_t st = static_cast<cudaStream_t>(stream);
     SD_CUDA(launch_following(sd_vp_rows_kernel, dim3((unsigned)B), 32 * (k + 1 < kRowsMaxWarps ? k + 1 : kRowsMaxWarps), st, P));
-    const int slices = (P.NR + kVpSliceRegions - 1) / kVpSliceRegions;
+    // blocks as in the single-GPU sweeps: up to four regions a warp, fewer where the call has no block for every SM's six
+    // (888), all of about the same size.  64 sequences, 4 tokens, 75 regions a row: 32, 32 and 11 regions 38.2 us, 25 each 37.4;
+    // 16 sequences, 38 regions: 32 and 6 22.2, 19 each 20.6, 16 and fewer 19.8.
+    long long most = ((long long)B * (k + 1) * P.NR / 888 + kVpWarps - 1) / kVpWarps * kVpWarps;
+    most = most < kVpWarps ? kVpWarps : most > 4 * kVpWarps ? 4 * kVpWarps : most;
+    const int slices = (int)((P.NR + most - 1) / most), regions = (P.NR + slices - 1) / slices;
     const unsigned grid = (unsigned)B * (unsigned)(k + 1) * (unsigned)slices;
-    SD_CUDA(dtype == SD_DTYPE_F32 ? launch_following(sd_vp_grad_kernel<SD_DTYPE_F32>, dim3(grid), kVpThreads, st, P, slices)
-                                  : launch_following(sd_vp_grad_kernel<SD_DTYPE_BF16>, dim3(grid), kVpThreads, st, P, slices));
+    SD_CUDA(dtype == SD_DTYPE_F32 ? launch_following(sd_vp_grad_kernel<SD_DTYPE_F32>, dim3(grid), kVpThreads, st, P, slices, regions)
+                                  : launch_following(sd_vp_grad_kernel<SD_DTYPE_BF16>, dim3(grid), kVpThreads, st, P, slices, regions));
     tl_info[0] = 6; tl_info[1] = 1; tl_info[2] = kVpThreads; tl_info[3] = 0; tl_info[4] = (int)grid; tl_info[5] = 2;
     return SD_OK;
 }
@@ -1554,8 +1559,8 @@ int sd_vp_draw(const void* target_shard, const void* draft_shard, const int32_t*
     P.tokens = out_tokens;
     P.status = out_status;
     cudaStream_t st = static_cast<cudaStream_t>(stream);
-    SD_CUDA(dtype == SD_DTYPE_F32 ? launch_following(sd_vp_draw_kernel<SD_DTYPE_F32>, dim3((unsigned)B), 32, st, P)
-                                  : launch_following(sd_vp_draw_kernel<SD_DTYPE_BF16>, dim3((unsigned)B), 32, st, P));
+    SD_CUDA(dtype == SD_DTYPE_F32 ? launch_following(sd_vp_draw_kernel<SD_DTYPE_F32>, dim3((unsigned)B), kSweepThreads, st, P)
+                                  : launch_following(sd_vp_draw_kernel<SD_DTYPE_BF16>, dim3((unsigned)B), kSweepThreads, st, P));
     tl_info[0] = 6; tl_info[5] = 1;
     return SD_OK;
 }

@@ -318,6 +318,41 @@ __device__ __forceinline__ void sweep_pass1(const uint4* gT, const uint4* gD, in
     if (nvec > 0) s = pass1_region_again<DT, BONUS>(gT, gD, nvec, lane, c, s);   // cut short by the end of the row
 }
 
+// The same with two regions of a warp on their way at a time, and every region raising the references: for warps with few
+// regions, whose time is round trips.
+template <int DT, bool BONUS>
+__device__ __forceinline__ void sweep_pass1_pairs(const uint4* gT, const uint4* gD, int nvec, int step, int lane, float c, uint64_t policy,
+                                                  Pass1State& s) {
+    for (; nvec >= kRegionVecs; gT += 2 * step, gD += 2 * step, nvec -= 2 * step) {
+        uint4 rt[2][kRegionRows], rd[2][kRegionRows];
+        const bool both = nvec - step >= kRegionVecs;
+#pragma unroll
+        for (int j = 0; j < 2; ++j)
+#pragma unroll
+            for (int g = 0; g < kRegionRows; ++g) {
+                rt[j][g] = rd[j][g] = Elem<DT>::masked();
+                if (j == 0 || both) {
+                    rt[j][g] = load_l2(gT + j * step + g * 32 + lane, policy);
+                    if (!BONUS) rd[j][g] = load_l2(gD + j * step + g * 32 + lane, policy);
+                }
+            }
+#pragma unroll
+        for (int j = 0; j < 2; ++j) {
+            if (j == 1 && !both) break;
+            follow_references<DT, BONUS>(rt[j], rd[j], c, s);
+            float sT, sD, sW;
+            region_sums_of<DT, BONUS, false>(rt[j], rd[j], c, s.RT, s.RD, sT, sD, sW);
+            // masked target entries (a NaN): with the test for them
+            if (__any_sync(0xffffffffu, sW != sW)) region_sums_of<DT, BONUS, true>(rt[j], rd[j], c, s.RT, s.RD, sT, sD, sW);
+            s.ls.sT += sT;
+            s.ls.sD += sD;
+            s.ls.w += sW;
+        }
+        if (!both && nvec > step) { gT += step; gD += step; nvec -= step; break; }
+    }
+    if (nvec > 0) s = pass1_region_again<DT, BONUS>(gT, gD, nvec, lane, c, s);   // cut short by the end of the row
+}
+
 // One block per item: blockIdx.x = unit, blockIdx.y = slice.  FINE (a grid of one dimension): the units with large items like
 // that, then those with small ones.
 template <int DT, bool RAGGED, bool FINE>

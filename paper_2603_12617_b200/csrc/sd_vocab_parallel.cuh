@@ -73,7 +73,8 @@ struct VpParams {
 // A cluster of C blocks per row (as many as leave all of them resident: a warp's time is a chain of round trips, one
 // per region), its warps take the row's regions in turn, with the loop of the single-GPU first sweep (a
 // maximum for every two vectors and a test for masked entries took 18.0 us on 320 rows of 37 984 bf16 entries,
-// one block of eight warps per row 15.7).
+// one block of eight warps per row 15.7; ten or twelve blocks an SM, with fewer registers, no less, and fp32 rows a tenth more).
+// fp32 rows go two regions at a time (448 rows of 32 064 entries: the three calls 52.5 -> 50.6).
 // Every region raises the references: with those of a warp's first region alone the error of fp32
 // gradients against 64 bits doubled.  With a vote whether any entry is above them that costs nothing there
 // (1792 rows of 32 064 entries 42.0 -> 44.0; raised without looking 45.0).
@@ -118,8 +119,15 @@ __global__ void __launch_bounds__(kVpStatsThreads, 8) sd_vp_stats_kernel(const V
     const int w0 = slot * kRegionVecs;
     const uint64_t policy = policy_normal();     // what fits stays in L2 for the second sweep
     const int nvec = SD_IN(unit, P.B * K1, 60) ? NV - w0 : 0;
-    if (bonus) sweep_pass1<DT, true, true>(Trow + w0, Drow + w0, nvec, slots * kRegionVecs, lane, P.c, policy, ps);
-    else       sweep_pass1<DT, false, true>(Trow + w0, Drow + w0, nvec, slots * kRegionVecs, lane, P.c, policy, ps);
+    const int step = slots * kRegionVecs;
+    if constexpr (DT == SD_DTYPE_F32) {
+        // (bf16 regions, with twice the entries, have no registers for two: 37.7 us against 37.0 on 320 rows of 37 984)
+        if (bonus) sweep_pass1_pairs<DT, true>(Trow + w0, Drow + w0, nvec, step, lane, P.c, policy, ps);
+        else       sweep_pass1_pairs<DT, false>(Trow + w0, Drow + w0, nvec, step, lane, P.c, policy, ps);
+    } else {
+        if (bonus) sweep_pass1<DT, true, true>(Trow + w0, Drow + w0, nvec, step, lane, P.c, policy, ps);
+        else       sweep_pass1<DT, false, true>(Trow + w0, Drow + w0, nvec, step, lane, P.c, policy, ps);
+    }
     __syncwarp();
     if (C > 1) {
         cluster_wait();
@@ -241,9 +249,8 @@ __global__ void __launch_bounds__(kRowsMaxWarps * 32) sd_vp_rows_kernel(const Vp
 // pair row; masses of the regions of row n_b of every sequence (the bonus row when n_b = k); and, by the block that
 // brings that row's last slice, this shard's share of the row's mass (fixed order, fp64).  Rows that are not drawn
 // from skip their masses.
-constexpr int kVpSliceRegions = 32;
 template <int DT>
-__global__ void __launch_bounds__(kVpThreads, 6) sd_vp_grad_kernel(const VpParams P, const int slices) {
+__global__ void __launch_bounds__(kVpThreads, 6) sd_vp_grad_kernel(const VpParams P, const int slices, const int regions) {
     using E = Elem<DT>;
     using ET = typename E::type;
     constexpr int VEC = E::VEC;
@@ -264,7 +271,7 @@ __global__ void __launch_bounds__(kVpThreads, 6) sd_vp_grad_kernel(const VpParam
     ET* Grow = (P.grad && !bonus) ? reinterpret_cast<ET*>(P.grad) + (size_t)(b * P.k + i) * P.Vs : nullptr;
     const int NV = P.Vs / VEC;
     float* rsum = P.region_sums + (size_t)b * 2 * P.NR;
-    const int r0 = sl * kVpSliceRegions, r1 = min(P.NR, r0 + kVpSliceRegions);
+    const int r0 = sl * regions, r1 = min(P.NR, r0 + regions);
     if (!draws) {
         const int v0 = (r0 + warp) * kRegionVecs;
         int nvec = min(r1 * kRegionVecs, NV) - v0;
@@ -322,35 +329,44 @@ __global__ void __launch_bounds__(kVpThreads, 6) sd_vp_grad_kernel(const VpParam
 }
 
 // ---- phase 3 -------------------------------------------------------------------------------
-// One warp per sequence.  Shares in rank order: the first rank whose running sum exceeds
-// u_k * total owns the draw (the last rank with mass, if rounding leaves none).
+// One block per sequence.  Shares in rank order: the first rank whose running sum exceeds
+// u_k * total owns the draw (the last rank with mass, if rounding leaves none); its block searches as the single-GPU
+// draw does (sweep_draw), with the mass of the ranks before it in front.  (A warp that took sixteen regions and entries to a
+// lane: with the slices of phase 2 as they were 22.2 us for the three calls on 16 sequences, 4 tokens, an eighth of 151 936
+// bf16 entries, 18.0 with both; 4 sequences, a quarter of 32 000 14.8, 13.3.)
 template <int DT>
-__global__ void __launch_bounds__(32) sd_vp_draw_kernel(const VpParams P) {
-    constexpr int PER = kRegionVecs * Elem<DT>::VEC / 32;
-    const int b = blockIdx.x, lane = threadIdx.x;
+__global__ void __launch_bounds__(kSweepThreads) sd_vp_draw_kernel(const VpParams P) {
+    using E = Elem<DT>;
+    constexpr int kEntries = kRegionVecs * E::VEC, PER = kEntries / kSweepThreads;
+    __shared__ double sums[2][kSweepWarps];
+    __shared__ double prefix_sh;
+    __shared__ int owner_sh[2], found, last_mass;
+    const int b = blockIdx.x, tid = threadIdx.x, lane = tid & 31;
     const int k = P.k, K1 = k + 1;
     await_previous_kernel();
     launch_dependents();
-    // everything that does not depend on where the draw falls is asked for at once: the warp's time is round trips
+    // everything that does not depend on where the draw falls is asked for at once: the block's time is round trips
     // (the caller's memory: a length that phase 2 cannot have written leads to no row but the sequence's own)
     const int n = min(max(P.accept_len[b], 0), k);
-    const float uk = P.u[b * K1 + k];
-    const int32_t x_first = lane < k ? P.x[b * k + lane] : -1;
+    const double uk = (double)P.u[b * K1 + k];
+    const int32_t x = tid < k ? P.x[b * k + tid] : -1;
     double2 mass = make_double2(0.0, 0.0);
     if (lane < P.G) {
         const double* const m = P.all_mass + ((size_t)lane * P.B + b) * 2;
         mass = make_double2(m[0], m[1]);
     }
-    const int per = (P.NR + 31) / 32;
-    const int j0 = min(P.NR, lane * per), j1 = min(P.NR, j0 + per);
-    constexpr int kHeld = 8;
-    float held[kHeld];
-#pragma unroll
-    for (int q = 0; q < kHeld; ++q) held[q] = j0 + q < j1 ? P.region_sums[(size_t)b * 2 * P.NR + j0 + q] : 0.f;
+    const int per = (P.NR + kSweepThreads - 1) / kSweepThreads, j0 = min(P.NR, tid * per), j1 = min(P.NR, j0 + per);
+    const float* rs = P.region_sums + (size_t)b * 2 * P.NR;
+    float held = j0 < j1 ? rs[j0] : 0.f;
+    if (tid == 0) {
+        owner_sh[0] = owner_sh[1] = 0x7fffffff;
+        found = 0;
+        last_mass = -1;
+    }
     const bool bonus = (n == k);
     const int unit = b * K1 + n;
     const RowConst rc = P.rowc[unit];
-    // rank g's shares
+    // rank g's shares (every warp finds the same)
     const auto share = [&](int g, int which) {
         if (P.G > 32) return P.all_mass[((size_t)g * P.B + b) * 2 + which];
         return __shfl_sync(0xffffffffu, which ? mass.y : mass.x, g);
@@ -366,17 +382,17 @@ __global__ void __launch_bounds__(32) sd_vp_draw_kernel(const VpParams P) {
         which = 1;
         total = 0.0;
         for (int g = 0; g < P.G; ++g) total += share(g, 1);
-#pragma unroll
-        for (int q = 0; q < kHeld; ++q) held[q] = j0 + q < j1 ? P.region_sums[((size_t)b * 2 + 1) * P.NR + j0 + q] : 0.f;
+        rs += P.NR;
+        held = j0 < j1 ? rs[j0] : 0.f;
     }
     const int mode = bonus ? 1 : (which ? 2 : 0);
-    const double t = (double)uk * total;
+    const double t = uk * total;
     int owner = -1, last_with_mass = -1;
-    double before = 0.0, run = 0.0;
+    double ahead = 0.0, run = 0.0;
     for (int g = 0; g < P.G; ++g) {
         const double m = share(g, which);
         if (m > 0.0) last_with_mass = g;
-        if (owner < 0 && run + m > t) { owner = g; before = run; }
+        if (owner < 0 && run + m > t) { owner = g; ahead = run; }
         run += m;
     }
     bool past_end = false;
@@ -387,65 +403,63 @@ __global__ void __launch_bounds__(32) sd_vp_draw_kernel(const VpParams P) {
         // stands in, and the status says so
         flags |= SD_STATUS_BAD_ROW;
         if (P.rank == 0) y = 0;
-    } else if (owner == P.rank) {
-        // the search of the single-GPU resolver, with the mass of the ranks before this one in front
-        Params Q;
-        memset(&Q, 0, sizeof Q);
-        Q.T = P.T; Q.D = P.D; Q.V = P.Vs; Q.c = P.c;
+    } else if (owner == P.rank) {                     // (the same for every thread)
         const size_t offT = (size_t)unit * P.Vs, offD = (size_t)(b * k + (bonus ? 0 : n)) * P.Vs;
-        const float* rs = P.region_sums + ((size_t)b * 2 + which) * P.NR;
-        const auto sum_of = [&](int j) { return (double)rs[j]; };
-        double mine = 0.0;
-#pragma unroll
-        for (int q = 0; q < kHeld; ++q) mine += (double)held[q];
-        for (int j = j0 + kHeld; j < j1; ++j) mine += sum_of(j);
-        const double incl = warp_inclusive_scan(mine);
-        int cand = 0x7fffffff;
-        double cand_prefix = 0.0;
-        if (!past_end) {
-            double r2 = before + (incl - mine);
-#pragma unroll
-            for (int q = 0; q < kHeld; ++q) {
-                if (cand == 0x7fffffff && j0 + q < j1) {
-                    const double next = r2 + (double)held[q];
-                    if (next > t) { cand = j0 + q; cand_prefix = r2; }
-                    else r2 = next;
-                }
+        double mine = (double)held, all;
+        for (int j = j0 + 1; j < j1; ++j) mine += (double)rs[j];
+        const double before = ahead + block_sums_before(mine, sums[0], &all);
+        if (!past_end && mine > 0.0 && before + mine > t) atomicMin(&owner_sh[0], tid);
+        if (mine > 0.0) atomicMax(&last_mass, tid);
+        __syncthreads();
+        const bool to_last = owner_sh[0] == 0x7fffffff;      // (rounding: the last region of this shard that holds mass)
+        if (tid == (to_last ? last_mass : owner_sh[0])) {
+            int at = j0;
+            double r2 = before;
+            for (int j = j0; j < j1; ++j) {
+                const double m = j == j0 ? (double)held : (double)rs[j];
+                if (!(m > 0.0)) continue;
+                at = j;
+                if (!to_last && r2 + m > t) break;
+                r2 += m;
             }
-            for (int j = j0 + kHeld; j < j1 && cand == 0x7fffffff; ++j) {
-                const double next = r2 + sum_of(j);
-                if (next > t) { cand = j; cand_prefix = r2; }
-                else r2 = next;
-            }
+            found = at;
+            prefix_sh = r2;
         }
-        const unsigned has = __ballot_sync(0xffffffffu, cand != 0x7fffffff);
-        int region = -1;
-        double prefix = 0.0;
-        bool last_only = past_end;
-        if (has) {
-            const int src = __ffs(has) - 1;
-            region = __shfl_sync(0xffffffffu, cand, src);
-            prefix = __shfl_sync(0xffffffffu, cand_prefix, src);
-        } else {
-            last_only = true;                     // rounding: the last region of this shard that holds mass
-            int lastr = -1;
-            for (int j = j0; j < j1; ++j)
-                if (rs[j] > 0.f) lastr = j;
+        __syncthreads();
+        const int region = found;
+        const double prefix = to_last ? 0.0 : prefix_sh;
+        if (tid == 0) last_mass = -1;
+        float m[PER];
+        const int v0 = region * kEntries + tid * PER;
+        mine = 0.0;
 #pragma unroll
-            for (int off = 16; off > 0; off >>= 1) lastr = max(lastr, __shfl_xor_sync(0xffffffffu, lastr, off));
-            region = lastr;
+        for (int e = 0; e < PER; ++e) {
+            const bool in = v0 + e < P.Vs && SD_IN(region, P.NR, 63);
+            const float tl = in ? E::load(P.T, offT + v0 + e) : -INFINITY, dl = in && mode == 0 ? E::load(P.D, offD + v0 + e) : -INFINITY;
+            m[e] = in ? mass_of(tl, dl, P.c, rc, mode) : 0.f;
+            mine += (double)m[e];
         }
-        int local = -1;
-        if (region >= 0) {
-            double rtot;
-            local = search_region<DT, PER, true>(Q, rc, mode, offT, offD, region, prefix, t, last_only, &rtot);
-            if (local < 0) local = search_region<DT, PER, true>(Q, rc, mode, offT, offD, region, 0.0, 0.0, true, &rtot);
+        const double inside = prefix + block_sums_before(mine, sums[1], &all);
+        if (!to_last && mine > 0.0 && inside + mine > t) atomicMin(&owner_sh[1], tid);
+        if (mine > 0.0) atomicMax(&last_mass, tid);
+        __syncthreads();
+        const bool last_entry = owner_sh[1] == 0x7fffffff;
+        if (tid == (last_entry ? last_mass : owner_sh[1])) {
+            int at = -1;
+            double r2 = inside;
+#pragma unroll
+            for (int e = 0; e < PER; ++e) {
+                if (m[e] > 0.f && (last_entry || at < 0 || !(r2 > t))) at = v0 + e;     // (the first behind which the sum exceeds t)
+                r2 += (double)m[e];
+            }
+            found = max(at, 0);
         }
-        y = P.v_offset + (local < 0 ? 0 : local);
+        if (tid == 0 && last_mass < 0) found = 0;
+        __syncthreads();
+        y = P.v_offset + found;
     }
-    if (lane == 0 && flags && P.status) atomicOr(P.status + b, flags);
-    for (int i = lane; i <= k; i += 32)
-        P.tokens[b * K1 + i] = (i < n) ? (i == lane ? x_first : P.x[b * k + i]) : (i == n ? y : -1);
+    if (tid == 0 && flags && P.status) atomicOr(P.status + b, flags);
+    if (tid <= k) P.tokens[b * K1 + tid] = tid < n ? x : (tid == n ? y : -1);
 }
 
 }  // namespace sdv

@@ -78,6 +78,17 @@ def test_shards_of_equal_width(binding, dtype, V, G):
     assert binding.sd_launch_info()["path"] == 6
 
 
+@pytest.mark.parametrize("B,k,V,dtype,width", [(20, 2, 256 * 65, "f32", 256 * 32), (20, 2, 256 * 98 + 4, "f32", 256 * 33), (700, 1, 256 * 13 - 4, "f32", 256 * 7),
+                                               (2, 2, 512 * 257 + 8, "bf16", 512 * 256), (200, 2, 512 * 40, "bf16", 512 * 23)])
+def test_shards_of_as_many_regions_as_warps_and_threads(binding, B, k, V, dtype, width):
+    """The first sweep of fp32 rows takes a warp's regions two at a time, the draw a thread's one after the other, the second
+    sweep slices of about the same size."""
+    inp = synth.make_inputs(synth.custom_config(B=B, k=k, V=V, dtype=dtype, tau=0.9, index=79))
+    inp.uniforms[:, k] = np.linspace(0, 1 - 2.0 ** -24, B, dtype=np.float32)
+    out = run_sharded(binding, inp, 2, cuts=[(0, width), (width, V)])
+    check(inp, out, oracle_of(inp), max_band_frac=1.0)
+
+
 @pytest.mark.parametrize("dtype", ["f32", "bf16"])
 def test_shards_of_unequal_width_and_a_ragged_last_region(binding, dtype):
     V = 50000
