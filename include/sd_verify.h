@@ -273,9 +273,9 @@ size_t sd_greedy_workspace_bytes(int B, int k);
  *                                      for the two sweeps; with a workspace the cluster kernel serves them)
  *   stream                        in   cudaStream_t
  * Rows must be whole 16-byte vectors and every tensor 16-byte aligned (SD_ERR_ALIGN otherwise:
- * there is no element-wise path for this entry point).  Two kernels are enqueued: one of the kernels
+ * there is no element-wise path for this entry point).  Two kernels are enqueued -- one of the kernels
  * of sd_verify_feedback over (sequence, row, learner) units (the persistent one, or that which holds
- * the rows), then a one-block reduction.
+ * the rows), then a one-block reduction -- or three, the two sweeps (five with more than four learners).
  */
 int sd_ensemble_feedback(const void* target_logits, const void* const* draft_logits, int n_learners,
                          float temperature, float epsilon, int B, int k, int V, int dtype,

@@ -298,14 +298,14 @@ int launch_stream(DeviceState& d, const Params& P, int C, int G, int lag, cudaSt
 // row: as long as every row has an SM to itself its time depends on the row's length alone, while that of
 // the sweeps grows with the rows; with more rows than that its time steps up.  So the length from which the
 // sweeps are faster grows with the rows, up to about 180 of them; from there a call's entries decide.
-// The line was drawn with sweeps a quarter slower than the present ones.  Calls back to back as the kernels are now,
-// element-wise / sweeps in us (4 tokens, i.e. 5 rows a sequence; * = calls to which the line gives the slower kernel):
-//     bf16  4 097 entries 80 rows 18.6 / 19.7, 320 28.1 / 22.0 *, 500 30.6 / 24.7;  8 201: 5 rows 21.2 / 18.3 *,
-//           100 21.9 / 21.0 *, 200 25.6 / 22.1 *, 320 39.2 / 24.2;  12 001: 20 rows 24.3 / 19.1, 145 28.6 / 22.4 *,
-//           200 34.1 / 23.0;  16 385: 145 34.7 / 22.6 *;  32 001: 5 rows 41.7 / 18.0, 320 119 / 33.4
-//     fp32  4 097: 5 rows 14.5 / 14.0 *, 180 16.5 / 16.7, 320 22.3 / 18.3 *, 640 30.7 / 21.5;  8 201: 40 rows 18.0 / 15.4,
-//           145 20.0 / 17.3 *, 320 30.2 / 21.2;  16 385: 145 rows 27.3 / 19.7 *, 320 47.8 / 25.5;  32 001: 5 rows 46.2 / 14.2
-// So the sweeps would now do from about 5 000 entries on whatever the rows, and below that from some 200 rows.
+// The line was drawn with sweeps half as slow again as the present ones, and tests hold it there.  Calls back to back as the
+// kernels are now, element-wise / sweeps in us (4 tokens, i.e. 5 rows a sequence; * = calls to which the line gives the slower kernel):
+//     bf16  4 097 entries 80 rows 18.6 / 14.9 *, 320 25.1 / 16.4 *, 500 27.1 / 19.1;  8 201: 5 rows 21.8 / 14.2 *,
+//           100 21.7 / 16.0 *, 200 22.6 / 16.7 *, 320 32.9 / 19.0;  12 001: 20 rows 24.4 / 14.7, 145 24.2 / 17.3 *,
+//           200 28.9 / 17.4;  16 385: 145 28.2 / 17.2 *;  32 001: 5 rows 41.5 / 14.1, 320 116 / 30.0
+//     fp32  4 097: 5 rows 16.1 / 12.6 *, 180 16.3 / 14.5 *, 320 21.5 / 15.5 *, 640 29.6 / 18.4;  8 201: 40 rows 18.7 / 13.3,
+//           145 18.9 / 14.9 *, 320 28.0 / 17.8;  16 385: 145 rows 25.2 / 17.0 *, 320 48.0 / 23.2;  32 001: 5 rows 48.2 / 12.7
+// So the sweeps would now do at every length and number of rows that they can take.
 bool use_ragged_sweeps(const void* D, const void* grad, const void* hint, long long units, int V, int dtype) {
     const int vec = vec_elems(dtype);
     if (hint || option(SD_OPT_FORCE_GENERIC) != 0 || V % vec == 0 || V < 8 * kRegionVecs * vec ||
@@ -380,12 +380,12 @@ bool held_room(const WorkspaceLayout& L) { return L.slices > 0 || L.NRmax * size
 // back to back on inputs from HBM:
 //     1 sequence, 4 tokens, 32 000 fp32 16.6 / - / 8.8;  8, 5, 32 000 bf16 23.0 / - / 10.9;  1, 4, 128 256 bf16
 //     20.6 / - / 12.6, in clusters of 16 with one region a warp 14.8;  3, 2, 152 064 fp32 22.9 / - / 13.2;
-//     15 rows of 128 256 fp32 - / 18.6 / 13.5;  33 of 128 256 bf16 - / 21.4 / 15.8;  147 of 32 000 bf16 - / 22.4 / 16.3
+//     15 rows of 128 256 fp32 - / 17.2 / 12.7;  33 of 128 256 bf16 - / 19.2 / 16.0;  147 of 32 000 bf16 - / 19.5 / 16.3
 // Of clusters whose size is no power of two, one fewer than the device says is resident has its SMs at once: 45 rows of
 // 65 536 bf16 (clusters of 3, all of them resident by that count) 19.3, 42 rows 14.4; 12 of 152 064 fp32
 // (clusters of 10) 19.2, 9 rows 12.6.
 // A second round costs as much as the first.  Where there are sweeps they are faster then (42 rows of 100 000 bf16 23.7,
-// sweeps 21.2; 48 of 128 256 27.7 and 22.4); the cluster kernel is not (35.0).  `second`: two rounds are allowed.
+// sweeps 19.5; 48 of 128 256 27.7 and 19.4); the cluster kernel is not (35.0).  `second`: two rounds are allowed.
 // Options that only the cluster kernel has, off their defaults, choose the cluster kernel.
 bool use_held(DeviceState& d, int V, long long units, int dtype, bool second, HeldShape* h) {
     if (option(SD_OPT_CLUSTER) != 0 || option(SD_OPT_LAG) != -1 || option(SD_OPT_PREFETCH) != 0 ||
@@ -598,9 +598,9 @@ int choose_stream(DeviceState& d, int V, long long units, int dtype, int* G_out,
 //           24 000: 256 MB (10) 101 / 100, 307 MB (12) 116 / 119;  20 000: 191 MB (9) 81.6 / 79.3, 213 MB (10) 85.5 / 87.8;
 //           16 384 and below: faster at every size, 440 MB 179 / 170 (the cluster kernel's stages fit such rows badly)
 // The smallest calls go to sd_held_kernel first (use_held); of the others the sweeps are the faster ones however small
-// they are (us, cluster kernel / sweeps as they are now): 100 sequences, 2 tokens, 8 192 bf16 entries, 8 MB 19.6 / 19.5;
-// 64, 8, 1 000 fp32, 4 MB 23.1 / 16.2; 64, 4, 8 192 fp32, 19 MB 24.0 / 19.8; 8, 5, 128 256 bf16, 23 MB 35.0 / 22.4;
-// 16, 5, 50 304 fp32, 35 MB 28.2 / 23.2; 8, 5, 128 256 fp32, 45 MB 35.4 / 26.1.
+// they are (us, cluster kernel / sweeps as they are now): 100 sequences, 2 tokens, 8 192 bf16 entries, 8 MB 19.6 / 16.3;
+// 64, 8, 1 000 fp32, 4 MB 23.1 / 15.1; 64, 4, 8 192 fp32, 19 MB 24.0 / 17.3; 8, 5, 128 256 bf16, 23 MB 35.0 / 19.6;
+// 16, 5, 50 304 fp32, 35 MB 28.2 / 20.7; 8, 5, 128 256 fp32, 45 MB 35.4 / 23.2.
 // Options that only the cluster kernel has, off their defaults, choose the cluster kernel.
 // (Nor can the second sweep have more blocks than a grid: a billion rows of one vector.)
 bool use_sweeps(DeviceState& d, int dtype, double bytes, long long units, int V, int slices) {

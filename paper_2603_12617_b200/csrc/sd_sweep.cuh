@@ -1,6 +1,6 @@
 // The step as two sweeps over the logits, grids of small independent blocks: no cluster, no ring, nobody
 // waits for anybody.  A unit (sequence, row) is cut into `slices` items of the same number of sampling
-// regions, a block takes one item, a warp every eighth region of it, straight from global memory into
+// regions (towards the end of a sweep smaller ones), a block takes one item, a warp every eighth region of it, straight from global memory into
 // registers.  Three kernels, each of which comes in as the one before goes out:
 //
 //   sd_sweep_stats_kernel  softmax sums of every item to the workspace.
@@ -19,15 +19,20 @@
 // sd_stream_kernel reads every logit from HBM once, but its 28 consumer warps share one ring and all blocks
 // read at the same time and compute at the same time, so at bf16, where the exponentials take as long as
 // the reads, it moves 2.9 TB/s.  Step on 32 sequences, 8 draft tokens, 128 256 bf16 entries: 71.1 us there,
-// 58.7 us here (61.6 before the first kernel was launched programmatically and the maxima taken of packed bf16);
-// 64 sequences, 4 tokens, 151 936: 93.4 and 72.9 us; 8, 5, 128 256: 35.0 and 22.
+// 56.1 us here; 64 sequences, 4 tokens, 151 936: 93.4 and 69.7 us; 8, 5, 128 256: 35.0 and 19.6.  Of the 57.4 us that the first
+// of these took with items of one size, clock stamps of every block: first sweep 29.5, the last 8 with fewer and fewer
+// blocks; 4.5 until the second sweep works, 2 of them in the rows kernel; second sweep 24.  16 sequences, 5 tokens, 65 536 bf16
+// entries, 19.6 us: 8, 4, 5, and 4 for the draws.
 // The rule which of the two a call takes is use_sweeps (host).
 //
 // Tried and dropped, on the first of these: one persistent kernel whose warps take both passes of an item
 // from per-warp rings of bulk copies (82 us: many 1 KiB copies in flight slow each other down) or of
 // cp.async (99: their instructions), from registers in teams of blocks that wait for their row (71), and
-// from a queue that mixes first and second passes so that the second hits L2 (70: an SM has no more
-// instruction slots for both than for one).
+// from a queue that mixes first and second passes so that the second hits L2 (70; again, on the present loops, with
+// sequences opened for the second pass by a flag: 118.  Under load a round trip is 2 to 3 us, and partial, counter, row and
+// flag are ten of them: more logits lie between the passes than L2 keeps).  The first sweep of a group of sequences in one
+// grid with the second of the group before, a rows kernel between: 60.6 with one group, 68 with two, 80 with three.  L2
+// prefetches of a block's or a warp's next regions: 59 to 68.  Items in row order: 57.5.
 #pragma once
 
 #include "sd_kernels.cuh"
@@ -109,8 +114,8 @@ __device__ __forceinline__ PartialStats load_partial_cg(const PartialStats* p) {
 // Regions at the ends of a row, where a vector would reach into another row or out of the tensor, are read
 // and written entry by entry, out of line and with registers of their own: with one set for both, filled by a
 // function for the ends, every region went through local memory (13 sequences, 8 tokens, 110 593 fp32 entries 67.3 us,
-// 42 since; 122, 4, 119 177 302 and 206; 64, 4, 100 001 bf16 84.9 and 64).  16 sequences, 5 tokens, 50 257 bf16
-// entries: 25.3 us, against 91.6 us for the element-wise kernel, whose one block per row reads two bytes a lane.
+// 41 since; 122, 4, 119 177 302 and 202; 64, 4, 100 001 bf16 84.9 and 61).  16 sequences, 5 tokens, 50 257 bf16
+// entries: 19.8 us, against 91.6 us for the element-wise kernel, whose one block per row reads two bytes a lane.
 template <int DT> struct RowFrame {
     const typename Elem<DT>::type *rowT, *rowD;
     const uint4 *T16, *D16;      // vector 0 of the regions, aligned: up to a vector before the row
