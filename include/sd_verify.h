@@ -268,9 +268,9 @@ size_t sd_greedy_workspace_bytes(int B, int k);
  *   out_weights     [N] float     out  device, sums to 1
  *   out_status      [B] uint32    out  device SD_STATUS_BAD_ROW / SD_STATUS_TIMEOUT bits, or NULL
  *   workspace                     in   device scratch of SD_ENSEMBLE_SCRATCH_BYTES, aligned to 256
- *                                      bytes, or NULL for the library's own (of which bf16 calls that are
- *                                      not held on the chip take 16 bytes and up to 1 KiB a row and learner,
- *                                      for the two sweeps; with a workspace the cluster kernel serves them)
+ *                                      bytes, or NULL for the library's own; of sd_ensemble_workspace_bytes
+ *                                      bytes, if the two sweeps are to serve the call where they are the
+ *                                      faster (with less of it the cluster kernel does)
  *   stream                        in   cudaStream_t
  * Rows must be whole 16-byte vectors and every tensor 16-byte aligned (SD_ERR_ALIGN otherwise:
  * there is no element-wise path for this entry point).  Two kernels are enqueued -- one of the kernels
@@ -282,6 +282,9 @@ int sd_ensemble_feedback(const void* target_logits, const void* const* draft_log
                          const double* cum_loss_in, float* out_loss, void* const* out_grad,
                          double* out_round_loss, double* out_cum_loss, float* out_weights,
                          uint32_t* out_status, void* workspace, size_t workspace_bytes, void* stream);
+
+/* Bytes of scratch with which sd_ensemble_feedback may take any of its kernels; 0 if the shape is invalid. */
+size_t sd_ensemble_workspace_bytes(int B, int k, int V, int dtype, int n_learners);
 
 /*
  * sd_verify_error_feedback -- the step with the feedback restricted to the error position, the

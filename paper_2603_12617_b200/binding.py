@@ -76,6 +76,8 @@ def _load() -> ctypes.CDLL:
     lib.sd_ensemble_feedback.restype = I
     lib.sd_ensemble_feedback.argtypes = [P, P, I, ctypes.c_float, ctypes.c_float, I, I, I, I, P, P, P, P, P, P, P,
                                          P, Z, P]
+    lib.sd_ensemble_workspace_bytes.restype = Z
+    lib.sd_ensemble_workspace_bytes.argtypes = [I, I, I, I, I]
     lib.sd_lmhead_grad.restype = I
     lib.sd_lmhead_grad.argtypes = [P, P, I, I, I, P, P, P]
     lib.sd_hint_workspace_bytes.restype = Z
@@ -126,7 +128,8 @@ def _load_native():
     # the entry points of the library that was loaded above, in the order of its struct Library
     module.bind(*[ctypes.cast(fn, ctypes.c_void_p).value for fn in (
         _lib.sd_verify_feedback, _lib.sd_verify_feedback_bf16, _lib.sd_verify_greedy, _lib.sd_verify_error_feedback,
-        _lib.sd_verify_feedback_hint, _lib.sd_ensemble_feedback, _lib.sd_lmhead_grad, _lib.sd_vp_partial, _lib.sd_vp_finish, _lib.sd_vp_draw)])
+        _lib.sd_verify_feedback_hint, _lib.sd_ensemble_feedback, _lib.sd_lmhead_grad, _lib.sd_vp_partial, _lib.sd_vp_finish, _lib.sd_vp_draw,
+        _lib.sd_ensemble_workspace_bytes)])
     return module
 
 
@@ -487,9 +490,13 @@ def sd_ensemble_feedback(target_logits: torch.Tensor, draft_logits, temperature:
     dptr = (ctypes.c_void_p * N)(*[d.data_ptr() for d in draft_logits])
     gptr = (ctypes.c_void_p * N)(*[g.data_ptr() for g in out.grad]) if out.grad is not None else None
     with _OnDevice(dev):
+        # scratch of the call's own (allocated on the stream that uses it): calls may overlap on the GPU
+        nbytes = int(_lib.sd_ensemble_workspace_bytes(B, k, V, code, N))
+        with torch.cuda.stream(stream):
+            ws = torch.empty(nbytes, dtype=torch.uint8, device=dev) if nbytes else None
         rc = _lib.sd_ensemble_feedback(_ptr(target_logits), dptr, N, float(temperature), float(epsilon), B, k, V, code,
                                        _ptr(cum_loss), _ptr(out.loss), gptr, _ptr(out.round_loss),
-                                       _ptr(out.cum_loss), _ptr(out.weights), _ptr(out.status), None, 0,
+                                       _ptr(out.cum_loss), _ptr(out.weights), _ptr(out.status), _ptr(ws), nbytes,
                                        _stream_ptr(stream))
     if rc != 0:
         raise SdVerifyError(rc, "sd_ensemble_feedback")

@@ -1051,6 +1051,11 @@ int launch_ensemble_sweeps(const Params& P, EnsembleSweep S, const HedgeArgs& H,
 }
 }  // namespace
 extern "C" {
+size_t sd_ensemble_workspace_bytes(int B, int k, int V, int dtype, int n_learners) {
+    if ((dtype != SD_DTYPE_F32 && dtype != SD_DTYPE_BF16) || !shape_ok(B, k, V) || n_learners < 1 || n_learners > SD_MAX_LEARNERS) return 0;
+    return dtype == SD_DTYPE_BF16 ? ensemble_layout(B, k, V, dtype, n_learners).total : SD_ENSEMBLE_SCRATCH_BYTES;
+}
+
 int sd_ensemble_feedback(const void* target_logits, const void* const* draft_logits, int n_learners,
                          float temperature, float epsilon, int B, int k, int V, int dtype,
                          const double* cum_loss_in, float* out_loss, void* const* out_grad,
@@ -1083,8 +1088,8 @@ int sd_ensemble_feedback(const void* target_logits, const void* const* draft_log
     HeldShape held;
     const bool holds = use_held(*d, V, (long long)B * k * n_learners, dtype, true, &held);
     const EnsembleLayout L = ensemble_layout(B, k, V, dtype, n_learners);
-    // (the sweeps' scratch is the library's: what a caller brings is a flag word)
-    const bool sweeps = !holds && !ws && use_ensemble_sweeps(dtype, (long long)B * k, L.slices) && (d->ws_bytes >= L.total || !capturing(st));
+    const bool sweeps = !holds && use_ensemble_sweeps(dtype, (long long)B * k, L.slices) &&
+                        (ws ? workspace_bytes >= L.total : d->ws_bytes >= L.total || !capturing(st));
     if (!ws) {
         Head head;                 // (cleared below; the flag word sits where other entry points expect zeros)
         const size_t need = sweeps ? L.total : SD_ENSEMBLE_SCRATCH_BYTES;

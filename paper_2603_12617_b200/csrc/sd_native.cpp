@@ -32,6 +32,7 @@ struct Library {
     decltype(&sd_vp_partial) vp_partial = nullptr;
     decltype(&sd_vp_finish) vp_finish = nullptr;
     decltype(&sd_vp_draw) vp_draw = nullptr;
+    decltype(&sd_ensemble_workspace_bytes) ensemble_bytes = nullptr;
 } lib;
 
 constexpr int kVpRecordBytes = 48;
@@ -260,11 +261,15 @@ PyObject* ensemble(PyObject*, PyObject* const* a, Py_ssize_t n) {
         g[i] = s.make({B, k, V}, T->scalar_type());
         G[i] = ptr(g[i]);
     }
+    // (scratch of the call's own: calls may overlap on the GPU)
+    const size_t bytes = lib.ensemble_bytes((int)B, (int)k, (int)V, code, (int)N);
+    const at::Tensor ws = bytes ? s.make({(int64_t)bytes}, at::kByte) : at::Tensor();
+    void* const wp = bytes ? ptr(ws) : nullptr;
     uint32_t* const sp = status.defined() ? (uint32_t*)ptr(status) : nullptr;
     void* const st = s.stream();
     const int rc = unlocked(lib.ensemble, ptr(*T), D, (int)N, tau, eps, (int)B, (int)k, (int)V, code, cum_in, (float*)ptr(loss),
                             grad ? G : nullptr,
-                            (double*)ptr(mean), (double*)ptr(cum), (float*)ptr(weights), sp, nullptr, 0, st);
+                            (double*)ptr(mean), (double*)ptr(cum), (float*)ptr(weights), sp, wp, bytes, st);
     PyObject* grads = Py_None;
     if (grad) {
         grads = PyList_New(N);
@@ -387,7 +392,7 @@ PyObject* vp_draw(PyObject*, PyObject* const* a, Py_ssize_t n) {
 PyObject* bind(PyObject*, PyObject* const* a, Py_ssize_t n) {
     void** const slots[] = {(void**)&lib.step_f32, (void**)&lib.step_bf16, (void**)&lib.greedy,    (void**)&lib.errors,
                             (void**)&lib.hint,     (void**)&lib.ensemble,   (void**)&lib.lmhead,
-                            (void**)&lib.vp_partial, (void**)&lib.vp_finish, (void**)&lib.vp_draw};
+                            (void**)&lib.vp_partial, (void**)&lib.vp_finish, (void**)&lib.vp_draw, (void**)&lib.ensemble_bytes};
     constexpr Py_ssize_t want = sizeof slots / sizeof slots[0];
     if (n != want) {
         PyErr_SetString(PyExc_TypeError, "bind: wrong number of entry points");

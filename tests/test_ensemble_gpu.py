@@ -323,3 +323,47 @@ def test_two_sweeps_in_a_graph(binding):
         assert torch.equal(again.tokens, step.tokens) and torch.equal(again.grad_draft, step.grad_draft)
         assert torch.equal(out.loss, want.loss) and torch.equal(out.weights, want.weights)
         assert all(torch.equal(a, b) for a, b in zip(out.grad, want.grad))
+
+
+def test_two_sweeps_on_two_streams_at_once(binding):
+    """Calls of the binding bring scratch of their own: they may overlap on the GPU."""
+    cfg = synth.custom_config(60, 3, 20000, dtype="bf16", tau=0.9, index=132)
+    inp = synth.make_inputs(cfg)
+    Ds = synth.ensemble_drafts(inp, 3)
+    T, dDs = dev(inp.target_logits), [dev(d) for d in Ds]
+    want = [binding.sd_ensemble_feedback(T, list(d), inp.tau, EPS) for d in (dDs, dDs[::-1])]
+    torch.cuda.synchronize()
+    streams = [torch.cuda.Stream(), torch.cuda.Stream()]
+    got = [[], []]
+    for _ in range(6):
+        for i, d in enumerate((dDs, dDs[::-1])):
+            with torch.cuda.stream(streams[i]):
+                got[i].append(binding.sd_ensemble_feedback(T, list(d), inp.tau, EPS))
+                assert binding.sd_launch_info()["threads"] == 256
+    torch.cuda.synchronize()
+    for w, outs in zip(want, got):
+        for o in outs:
+            assert torch.equal(o.loss, w.loss) and torch.equal(o.weights, w.weights) and all(torch.equal(a, b) for a, b in zip(o.grad, w.grad))
+
+
+def test_a_workspace_without_room_for_the_sweeps_takes_the_cluster_kernel(binding):
+    """Callers that bring a flag word are served as before, and the library's own scratch takes the sweeps."""
+    import ctypes
+    cfg = synth.custom_config(60, 3, 20000, dtype="bf16", tau=0.9, index=133)
+    inp = synth.make_inputs(cfg)
+    Ds = synth.ensemble_drafts(inp, 3)
+    T, dDs = dev(inp.target_logits), [dev(d) for d in Ds]
+    want = binding.sd_ensemble_feedback(T, dDs, inp.tau, EPS)
+    need = binding._lib.sd_ensemble_workspace_bytes(cfg.B, cfg.k, cfg.V, binding.SD_DTYPE_BF16, 3)
+    dptr = (ctypes.c_void_p * 3)(*[d.data_ptr() for d in dDs])
+    for nbytes, threads in ((256, 1024), (need - 256, 1024), (need, 256), (0, 256)):
+        ws = torch.full((nbytes,), 0xA5, dtype=torch.uint8, device="cuda")
+        loss = torch.empty_like(want.loss)
+        small = [torch.empty(3, dtype=torch.float64, device="cuda") for _ in range(2)] + [torch.empty(3, device="cuda")]
+        rc = binding._lib.sd_ensemble_feedback(T.data_ptr(), dptr, 3, float(inp.tau), EPS, cfg.B, cfg.k, cfg.V, binding.SD_DTYPE_BF16, None,
+                                               loss.data_ptr(), None, *[t.data_ptr() for t in small], None,
+                                               ws.data_ptr() if nbytes else None, nbytes, None)
+        torch.cuda.synchronize()
+        assert rc == 0 and binding.sd_launch_info()["threads"] == threads
+        err = (loss - want.loss).abs()
+        assert torch.equal(loss, want.loss) if threads == 256 else (err <= 1e-4 * want.loss.abs() + 4e-7).all()
