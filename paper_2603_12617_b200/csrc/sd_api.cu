@@ -1097,10 +1097,10 @@ int sd_ensemble_feedback(const void* target_logits, const void* const* draft_log
         if (rc != SD_OK) return rc;
         ws = static_cast<unsigned char*>(d->ws);
     }
-    if (!sweeps) {
-        SD_CUDA(cudaMemsetAsync(ws, 0, SD_ENSEMBLE_SCRATCH_BYTES, st));
-        if (out_status) SD_CUDA(cudaMemsetAsync(out_status, 0, (size_t)B * 4, st));
-    }
+    // (held rows wait for nobody and want no flag word; with one cleared before every call, 2 sequences, 5 tokens, 4 learners of
+    // 97 472 bf16 entries took 16.3 us, 15.7 without)
+    if (!sweeps && !holds) SD_CUDA(cudaMemsetAsync(ws, 0, SD_ENSEMBLE_SCRATCH_BYTES, st));
+    if (!sweeps && out_status) SD_CUDA(cudaMemsetAsync(out_status, 0, (size_t)B * 4, st));
 
     Params P;
     memset(&P, 0, sizeof P);
@@ -1144,7 +1144,7 @@ int sd_ensemble_feedback(const void* target_logits, const void* const* draft_log
     }
     if (rc != SD_OK) return rc;
     SD_CUDA(launch_following(sd_hedge_kernel, dim3(1), kHedgeThreads, st, (const float*)out_loss, n_learners, (long long)B * k, (double)epsilon,
-                             cum_loss_in, out_round_loss, out_cum_loss, out_weights, (const uint32_t*)P.sticky, out_status, B));
+                             cum_loss_in, out_round_loss, out_cum_loss, out_weights, (const uint32_t*)(holds ? nullptr : P.sticky), out_status, B));
     tl_info[0] = 3; tl_info[5] = 2;
     return SD_OK;
 }

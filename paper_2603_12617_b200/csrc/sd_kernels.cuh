@@ -1085,8 +1085,8 @@ __global__ void __launch_bounds__(kHedgeThreads) sd_hedge_kernel(const float* lo
         const int i = min(lane, N - 1);
         hedge_weights(N, ((part[i][0] + part[i][1]) + (part[i][2] + part[i][3])) / (double)per, eps, cum_in, round_loss, cum_out, weights);
     }
-    // a bounded wait gave up somewhere in the feedback kernel: nothing of this round is valid
-    if (status && *sticky != 0)
+    // a bounded wait gave up somewhere in the feedback kernel (null: it has none): nothing of this round is valid
+    if (status && sticky && *sticky != 0)
         for (int b = tid; b < B; b += kHedgeThreads) atomicOr(status + b, kStatusTimeout);
 }
 
