@@ -506,6 +506,76 @@ __device__ __noinline__ double block_sums_before(double mine, double* sums, doub
     return before + (incl - mine);
 }
 
+// Where a rejection leaves no residual mass: an entry drawn from p_n, in every thread.  There are no region masses of p_n, so
+// a warp adds up an eighth of the row's regions and the warp into whose share the draw falls takes them once more; sums,
+// prefixes and totals in fp64, from the entries on.  (Four entries at a time, taken again where they are searched: the
+// registers are those of the kernel's loops.)
+template <int DT>
+__device__ __noinline__ int sweep_draw_from_p(const Params& P, const RowConst& rc, size_t offT, double u, int lead) {
+    using E = Elem<DT>;
+    constexpr int kEntries = kRegionVecs * E::VEC, PER = kEntries / 32;
+    __shared__ double share[kSweepWarps];
+    __shared__ int drawn;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int per = (P.NR + kSweepWarps - 1) / kSweepWarps, j0 = min(P.NR, warp * per), j1 = min(P.NR, j0 + per);
+    const auto mass = [&](int v) {
+        return v >= 0 && v < P.V && SD_IN(v, P.V, 24) ? (double)prob_elem(E::load(P.T, offT + v), P.c, rc) : 0.0;
+    };
+    // a lane's entries of region j
+    const auto lane_sum = [&](int j) {
+        const int v0 = j * kEntries + lane * PER - lead;
+        double s = 0.0;
+#pragma unroll 4
+        for (int e = 0; e < PER; ++e) s += mass(v0 + e);
+        return s;
+    };
+    double mine = 0.0;
+    for (int j = j0; j < j1; ++j) mine += warp_sum(lane_sum(j));
+    if (threadIdx.x == 0) drawn = 0;
+    if (lane == 0) share[warp] = mine;
+    __syncthreads();
+    // the first share whose end exceeds t, or (rounding pushed t to the total) the last one with mass
+    double total = 0.0, before = 0.0, run = 0.0;
+    for (int w = 0; w < kSweepWarps; ++w) total += share[w];
+    const double t = u * total;
+    int owner = -1;
+    bool found = false;
+#pragma unroll 1
+    for (int w = 0; w < kSweepWarps && !found; ++w) {
+        if (share[w] > 0.0) { owner = w; before = run; found = run + share[w] > t; }
+        run += share[w];
+    }
+    if (warp == owner && isfinite(total)) {
+        int at = -1;                                     // the first entry behind which the sum exceeds t, or the last with mass
+        found = false;
+        for (int j = j0; j < j1 && !found; ++j) {
+            const double s = lane_sum(j), incl = warp_inclusive_scan(s);
+            const int v0 = j * kEntries + lane * PER - lead;
+            double sum = before + (incl - s);
+            int first = 0x7fffffff, last = -1;
+#pragma unroll 1
+            for (int e = 0; e < PER; ++e) {
+                const double m = mass(v0 + e);
+                sum += m;
+                if (!(m > 0.0)) continue;
+                last = v0 + e;
+                if (first == 0x7fffffff && sum > t) first = v0 + e;
+            }
+#pragma unroll
+            for (int off = 16; off > 0; off >>= 1) {
+                first = min(first, __shfl_xor_sync(0xffffffffu, first, off));
+                last = max(last, __shfl_xor_sync(0xffffffffu, last, off));
+            }
+            found = first != 0x7fffffff;
+            at = found ? first : max(at, last);
+            before += __shfl_sync(0xffffffffu, incl, 31);
+        }
+        if (lane == 0) drawn = max(at, 0);
+    }
+    __syncthreads();
+    return drawn;
+}
+
 // The extra token of a sequence, and what the sequence puts out, by the block that brought the last item of the row that
 // it is drawn from, `unit`, once that row's region masses are all there.  Its end is the call's where the sweep is short, and what it consists of is
 // round trips and sums that wait for one another; so a block does it, a region or two to a thread and then an entry or
@@ -525,7 +595,7 @@ __device__ __noinline__ void sweep_draw(const Params& P, int unit, int lead) {
     const int b = unit / (k + 1), n = unit - b * (k + 1);
     const bool bonus = n == k;
     if (!SD_IN(unit, P.B * (k + 1), 23)) return;
-    float* const rs = P.region_sums + (size_t)unit * NR;
+    const float* const rs = P.region_sums + (size_t)unit * NR;
     const size_t offT = (size_t)unit * P.V, offD = (size_t)(b * k + (bonus ? 0 : n)) * P.V;
     // (everything that depends on nothing, at once)
     const float4 rcv = __ldcg(reinterpret_cast<const float4*>(P.rowc + unit));
@@ -539,39 +609,20 @@ __device__ __noinline__ void sweep_draw(const Params& P, int unit, int lead) {
         last_mass = -1;
     }
     const int per = (NR + kSweepThreads - 1) / kSweepThreads, j0 = tid * per, j1 = min(NR, j0 + per);
-    int mode = bonus ? 1 : 0, y = 0;
-    double all, t;
-    for (;;) {
-        // (the first two regions of a thread stay in registers: rows of up to 512 regions)
-        float held[2];
+    const int mode = bonus ? 1 : 0;
+    int y = 0;
+    // (the first two regions of a thread stay in registers: rows of up to 512 regions)
+    float held[2];
 #pragma unroll
-        for (int q = 0; q < 2; ++q) held[q] = j0 + q < j1 ? __ldcg(rs + j0 + q) : 0.f;
-        double mine = (double)held[0] + (double)held[1];
-        for (int j = j0 + 2; j < j1; ++j) mine += (double)__ldcg(rs + j);
-        const double before = block_sums_before(mine, sums[0], &all);
-        t = uk * all;
-        if (!(all > 0.0) || !isfinite(all)) {                      // (the same for every thread)
-            if (mode != 0) {
-                if (bonus) flags |= SD_STATUS_BAD_ROW;
-                break;
-            }
-            // a rejection whose residual has no mass: the masses of p_n in their place
-            flags |= SD_STATUS_ZERO_RESIDUAL;
-            mode = 2;
-            const int lane = tid & 31;
-            for (int j = tid >> 5; j < NR; j += kSweepWarps) {
-                float m = 0.f;
-                for (int e = lane; e < kEntries; e += 32) {
-                    const int v = j * kEntries + e - lead;
-                    if (v >= 0 && v < P.V) m += prob_elem(E::load(P.T, offT + v), P.c, rc);
-                }
-#pragma unroll
-                for (int off = 16; off > 0; off >>= 1) m += __shfl_xor_sync(0xffffffffu, m, off);
-                if (lane == 0) rs[j] = m;
-            }
-            __syncthreads();
-            continue;
-        }
+    for (int q = 0; q < 2; ++q) held[q] = j0 + q < j1 ? __ldcg(rs + j0 + q) : 0.f;
+    double all, mine = (double)held[0] + (double)held[1];
+    for (int j = j0 + 2; j < j1; ++j) mine += (double)__ldcg(rs + j);
+    const double before = block_sums_before(mine, sums[0], &all);
+    const double t = uk * all;
+    if (!(all > 0.0) || !isfinite(all)) {                          // (the same for every thread)
+        flags |= bonus ? SD_STATUS_BAD_ROW : SD_STATUS_ZERO_RESIDUAL;
+        if (!bonus) y = sweep_draw_from_p<DT>(P, rc, offT, uk, lead);
+    } else {
         // the first region whose running sum exceeds t, or (rounding pushed u * R to the total) the last with mass
         if (mine > 0.0 && before + mine > t) atomicMin(&owner[0], tid);
         if (mine > 0.0) atomicMax(&last_mass, tid);
@@ -625,7 +676,6 @@ __device__ __noinline__ void sweep_draw(const Params& P, int unit, int lead) {
         if (tid == 0 && last_mass < 0) found = 0;
         __syncthreads();
         y = found;
-        break;
     }
     if (tid == 0) {
         P.accept_len[b] = n;
@@ -780,7 +830,6 @@ sd_sweep_grad_kernel(const __grid_constant__ Params P, const __grid_constant__ S
     if (!is_last) return;
     if ((HINT || S.all_rows) && !ur.bonus && warp == 0) sweep_row_sums<HINT>(P, S, unit, ur.d_row);
     if (!draws) return;
-    if (S.all_rows) __syncthreads();                  // (the draw may put other masses in place of the row's)
     sweep_draw<DT>(P, unit, RAGGED ? row_frame<DT>(P, ur).lead : 0);
 }
 
