@@ -117,12 +117,12 @@ int sweep_regions(long long units, int V, int dtype) {
 // Room for that many items, never less for more units or longer rows: a buffer that was sized for the
 // largest batch does for every smaller one.  (sweep_regions takes steps of eight, with which units * slices
 // alone goes up and down: 11 sequences of 6 x 50 257 bf16 entries have 858 items, 14 have 588.)  Below four regions per
-// warp there are at most 9/8 of 888 items and one more per unit.
-size_t sweep_item_room(size_t units, int V, int dtype) {
+// warp, where items are so large that `blocks` of them go at a time, there are at most 9/8 of that many and one more per unit.
+size_t sweep_item_room(size_t units, int V, int dtype, size_t blocks = 888) {
     const int vec = vec_elems(dtype);
     const size_t R = ((size_t)V + 2 * vec - 2) / vec / kRegionVecs + 1;       // at least sweep_row_regions of any V up to this one
     const auto most = [&](size_t regions) { const size_t s = (R + regions - 1) / regions; return units * (s < kMaxSlices ? s : kMaxSlices); };
-    const size_t few = most(kSweepWarps) < units + 1000 ? most(kSweepWarps) : units + 1000, many = most(4 * kSweepWarps);
+    const size_t below = units + blocks + blocks / 8 + 1, few = most(kSweepWarps) < below ? most(kSweepWarps) : below, many = most(4 * kSweepWarps);
     return few > many ? few : many;
 }
 
@@ -1005,7 +1005,9 @@ EnsembleLayout ensemble_layout(int B, int k, int V, int dtype, int n_learners) {
     L.slices = (int)(s > kMaxSlices ? kMaxSlices : s);
     L.rowc = kAlign;
     L.part = align_up(L.rowc + rows * sizeof(RowConst), kAlign);
-    L.total = align_up(L.part + rows * L.slices * sizeof(PartialStats), kAlign);
+    // (the room does for every smaller call, as that of the step's sweeps does: 8 tokens of 128 256 entries have 640 items with
+    // 5 sequences and 528 with 6)
+    L.total = align_up(L.part + n_learners * sweep_item_room((size_t)positions, V, dtype, 592) * sizeof(PartialStats), kAlign);
     return L;
 }
 
