@@ -1092,14 +1092,15 @@ int sd_ensemble_feedback(const void* target_logits, const void* const* draft_log
     const EnsembleLayout L = ensemble_layout(B, k, V, dtype, n_learners);
     const bool sweeps = !holds && use_ensemble_sweeps(dtype, (long long)B * k, L.slices) &&
                         (ws ? workspace_bytes >= L.total : d->ws_bytes >= L.total || !capturing(st));
-    if (!ws) {
-        Head head;                 // (cleared below; the flag word sits where other entry points expect zeros)
+    if (!ws && !holds) {
+        // (the cluster kernel's flag word is cleared below and the sweeps write wherever they like: nothing is known of the head any more)
+        Head head;
         const size_t need = sweeps ? L.total : SD_ENSEMBLE_SCRATCH_BYTES;
         rc = own_scratch(d, need, need, st, &head);
         if (rc != SD_OK) return rc;
         ws = static_cast<unsigned char*>(d->ws);
     }
-    // (held rows wait for nobody and want no flag word; with one cleared before every call, 2 sequences, 5 tokens, 4 learners of
+    // (held rows wait for nobody and want no scratch; with a flag word cleared before every call, 2 sequences, 5 tokens, 4 learners of
     // 97 472 bf16 entries took 16.3 us, 15.7 without)
     if (!sweeps && !holds) SD_CUDA(cudaMemsetAsync(ws, 0, SD_ENSEMBLE_SCRATCH_BYTES, st));
     if (!sweeps && out_status) SD_CUDA(cudaMemsetAsync(out_status, 0, (size_t)B * 4, st));
@@ -1113,7 +1114,7 @@ int sd_ensemble_feedback(const void* target_logits, const void* const* draft_log
     P.inv_tau = 1.0 / (double)temperature;
     P.loss = out_loss;
     P.status = out_status;
-    P.sticky = reinterpret_cast<uint32_t*>(ws);
+    P.sticky = holds ? nullptr : reinterpret_cast<uint32_t*>(ws);
     P.learners = n_learners;
     P.wait_polls = wait_polls();
     for (int n = 0; n < n_learners; ++n) {
@@ -1146,7 +1147,7 @@ int sd_ensemble_feedback(const void* target_logits, const void* const* draft_log
     }
     if (rc != SD_OK) return rc;
     SD_CUDA(launch_following(sd_hedge_kernel, dim3(1), kHedgeThreads, st, (const float*)out_loss, n_learners, (long long)B * k, (double)epsilon,
-                             cum_loss_in, out_round_loss, out_cum_loss, out_weights, (const uint32_t*)(holds ? nullptr : P.sticky), out_status, B));
+                             cum_loss_in, out_round_loss, out_cum_loss, out_weights, (const uint32_t*)P.sticky, out_status, B));
     tl_info[0] = 3; tl_info[5] = 2;
     return SD_OK;
 }

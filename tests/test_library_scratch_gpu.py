@@ -1,6 +1,9 @@
 """The library's own scratch (calls without a workspace) under CUDA graphs and after a wait that ran out:
 what the host believes of its contents must hold whenever a call runs, not only when it was issued.
 Every answer is compared, bit for bit, with the call on a fresh caller workspace."""
+import ctypes
+import types
+
 import pytest
 import torch
 
@@ -147,4 +150,41 @@ def test_a_captured_call_keeps_its_scratch_when_a_larger_call_needs_more(binding
     call.check("replay on the buffer that was outgrown")
     larger.run("larger again")
     assert all(bool((f == 0xFF).all()) for f in fill)
+    del graph
+
+
+class EnsembleCall(Call):
+    """An ensemble on the library's scratch (the Python wrapper brings its own), two learners."""
+
+    def __init__(self, binding, shape, index):
+        B, k, V, dtype = shape
+        inp = synth.make_inputs(synth.custom_config(B=B, k=k, V=V, dtype=dtype, tau=0.9, index=index))
+        T, D, _, _ = to_device(inp)
+        Ds = [D, D.roll(1, 0).contiguous()]
+        o = binding.sd_ensemble_feedback(T, Ds, inp.tau, 10.0, want_status=True)
+        torch.cuda.synchronize()
+        self.out = types.SimpleNamespace(loss=o.loss, grad0=o.grad[0], grad1=o.grad[1], round_loss=o.round_loss, cum_loss=o.cum_loss,
+                                         weights=o.weights, status=o.status)
+        self.want = {n: t.clone() for n, t in vars(self.out).items()}
+        dptr, gptr = ((ctypes.c_void_p * 2)(*[t.data_ptr() for t in ts]) for ts in (Ds, o.grad))
+
+        def fn(keep=(T, Ds, dptr, gptr)):
+            rc = binding._lib.sd_ensemble_feedback(T.data_ptr(), dptr, 2, float(inp.tau), 10.0, B, k, V, binding._dtype_code(T), None,
+                                                   o.loss.data_ptr(), gptr, o.round_loss.data_ptr(), o.cum_loss.data_ptr(),
+                                                   o.weights.data_ptr(), o.status.data_ptr(), None, 0,
+                                                   torch.cuda.current_stream().cuda_stream)
+            assert rc == 0
+        self.fn = fn
+
+
+def test_a_held_ensemble_wants_no_scratch(binding):
+    """Rows on the chip: nothing to allocate, so there need be none when the call is captured."""
+    call = EnsembleCall(binding, (2, 3, 8192, "bf16"), 116)
+    assert binding.sd_launch_info()["threads"] == 512
+    call.run("eager")
+    binding.sd_release_cached_buffers()
+    graph = call.capture()
+    call.forget()
+    graph.replay()
+    call.check("replay")
     del graph
