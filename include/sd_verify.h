@@ -275,7 +275,8 @@ size_t sd_greedy_workspace_bytes(int B, int k);
  * Rows must be whole 16-byte vectors and every tensor 16-byte aligned (SD_ERR_ALIGN otherwise:
  * there is no element-wise path for this entry point).  Two kernels are enqueued -- one of the kernels
  * of sd_verify_feedback over (sequence, row, learner) units (the persistent one, or that which holds
- * the rows), then a one-block reduction -- or three, the two sweeps (five with more than four learners).
+ * the rows), then a one-block reduction -- or three, the two sweeps; with more than four learners five, or four if
+ * no gradient of the later half of them is wanted.
  */
 int sd_ensemble_feedback(const void* target_logits, const void* const* draft_logits, int n_learners,
                          float temperature, float epsilon, int B, int k, int V, int dtype,
@@ -454,8 +455,8 @@ long long sd_get_option(int option_id);
  * thread was launched: path (0 = generic, 1 = fast path (one kernel: cluster kernel or, with 512 threads a
  * block, held rows; three: the two sweeps), 2 = greedy verification, 3 = ensemble feedback, 4 = error-position feedback, 5 = output-layer gradient,
  * 6 = vocabulary-parallel step), cluster size, threads per block, dynamic shared memory per block, blocks
- * launched, kernels launched (sd_verify_feedback_host: of all its slices).  Any pointer may be NULL.
- * Diagnostic only.
+ * launched (of the two sweeps: by the first), kernels launched (sd_verify_feedback_host: of all its slices).
+ * Any pointer may be NULL.  Diagnostic only.
  */
 void sd_launch_info(int* path, int* cluster_size, int* threads, int* smem_bytes, int* blocks,
                     int* kernels);

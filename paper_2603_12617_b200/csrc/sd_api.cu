@@ -445,6 +445,7 @@ int launch_sweeps_of(const Params& P, const Sweep& S, long long units, bool all,
     const long long rows = (long long)P.B * P.k, fine = FINE2 ? S.fine_rows : 0;
     const unsigned second = (unsigned)S.draw_blocks + (all ? (unsigned)((rows - fine) * S.slices + fine * S.fine_slices) : 0u);
     SD_CUDA(launch_following(sd_sweep_grad_kernel<DT, MODE, RAGGED, FINE2>, dim3(second), kSweepThreads, stream, P, S));
+    tl_info[4] = (int)(first.x * first.y);
     return SD_OK;
 }
 
@@ -501,8 +502,7 @@ int launch_sweeps(const Params& P, Sweep& S, long long units, int dtype, cudaStr
         rc = dtype == SD_DTYPE_F32 ? launch_sweeps_of<SD_DTYPE_F32, MODE, RAGGED, false>(P, S, units, all, stream)
                                    : launch_sweeps_of<SD_DTYPE_BF16, MODE, RAGGED, false>(P, S, units, all, stream);
     if (rc != SD_OK) return rc;
-    tl_info[0] = 1; tl_info[1] = 1; tl_info[2] = kSweepThreads; tl_info[3] = 0;
-    tl_info[4] = (int)(units * S.slices); tl_info[5] = 3;
+    tl_info[0] = 1; tl_info[1] = 1; tl_info[2] = kSweepThreads; tl_info[3] = 0; tl_info[5] = 3;
     return SD_OK;
 }
 
@@ -1016,12 +1016,14 @@ int launch_ensemble_group(const Params& P, const EnsembleSweep& S, const HedgeAr
     const long long positions = (long long)P.B * P.k;
     if (!second) {
         SD_CUDA(launch_following(sd_ensemble_stats_kernel<DT, NL>, dim3((unsigned)positions, (unsigned)S.slices), kSweepThreads, stream, P, S));
+        ++tl_info[5];
         return SD_OK;
     }
     bool wanted = false;
     for (int n = 0; n < NL; ++n) wanted = wanted || P.Gn[S.n0 + n] != nullptr;
     if (!wanted && S.n0 != 0) return SD_OK;
     SD_CUDA(launch_following(sd_ensemble_grad_kernel<DT, NL>, dim3(1u + (wanted ? (unsigned)(positions * S.slices) : 0u)), kSweepThreads, stream, P, S, H));
+    ++tl_info[5];
     return SD_OK;
 }
 
@@ -1030,6 +1032,7 @@ int launch_ensemble_sweeps(const Params& P, EnsembleSweep S, const HedgeArgs& H,
     // groups of learners of the same size or one less
     const int groups = (P.learners + kEnsembleGroup - 1) / kEnsembleGroup;
     S.kept = (80u << 20) / (unsigned)(S.regions * kRegionVecs * 16 * ((P.learners + groups - 1) / groups + 1));
+    tl_info[5] = 0;
     for (int second = 0; second < 2; ++second) {
         for (int g = 0; g < groups; ++g) {
             S.n0 = P.learners * g / groups;
@@ -1045,10 +1048,11 @@ int launch_ensemble_sweeps(const Params& P, EnsembleSweep S, const HedgeArgs& H,
         if (!second) {
             const long long rows = (long long)P.B * P.k * P.learners;
             SD_CUDA(launch_following(sd_ensemble_rows_kernel, dim3((unsigned)((rows + kSweepWarps - 1) / kSweepWarps)), kSweepThreads, stream, P, S));
+            ++tl_info[5];
         }
     }
     tl_info[1] = 1; tl_info[2] = kSweepThreads; tl_info[3] = 0;
-    tl_info[4] = (int)(P.B * P.k * S.slices); tl_info[5] = 2 * groups + 1;
+    tl_info[4] = (int)(P.B * P.k * S.slices);
     return SD_OK;
 }
 }  // namespace

@@ -367,3 +367,15 @@ def test_a_workspace_without_room_for_the_sweeps_takes_the_cluster_kernel(bindin
         assert rc == 0 and binding.sd_launch_info()["threads"] == threads
         err = (loss - want.loss).abs()
         assert torch.equal(loss, want.loss) if threads == 256 else (err <= 1e-4 * want.loss.abs() + 4e-7).all()
+
+
+def test_two_sweeps_count_their_kernels(binding):
+    """No second sweep of a group of learners without a gradient; the first group's does the round in any case."""
+    cfg = synth.custom_config(40, 3, 20000, dtype="bf16", tau=0.9, index=134)
+    inp = synth.make_inputs(cfg)
+    T, Ds = dev(inp.target_logits), [dev(d) for d in synth.ensemble_drafts(inp, 5)]
+    for N, grad, kernels in ((4, True, 3), (4, False, 3), (5, True, 5), (5, False, 4)):
+        binding.sd_ensemble_feedback(T, Ds[:N], inp.tau, EPS, want_grad=grad)
+        info = binding.sd_launch_info()
+        assert (info["threads"], info["kernels"]) == (256, kernels)
+    torch.cuda.synchronize()
