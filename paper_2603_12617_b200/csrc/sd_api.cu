@@ -440,8 +440,9 @@ int launch_sweeps_of(const Params& P, const Sweep& S, long long units, bool all,
                             : dim3((unsigned)units, (unsigned)S.slices);
     SD_CUDA(launch_following(sd_sweep_stats_kernel<DT, RAGGED, FINE>, first, kSweepThreads, stream, P, S));
     SD_CUDA(launch_following(sd_sweep_rows_kernel<DT>, dim3((unsigned)P.B), rows_threads(P.k), stream, P, S));
-    // the rows that are drawn from, then (if anything of them is wanted) all pair rows; the hint error is summed by items of one size
-    constexpr bool FINE2 = FINE && MODE != kSweepHint;
+    // the rows that are drawn from, then (if anything of them is wanted) all pair rows; the hint error is summed by items of one
+    // size, and the error feedback has nothing but the rows that are drawn from
+    constexpr bool FINE2 = FINE && MODE == kSweepStepMode;
     const long long rows = (long long)P.B * P.k, fine = FINE2 ? S.fine_rows : 0;
     const unsigned second = (unsigned)S.draw_blocks + (all ? (unsigned)((rows - fine) * S.slices + fine * S.fine_slices) : 0u);
     SD_CUDA(launch_following(sd_sweep_grad_kernel<DT, MODE, RAGGED, FINE2>, dim3(second), kSweepThreads, stream, P, S));
