@@ -496,6 +496,12 @@ int launch_sweeps(const Params& P, Sweep& S, long long units, int dtype, cudaStr
         }
     }
     S.draw_blocks = P.B * S.draw_slices;
+    // Where all sequences draw at about the same time, instructions are what a draw costs, and half a block has the fewer; alone a
+    // whole block is the sooner done.  Step, whole / half blocks / the warp that drew once, us: 500 sequences, 8 tokens, 2 048 bf16 entries
+    // 32.8 / 31.8 / 32.1, 800, 1, 8 192 28.5 / 27.7 / 27.2, 400, 4, 8 192 fp32 45.0 / 44.1 / 46.2, 256, 4, 16 384 55.9 / 55.6 / 56.0,
+    // 100, 2, 8 192 16.1 / 15.4 / 16.9; 64, 4, 151 936 bf16, error feedback 49.2 / 49.6 / 51.2, 16, 5, 50 257 19.3 / 19.6 / 25.1, 12, 4, 128 256
+    // fp32 21.5 / 21.7 / 23.5.
+    S.draw_threads = P.B > 64 ? kSweepThreads / 2 : kSweepThreads;
     int rc;
     if (!RAGGED && S.fine_units > 0)
         rc = launch_sweeps_of<SD_DTYPE_BF16, MODE, false, true>(P, S, units, all, stream);

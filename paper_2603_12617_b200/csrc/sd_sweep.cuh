@@ -53,6 +53,7 @@ struct Sweep {
     int part_stride;         // room for a unit's partials
     PartialStats* part;      // workspace [units][part_stride]; its memory is region_sums' from the second sweep on
     uint32_t* arrived;       // workspace [units], zero on entry and zero again on exit
+    int draw_threads;        // of a block that draws
     unsigned kept;           // items, from the last one backwards, that L2 is asked to keep between the sweeps
     int all_rows;            // second sweep: masses of every row wanted (acceptance probabilities)
     int draw_blocks;         // second sweep: its first blocks, those of the rows that are drawn from,
@@ -489,35 +490,44 @@ __device__ __forceinline__ void sweep_pass2(const uint4* gT, const uint4* gD, co
 }
 
 // ---- the draw -----------------------------------------------------------------------------------
-// Sums of the threads of a block before a thread's own, and of all of them, in a fixed order.  All threads; `sums` is
-// free again after the next barrier.
-__device__ __noinline__ double block_sums_before(double mine, double* sums, double* all) {
+// A draw is done by a team, the first T threads of a block.
+template <int T>
+__device__ __forceinline__ void team_sync() {
+    if constexpr (T == kSweepThreads) __syncthreads();
+    else asm volatile("bar.sync 1, %0;" ::"n"(T) : "memory");
+}
+
+// Sums of the team's threads before a thread's own, and of all of them, in a fixed order.  `sums` is free again after
+// the team's next barrier.
+template <int T>
+__device__ __noinline__ double team_sums_before(double mine, double* sums, double* all) {
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const double incl = warp_inclusive_scan(mine);
     if (lane == 31) sums[warp] = incl;
-    __syncthreads();
-    double before = 0.0, total = 0.0;
-#pragma unroll 1
-    for (int w = 0; w < kSweepWarps; ++w) {
-        if (w == warp) before = total;
-        total += sums[w];
+    team_sync<T>();
+    double warps = lane < T / 32 ? sums[lane] : 0.0;
+#pragma unroll
+    for (int off = 1; off < T / 32; off <<= 1) {
+        const double o = __shfl_up_sync(0xffffffffu, warps, off);
+        if (lane >= off) warps += o;
     }
-    *all = total;
-    return before + (incl - mine);
+    *all = __shfl_sync(0xffffffffu, warps, T / 32 - 1);
+    const double before = __shfl_sync(0xffffffffu, warps, max(warp - 1, 0));
+    return (warp > 0 ? before : 0.0) + (incl - mine);
 }
 
 // Where a rejection leaves no residual mass: an entry drawn from p_n, in every thread.  There are no region masses of p_n, so
-// a warp adds up an eighth of the row's regions and the warp into whose share the draw falls takes them once more; sums,
+// every warp adds up a share of the row's regions and the one into whose share the draw falls takes it once more; sums,
 // prefixes and totals in fp64, from the entries on.  (Four entries at a time, taken again where they are searched: the
 // registers are those of the kernel's loops.)
-template <int DT>
+template <int DT, int T>
 __device__ __noinline__ int sweep_draw_from_p(const Params& P, const RowConst& rc, size_t offT, double u, int lead) {
     using E = Elem<DT>;
-    constexpr int kEntries = kRegionVecs * E::VEC, PER = kEntries / 32;
-    __shared__ double share[kSweepWarps];
+    constexpr int kEntries = kRegionVecs * E::VEC, PER = kEntries / 32, kWarps = T / 32;
+    __shared__ double share[kWarps];
     __shared__ int drawn;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const int per = (P.NR + kSweepWarps - 1) / kSweepWarps, j0 = min(P.NR, warp * per), j1 = min(P.NR, j0 + per);
+    const int per = (P.NR + kWarps - 1) / kWarps, j0 = min(P.NR, warp * per), j1 = min(P.NR, j0 + per);
     const auto mass = [&](int v) {
         return v >= 0 && v < P.V && SD_IN(v, P.V, 24) ? (double)prob_elem(E::load(P.T, offT + v), P.c, rc) : 0.0;
     };
@@ -533,15 +543,15 @@ __device__ __noinline__ int sweep_draw_from_p(const Params& P, const RowConst& r
     for (int j = j0; j < j1; ++j) mine += warp_sum(lane_sum(j));
     if (threadIdx.x == 0) drawn = 0;
     if (lane == 0) share[warp] = mine;
-    __syncthreads();
+    team_sync<T>();
     // the first share whose end exceeds t, or (rounding pushed t to the total) the last one with mass
     double total = 0.0, before = 0.0, run = 0.0;
-    for (int w = 0; w < kSweepWarps; ++w) total += share[w];
+    for (int w = 0; w < kWarps; ++w) total += share[w];
     const double t = u * total;
     int owner = -1;
     bool found = false;
 #pragma unroll 1
-    for (int w = 0; w < kSweepWarps && !found; ++w) {
+    for (int w = 0; w < kWarps && !found; ++w) {
         if (share[w] > 0.0) { owner = w; before = run; found = run + share[w] > t; }
         run += share[w];
     }
@@ -572,7 +582,7 @@ __device__ __noinline__ int sweep_draw_from_p(const Params& P, const RowConst& r
         }
         if (lane == 0) drawn = max(at, 0);
     }
-    __syncthreads();
+    team_sync<T>();
     return drawn;
 }
 
@@ -583,12 +593,12 @@ __device__ __noinline__ int sweep_draw_from_p(const Params& P, const RowConst& r
 // warp with sixteen regions and entries to a lane, one after the other, 7.5: 16 sequences, 5 tokens, 50 257 bf16 entries
 // 25.4 -> 20.2 us, 16, 5, 65 536 21.0 -> 19.2, 12, 4, 128 256 fp32 27.9 -> 26.2; error feedback 64, 4, 151 936 bf16
 // 52.0 -> 50.6.  (Run once beforehand by blocks that wait anyway, so that its instructions are there: slower, 52.6.)
-template <int DT>
+template <int DT, int T>
 __device__ __noinline__ void sweep_draw(const Params& P, int unit, int lead) {
     using E = Elem<DT>;
-    constexpr int kEntries = kRegionVecs * E::VEC, PER = kEntries / kSweepThreads;
-    static_assert(SD_MAX_K < kSweepThreads, "a thread for every token");
-    __shared__ double sums[2][kSweepWarps];
+    constexpr int kEntries = kRegionVecs * E::VEC, PER = kEntries / T;
+    static_assert(SD_MAX_K < T, "a thread for every token");
+    __shared__ double sums[2][T / 32];
     __shared__ double prefix_sh;
     __shared__ int owner[2], found, last_mass;
     const int tid = threadIdx.x, k = P.k, NR = P.NR;
@@ -608,7 +618,7 @@ __device__ __noinline__ void sweep_draw(const Params& P, int unit, int lead) {
         owner[0] = owner[1] = found = 0x7fffffff;
         last_mass = -1;
     }
-    const int per = (NR + kSweepThreads - 1) / kSweepThreads, j0 = tid * per, j1 = min(NR, j0 + per);
+    const int per = (NR + T - 1) / T, j0 = tid * per, j1 = min(NR, j0 + per);
     const int mode = bonus ? 1 : 0;
     int y = 0;
     // (the first two regions of a thread stay in registers: rows of up to 512 regions)
@@ -617,16 +627,16 @@ __device__ __noinline__ void sweep_draw(const Params& P, int unit, int lead) {
     for (int q = 0; q < 2; ++q) held[q] = j0 + q < j1 ? __ldcg(rs + j0 + q) : 0.f;
     double all, mine = (double)held[0] + (double)held[1];
     for (int j = j0 + 2; j < j1; ++j) mine += (double)__ldcg(rs + j);
-    const double before = block_sums_before(mine, sums[0], &all);
+    const double before = team_sums_before<T>(mine, sums[0], &all);
     const double t = uk * all;
     if (!(all > 0.0) || !isfinite(all)) {                          // (the same for every thread)
         flags |= bonus ? SD_STATUS_BAD_ROW : SD_STATUS_ZERO_RESIDUAL;
-        if (!bonus) y = sweep_draw_from_p<DT>(P, rc, offT, uk, lead);
+        if (!bonus) y = sweep_draw_from_p<DT, T>(P, rc, offT, uk, lead);
     } else {
         // the first region whose running sum exceeds t, or (rounding pushed u * R to the total) the last with mass
         if (mine > 0.0 && before + mine > t) atomicMin(&owner[0], tid);
         if (mine > 0.0) atomicMax(&last_mass, tid);
-        __syncthreads();
+        team_sync<T>();
         const bool past_end = owner[0] == 0x7fffffff;
         if (tid == (past_end ? last_mass : owner[0])) {
             int at = -1;
@@ -641,7 +651,7 @@ __device__ __noinline__ void sweep_draw(const Params& P, int unit, int lead) {
             found = max(at, 0);
             prefix_sh = run;
         }
-        __syncthreads();
+        team_sync<T>();
         const int region = found;
         const double prefix = past_end ? 0.0 : prefix_sh;
         if (tid == 0) last_mass = -1;
@@ -657,10 +667,10 @@ __device__ __noinline__ void sweep_draw(const Params& P, int unit, int lead) {
             mine += (double)m[e];
         }
         double region_all;
-        const double inside = prefix + block_sums_before(mine, sums[1], &region_all);
+        const double inside = prefix + team_sums_before<T>(mine, sums[1], &region_all);
         if (!past_end && mine > 0.0 && inside + mine > t) atomicMin(&owner[1], tid);
         if (mine > 0.0) atomicMax(&last_mass, tid);
-        __syncthreads();
+        team_sync<T>();
         // (region sum and re-summed entries may disagree in the last bits: the last entry with mass then, too)
         const bool to_last = owner[1] == 0x7fffffff;
         if (tid == (to_last ? last_mass : owner[1])) {
@@ -674,7 +684,7 @@ __device__ __noinline__ void sweep_draw(const Params& P, int unit, int lead) {
             found = max(at, 0);
         }
         if (tid == 0 && last_mass < 0) found = 0;
-        __syncthreads();
+        team_sync<T>();
         y = found;
     }
     if (tid == 0) {
@@ -829,8 +839,10 @@ sd_sweep_grad_kernel(const __grid_constant__ Params P, const __grid_constant__ S
     else __syncwarp();
     if (!is_last) return;
     if ((HINT || S.all_rows) && !ur.bonus && warp == 0) sweep_row_sums<HINT>(P, S, unit, ur.d_row);
-    if (!draws) return;
-    sweep_draw<DT>(P, unit, RAGGED ? row_frame<DT>(P, ur).lead : 0);
+    if (!draws || tid >= S.draw_threads) return;
+    const int lead = RAGGED ? row_frame<DT>(P, ur).lead : 0;
+    if (S.draw_threads == kSweepThreads) sweep_draw<DT, kSweepThreads>(P, unit, lead);
+    else                                 sweep_draw<DT, kSweepThreads / 2>(P, unit, lead);
 }
 
 }  // namespace sdv

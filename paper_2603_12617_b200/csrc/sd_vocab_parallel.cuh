@@ -407,7 +407,7 @@ __global__ void __launch_bounds__(kSweepThreads) sd_vp_draw_kernel(const VpParam
         const size_t offT = (size_t)unit * P.Vs, offD = (size_t)(b * k + (bonus ? 0 : n)) * P.Vs;
         double mine = (double)held, all;
         for (int j = j0 + 1; j < j1; ++j) mine += (double)rs[j];
-        const double before = ahead + block_sums_before(mine, sums[0], &all);
+        const double before = ahead + team_sums_before<kSweepThreads>(mine, sums[0], &all);
         if (!past_end && mine > 0.0 && before + mine > t) atomicMin(&owner_sh[0], tid);
         if (mine > 0.0) atomicMax(&last_mass, tid);
         __syncthreads();
@@ -439,7 +439,7 @@ __global__ void __launch_bounds__(kSweepThreads) sd_vp_draw_kernel(const VpParam
             m[e] = in ? mass_of(tl, dl, P.c, rc, mode) : 0.f;
             mine += (double)m[e];
         }
-        const double inside = prefix + block_sums_before(mine, sums[1], &all);
+        const double inside = prefix + team_sums_before<kSweepThreads>(mine, sums[1], &all);
         if (!to_last && mine > 0.0 && inside + mine > t) atomicMin(&owner_sh[1], tid);
         if (mine > 0.0) atomicMax(&last_mass, tid);
         __syncthreads();
