@@ -435,11 +435,16 @@ cudaError_t launch_following(K kern, dim3 grid, int threads, cudaStream_t stream
 int rows_threads(int k) { return 32 * (k < 8 ? 8 : k + 1 < kRowsMaxWarps ? k + 1 : kRowsMaxWarps); }
 
 template <int DT, int MODE, bool RAGGED, bool FINE>
-int launch_sweeps_of(const Params& P, const Sweep& S, long long units, bool all, cudaStream_t stream) {
+int launch_sweeps_of(const Params& P, const Sweep& S, long long units, bool all, int sms, cudaStream_t stream) {
     const dim3 first = FINE ? dim3((unsigned)((units - S.fine_units) * S.slices + (long long)S.fine_units * S.fine_slices))
                             : dim3((unsigned)units, (unsigned)S.slices);
     SD_CUDA(launch_following(sd_sweep_stats_kernel<DT, RAGGED, FINE>, first, kSweepThreads, stream, P, S));
-    SD_CUDA(launch_following(sd_sweep_rows_kernel<DT>, dim3((unsigned)P.B), rows_threads(P.k), stream, P, S));
+    // With registers as the compiler takes them four blocks of the rows kernel fit an SM; a call with more sequences than
+    // that would have a second round of them and takes the kernel that is held to 40 (six).  Step, 49 / 40 registers, us: 800 sequences,
+    // 1 token, 8 192 bf16 entries 27.6 / 25.8, 700, 2, 8 192 32.6 / 30.8, 2000, 4, 504 64.5 / 63.1, 600, 1, 8 201 fp32 34.4 / 33.2, 700, 16, 1 000 bf16
+    // 72.8 / 70.8; with one round 500, 8, 2 048 31.8 / 32.7, 400, 4, 8 192 fp32 44.1 / 45.0.
+    SD_CUDA(P.B > 4 * sms ? launch_following(sd_sweep_rows_kernel<DT, true>, dim3((unsigned)P.B), rows_threads(P.k), stream, P, S)
+                          : launch_following(sd_sweep_rows_kernel<DT, false>, dim3((unsigned)P.B), rows_threads(P.k), stream, P, S));
     // the rows that are drawn from, then (if anything of them is wanted) all pair rows; the hint error is summed by items of one
     // size, and the error feedback has nothing but the rows that are drawn from
     constexpr bool FINE2 = FINE && MODE == kSweepStepMode;
@@ -451,7 +456,7 @@ int launch_sweeps_of(const Params& P, const Sweep& S, long long units, bool all,
 }
 
 template <int MODE, bool RAGGED = false>
-int launch_sweeps(const Params& P, Sweep& S, long long units, int dtype, cudaStream_t stream) {
+int launch_sweeps(const DeviceState& d, const Params& P, Sweep& S, long long units, int dtype, cudaStream_t stream) {
     S.regions = (P.NR + S.slices - 1) / S.slices;
     // What the first sweep reads last stays in L2 for the second, which starts there: 80 MiB of 126 (measured
     // on 288 rows of 128 256 bf16 entries: 0 MiB 70.5 us, 48 69.7, 64 69.1, 80 68.4, 96 68.8, before the draws
@@ -504,10 +509,10 @@ int launch_sweeps(const Params& P, Sweep& S, long long units, int dtype, cudaStr
     S.draw_threads = P.B > 64 ? kSweepThreads / 2 : kSweepThreads;
     int rc;
     if (!RAGGED && S.fine_units > 0)
-        rc = launch_sweeps_of<SD_DTYPE_BF16, MODE, false, true>(P, S, units, all, stream);
+        rc = launch_sweeps_of<SD_DTYPE_BF16, MODE, false, true>(P, S, units, all, d.sm_count, stream);
     else
-        rc = dtype == SD_DTYPE_F32 ? launch_sweeps_of<SD_DTYPE_F32, MODE, RAGGED, false>(P, S, units, all, stream)
-                                   : launch_sweeps_of<SD_DTYPE_BF16, MODE, RAGGED, false>(P, S, units, all, stream);
+        rc = dtype == SD_DTYPE_F32 ? launch_sweeps_of<SD_DTYPE_F32, MODE, RAGGED, false>(P, S, units, all, d.sm_count, stream)
+                                   : launch_sweeps_of<SD_DTYPE_BF16, MODE, RAGGED, false>(P, S, units, all, d.sm_count, stream);
     if (rc != SD_OK) return rc;
     tl_info[0] = 1; tl_info[1] = 1; tl_info[2] = kSweepThreads; tl_info[3] = 0; tl_info[5] = 3;
     return SD_OK;
@@ -721,9 +726,9 @@ int run_device(DeviceState& d, const void* T, const void* D, const int32_t* x, c
         P.blocks_per_unit = L.slices;
         P.RE = kRegionVecs * vec_elems(dtype);
         P.NR = (int)sweep_row_regions(V, dtype);
-        if (ragged) return launch_sweeps<kSweepStepMode, true>(P, S, units, dtype, stream);
-        return hint ? launch_sweeps<kSweepHint>(P, S, units, dtype, stream)
-                    : launch_sweeps<kSweepStepMode>(P, S, units, dtype, stream);
+        if (ragged) return launch_sweeps<kSweepStepMode, true>(d, P, S, units, dtype, stream);
+        return hint ? launch_sweeps<kSweepHint>(d, P, S, units, dtype, stream)
+                    : launch_sweeps<kSweepStepMode>(d, P, S, units, dtype, stream);
     }
     if (status) SD_CUDA(cudaMemsetAsync(status, 0, (size_t)B * 4, stream));   // bits are ORed in on the device
     int C = 0, G = 0, lag = 0, per = 0;
@@ -1226,7 +1231,7 @@ int sd_verify_error_feedback(const void* target_logits, const void* draft_logits
         S.arrived = reinterpret_cast<uint32_t*>(ws + L.arrived);
         S.all_rows = 0;
         P.blocks_per_unit = L.slices;
-        rc = launch_sweeps<kSweepErrors>(P, S, units, dtype, st);
+        rc = launch_sweeps<kSweepErrors>(*d, P, S, units, dtype, st);
         if (rc != SD_OK) return rc;
         if (!workspace) keep_scratch(d, L.accept, head);
         tl_info[0] = 4;

@@ -417,10 +417,11 @@ sd_sweep_stats_kernel(const __grid_constant__ Params P, const __grid_constant__ 
 }
 
 // A block per sequence, a warp per row (up to kRowsMaxWarps of them at a time).  Leaves the sequence's first rejected
-// position (k if there is none) in P.accept[b * k].
+// position (k if there is none) in P.accept[b * k].  MANY: held to 40 registers, six blocks of eight warps to an SM (rule and
+// figures: launch_sweeps_of, host).
 constexpr int kRowsMaxWarps = 16;
-template <int DT>
-__global__ void __launch_bounds__(kRowsMaxWarps * 32)
+template <int DT, bool MANY>
+__global__ void __launch_bounds__(kRowsMaxWarps * 32, MANY ? 3 : 0)
 sd_sweep_rows_kernel(const __grid_constant__ Params P, const __grid_constant__ Sweep S) {
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, warps = (int)blockDim.x >> 5;
     const int b = blockIdx.x;
