@@ -1583,8 +1583,12 @@ int sd_vp_draw(const void* target_shard, const void* draft_shard, const int32_t*
     P.tokens = out_tokens;
     P.status = out_status;
     cudaStream_t st = static_cast<cudaStream_t>(stream);
-    SD_CUDA(dtype == SD_DTYPE_F32 ? launch_following(sd_vp_draw_kernel<SD_DTYPE_F32>, dim3((unsigned)B), kSweepThreads, st, P)
-                                  : launch_following(sd_vp_draw_kernel<SD_DTYPE_BF16>, dim3((unsigned)B), kSweepThreads, st, P));
+    const bool many = B > 4 * ds->sm_count;             // (figures: sd_vp_draw_kernel)
+    const dim3 grid((unsigned)B);
+    if (dtype == SD_DTYPE_F32)
+        SD_CUDA(many ? launch_following(sd_vp_draw_kernel<SD_DTYPE_F32, 64>, grid, 64, st, P) : launch_following(sd_vp_draw_kernel<SD_DTYPE_F32, 128>, grid, 128, st, P));
+    else
+        SD_CUDA(many ? launch_following(sd_vp_draw_kernel<SD_DTYPE_BF16, 64>, grid, 64, st, P) : launch_following(sd_vp_draw_kernel<SD_DTYPE_BF16, 128>, grid, 128, st, P));
     tl_info[0] = 6; tl_info[5] = 1;
     return SD_OK;
 }

@@ -329,16 +329,17 @@ __global__ void __launch_bounds__(kVpThreads, 6) sd_vp_grad_kernel(const VpParam
 }
 
 // ---- phase 3 -------------------------------------------------------------------------------
-// One block per sequence.  Shares in rank order: the first rank whose running sum exceeds
+// One block of T threads per sequence.  Shares in rank order: the first rank whose running sum exceeds
 // u_k * total owns the draw (the last rank with mass, if rounding leaves none); its block searches as the single-GPU
-// draw does (sweep_draw), with the mass of the ranks before it in front.  (A warp that took sixteen regions and entries to a
-// lane: with the slices of phase 2 as they were 22.2 us for the three calls on 16 sequences, 4 tokens, an eighth of 151 936
-// bf16 entries, 18.0 with both; 4 sequences, a quarter of 32 000 14.8, 13.3.)
-template <int DT>
-__global__ void __launch_bounds__(kSweepThreads) sd_vp_draw_kernel(const VpParams P) {
+// draw does (sweep_draw), with the mass of the ranks before it in front.  128 threads, 64 where there are more than four blocks to
+// an SM.  This kernel alone, the warp that drew once / 64 / 128 / 256 threads, us: 64 sequences, 37 984 bf16 entries 4.6 / 4.3 / 3.8 /
+// 3.8, 512 of 8 000 5.1 / 4.4 / 4.2 / 5.9, 1000 of 16 000 4.8 / 4.4 / 5.1 / 6.5; fp32 256 of 19 000 3.8 / 4.1 / 3.7 / 3.9, 512 of 8 000 4.2 / 4.2 / 4.2 /
+// 5.8, 1000 of 512 3.8 / 4.0 / 5.5 / 6.4, 2000 of 256 4.8 / 5.5 / 6.5 / 9.8.
+template <int DT, int T>
+__global__ void __launch_bounds__(T) sd_vp_draw_kernel(const VpParams P) {
     using E = Elem<DT>;
-    constexpr int kEntries = kRegionVecs * E::VEC, PER = kEntries / kSweepThreads;
-    __shared__ double sums[2][kSweepWarps];
+    constexpr int kEntries = kRegionVecs * E::VEC, PER = kEntries / T;
+    __shared__ double sums[2][T / 32];
     __shared__ double prefix_sh;
     __shared__ int owner_sh[2], found, last_mass;
     const int b = blockIdx.x, tid = threadIdx.x, lane = tid & 31;
@@ -355,7 +356,7 @@ __global__ void __launch_bounds__(kSweepThreads) sd_vp_draw_kernel(const VpParam
         const double* const m = P.all_mass + ((size_t)lane * P.B + b) * 2;
         mass = make_double2(m[0], m[1]);
     }
-    const int per = (P.NR + kSweepThreads - 1) / kSweepThreads, j0 = min(P.NR, tid * per), j1 = min(P.NR, j0 + per);
+    const int per = (P.NR + T - 1) / T, j0 = min(P.NR, tid * per), j1 = min(P.NR, j0 + per);
     const float* rs = P.region_sums + (size_t)b * 2 * P.NR;
     float held = j0 < j1 ? rs[j0] : 0.f;
     if (tid == 0) {
@@ -407,10 +408,10 @@ __global__ void __launch_bounds__(kSweepThreads) sd_vp_draw_kernel(const VpParam
         const size_t offT = (size_t)unit * P.Vs, offD = (size_t)(b * k + (bonus ? 0 : n)) * P.Vs;
         double mine = (double)held, all;
         for (int j = j0 + 1; j < j1; ++j) mine += (double)rs[j];
-        const double before = ahead + team_sums_before<kSweepThreads>(mine, sums[0], &all);
+        const double before = ahead + team_sums_before<T>(mine, sums[0], &all);
         if (!past_end && mine > 0.0 && before + mine > t) atomicMin(&owner_sh[0], tid);
         if (mine > 0.0) atomicMax(&last_mass, tid);
-        __syncthreads();
+        team_sync<T>();
         const bool to_last = owner_sh[0] == 0x7fffffff;      // (rounding: the last region of this shard that holds mass)
         if (tid == (to_last ? last_mass : owner_sh[0])) {
             int at = j0;
@@ -425,7 +426,7 @@ __global__ void __launch_bounds__(kSweepThreads) sd_vp_draw_kernel(const VpParam
             found = at;
             prefix_sh = r2;
         }
-        __syncthreads();
+        team_sync<T>();
         const int region = found;
         const double prefix = to_last ? 0.0 : prefix_sh;
         if (tid == 0) last_mass = -1;
@@ -439,10 +440,10 @@ __global__ void __launch_bounds__(kSweepThreads) sd_vp_draw_kernel(const VpParam
             m[e] = in ? mass_of(tl, dl, P.c, rc, mode) : 0.f;
             mine += (double)m[e];
         }
-        const double inside = prefix + team_sums_before<kSweepThreads>(mine, sums[1], &all);
+        const double inside = prefix + team_sums_before<T>(mine, sums[1], &all);
         if (!to_last && mine > 0.0 && inside + mine > t) atomicMin(&owner_sh[1], tid);
         if (mine > 0.0) atomicMax(&last_mass, tid);
-        __syncthreads();
+        team_sync<T>();
         const bool last_entry = owner_sh[1] == 0x7fffffff;
         if (tid == (last_entry ? last_mass : owner_sh[1])) {
             int at = -1;
@@ -455,11 +456,11 @@ __global__ void __launch_bounds__(kSweepThreads) sd_vp_draw_kernel(const VpParam
             found = max(at, 0);
         }
         if (tid == 0 && last_mass < 0) found = 0;
-        __syncthreads();
+        team_sync<T>();
         y = P.v_offset + found;
     }
     if (tid == 0 && flags && P.status) atomicOr(P.status + b, flags);
-    if (tid <= k) P.tokens[b * K1 + tid] = tid < n ? x : (tid == n ? y : -1);
+    for (int i = tid; i <= k; i += T) P.tokens[b * K1 + i] = i < n ? (i == tid ? x : P.x[b * k + i]) : (i == n ? y : -1);
 }
 
 }  // namespace sdv
