@@ -1514,8 +1514,15 @@ int sd_vp_partial(const void* target_shard, const void* draft_shard, const int32
     if (C > (unsigned)((NR + kVpStatsWarps - 1) / kVpStatsWarps)) C = (unsigned)((NR + kVpStatsWarps - 1) / kVpStatsWarps);
     if (C > (unsigned)kVpMaxCluster) C = kVpMaxCluster;
     if (C < 1) C = 1;
-    SD_CUDA(dtype == SD_DTYPE_F32 ? launch_following_clusters(sd_vp_stats_kernel<SD_DTYPE_F32>, dim3(units * C), kVpStatsThreads, C, st, P)
-                                  : launch_following_clusters(sd_vp_stats_kernel<SD_DTYPE_BF16>, dim3(units * C), kVpStatsThreads, C, st, P));
+    // fp32 warps with enough regions take them two at a time; with few the second of the last pair is the work of a region for nothing.
+    // One at a time / in pairs, us, regions a warp in brackets: one block a row 128 sequences, 4 tokens, 4 000 entries (4) 6.1 / 6.3, 256, 4, 6 144
+    // (6) 9.2 / 9.3, 7 168 (7) 11.1 / 10.7, 8 192 (8) 12.5 / 11.6; several 64, 4, 8 000 (3) 5.6 / 5.9, 20 000 (7) 8.8 / 9.2, 37 984 (12) 15.3 / 15.3,
+    // 64, 6, 32 064 (16) 20.2 / 19.6, 2, 2, 500 000 (61) 23.1 / 18.8; 32, 8, 16 032 (4), on the wrong side, 8.4 / 8.2.  bf16 regions, with twice the
+    // entries, have no registers for two (37.7 against 37.0 on 320 rows of 37 984).
+    const bool pairs = dtype == SD_DTYPE_F32 && NR > (C == 1 ? 6 : 12) * (int)C * kVpStatsWarps;
+    SD_CUDA(pairs                   ? launch_following_clusters(sd_vp_stats_kernel<SD_DTYPE_F32, true>, dim3(units * C), kVpStatsThreads, C, st, P)
+            : dtype == SD_DTYPE_F32 ? launch_following_clusters(sd_vp_stats_kernel<SD_DTYPE_F32, false>, dim3(units * C), kVpStatsThreads, C, st, P)
+                                    : launch_following_clusters(sd_vp_stats_kernel<SD_DTYPE_BF16, false>, dim3(units * C), kVpStatsThreads, C, st, P));
     tl_info[0] = 6; tl_info[1] = (int)C; tl_info[2] = kVpStatsThreads; tl_info[3] = 0; tl_info[4] = (int)(units * C); tl_info[5] = 1;
     return SD_OK;
 }

@@ -74,14 +74,14 @@ struct VpParams {
 // per region), its warps take the row's regions in turn, with the loop of the single-GPU first sweep (a
 // maximum for every two vectors and a test for masked entries took 18.0 us on 320 rows of 37 984 bf16 entries,
 // one block of eight warps per row 15.7; ten or twelve blocks an SM, with fewer registers, no less, and fp32 rows a tenth more).
-// fp32 rows go two regions at a time (448 rows of 32 064 entries: the three calls 52.5 -> 50.6).
+// PAIRS: a warp's regions two at a time (fp32 rows; rule and figures: sd_vp_partial, host).
 // Every region raises the references: with those of a warp's first region alone the error of fp32
 // gradients against 64 bits doubled.  With a vote whether any entry is above them that costs nothing there
 // (1792 rows of 32 064 entries 42.0 -> 44.0; raised without looking 45.0).
 constexpr int kVpStatsWarps = 4;
 constexpr int kVpStatsThreads = kVpStatsWarps * 32;
 constexpr int kVpMaxCluster = 8;
-template <int DT>
+template <int DT, bool PAIRS>
 __global__ void __launch_bounds__(kVpStatsThreads, 8) sd_vp_stats_kernel(const VpParams P) {
     using E = Elem<DT>;
     using ET = typename E::type;
@@ -120,8 +120,7 @@ __global__ void __launch_bounds__(kVpStatsThreads, 8) sd_vp_stats_kernel(const V
     const uint64_t policy = policy_normal();     // what fits stays in L2 for the second sweep
     const int nvec = SD_IN(unit, P.B * K1, 60) ? NV - w0 : 0;
     const int step = slots * kRegionVecs;
-    if constexpr (DT == SD_DTYPE_F32) {
-        // (bf16 regions, with twice the entries, have no registers for two: 37.7 us against 37.0 on 320 rows of 37 984)
+    if constexpr (PAIRS) {
         if (bonus) sweep_pass1_pairs<DT, true>(Trow + w0, Drow + w0, nvec, step, lane, P.c, policy, ps);
         else       sweep_pass1_pairs<DT, false>(Trow + w0, Drow + w0, nvec, step, lane, P.c, policy, ps);
     } else {

@@ -80,9 +80,10 @@ def test_shards_of_equal_width(binding, dtype, V, G):
 
 @pytest.mark.parametrize("B,k,V,dtype,width", [(20, 2, 256 * 65, "f32", 256 * 32), (20, 2, 256 * 98 + 4, "f32", 256 * 33), (700, 1, 256 * 13 - 4, "f32", 256 * 7),
                                                (2, 2, 512 * 257 + 8, "bf16", 512 * 256), (200, 2, 512 * 40, "bf16", 512 * 23),
+                                               (400, 2, 256 * 49, "f32", 256 * 24), (400, 2, 256 * 51 - 4, "f32", 256 * 25), (1, 2, 256 * 770 + 4, "f32", 256 * 385),
                                                (4, 1, 256 * 258, "f32", 256 * 129), (600, 1, 512 * 66, "bf16", 512 * 65), (600, 64, 264, "bf16", 136)])
 def test_shards_of_as_many_regions_as_warps_and_threads(binding, B, k, V, dtype, width):
-    """The first sweep of fp32 rows takes a warp's regions two at a time, the draw a thread's one after the other (of 128 threads,
+    """The first sweep of fp32 rows takes a warp's regions two at a time (one at a time, if it has few), the draw a thread's one after the other (of 128 threads,
     of 64 with very many sequences, which then may have more tokens than that), the second sweep slices of about the same size."""
     inp = synth.make_inputs(synth.custom_config(B=B, k=k, V=V, dtype=dtype, tau=0.9, index=79))
     inp.uniforms[:, k] = np.linspace(0, 1 - 2.0 ** -24, B, dtype=np.float32)
