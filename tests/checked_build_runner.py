@@ -25,12 +25,27 @@ KERNEL = {1024: "cluster", 512: "held", 256: "sweeps"}
 SEEN = set()
 
 
-def took(entry):
+def took(entry, sweeps=3):
     info = b.sd_launch_info()
     kernel = "element-wise" if info["path"] == 0 else KERNEL[info["threads"]]
-    assert info["kernels"] == {"sweeps": 3}.get(kernel, 2 if entry in ("errors", "ensemble") else 1), (entry, info)
+    assert info["kernels"] == {"sweeps": sweeps}.get(kernel, 2 if entry in ("errors", "ensemble") else 1), (entry, info)
     SEEN.add((entry, kernel))
     return kernel
+
+
+def sharded(T, D, x, u, tau, cuts):
+    """The vocabulary-parallel step, every rank's calls."""
+    B, k, V = D.shape
+    code, G = (b.SD_DTYPE_F32 if T.dtype == torch.float32 else b.SD_DTYPE_BF16), len(cuts)
+    Ts = [T[:, :, a:c].contiguous() for a, c in cuts]
+    Ds = [D[:, :, a:c].contiguous() for a, c in cuts]
+    ws = [torch.empty(max(256, b.sd_vp_workspace_bytes(B, k, c - a, code)), dtype=torch.uint8, device="cuda") for a, c in cuts]
+    recs = torch.stack([b.sd_vp_partial(Ts[r], Ds[r], x, tau, cuts[r][0], V, ws[r]) for r in range(G)], 0).contiguous()
+    fins = [b.sd_vp_finish(Ts[r], Ds[r], x, u, tau, cuts[r][0], V, recs, G, r, ws[r]) for r in range(G)]
+    m = torch.stack([f.local_mass for f in fins], 0).contiguous()
+    tokens = torch.stack([b.sd_vp_draw(Ts[r], Ds[r], x, u, tau, cuts[r][0], V, fins[r].accept_len, m, G, r, fins[r].status, ws[r])
+                          for r in range(G)], 0).max(0).values
+    return fins[0].accept_len, tokens
 
 
 def main():
@@ -68,23 +83,12 @@ def main():
         g = b.sd_verify_greedy(T, x)
         gref = sd_oracle.verify_greedy(inp.target_logits, inp.draft_tokens)
         assert (g.accept_len.cpu().numpy() == gref.accept_len).all() and (g.tokens.cpu().numpy() == gref.tokens).all()
-        if whole:
-            if V // (16 // es) >= 2:
-                code = b.SD_DTYPE_F32 if dt == "f32" else b.SD_DTYPE_BF16
-                cuts = shard.vocab_cuts(V, 2, es)
-                Ts = [T[:, :, a:c].contiguous() for a, c in cuts]
-                Ds = [D[:, :, a:c].contiguous() for a, c in cuts]
-                ws = [torch.empty(max(256, b.sd_vp_workspace_bytes(B, k, c - a, code)), dtype=torch.uint8, device="cuda")
-                      for a, c in cuts]
-                recs = torch.stack([b.sd_vp_partial(Ts[r], Ds[r], x, inp.tau, cuts[r][0], V, ws[r]) for r in range(2)], 0).contiguous()
-                fins = [b.sd_vp_finish(Ts[r], Ds[r], x, u, inp.tau, cuts[r][0], V, recs, 2, r, ws[r]) for r in range(2)]
-                m = torch.stack([f.local_mass for f in fins], 0).contiguous()
-                for r in range(2):
-                    b.sd_vp_draw(Ts[r], Ds[r], x, u, inp.tau, cuts[r][0], V, fins[r].accept_len, m, 2, r, fins[r].status, ws[r])
+        if whole and V // (16 // es) >= 2:
+            sharded(T, D, x, u, inp.tau, [(0, V // 2 // (16 // es) * (16 // es)), (V // 2 // (16 // es) * (16 // es), V)])
         torch.cuda.synchronize()
 
     # the two sweeps: whole-vector rows of more than fit the chip at once, odd rows wherever they start
-    for (B, k, V, dt, leadT, leadD) in [(40, 3, 58000, "bf16", 0, 0), (24, 3, 72004, "f32", 0, 0), (1300, 2, 4104, "bf16", 0, 0),
+    for (B, k, V, dt, leadT, leadD) in [(40, 3, 58000, "bf16", 0, 0), (24, 3, 72004, "f32", 0, 0), (1300, 2, 4104, "bf16", 0, 0), (1300, 2, 504, "bf16", 0, 0),
                                         (200, 2, 4097, "bf16", 1, 6), (150, 3, 2051, "f32", 2, 1), (3, 2, 50257, "bf16", 0, 0),
                                         (2, 2, 512 * 65 - 1, "bf16", 3, 0), (3, 2, 40003, "f32", 3, 3)]:
         cfg = synth.custom_config(B, k, V, dtype=dt, tau=0.9, index=91)
@@ -106,10 +110,27 @@ def main():
             h = b.sd_verify_feedback_hint(T, D, x, u, inp.tau, torch.zeros_like(D))
             assert took("hint") == "sweeps"
             assert torch.equal(e.tokens, out.tokens) and torch.equal(h.tokens, out.tokens)
+        if dt == "bf16" and V % 8 == 0:
+            # (one and two groups of learners; sums of another order than the step's, so its values to rounding)
+            for N, grad in ((2, True), (4, False), (5, True), (5, False)):
+                m = b.sd_ensemble_feedback(T, [D.roll(n, 0) for n in range(N)], inp.tau, 10.0, want_grad=grad)
+                assert took("ensemble", 3 if N <= 4 else 5 if grad else 4) == "sweeps"
+                assert ((m.loss[0] - out.loss).abs() <= 1e-5 * out.loss + 4e-7).all()
+                if grad:
+                    assert ((m.grad[0].float() - out.grad_draft.float()).abs() <= 2.0 ** -7 * out.grad_draft.float().abs() + 1e-6).all()
         torch.cuda.synchronize()
+
+    # the sharded step with regions one and two at a time, and with both sizes of the draw's blocks
+    for (B, k, V, dt, cut) in [(700, 1, 256 * 13, "f32", 256 * 7), (400, 2, 256 * 52, "f32", 256 * 26 + 4), (600, 2, 512 * 3 + 8, "bf16", 512), (4, 2, 512 * 300, "bf16", 512 * 170)]:
+        inp = synth.make_inputs(synth.custom_config(B, k, V, dtype=dt, tau=0.9, index=92))
+        T, D, x, u = to_device(inp)
+        accept_len, tokens = sharded(T, D, x, u, inp.tau, [(0, cut), (cut, V)])
+        ref = oracle_of(inp)
+        safe = (ref.accept_band.sum(1) == 0) & (ref.cdf_margin > 1e-6)
+        assert (accept_len.cpu().numpy() == ref.accept_len)[safe].all() and (tokens.cpu().numpy() == ref.tokens)[safe].all()
     # a later rule may not take a kernel out of this run
-    assert SEEN == {(e, n) for e in ("step", "hint", "errors", "ensemble") for n in ("cluster", "held", "sweeps")
-                    if (e, n) != ("ensemble", "sweeps")} | {("step", "element-wise"), ("hint", "element-wise")}, SEEN
+    assert SEEN == {(e, n) for e in ("step", "hint", "errors", "ensemble") for n in ("cluster", "held", "sweeps")} \
+        | {("step", "element-wise"), ("hint", "element-wise")}, SEEN
     print("REPORT " + json.dumps(b.sd_bounds_report()))
 
 

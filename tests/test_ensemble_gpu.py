@@ -302,8 +302,56 @@ def test_two_sweeps_special_rows(binding):
     assert torch.equal(bad.loss[:, keep], out.loss[:, keep])
 
 
+def test_two_sweeps_keep_a_bad_draft_row_to_itself(binding):
+    """A draft row without a finite entry -- of the first learner, whose constants the group takes the target's from, or of the
+    last -- leaves everybody else's losses and gradients as they are, to the last bit."""
+    B, k, V = 60, 3, 20000
+    inp = synth.make_inputs(synth.custom_config(B, k, V, dtype="bf16", tau=0.9, index=135))
+    for N in (3, 5):
+        Ds = [dev(d) for d in synth.ensemble_drafts(inp, N)]
+        T = dev(inp.target_logits)
+        want = binding.sd_ensemble_feedback(T, Ds, inp.tau, EPS)
+        torch.cuda.synchronize()
+        bad = [(0, 9, 0), (N - 1, 20, 2)]
+        for n, b, i in bad:
+            Ds[n][b, i] = float("-inf")
+        out = binding.sd_ensemble_feedback(T, Ds, inp.tau, EPS, want_status=True)
+        assert binding.sd_launch_info()["threads"] == 256
+        torch.cuda.synchronize()
+        good = torch.ones(N, B, k, dtype=torch.bool, device="cuda")
+        for n, b, i in bad:
+            good[n, b, i] = False
+        assert torch.equal(out.loss[good], want.loss[good])
+        for n in range(N):
+            assert torch.equal(out.grad[n][good[n]], want.grad[n][good[n]])
+        assert [b for b in range(B) if out.status[b] != 0] == [9, 20] and (out.status[[9, 20]] == binding.SD_STATUS_BAD_ROW).all()
+
+
+@pytest.mark.parametrize("N,left_out", [(3, (0, 1)), (3, (2,)), (5, (0, 4)), (5, (0, 1)), (5, (2, 3, 4)), (2, (0, 1))])
+def test_two_sweeps_without_the_gradients_of_some_learners(binding, N, left_out):
+    """Some of a group, a whole group (5 learners go as 2 and 3), all."""
+    import ctypes
+    cfg = synth.custom_config(60, 3, 20008, dtype="bf16", tau=0.9, index=136)
+    inp = synth.make_inputs(cfg)
+    T, Ds = dev(inp.target_logits), [dev(d) for d in synth.ensemble_drafts(inp, N)]
+    full = binding.sd_ensemble_feedback(T, Ds, inp.tau, EPS)
+    need = binding._lib.sd_ensemble_workspace_bytes(cfg.B, cfg.k, cfg.V, binding.SD_DTYPE_BF16, N)
+    ws = torch.empty(need, dtype=torch.uint8, device="cuda")
+    grads = [torch.full_like(g, 7.0) for g in full.grad]
+    loss, small = torch.empty_like(full.loss), [torch.empty_like(t) for t in (full.round_loss, full.cum_loss, full.weights)]
+    dptr = (ctypes.c_void_p * N)(*[d.data_ptr() for d in Ds])
+    gptr = (ctypes.c_void_p * N)(*[None if n in left_out else g.data_ptr() for n, g in enumerate(grads)])
+    rc = binding._lib.sd_ensemble_feedback(T.data_ptr(), dptr, N, float(inp.tau), EPS, cfg.B, cfg.k, cfg.V, binding.SD_DTYPE_BF16, None,
+                                           loss.data_ptr(), gptr, *[t.data_ptr() for t in small], None, ws.data_ptr(), need, None)
+    torch.cuda.synchronize()
+    assert rc == 0 and binding.sd_launch_info()["threads"] == 256
+    assert torch.equal(loss, full.loss) and torch.equal(small[2], full.weights)
+    for n, g in enumerate(grads):
+        assert (g == 7.0).all() if n in left_out else torch.equal(g, full.grad[n])
+
+
 def test_two_sweeps_in_a_graph(binding):
-    """A replay and eager calls on the library's scratch, one after the other."""
+    """A replay, whose scratch is the graph's, beside eager steps."""
     cfg = synth.custom_config(60, 3, 20000, dtype="bf16", tau=0.9, index=131)
     inp = synth.make_inputs(cfg)
     Ds = synth.ensemble_drafts(inp, 3)

@@ -188,3 +188,25 @@ def test_a_held_ensemble_wants_no_scratch(binding):
     graph.replay()
     call.check("replay")
     del graph
+
+
+def test_ensembles_and_other_calls_share_the_scratch(binding):
+    """The ensemble's sweeps write where other calls keep words that must be zero, when they are issued and whenever a graph replays them."""
+    call = EnsembleCall(binding, (60, 3, 20000, "bf16"), 117)
+    assert binding.sd_launch_info()["threads"] == 256
+    other = Call(binding, "step", LARGE, 118)
+    call.run("first")
+    other.run("other after an ensemble")
+    call.run("second")
+    other.run("other, again")
+    graph = call.capture()
+    assert binding.sd_launch_info()["threads"] == 256
+    for turn in range(2):
+        other.run("other, between")
+        call.forget()
+        graph.replay()
+        call.check(f"replay {turn}")
+        other.run("other after a replay")
+        call.run("eager")
+        other.run("other after both")
+    del graph
