@@ -10,7 +10,10 @@
 // What bounds it: HBM, where every logit is read twice but for the 80 MiB that L2 keeps.  3 learners, 32 sequences, 8
 // tokens, 128 256 bf16 entries 122 us (at the copy bandwidth: 70 us for every logit once, 98 for what is moved), 144 on
 // the cluster kernel, which takes the learners one after the other and the target's exponentials with each.  A group of four
-// learners has three blocks an SM (four spill: 158 us against 155), smaller ones four (2 learners 87, with three blocks 90).
+// learners has three blocks an SM (four spill: 158 us against 155), smaller ones four (2 learners 87, with three blocks 90).  Three
+// learners spill at four blocks, too (92 bytes of stores in the first sweep, 8 in the second; at three blocks none), and are no slower for
+// it, us, four blocks / three in the first sweep / in both: 256 positions of 128 256 entries 120.8 / 121.2 / 120.3, 600 of 151 936 328 / 333 /
+// 331, 144 of 32 000 20.4 / 20.4 / 20.8; 6 learners 655 / 666 / 662 and 41.2 / 43.2 / 44.6.
 // bf16 rows only (rule and figures: use_ensemble_sweeps, host).
 #pragma once
 

@@ -19,10 +19,10 @@
 // sd_stream_kernel reads every logit from HBM once, but its 28 consumer warps share one ring and all blocks
 // read at the same time and compute at the same time, so at bf16, where the exponentials take as long as
 // the reads, it moves 2.9 TB/s.  Step on 32 sequences, 8 draft tokens, 128 256 bf16 entries: 71.1 us there,
-// 56.1 us here; 64 sequences, 4 tokens, 151 936: 93.4 and 69.7 us; 8, 5, 128 256: 35.0 and 19.6.  Of the 57.4 us that the first
+// 56.1 us here; 64 sequences, 4 tokens, 151 936: 93.4 and 69.7 us; 8, 5, 128 256: 35.0 and 18.9.  Of the 57.4 us that the first
 // of these took with items of one size, clock stamps of every block: first sweep 29.5, the last 8 with fewer and fewer
 // blocks; 4.5 until the second sweep works, 2 of them in the rows kernel; second sweep 24.  16 sequences, 5 tokens, 65 536 bf16
-// entries, 19.6 us: 8, 4, 5, and 4 for the draws.
+// entries, when it took 19.6 us (18.4 now): 8, 4, 5, and 4 for the draws.
 // The rule which of the two a call takes is use_sweeps (host).
 //
 // Tried and dropped, on the first of these: one persistent kernel whose warps take both passes of an item
@@ -116,7 +116,7 @@ __device__ __forceinline__ PartialStats load_partial_cg(const PartialStats* p) {
 // and written entry by entry, out of line and with registers of their own: with one set for both, filled by a
 // function for the ends, every region went through local memory (13 sequences, 8 tokens, 110 593 fp32 entries 67.3 us,
 // 41 since; 122, 4, 119 177 302 and 202; 64, 4, 100 001 bf16 84.9 and 61).  16 sequences, 5 tokens, 50 257 bf16
-// entries: 19.8 us, against 91.6 us for the element-wise kernel, whose one block per row reads two bytes a lane.
+// entries: 19.4 us, against 91.6 us for the element-wise kernel, whose one block per row reads two bytes a lane.
 template <int DT> struct RowFrame {
     const typename Elem<DT>::type *rowT, *rowD;
     const uint4 *T16, *D16;      // vector 0 of the regions, aligned: up to a vector before the row
@@ -593,13 +593,14 @@ __device__ __noinline__ int sweep_draw_from_p(const Params& P, const RowConst& r
     return drawn;
 }
 
-// The extra token of a sequence, and what the sequence puts out, by the block that brought the last item of the row that
-// it is drawn from, `unit`, once that row's region masses are all there.  Its end is the call's where the sweep is short, and what it consists of is
-// round trips and sums that wait for one another; so a block does it, a region or two to a thread and then an entry or
-// two of the region.  `lead`: entries of region 0 before the row.  From the last item to the end of the call 4 us, by one
-// warp with sixteen regions and entries to a lane, one after the other, 7.5: 16 sequences, 5 tokens, 50 257 bf16 entries
-// 25.4 -> 20.2 us, 16, 5, 65 536 21.0 -> 19.2, 12, 4, 128 256 fp32 27.9 -> 26.2; error feedback 64, 4, 151 936 bf16
-// 52.0 -> 50.6.  (Run once beforehand by blocks that wait anyway, so that its instructions are there: slower, 52.6.)
+// The extra token of a sequence, and what the sequence puts out, by the first T threads of the block that brought the last item of
+// the row that it is drawn from, `unit`, once that row's region masses are all there.  `lead`: entries of region 0 before the row.
+// Its end is the call's where the sweep is short, and what it consists of is round trips and sums that wait for one another; so many
+// threads do it, a region or two to a thread and then a few entries of one (how many: rule and figures at launch_sweeps, host).
+// From the last item to the end of the call 4 us; by one warp with sixteen regions and entries to a lane, one after the other,
+// 7.5.  Calls, one warp / 256 threads, normal logits, back to back in one run: 16 sequences, 5 tokens, 50 257 bf16 entries 25.1 / 19.3 us,
+// 16, 5, 65 536 20.8 / 18.4, 12, 4, 128 256 fp32 23.5 / 21.5, error feedback 64, 4, 151 936 bf16 51.2 / 49.2.  (Run once beforehand
+// by blocks that wait anyway, so that its instructions are there: slower, 52.6 for 51.2 as it was then.)
 template <int DT, int T>
 __device__ __noinline__ void sweep_draw(const Params& P, int unit, int lead) {
     using E = Elem<DT>;
