@@ -439,12 +439,14 @@ int launch_sweeps_of(const Params& P, const Sweep& S, long long units, bool all,
     const dim3 first = FINE ? dim3((unsigned)((units - S.fine_units) * S.slices + (long long)S.fine_units * S.fine_slices))
                             : dim3((unsigned)units, (unsigned)S.slices);
     SD_CUDA(launch_following(sd_sweep_stats_kernel<DT, RAGGED, FINE>, first, kSweepThreads, stream, P, S));
-    // With registers as the compiler takes them four blocks of the rows kernel fit an SM; a call with more sequences than
-    // that would have a second round of them and takes the kernel that is held to 40 (six).  Step, 49 / 40 registers, us: 800 sequences,
-    // 1 token, 8 192 bf16 entries 27.6 / 25.8, 700, 2, 8 192 32.6 / 30.8, 2000, 4, 504 64.5 / 63.1, 600, 1, 8 201 fp32 34.4 / 33.2, 700, 16, 1 000 bf16
-    // 72.8 / 70.8; with one round 500, 8, 2 048 31.8 / 32.7, 400, 4, 8 192 fp32 44.1 / 45.0.
-    SD_CUDA(P.B > 4 * sms ? launch_following(sd_sweep_rows_kernel<DT, true>, dim3((unsigned)P.B), rows_threads(P.k), stream, P, S)
-                          : launch_following(sd_sweep_rows_kernel<DT, false>, dim3((unsigned)P.B), rows_threads(P.k), stream, P, S));
+    // With registers as the compiler takes them (49, 56 of them to a thread) four blocks of eight warps of the rows kernel fit an SM, two
+    // of sixteen; a call with more sequences than that would have a second round of them and takes the kernel that is held to 40 (six and
+    // three).  Step, 49 / 40 registers, us: 800 sequences, 1 token, 8 192 bf16 entries 27.6 / 25.8, 700, 2, 8 192 32.6 / 30.8, 2000, 4, 504 64.5 /
+    // 63.1, 600, 1, 8 201 fp32 34.4 / 33.2, 320, 16, 1 000 bf16 36.7 / 35.6, 380, 16, 4 096 59.9 / 58.3, 400, 12, 2 048 fp32 40.1 / 38.8; with one round
+    // 500, 8, 2 048 bf16 31.8 / 32.7, 400, 4, 8 192 fp32 44.1 / 45.0.
+    const int resident = sms * (65536 / (rows_threads(P.k) * 56));
+    SD_CUDA(P.B > resident ? launch_following(sd_sweep_rows_kernel<DT, true>, dim3((unsigned)P.B), rows_threads(P.k), stream, P, S)
+                           : launch_following(sd_sweep_rows_kernel<DT, false>, dim3((unsigned)P.B), rows_threads(P.k), stream, P, S));
     // the rows that are drawn from, then (if anything of them is wanted) all pair rows; the hint error is summed by items of one
     // size, and the error feedback has nothing but the rows that are drawn from
     constexpr bool FINE2 = FINE && MODE == kSweepStepMode;
