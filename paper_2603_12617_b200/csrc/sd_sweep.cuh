@@ -779,10 +779,12 @@ sd_sweep_grad_kernel(const __grid_constant__ Params P, const __grid_constant__ S
         unit = b * (P.k + 1) + n;
         if (!SD_IN(unit, total_units<false>(P), 20)) return;
         rc = P.rowc[unit];
-    } else if (unit - b * (P.k + 1) == n) {
-        return;                                       // the first blocks have it
     }
-    const UnitRef ur = unit_ref<false>(P, unit);
+    const int i = unit - b * (P.k + 1);
+    if (!draws && i == n) return;                     // the first blocks have it
+    // (not from the unit: another division, on the way of every block)
+    const bool bonus = draws && n == P.k;
+    const UnitRef ur{b, i, 0, bonus, (size_t)unit, (size_t)b * P.k + (bonus ? 0 : i)};
     const int v0 = (slice * regions + warp) * kRegionVecs;
     float herr = 0.f;
     float* const rsum = P.region_sums + (size_t)unit * P.NR + slice * regions + warp;
