@@ -300,11 +300,11 @@ int launch_stream(DeviceState& d, const Params& P, int C, int G, int lag, cudaSt
 // sweeps are faster grows with the rows, up to about 180 of them; from there a call's entries decide.
 // The line was drawn with sweeps half as slow again as the present ones, and tests hold it there.  Calls back to back as the
 // kernels are now, element-wise / sweeps in us (4 tokens, i.e. 5 rows a sequence; * = calls to which the line gives the slower kernel):
-//     bf16  4 097 entries 80 rows 18.6 / 14.5 *, 320 25.2 / 16.1 *, 500 27.2 / 18.9;  8 201: 5 rows 21.6 / 13.7 *,
-//           100 21.8 / 15.6 *, 200 22.8 / 16.4 *, 320 32.7 / 18.7;  12 001: 20 rows 24.4 / 14.3, 145 24.3 / 16.9 *,
-//           200 28.0 / 17.0;  16 385: 145 28.2 / 16.8 *;  32 001: 5 rows 40.7 / 13.5, 320 116 / 29.9
-//     fp32  4 097: 5 rows 15.6 / 12.2 *, 180 15.9 / 14.3 *, 320 21.0 / 15.3 *, 640 28.8 / 17.9;  8 201: 40 rows 18.2 / 12.9,
-//           145 18.5 / 14.6 *, 320 27.4 / 17.4;  16 385: 145 rows 24.7 / 16.6 *, 320 47.5 / 23.1;  32 001: 5 rows 47.1 / 12.4
+//     bf16  4 097 entries 80 rows 18.4 / 14.1 *, 320 25.1 / 15.9 *, 500 27.1 / 18.8;  8 201: 5 rows 18.6 / 11.6 *,
+//           100 21.7 / 15.3 *, 200 22.7 / 16.0 *, 320 32.7 / 18.5;  12 001: 20 rows 24.4 / 13.0, 145 24.2 / 16.6 *,
+//           200 28.5 / 16.8;  16 385: 145 28.2 / 16.5 *;  32 001: 5 rows 38.2 / 12.2, 320 116 / 29.2
+//     fp32  4 097: 5 rows 14.5 / 10.4 *, 180 15.9 / 14.1 *, 320 21.0 / 15.2 *, 640 28.9 / 17.8;  8 201: 40 rows 18.1 / 12.6,
+//           145 18.6 / 14.4 *, 320 27.3 / 17.2;  16 385: 145 rows 23.9 / 16.4 *, 320 47.3 / 22.6;  32 001: 5 rows 45.4 / 10.8
 // So the sweeps would now do at every length and number of rows that they can take.
 bool use_ragged_sweeps(const void* D, const void* grad, const void* hint, long long units, int V, int dtype) {
     const int vec = vec_elems(dtype);
@@ -380,12 +380,12 @@ bool held_room(const WorkspaceLayout& L) { return L.slices > 0 || L.NRmax * size
 // back to back on inputs from HBM:
 //     1 sequence, 4 tokens, 32 000 fp32 16.6 / - / 8.8;  8, 5, 32 000 bf16 23.0 / - / 10.9;  1, 4, 128 256 bf16
 //     20.6 / - / 12.6, in clusters of 16 with one region a warp 14.8;  3, 2, 152 064 fp32 22.9 / - / 13.2;
-//     15 rows of 128 256 fp32 - / 16.5 / 12.8;  33 of 128 256 bf16 - / 18.5 / 16.0;  147 of 32 000 bf16 - / 18.8 / 16.4
+//     15 rows of 128 256 fp32 - / 16.6 / 12.8;  33 of 128 256 bf16 - / 18.2 / 16.1;  147 of 32 000 bf16 - / 18.6 / 16.4
 // Of clusters whose size is no power of two, one fewer than the device says is resident has its SMs at once: 45 rows of
 // 65 536 bf16 (clusters of 3, all of them resident by that count) 19.3, 42 rows 14.4; 12 of 152 064 fp32
 // (clusters of 10) 19.2, 9 rows 12.6.
 // A second round costs as much as the first.  Where there are sweeps they are faster then (42 rows of 100 000 bf16 23.7,
-// sweeps 18.8; 48 of 128 256 27.7 and 18.7); the cluster kernel is not (35.0).  `second`: two rounds are allowed.
+// sweeps 18.4; 48 of 128 256 27.7 and 18.4); the cluster kernel is not (35.0).  `second`: two rounds are allowed.
 // Options that only the cluster kernel has, off their defaults, choose the cluster kernel.
 bool use_held(DeviceState& d, int V, long long units, int dtype, bool second, HeldShape* h) {
     if (option(SD_OPT_CLUSTER) != 0 || option(SD_OPT_LAG) != -1 || option(SD_OPT_PREFETCH) != 0 ||
@@ -612,9 +612,9 @@ int choose_stream(DeviceState& d, int V, long long units, int dtype, int* G_out,
 //           24 000: 256 MB (10) 101 / 100, 307 MB (12) 116 / 119;  20 000: 191 MB (9) 81.6 / 79.3, 213 MB (10) 85.5 / 87.8;
 //           16 384 and below: faster at every size, 440 MB 179 / 170 (the cluster kernel's stages fit such rows badly)
 // The smallest calls go to sd_held_kernel first (use_held); of the others the sweeps are the faster ones however small
-// they are (us, cluster kernel / sweeps as they are now): 100 sequences, 2 tokens, 8 192 bf16 entries, 8 MB 19.6 / 15.5;
-// 64, 8, 1 000 fp32, 4 MB 23.1 / 14.2; 64, 4, 8 192 fp32, 19 MB 24.0 / 16.4; 8, 5, 128 256 bf16, 23 MB 35.0 / 18.9;
-// 16, 5, 50 304 fp32, 35 MB 28.2 / 20.0; 8, 5, 128 256 fp32, 45 MB 35.4 / 22.4.
+// they are (us, cluster kernel / sweeps as they are now): 100 sequences, 2 tokens, 8 192 bf16 entries, 8 MB 19.6 / 15.3;
+// 64, 8, 1 000 fp32, 4 MB 23.1 / 14.2; 64, 4, 8 192 fp32, 19 MB 24.0 / 16.4; 8, 5, 128 256 bf16, 23 MB 35.0 / 18.6;
+// 16, 5, 50 304 fp32, 35 MB 28.2 / 19.8; 8, 5, 128 256 fp32, 45 MB 35.4 / 22.4.
 // Options that only the cluster kernel has, off their defaults, choose the cluster kernel.
 // (Nor can the second sweep have more blocks than a grid: a billion rows of one vector.)
 bool use_sweeps(DeviceState& d, int dtype, double bytes, long long units, int V, int slices) {

@@ -19,10 +19,10 @@
 // sd_stream_kernel reads every logit from HBM once, but its 28 consumer warps share one ring and all blocks
 // read at the same time and compute at the same time, so at bf16, where the exponentials take as long as
 // the reads, it moves 2.9 TB/s.  Step on 32 sequences, 8 draft tokens, 128 256 bf16 entries: 71.1 us there,
-// 56.1 us here; 64 sequences, 4 tokens, 151 936: 93.4 and 69.7 us; 8, 5, 128 256: 35.0 and 18.9.  Of the 57.4 us that the first
+// 56.1 us here; 64 sequences, 4 tokens, 151 936: 93.4 and 69.2 us; 8, 5, 128 256: 35.0 and 18.6.  Of the 57.4 us that the first
 // of these took with items of one size, clock stamps of every block: first sweep 29.5, the last 8 with fewer and fewer
 // blocks; 4.5 until the second sweep works, 2 of them in the rows kernel; second sweep 24.  16 sequences, 5 tokens, 65 536 bf16
-// entries, when it took 19.6 us (18.4 now): 8, 4, 5, and 4 for the draws.
+// entries, when it took 19.6 us (18.2 now): 8, 4, 5, and 4 for the draws.
 // The rule which of the two a call takes is use_sweeps (host).
 //
 // Tried and dropped, on the first of these: one persistent kernel whose warps take both passes of an item
@@ -115,8 +115,8 @@ __device__ __forceinline__ PartialStats load_partial_cg(const PartialStats* p) {
 // Regions at the ends of a row, where a vector would reach into another row or out of the tensor, are read
 // and written entry by entry, out of line and with registers of their own: with one set for both, filled by a
 // function for the ends, every region went through local memory (13 sequences, 8 tokens, 110 593 fp32 entries 67.3 us,
-// 41 since; 122, 4, 119 177 302 and 202; 64, 4, 100 001 bf16 84.9 and 61).  16 sequences, 5 tokens, 50 257 bf16
-// entries: 19.4 us, against 91.6 us for the element-wise kernel, whose one block per row reads two bytes a lane.
+// 40 since; 122, 4, 119 177 302 and 200; 64, 4, 100 001 bf16 84.9 and 60).  16 sequences, 5 tokens, 50 257 bf16
+// entries: 19.3 us, against 91.6 us for the element-wise kernel, whose one block per row reads two bytes a lane.
 template <int DT> struct RowFrame {
     const typename Elem<DT>::type *rowT, *rowD;
     const uint4 *T16, *D16;      // vector 0 of the regions, aligned: up to a vector before the row
@@ -782,7 +782,7 @@ sd_sweep_grad_kernel(const __grid_constant__ Params P, const __grid_constant__ S
     }
     const int i = unit - b * (P.k + 1);
     if (!draws && i == n) return;                     // the first blocks have it
-    // (not from the unit: another division, on the way of every block)
+    // (not from the unit: another division, on the way of every block; 450 sequences, 16 tokens, 1 000 bf16 entries 48.0 -> 45.2 us)
     const bool bonus = draws && n == P.k;
     const UnitRef ur{b, i, 0, bonus, (size_t)unit, (size_t)b * P.k + (bonus ? 0 : i)};
     const int v0 = (slice * regions + warp) * kRegionVecs;
