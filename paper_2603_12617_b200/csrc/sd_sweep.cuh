@@ -19,7 +19,7 @@
 // sd_stream_kernel reads every logit from HBM once, but its 28 consumer warps share one ring and all blocks
 // read at the same time and compute at the same time, so at bf16, where the exponentials take as long as
 // the reads, it moves 2.9 TB/s.  Step on 32 sequences, 8 draft tokens, 128 256 bf16 entries: 71.1 us there,
-// 56.1 us here; 64 sequences, 4 tokens, 151 936: 93.4 and 69.2 us; 8, 5, 128 256: 35.0 and 18.6.  Of the 57.4 us that the first
+// 55.6 us here; 64 sequences, 4 tokens, 151 936: 93.4 and 69.0 us; 8, 5, 128 256: 35.0 and 18.6.  Of the 57.4 us that the first
 // of these took with items of one size, clock stamps of every block: first sweep 29.5, the last 8 with fewer and fewer
 // blocks; 4.5 until the second sweep works, 2 of them in the rows kernel; second sweep 24.  16 sequences, 5 tokens, 65 536 bf16
 // entries, when it took 19.6 us (18.2 now): 8, 4, 5, and 4 for the draws.
